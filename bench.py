@@ -289,8 +289,8 @@ def kernel_bytes(stats: dict, kid: int, sort_passes: int) -> float:
 
 
 KERNEL_NAMES = {1: "k_get (probe + row gather)", 2: "k_probe", 3: "k_sort_scatter",
-                4: "k_short (run sum + Adagrad)", 5: "k_long_sum (chunk sums of long runs)",
-                6: "k_heads (runs found in the sorted ids)", 7: "k_long_combine (chunk sums + Adagrad)",
+                4: "k_short (run sum + Adagrad)", 5: "k_long (chunk sums of long runs)",
+                6: "k_heads (runs found in the sorted ids)", 7: "k_combine (chunk sums + Adagrad)",
                 8: "k_tier_fetch (host <-> HBM row swap)", 9: "k_put_scatter (Put: last occurrence writes)",
                 10: "k_single (runs of one lookup + Adagrad)", 11: "k_small (runs of 2-4 lookups + Adagrad)"}
 KERNEL_SOURCES = {1: "mlkv_index.cu", 2: "mlkv_index.cu", 3: "mlkv_sort.cu", 4: "mlkv_apply.cu",
@@ -300,7 +300,7 @@ KERNEL_SOURCES = {1: "mlkv_index.cu", 2: "mlkv_index.cu", 3: "mlkv_sort.cu", 4: 
 
 # ncu kernel names (demangled, without the namespace) -> kernel class
 KERNEL_PATTERNS = [("k_get_bulk<", 1), ("k_get<", 1), ("k_probe<", 2), ("k_sort_scatter", 3), ("k_short<", 4),
-                   ("k_long_sum<", 5), ("k_heads", 6), ("k_long_combine<", 7), ("k_tier_fetch", 8),
+                   ("k_long<", 5), ("k_heads", 6), ("k_combine<", 7), ("k_tier_fetch", 8),
                    ("k_put_scatter", 9), ("k_single<", 10), ("k_small<", 11)]
 TRAFFIC_PATH = os.path.join(ROOT, "profiles", "traffic.json")
 

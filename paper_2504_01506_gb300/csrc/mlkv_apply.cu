@@ -16,34 +16,40 @@
 //                 per block and list; any order: every run is summed on its
 //                 own), longer ones are measured (a warp-wide search for their
 //                 end) and listed for k_long_*.
-//  k_single       one lane group per run of one lookup: row, state and the
-//                 gradient row loaded together, then the Adagrad step.
-//  k_small        one lane group per run of 2 .. kSmallRun lookups, whose
-//                 positions k_heads wrote into the run's record: row, state and
-//                 every gradient row in one round trip, the occurrence-order
-//                 sum, then the Adagrad step.
-//  k_short        one lane group per run of kSmallRun + 1 ..
-//                 MLKV_SEQ_SEGMENT_MAX lookups: the row, the state, the first
-//                 gradient row and the run's other positions are loaded
-//                 together, the rest summed in occurrence order, then the
-//                 Adagrad step.
-//  k_long_sum     one lane group per chunk of 64 lookups (16 in calls of
-//                 fewer than 2^19 lookups) of a long run
+//  k_single       runs of one lookup: row, state and the gradient row loaded
+//                 together, then the Adagrad step.
+//  k_small        runs of 2 .. kSmallRun lookups, whose positions k_heads wrote
+//                 into the run's record: row, state and every gradient row in
+//                 one round trip, the occurrence-order sum, the Adagrad step.
+//  k_short        runs of kSmallRun + 1 .. MLKV_SEQ_SEGMENT_MAX lookups: row,
+//                 state, first gradient row and the run's other positions
+//                 loaded together, the rest summed in occurrence order, then
+//                 the Adagrad step.
+//  k_long         chunks of 64 lookups (16 in calls of fewer than 2^19 lookups,
+//                 but 64 there too for runs of more than 4,096) of a long run
 //                 (Zipf-hot keys reach 10^4-10^5 lookups): the chunk's sum,
 //                 compensated, to scratch as a (sum, compensation) pair.
-//  k_long_combine per long run: the chunk pairs added in a fixed order with
-//                 compensation (split over a whole block's lane groups for the
-//                 runs of many chunks, one lane group for the others), the sum
-//                 rounded once, and the row updated.
+//  k_combine      per long run: the chunk pairs added in a fixed order with
+//                 compensation, the sum rounded once, and the row updated.
+//
+// The row kernels' unit of work is one segment of a run: a lane group (G
+// lanes, the power of two that holds a row of up to 32 vectors) reduces G
+// vectors of the row at a time, and a wider row is nseg units.  Every operation
+// is element-wise, so the segments are independent, and a segment takes the
+// registers of a narrow row.  (With a wide row's vectors all held by one lane
+// group, 4 a lane at dim 512, k_single spilled at its 40 registers and took
+// 172 us for 65,536 lookups, Zipf(0.8), of dim 512; by segments it takes 67,
+// and the apply + Get 190 us instead of 319.)
+//
 // Long runs are summed with compensation because the Adagrad step is
 // ill-conditioned where a summed gradient element lands near eps (with zero
 // state, u = lr * g / (|g| + eps) changes fast in g there): a plain fp32 sum
 // of 10^2-10^4 terms can then move the update by more than 1e-5, while the
 // compensated sum stays within about one rounding of the exact sum.
-// Each is tuned for requests in flight (resident warps against rows in flight
-// per warp): the access pattern is random 512-byte rows, which HBM serves near
-// its copy bandwidth only with many requests in flight.  Results do not depend
-// on scheduling.
+// Each kernel is tuned for requests in flight (resident warps against rows in
+// flight per warp): the access pattern is random 512-byte rows, which HBM
+// serves near its copy bandwidth only with many requests in flight.  Results do
+// not depend on scheduling.
 #include <algorithm>
 
 #include "mlkv_internal.cuh"
@@ -62,70 +68,51 @@ namespace {
 #define MLKV_CHUNK_SMALL 16
 #endif
 constexpr uint32_t kChunkLarge = 64, kChunkSmall = MLKV_CHUNK_SMALL, kSmallBatch = MLKV_SMALL_BATCH;
-// Long runs of more than `big` chunk sums (the hottest rows) are combined by a
-// whole block of k_long_combine (MLKV_COMBINE_THREADS); the rest by one lane
-// group each.
-// In calls of at least kSmallBatch lookups, big = kBigRunLarge (many long
-// runs: lane groups keep the SMs busy); below, kBigRunSmall (few long runs:
-// blocks sum their chunks in parallel).
-constexpr uint32_t kBigRunLarge = 32, kBigRunSmall = 4;
+// In a small call a run of more small chunks than this is cut into large ones:
+// up to here a block combines them in one node.  (At 64, a knowledge-graph step
+// of 200k lookups lost 7 us in k_long: its runs of some thousand lookups were
+// cut into too few chunks to fill the GPU.)
+constexpr uint32_t kFewChunks = 256;
 
-// Tuning (set at build time): gradient rows in flight per lane group, and the
-// minimum resident blocks per SM the register allocation must allow.
-#ifndef MLKV_REDUCE_ROWS_IN_FLIGHT
-#define MLKV_REDUCE_ROWS_IN_FLIGHT 8
+// Lookups per chunk of a long run of len lookups (`chunk`: the call's).
+__device__ __forceinline__ uint32_t run_chunk(uint32_t len, uint32_t chunk) {
+    return len > chunk * kFewChunks ? kChunkLarge : chunk;
+}
+#ifndef MLKV_GROUP_CHUNKS
+#define MLKV_GROUP_CHUNKS 16
+#endif
+#ifndef MLKV_NODE
+#define MLKV_NODE 256
+#endif
+constexpr uint32_t NONE = 0xFFFFFFFFu;  // no position (a small run's record past its end)
+// k_combine: a lane group adds up the chunk sums of a run of at most
+// kGroupChunks chunks; of longer runs, a block takes kNode chunks at a time.
+constexpr uint32_t kGroupChunks = MLKV_GROUP_CHUNKS, kNode = MLKV_NODE;
+
+// Tuning (set at build time): gradient rows in flight per lane group in a long
+// chunk and in a run of 5-32 lookups, and the resident blocks per SM the
+// register allocations must allow.
+#ifndef MLKV_LONG_ROWS
+#define MLKV_LONG_ROWS 8
+#endif
+#ifndef MLKV_SHORT_ROWS
+#define MLKV_SHORT_ROWS 8
+#endif
+#ifndef MLKV_LONG_MIN_BLOCKS
+#define MLKV_LONG_MIN_BLOCKS 2
 #endif
 #ifndef MLKV_SHORT_MIN_BLOCKS
 #define MLKV_SHORT_MIN_BLOCKS 2
 #endif
-// k_short: runs a lane group claims at a time.
-#ifndef MLKV_SHORT_GRAB
-#define MLKV_SHORT_GRAB 4
-#endif
-// k_single: runs of one lookup in flight per lane group, and blocks per SM.
-#ifndef MLKV_SINGLES
-#define MLKV_SINGLES 1
+#ifndef MLKV_SMALL_MIN_BLOCKS
+#define MLKV_SMALL_MIN_BLOCKS 4
 #endif
 #ifndef MLKV_SINGLE_MIN_BLOCKS
 #define MLKV_SINGLE_MIN_BLOCKS 6
 #endif
-// The apply's reduce kernels on three streams (0: one after the other).
-#ifndef MLKV_REDUCE_BRANCHES
-#define MLKV_REDUCE_BRANCHES 1
-#endif
-// Narrow rows (a row on at most 16 lanes: dim <= 64): runs of one lookup two
-// at a time per lane group on at most 3 blocks per SM, runs of 5-32 lookups
-// with 4 gradient rows in flight at 3 blocks per SM (more warps); 0: the
-// wide rows' kernels for every dim.
-#ifndef MLKV_NARROW_ROWS
-#define MLKV_NARROW_ROWS 1
-#endif
-// k_single on at most this many blocks per SM (0: as many as fit).
-#ifndef MLKV_SINGLE_PER_SM
-#define MLKV_SINGLE_PER_SM 0
-#endif
-// Launch order of the reduce kernels.  MLKV_SHORT_FIRST: the runs of 5-32 launched before those of 2-4 (0: never,
-// 1: always, 2: in calls of fewer than kSmallBatch lookups).
-#ifndef MLKV_SHORT_FIRST
-#define MLKV_SHORT_FIRST 2
-#endif
-// k_long_combine's block (a big run's chunks are split over its lane groups):
-// 256 threads fit the slots that retiring blocks of the other reduce kernels
-// free, where a 1024-thread block waited for a whole SM to drain (DLRM: the
-// combine started 70 us after its chunk sums were done).
-#ifndef MLKV_COMBINE_THREADS
-#define MLKV_COMBINE_THREADS 256
-#endif
-// k_small: blocks per SM the register allocation must allow.
-#ifndef MLKV_SMALL_MIN_BLOCKS
-#define MLKV_SMALL_MIN_BLOCKS 4
-#endif
-constexpr uint32_t NONE = 0xFFFFFFFFu;  // no position (a small run's record past its end)
-#ifndef MLKV_LONG_ROWS_IN_FLIGHT
-#define MLKV_LONG_ROWS_IN_FLIGHT 8
-#endif
-#ifndef MLKV_LONG_MIN_BLOCKS
-#define MLKV_LONG_MIN_BLOCKS 2
+// k_short: runs a lane group claims at a time.
+#ifndef MLKV_SHORT_GRAB
+#define MLKV_SHORT_GRAB 4
 #endif
 
 struct RowArgs {
@@ -134,15 +121,20 @@ struct RowArgs {
     int dpad;
     int NV;
     int G;
+    int gshift;      // log2 of G
     int d;
+    uint32_t nseg;   // segments of G vectors per row: a lane group reduces one segment of a run at a time
     uint32_t nrows;  // rows of the slot array (bounds-checked build)
 };
 
 // Sites of the bounds-checked build (in_bounds).
 enum CheckSite : uint32_t {
     kChkSingleRow = 1, kChkSinglePos, kChkSmallRow, kChkSmallPos, kChkShortRun, kChkShortRow, kChkShortPos,
-    kChkLongItem, kChkLongPos, kChkCombineRun, kChkCombineRow, kChkHeadsPos, kChkListEntry
+    kChkLongItem, kChkLongPos, kChkLongRow, kChkHeadsPos, kChkListEntry
 };
+
+constexpr uint32_t kItemLenBits = 7;  // a chunk holds at most 64 lookups; a run at most 2^24 chunks of 64
+static_assert(kChunkLarge < (1u << kItemLenBits) && kChunkSmall < (1u << kItemLenBits), "chunk lengths fit their bits");
 
 struct RunArgs {
     const float* grads;
@@ -157,18 +149,17 @@ struct RunArgs {
     uint4* smalls;         // [max_batch] runs of 2 .. kSmallRun lookups: (row, p0, p1, p2), positions in
                            //   occurrence order, NONE past the run's end
     uint32_t* small_p3;    // [max_batch] their fourth position (or NONE)
-    uint32_t* long_s;      // [max_long] first sorted position
-    uint32_t* long_e;      // [max_long] one past the last
-    uint32_t* long_row;    // [max_long]
-    uint32_t* long_base;   // [max_long] first chunk item
-    uint32_t* item_s;      // [max_items] first sorted position of each chunk
-    uint32_t* item_e;      // [max_items] one past its last
-    uint32_t* big_runs;    // [max_long] long runs of more than `big` chunks
-    float* partial;        // [max_items][dpad]
+    uint4* long_runs;      // [max_long] long runs of at most kGroupChunks chunks: (first chunk, chunks, row, -)
+    uint4* nodes;          // [max_nodes] kNode chunks each of the longer runs: (the run's first chunk, its chunks,
+                           //   row, node of the run)
+    uint4* items;          // [max_items] chunks of the long runs: (first sorted position, lookups |
+                           //   chunks of the run << kItemLenBits, row, the run's first chunk)
+    float* partial;        // [max_items][2][dpad] sums of chunks, and of nodes in their first chunk's place
+    uint32_t* node_cnt;    // [max_items][nseg] nodes of a run done (at its first chunk's entry), zero at rest
     uint32_t max_long;
+    uint32_t max_nodes;
     uint32_t max_items;
     uint32_t chunk;        // lookups per chunk of a long run (kChunkLarge or kChunkSmall)
-    uint32_t big;          // long runs of more chunks than this are combined by a whole block
     ErrSink err;
     float lr, eps;
     uint32_t release;      // non-zero in the apply's last kernels: the blocks of all of them (release_counters)
@@ -178,84 +169,68 @@ __device__ __forceinline__ unsigned group_mask(int G, int gid) {
     return G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (gid * G));
 }
 
-// acc += the gradient rows of sorted positions s .. s+len-1, in that order.
-// The group loads up to G positions at a time (one per lane) and hands them
-// round with group shuffles.  With PRE the first G positions were loaded by
-// the caller (pl_first, one per lane).  With COMP every addition is
-// compensated (comp_add): acc + cmp is then the sum to about twice fp32's
-// precision; without it cmp is not touched.
-template <int V, int KV, int ROWS = MLKV_REDUCE_ROWS_IN_FLIGHT, bool PRE = false, bool COMP = false>
-__device__ __forceinline__ void sum_rows(typename Vec<V>::T (&acc)[KV], typename Vec<V>::T (&cmp)[KV],
-                                         const float* __restrict__ grads,
-                                         const uint32_t* __restrict__ spos, uint32_t s, uint32_t len, int d,
-                                         int NV, int G, int glane, unsigned gmask, const ErrSink& err,
-                                         uint32_t site, uint32_t n, uint32_t pl_first = 0u) {
+// acc += the gradient vectors (this lane's column j, live when j < NV) of
+// sorted positions s .. s+len-1, in that order, ROWS in flight.  The group
+// loads up to G positions at a time (one per lane) and hands them round with
+// group shuffles.  With PRE the first G positions were loaded by the caller
+// (pl_first, one per lane).  With COMP every addition is compensated
+// (comp_add): acc + cmp is then the sum to about twice fp32's precision;
+// without it cmp is not touched.
+template <int V, int ROWS, bool PRE, bool COMP>
+__device__ __forceinline__ void sum_rows(typename Vec<V>::T& acc, typename Vec<V>::T& cmp,
+                                         const float* __restrict__ grads, const uint32_t* __restrict__ spos,
+                                         uint32_t s, uint32_t len, int d, int j, bool act, int G, int glane,
+                                         unsigned gmask, const ErrSink& err, uint32_t site, uint32_t n,
+                                         uint32_t pl_first = 0u) {
     using VT = typename Vec<V>::T;
-    constexpr int UNR = KV >= ROWS ? 1 : ROWS / KV;
     for (uint32_t base = 0; base < len; base += G) {
         const uint32_t cnt = min((uint32_t)G, len - base);
         if (MLKV_CHECK && !in_bounds(err, site, s + base + cnt - 1, n)) return;
         const uint32_t pl = (PRE && base == 0) ? pl_first
                             : (uint32_t)glane < cnt ? __ldg(spos + s + base + glane) : 0u;
-        for (uint32_t x = 0; x < cnt; x += UNR) {
-            VT g[UNR][KV];
+        for (uint32_t x = 0; x < cnt; x += ROWS) {
+            VT g[ROWS];
 #pragma unroll
-            for (int u = 0; u < UNR; ++u) {
+            for (int u = 0; u < ROWS; ++u) {
                 uint32_t p = __shfl_sync(gmask, pl, (int)(x + u) & (G - 1), G);
                 if (MLKV_CHECK && x + u < cnt && !in_bounds(err, site, p, n)) p = 0;
-                const VT* src = reinterpret_cast<const VT*>(grads + (size_t)p * d);
-#pragma unroll
-                for (int k = 0; k < KV; ++k) {
-                    const int j = glane + G * k;
-                    if (x + u < cnt && j < NV) g[u][k] = __ldcs(src + j);
-                }
+                if (x + u < cnt && act) g[u] = __ldcs(reinterpret_cast<const VT*>(grads + (size_t)p * d) + j);
             }
 #pragma unroll
-            for (int u = 0; u < UNR; ++u)
-#pragma unroll
-                for (int k = 0; k < KV; ++k)
-                    if (x + u < cnt && glane + G * k < NV) {
-                        if (COMP) Vec<V>::cadd(acc[k], cmp[k], g[u][k]);
-                        else Vec<V>::add(acc[k], g[u][k]);
-                    }
+            for (int u = 0; u < ROWS; ++u)
+                if (x + u < cnt && act) {
+                    if (COMP) Vec<V>::cadd(acc, cmp, g[u]);
+                    else Vec<V>::add(acc, g[u]);
+                }
         }
     }
 }
 
-template <int V, int KV>
-__device__ __forceinline__ void load_row_state(const RowArgs& ra, uint32_t row, typename Vec<V>::T (&w)[KV],
-                                               typename Vec<V>::T (&G)[KV], int glane) {
-    using VT = typename Vec<V>::T;
-    const float* slot = ra.slots + (size_t)row * ra.stride;
-    const VT* wv = reinterpret_cast<const VT*>(slot);
-    const VT* gv = reinterpret_cast<const VT*>(slot + ra.dpad);
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-        const int j = glane + ra.G * k;
-        if (j < ra.NV) {
-            w[k] = wv[j];
-            G[k] = gv[j];
-        }
-    }
+// This lane's vectors (column j) of a row and of its state.
+template <int V>
+__device__ __forceinline__ typename Vec<V>::T* row_vec(const RowArgs& ra, uint32_t row, int j) {
+    return reinterpret_cast<typename Vec<V>::T*>(ra.slots + (size_t)row * ra.stride) + j;
 }
 
-template <int V, int KV>
-__device__ __forceinline__ void adagrad_store(const RowArgs& ra, uint32_t row, typename Vec<V>::T (&w)[KV],
-                                              typename Vec<V>::T (&G)[KV], const typename Vec<V>::T (&g)[KV],
-                                              int glane, float lr, float eps) {
-    using VT = typename Vec<V>::T;
-    float* slot = ra.slots + (size_t)row * ra.stride;
-    VT* wv = reinterpret_cast<VT*>(slot);
-    VT* gv = reinterpret_cast<VT*>(slot + ra.dpad);
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-        const int j = glane + ra.G * k;
-        if (j < ra.NV) {
-            Vec<V>::adagrad(w[k], G[k], g[k], lr, eps);
-            wv[j] = w[k];
-            gv[j] = G[k];
-        }
-    }
+// The state's (or a pair's compensation's) vector beside p.
+template <class VT>
+__device__ __forceinline__ VT* beside(const RowArgs& ra, VT* p) {
+    return reinterpret_cast<VT*>(reinterpret_cast<float*>(p) + ra.dpad);
+}
+template <class VT>
+__device__ __forceinline__ const VT* beside(const RowArgs& ra, const VT* p) {
+    return reinterpret_cast<const VT*>(reinterpret_cast<const float*>(p) + ra.dpad);
+}
+
+// The Adagrad step on loaded row and state vectors, and their stores.
+template <int V>
+__device__ __forceinline__ void adagrad_store(const RowArgs& ra, uint32_t row, int j, typename Vec<V>::T w,
+                                              typename Vec<V>::T G, const typename Vec<V>::T& g, float lr,
+                                              float eps) {
+    typename Vec<V>::T* p = row_vec<V>(ra, row, j);
+    Vec<V>::adagrad(w, G, g, lr, eps);
+    *p = w;
+    *beside(ra, p) = G;
 }
 
 // Where the run of `row` that starts at sorted position s ends: the first
@@ -315,76 +290,56 @@ __device__ __forceinline__ uint32_t scan_end(const uint32_t* __restrict__ srow, 
     return run_end(srow, n, q0 + 1023u, row, lane);
 }
 
-// Chunks of `chunk` lookups of the long runs qs[k] .. qe[k] (k < nq): this
-// lane's run's count, and the exclusive prefix over the lanes (the whole warp).
-__device__ __forceinline__ uint32_t long_chunks(const uint32_t* qs, const uint32_t* qe, int nq, int lane,
-                                                uint32_t chunk, uint32_t& excl) {
-    const uint32_t nit = lane < nq ? (qe[lane] - qs[lane] + chunk - 1) / chunk : 0u;
-    uint32_t x = nit;
+// What the long runs qs[k] .. qe[k] (k < nq) add to the lists: chunks, runs
+// combined by a lane group, and nodes.
+struct LongCounts {
+    uint32_t items, runs, nodes;
+};
+
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t x, int lane) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    excl = x - nit;
-    return __shfl_sync(0xffffffffu, x, 31);  // all the runs' chunks
+    return x;
 }
 
-// Writes the long runs qs[k], qe[k], qr[k] (k < nq: start, end, row) at list
-// entries h0.. and their chunks at items ib0.. for k_long_sum / k_long_combine
+// This lane's run's counts, their exclusive prefix over the lanes, and the sums
 // (the whole warp).
-__device__ __forceinline__ void write_long_runs(const RunArgs& a, const uint32_t* qs, const uint32_t* qe,
-                                                const uint32_t* qr, int nq, uint32_t h0, uint32_t ib0,
-                                                int lane) {
-    uint32_t excl;
-    const uint32_t chunk = a.chunk;
-    long_chunks(qs, qe, nq, lane, chunk, excl);
-    if (lane < nq) {
-        a.long_s[h0 + lane] = qs[lane];
-        a.long_e[h0 + lane] = qe[lane];
-        a.long_row[h0 + lane] = qr[lane];
-        a.long_base[h0 + lane] = ib0 + excl;
-        if ((qe[lane] - qs[lane] + chunk - 1) / chunk > a.big) a.big_runs[atomicAdd(&a.cur->n_big, 1u)] = h0 + lane;
-    }
-    for (int k = 0; k < nq; ++k) {
-        const uint32_t s = qs[k], e = qe[k];
-        const uint32_t m = (e - s + chunk - 1) / chunk;
-        const uint32_t ib = ib0 + __shfl_sync(0xffffffffu, excl, k);
-        for (uint32_t c = lane; c < m; c += 32) {
-            a.item_s[ib + c] = s + c * chunk;
-            a.item_e[ib + c] = min(s + (c + 1) * chunk, e);
-        }
-    }
+__device__ __forceinline__ LongCounts long_counts(const uint32_t* qs, const uint32_t* qe, int nq, int lane,
+                                                  uint32_t chunk, LongCounts& mine, LongCounts& excl) {
+    const uint32_t len = lane < nq ? qe[lane] - qs[lane] : 0u;
+    const uint32_t c = run_chunk(len, chunk);
+    mine.items = (len + c - 1) / c;
+    mine.runs = lane < nq && mine.items <= kGroupChunks;
+    mine.nodes = mine.items > kGroupChunks ? (mine.items + kNode - 1) / kNode : 0u;
+    const LongCounts in = {warp_inclusive(mine.items, lane), warp_inclusive(mine.runs, lane),
+                           warp_inclusive(mine.nodes, lane)};
+    excl = {in.items - mine.items, in.runs - mine.runs, in.nodes - mine.nodes};
+    return {__shfl_sync(0xffffffffu, in.items, 31), __shfl_sync(0xffffffffu, in.runs, 31),
+            __shfl_sync(0xffffffffu, in.nodes, 31)};
 }
 
-// One short run [s, s + len) of `row`, first lookup p0, by one lane group: the
-// row, the state and the first gradient row are loaded together, the rest of
-// the gradient rows are added in occurrence order, then the Adagrad step.
-template <int V, int KV, int ROWS = MLKV_REDUCE_ROWS_IN_FLIGHT>
-__device__ __forceinline__ void short_run(const RowArgs& ra, const RunArgs& a, uint32_t s, uint32_t len,
-                                          uint32_t row, uint32_t p0, int glane, unsigned gmask) {
-    using VT = typename Vec<V>::T;
-    if (MLKV_CHECK && !(in_bounds(a.err, kChkShortRun, s + len, (unsigned long long)a.n + 1) &&
-                        in_bounds(a.err, kChkShortRun, 1, len) && in_bounds(a.err, kChkShortRow, row, ra.nrows) &&
-                        in_bounds(a.err, kChkShortPos, p0, a.n)))
-        return;
-    VT w[KV], Gs[KV], acc[KV];
-    // the positions of the run's other lookups load beside its row, state and
-    // first gradient row, so a run of a few lookups costs two round trips
-    const uint32_t rest = len - 1;
-    const uint32_t pl0 = (uint32_t)glane < min(rest, (uint32_t)ra.G) ? __ldg(a.spos + s + 1 + glane) : 0u;
-    load_row_state<V, KV>(ra, row, w, Gs, glane);
-    const VT* g0 = reinterpret_cast<const VT*>(a.grads + (size_t)p0 * ra.d);
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-        acc[k] = Vec<V>::zero();
-        const int j = glane + ra.G * k;
-        if (j < ra.NV) Vec<V>::add(acc[k], __ldcs(g0 + j));  // 0 + g: first term, in order
+// Writes the chunks of the long runs qs[k], qe[k], qr[k] (k < nq: start, end,
+// row) and their runs or nodes at list entries base.. (the whole warp).
+__device__ __forceinline__ void write_long_runs(const RunArgs& a, const uint32_t* qs, const uint32_t* qe,
+                                                const uint32_t* qr, int nq, const LongCounts& base, int lane) {
+    LongCounts mine, excl;
+    long_counts(qs, qe, nq, lane, a.chunk, mine, excl);
+    if (mine.runs) a.long_runs[base.runs + excl.runs] = make_uint4(base.items + excl.items, mine.items, qr[lane], 0u);
+    for (int k = 0; k < nq; ++k) {
+        const uint32_t s = qs[k], e = qe[k], row = qr[k], chunk = run_chunk(e - s, a.chunk);
+        const uint32_t m = __shfl_sync(0xffffffffu, mine.items, k);
+        const uint32_t ib = base.items + __shfl_sync(0xffffffffu, excl.items, k);
+        const uint32_t nodes = __shfl_sync(0xffffffffu, mine.nodes, k);
+        const uint32_t nb = base.nodes + __shfl_sync(0xffffffffu, excl.nodes, k);
+        for (uint32_t c = lane; c < m; c += 32) {
+            const uint32_t cs = s + c * chunk;
+            a.items[ib + c] = make_uint4(cs, min(chunk, e - cs) | m << kItemLenBits, row, ib);
+        }
+        for (uint32_t c = lane; c < nodes; c += 32) a.nodes[nb + c] = make_uint4(ib, m, row, c);
     }
-    if (len > 1)
-        sum_rows<V, KV, ROWS, true>(acc, acc, a.grads, a.spos, s + 1, rest, ra.d, ra.NV,
-                                                          ra.G, glane, gmask, a.err, kChkShortPos, a.n, pl0);
-    adagrad_store<V, KV>(ra, row, w, Gs, acc, glane, a.lr, a.eps);
 }
 
 // A warp per window of 32 sorted positions (windows dealt out grid-stride).
@@ -393,10 +348,9 @@ __device__ __forceinline__ void short_run(const RowArgs& ra, const RunArgs& a, u
 // that sort last) or, for the window's last run, where the next window's row
 // ids first differ (past that, it is long and its end is searched for after
 // the windows).  Runs of one lookup and the other runs of <=
-// MLKV_SEQ_SEGMENT_MAX lookups are staged in the warp's two shared-memory
-// lists, long ones in its queue; at the end the block reserves room in the
-// two run lists, the long-run list and the chunk list with one atomic each and
-// the warps copy their runs out.  (Counters that every warp bumps queue up at
+// MLKV_SEQ_SEGMENT_MAX lookups are staged in the warp's shared-memory lists,
+// long ones in its queue; at the end the block reserves room in the run lists
+// and the chunk list with one atomic each and the warps copy their runs out.  (Counters that every warp bumps queue up at
 // the end of the kernel.)
 #ifndef MLKV_HEADS_MIN_BLOCKS
 #define MLKV_HEADS_MIN_BLOCKS 4
@@ -409,7 +363,8 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
     __shared__ uint4 sml[8][kListS];  // (row, p0, p1, p2) of small runs
     __shared__ uint32_t sp3[8][kListS];  // ... and their p3
     __shared__ uint32_t qs[8][kQueue], qr[8][kQueue], qe[8][kQueue];  // long runs: start, row, end (0: unknown)
-    __shared__ uint32_t wsh[8], wlg[8], wit[8], ws1[8], ws2[8];  // per warp: short runs, long runs, chunks,
+    __shared__ LongCounts wlc[8];  // per warp: what its long runs add to the lists; then their bases
+    __shared__ uint32_t wsh[8], wlg[8], ws1[8], ws2[8];  // per warp: short runs, long runs,
                                                                  // runs of one lookup, small runs; then
                                                                  // their bases
     const uint32_t n = a.n, sent = a.sent;
@@ -453,8 +408,12 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
             }
         }
     };
-    auto emit_long = [&](uint32_t h0, uint32_t ib0) {
-        if (nq) write_long_runs(a, qs[wib], qe[wib], qr[wib], nq, h0, ib0, lane);
+    auto room = [&](const LongCounts& base, const LongCounts& tot) {
+        return base.items + tot.items <= a.max_items && base.runs + tot.runs <= a.max_long &&
+               base.nodes + tot.nodes <= a.max_nodes;
+    };
+    auto emit_long = [&](const LongCounts& base) {
+        if (nq) write_long_runs(a, qs[wib], qe[wib], qr[wib], nq, base, lane);
         nq = 0;
         __syncwarp();
     };
@@ -519,19 +478,22 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
             const int i = __ffs(lm) - 1;
             if (nq == kQueue) {
                 measure();
-                uint32_t excl, h0 = 0, ib0 = 0;
-                const uint32_t items = long_chunks(qs[wib], qe[wib], nq, lane, a.chunk, excl);
+                LongCounts mine, excl, base = {0u, 0u, 0u};
+                const LongCounts tot = long_counts(qs[wib], qe[wib], nq, lane, a.chunk, mine, excl);
                 if (lane == 0) {
-                    h0 = atomicAdd(&a.cur->n_long, (uint32_t)nq);
-                    ib0 = atomicAdd(&a.cur->n_items, items);
+                    atomicAdd(&a.cur->n_long, (uint32_t)nq);
+                    base.items = atomicAdd(&a.cur->n_items, tot.items);
+                    base.runs = atomicAdd(&a.cur->n_group, tot.runs);
+                    base.nodes = atomicAdd(&a.cur->n_nodes, tot.nodes);
                 }
-                h0 = __shfl_sync(0xffffffffu, h0, 0);
-                ib0 = __shfl_sync(0xffffffffu, ib0, 0);
-                if (h0 + nq > a.max_long || ib0 + items > a.max_items) {
+                base.items = __shfl_sync(0xffffffffu, base.items, 0);
+                base.runs = __shfl_sync(0xffffffffu, base.runs, 0);
+                base.nodes = __shfl_sync(0xffffffffu, base.nodes, 0);
+                if (!room(base, tot)) {
                     if (lane == 0) record_error(a.err, MLKV_ERR_FULL);
                     nq = 0;
                 } else {
-                    emit_long(h0, ib0);
+                    emit_long(base);
                 }
             }
             const uint32_t row = __shfl_sync(0xffffffffu, r, i);
@@ -545,40 +507,42 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
         }
     }
     measure();
-    uint32_t excl;
-    const uint32_t items = long_chunks(qs[wib], qe[wib], nq, lane, a.chunk, excl);
+    LongCounts mine, excl;
+    const LongCounts tot = long_counts(qs[wib], qe[wib], nq, lane, a.chunk, mine, excl);
     if (lane == 0) {
         wsh[wib] = (uint32_t)cnt;
         wlg[wib] = (uint32_t)nq;
-        wit[wib] = items;
+        wlc[wib] = tot;
         ws1[wib] = (uint32_t)cnt1;
         ws2[wib] = (uint32_t)cnt2;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        uint32_t ts = 0, tl = 0, ti = 0, t1 = 0, t2 = 0;
+        uint32_t ts = 0, tl = 0, t1 = 0, t2 = 0;
+        LongCounts t = {0u, 0u, 0u};
         for (int k = 0; k < 8; ++k) {
             ts += wsh[k];
             tl += wlg[k];
-            ti += wit[k];
+            t = {t.items + wlc[k].items, t.runs + wlc[k].runs, t.nodes + wlc[k].nodes};
             t1 += ws1[k];
             t2 += ws2[k];
         }
         uint32_t bs = ts ? atomicAdd(&a.cur->n_short, ts) : 0u;
-        uint32_t bl = tl ? atomicAdd(&a.cur->n_long, tl) : 0u;
-        uint32_t bi = ti ? atomicAdd(&a.cur->n_items, ti) : 0u;
+        if (tl) atomicAdd(&a.cur->n_long, tl);
+        LongCounts b = {t.items ? atomicAdd(&a.cur->n_items, t.items) : 0u,
+                        t.runs ? atomicAdd(&a.cur->n_group, t.runs) : 0u,
+                        t.nodes ? atomicAdd(&a.cur->n_nodes, t.nodes) : 0u};
         uint32_t b1 = t1 ? atomicAdd(&a.cur->n_single, t1) : 0u;
         uint32_t b2 = t2 ? atomicAdd(&a.cur->n_small, t2) : 0u;
         for (int k = 0; k < 8; ++k) {
-            const uint32_t c0 = wsh[k], c1 = wlg[k], c2 = wit[k], c3 = ws1[k], c4 = ws2[k];
+            const uint32_t c0 = wsh[k], c3 = ws1[k], c4 = ws2[k];
+            const LongCounts c = wlc[k];
             wsh[k] = bs;
-            wlg[k] = bl;
-            wit[k] = bi;
+            wlc[k] = b;
             ws1[k] = b1;
             ws2[k] = b2;
             bs += c0;
-            bl += c1;
-            bi += c2;
+            b = {b.items + c.items, b.runs + c.runs, b.nodes + c.nodes};
             b1 += c3;
             b2 += c4;
         }
@@ -590,44 +554,293 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
         a.smalls[ws2[wib] + k] = sml[wib][k];
         a.small_p3[ws2[wib] + k] = sp3[wib][k];
     }
-    if (wlg[wib] + nq > a.max_long || wit[wib] + items > a.max_items) {
+    const LongCounts base = wlc[wib];
+    if (!room(base, tot)) {
         if (lane == 0 && nq) record_error(a.err, MLKV_ERR_FULL);
         return;
     }
-    emit_long(wlg[wib], wit[wib]);
+    emit_long(base);
 }
 
-// One lane group per listed run of 2 .. MLKV_SEQ_SEGMENT_MAX lookups.  The
-// run's record (bounds, row, first lookup position) is loaded one run ahead;
-// its row, state, first gradient row and the positions of its other lookups
-// then load together, and the other gradient rows after them.
-__device__ __forceinline__ uint4 run_meta(const RunArgs& a, uint32_t u, uint32_t U) {
-    return u < U ? __ldg(a.runs + u) : make_uint4(0u, 0u, 0u, 0u);
+// (acc, cmp) = the pairs of tree entries slot0, slot0 + stride, ... (cnt of
+// them, in that order): each entry's sum added with compensation, then its own
+// compensation added to cmp.
+template <int V>
+__device__ __forceinline__ void sum_pairs(typename Vec<V>::T& acc, typename Vec<V>::T& cmp, const RowArgs& ra,
+                                          const float* partial, uint32_t slot0, uint32_t stride, uint32_t cnt, int j,
+                                          bool act) {
+    using VT = typename Vec<V>::T;
+    constexpr int UNR = 4;
+    acc = Vec<V>::zero();
+    cmp = Vec<V>::zero();
+    if (!act) return;
+    for (uint32_t x = 0; x < cnt; x += UNR) {
+        VT g[UNR], c[UNR];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u)
+            if (x + u < cnt) {
+                const VT* src =
+                    reinterpret_cast<const VT*>(partial + (size_t)(slot0 + (x + u) * stride) * 2 * ra.dpad) + j;
+                g[u] = __ldcg(src);
+                c[u] = __ldcg(beside(ra, src));
+            }
+#pragma unroll
+        for (int u = 0; u < UNR; ++u)
+            if (x + u < cnt) {
+                Vec<V>::cadd(acc, cmp, g[u]);
+                Vec<V>::add(cmp, c[u]);
+            }
+    }
 }
 
-template <int V, int KV, int ROWS = MLKV_REDUCE_ROWS_IN_FLIGHT>
+// The compensated sum of one segment of chunk rec of a long run, by one lane group.
+template <int V>
+__device__ __forceinline__ bool chunk_sum(typename Vec<V>::T& acc, typename Vec<V>::T& cmp, const RowArgs& ra,
+                                          const RunArgs& a, const uint4& rec, int j, int G, int glane,
+                                          unsigned gmask) {
+    const uint32_t len = rec.y & ((1u << kItemLenBits) - 1);
+    if (MLKV_CHECK && !(in_bounds(a.err, kChkLongItem, rec.x + len, (unsigned long long)a.n + 1) &&
+                        in_bounds(a.err, kChkLongItem, rec.w + (rec.y >> kItemLenBits),
+                                  (unsigned long long)a.max_items + 1) &&
+                        in_bounds(a.err, kChkLongRow, rec.z, ra.nrows)))
+        return false;
+    acc = Vec<V>::zero();
+    cmp = Vec<V>::zero();
+    sum_rows<V, MLKV_LONG_ROWS, false, true>(acc, cmp, a.grads, a.spos, rec.x, len, ra.d, j, j < ra.NV, G, glane,
+                                             gmask, a.err, kChkLongPos, a.n);
+    return true;
+}
+
+// Tree entry `slot`'s (sum, compensation) pair: this lane's vectors.
+template <int V>
+__device__ __forceinline__ void store_pair(const RowArgs& ra, const RunArgs& a, uint32_t slot, int j,
+                                           const typename Vec<V>::T& acc, const typename Vec<V>::T& cmp) {
+    typename Vec<V>::T* part = reinterpret_cast<typename Vec<V>::T*>(a.partial + (size_t)slot * 2 * ra.dpad) + j;
+    __stcg(part, acc);
+    __stcg(beside(ra, part), cmp);
+}
+
+// The sum acc + cmp rounded once, and the Adagrad step of `row` with it.
+template <int V>
+__device__ __forceinline__ void finish_long(const RowArgs& ra, const RunArgs& a, uint32_t row, int j,
+                                            typename Vec<V>::T acc, const typename Vec<V>::T& cmp) {
+    Vec<V>::add(acc, cmp);
+    const typename Vec<V>::T* p = row_vec<V>(ra, row, j);
+    adagrad_store<V>(ra, row, j, *p, *beside(ra, p), acc, a.lr, a.eps);
+}
+
+// One segment of a run of kSmallRun + 1 .. MLKV_SEQ_SEGMENT_MAX lookups (sorted
+// positions s .. e-1, first lookup p0), by one lane group: the row, the state,
+// the first gradient row and the other lookups' positions load together, the
+// rest of the gradient rows are added in occurrence order, then the Adagrad
+// step.
+template <int V, int ROWS>
+__device__ __forceinline__ void short_run(const RowArgs& ra, const RunArgs& a, uint32_t s, uint32_t e, uint32_t row,
+                                          uint32_t p0, int j, int G, int glane, unsigned gmask) {
+    using VT = typename Vec<V>::T;
+    if (MLKV_CHECK && !(in_bounds(a.err, kChkShortRun, e, (unsigned long long)a.n + 1) &&
+                        in_bounds(a.err, kChkShortRun, s, e) && in_bounds(a.err, kChkShortRow, row, ra.nrows) &&
+                        in_bounds(a.err, kChkShortPos, p0, a.n)))
+        return;
+    const bool act = j < ra.NV;
+    const uint32_t rest = e - s - 1;
+    const uint32_t pl0 = (uint32_t)glane < min(rest, (uint32_t)G) ? __ldg(a.spos + s + 1 + glane) : 0u;
+    VT w, Gs, acc = Vec<V>::zero();
+    if (act) {
+        const VT* p = row_vec<V>(ra, row, j);
+        w = p[0];
+        Gs = *beside(ra, p);
+        Vec<V>::add(acc, __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)p0 * ra.d) + j));  // 0 + g: in order
+    }
+    sum_rows<V, ROWS, true, false>(acc, acc, a.grads, a.spos, s + 1, rest, ra.d, j, act, G, glane, gmask, a.err,
+                                   kChkShortPos, a.n, pl0);
+    if (act) adagrad_store<V>(ra, row, j, w, Gs, acc, a.lr, a.eps);
+}
+
+// One segment of a run of 2 .. kSmallRun lookups, whose positions are in its
+// record: the row, the state and every gradient row load together, then the
+// sum 0 + g0 + g1 + ... in occurrence order and the Adagrad step.
+template <int V>
+__device__ __forceinline__ void small_run(const RowArgs& ra, const RunArgs& a, const uint4& m, uint32_t p3, int j) {
+    using VT = typename Vec<V>::T;
+    if (j >= ra.NV) return;
+    const uint32_t ps[kSmallRun] = {m.y, m.z, m.w, p3};
+    if (MLKV_CHECK && !(in_bounds(a.err, kChkSmallRow, m.x, ra.nrows) && in_bounds(a.err, kChkSmallPos, m.y, a.n) &&
+                        in_bounds(a.err, kChkSmallPos, m.z, a.n) &&
+                        (m.w == NONE || in_bounds(a.err, kChkSmallPos, m.w, a.n)) &&
+                        (p3 == NONE || in_bounds(a.err, kChkSmallPos, p3, a.n))))
+        return;
+    const VT* p = row_vec<V>(ra, m.x, j);
+    const VT w = p[0], Gs = *beside(ra, p);
+    VT g[kSmallRun];
+#pragma unroll
+    for (int i = 0; i < kSmallRun; ++i)
+        if (ps[i] != NONE) g[i] = __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)ps[i] * ra.d) + j);
+    VT acc = Vec<V>::zero();
+#pragma unroll
+    for (int i = 0; i < kSmallRun; ++i)
+        if (ps[i] != NONE) Vec<V>::add(acc, g[i]);
+    adagrad_store<V>(ra, m.x, j, w, Gs, acc, a.lr, a.eps);
+}
+
+// --- a kernel per run length, on three streams ---------------------------------
+// Work items are run segments: v = run * nseg + segment (SEG; without it a row is
+// one segment).
+
+// The chunks of the long runs: their sums, compensated, to scratch.  (Combining
+// them here too, by the last chunk of a run to arrive, cost a fence a chunk: a
+// recommendation step of 1.7M lookups took 600 us instead of 556.)
+template <int V, bool SEG>
+__global__ void __launch_bounds__(256, MLKV_LONG_MIN_BLOCKS) k_long(RowArgs ra, RunArgs a) {
+    pdl_enter();
+    using VT = typename Vec<V>::T;
+    const uint32_t nseg = SEG ? ra.nseg : 1u, N = min(a.cur->n_items, a.max_items) * nseg;
+    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane >> ra.gshift;
+    const unsigned gmask = group_mask(G, gid);
+    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) >> ra.gshift;
+    const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
+    for (uint32_t v = group; v < N; v += ngroups) {
+        const uint32_t it = SEG ? v / nseg : v;
+        const int j = glane + G * (int)(v - it * nseg);
+        VT acc, cmp;
+        if (chunk_sum<V>(acc, cmp, ra, a, __ldg(a.items + it), j, G, glane, gmask) && j < ra.NV)
+            store_pair<V>(ra, a, it, j, acc, cmp);
+    }
+}
+
+// The long runs' chunk sums combined, always in chunk order, and their rows
+// updated.  A node of up to kNode chunks of a run takes a block (one segment of
+// its rows): the lane groups split its chunk sums in a fixed way and group 0
+// adds the groups' results up; where the run has more nodes, the pair goes to
+// scratch and the block that finishes the run's last node adds the nodes' pairs
+// up the same way (nodes counted by an atomic: no block waits for another).
+// Every run of at most kGroupChunks chunks takes one lane group.  (With one
+// block for all chunks of a run, 8 lane groups each added up to a hundred
+// chunks one after another: 100,003 lookups, Zipf(1.0), dim 50, took 119 us for
+// apply + export, 113 with nodes.)  kGroupChunks = 16: 4 and 32 cost the 1.7M-
+// and 200k-lookup steps 1-2 us.
+// 256 threads fit the slots that retiring blocks of the other reduce kernels
+// free, where a 1024-thread block waits for a whole SM to drain.
+constexpr int kCombineThreads = 256;
+
+// acc, cmp of group 0: entries slot0, slot0 + stride, ... (cnt of them) added
+// up by the block's lane groups.  sh: the groups' pairs, G vectors each.
+template <int V>
+__device__ __forceinline__ void block_pairs(typename Vec<V>::T& acc, typename Vec<V>::T& cmp, const RowArgs& ra,
+                                            const float* partial, uint32_t slot0, uint32_t stride, uint32_t cnt,
+                                            int j, int group, int ngroups, typename Vec<V>::T* sh) {
+    const int G = ra.G, glane = threadIdx.x & (G - 1);
+    const bool act = j < ra.NV;
+    const uint32_t per = (cnt + ngroups - 1) / ngroups;
+    const uint32_t k0 = min(cnt, group * per), k1 = min(cnt, k0 + per);
+    sum_pairs<V>(acc, cmp, ra, partial, slot0 + k0 * stride, stride, k1 - k0, j, act);
+    sh[(group * 2) * G + glane] = acc;
+    sh[(group * 2 + 1) * G + glane] = cmp;
+    __syncthreads();
+    if (group == 0) {
+        acc = Vec<V>::zero();
+        cmp = Vec<V>::zero();
+        for (int x = 0; x < ngroups; ++x) {
+            Vec<V>::cadd(acc, cmp, sh[(x * 2) * G + glane]);
+            Vec<V>::add(cmp, sh[(x * 2 + 1) * G + glane]);
+        }
+    }
+    __syncthreads();
+}
+
+template <int V>
+__global__ void __launch_bounds__(kCombineThreads, 3) k_combine(RowArgs ra, RunArgs a, DevState* ds) {
+    pdl_enter();
+    using VT = typename Vec<V>::T;
+    __shared__ VT sh[2 * kCombineThreads];
+    __shared__ int last_node;
+    const uint32_t nseg = ra.nseg;
+    const uint32_t NR = min(a.cur->n_group, a.max_long) * nseg, NN = min(a.cur->n_nodes, a.max_nodes) * nseg;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        ds->last_unique = a.cur->n_single + a.cur->n_small + a.cur->n_short + a.cur->n_long;  // one run per row
+    const int G = ra.G, glane = threadIdx.x & (G - 1), group = threadIdx.x >> ra.gshift;
+    const int ngroups = kCombineThreads >> ra.gshift;
+    for (uint32_t v = blockIdx.x; v < NN; v += gridDim.x) {  // block-uniform
+        const uint32_t x = v / nseg, seg = v - x * nseg;
+        const uint4 nd = __ldg(a.nodes + x);  // (the run's first chunk, its chunks, row, node)
+        const uint32_t first = nd.w * kNode, nodes = (nd.y + kNode - 1) / kNode;
+        const int j = glane + G * (int)seg;
+        if (MLKV_CHECK && !(in_bounds(a.err, kChkLongItem, nd.x + nd.y, (unsigned long long)a.max_items + 1) &&
+                            in_bounds(a.err, kChkLongRow, nd.z, ra.nrows)))
+            continue;
+        VT acc, cmp;
+        bool done = nodes == 1;
+        uint32_t slot0 = nd.x + first, stride = 1, cnt = min(kNode, nd.y - first);
+        while (true) {  // the node's chunks, then, in the run's last block, its nodes
+            block_pairs<V>(acc, cmp, ra, a.partial, slot0, stride, cnt, j, group, ngroups, sh);
+            if (done) break;
+            if (group == 0) {
+                if (j < ra.NV) store_pair<V>(ra, a, nd.x + first, j, acc, cmp);
+                __threadfence();
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                uint32_t* ctr = a.node_cnt + (size_t)nd.x * nseg + seg;
+                last_node = atomicAdd(ctr, 1u) == nodes - 1;
+                if (last_node) *ctr = 0u;  // zero again for the next call
+                __threadfence();
+            }
+            __syncthreads();
+            if (!last_node) break;
+            done = true;
+            slot0 = nd.x;
+            stride = kNode;
+            cnt = nodes;
+        }
+        if (!done) continue;
+        if (group == 0 && j < ra.NV) finish_long<V>(ra, a, nd.z, j, acc, cmp);
+    }
+    // the other long runs: on the blocks that took no node (all blocks when the
+    // nodes outnumber them)
+    const uint32_t b0 = NN < gridDim.x ? NN : 0u;
+    const uint32_t gg = (blockIdx.x - b0) * ngroups + group, ngg = (gridDim.x - b0) * ngroups;
+    for (uint32_t v = blockIdx.x < b0 ? NR : gg; v < NR; v += ngg) {  // uniform within the group
+        const uint32_t x = v / nseg;
+        const uint4 r = __ldg(a.long_runs + x);  // (first chunk, chunks, row, -)
+        const int j = glane + G * (int)(v - x * nseg);
+        if (MLKV_CHECK && !(in_bounds(a.err, kChkLongItem, r.x + r.y, (unsigned long long)a.max_items + 1) &&
+                            in_bounds(a.err, kChkLongRow, r.z, ra.nrows)))
+            continue;
+        if (j >= ra.NV) continue;
+        const VT* p = row_vec<V>(ra, r.z, j);
+        const VT w = p[0], Gs = *beside(ra, p);  // beside the chunk sums
+        VT acc, cmp;
+        sum_pairs<V>(acc, cmp, ra, a.partial, r.x, 1, r.y, j, true);
+        Vec<V>::add(acc, cmp);  // the sum, rounded once
+        adagrad_store<V>(ra, r.z, j, w, Gs, acc, a.lr, a.eps);
+    }
+    if (a.release) release_counters(a.cur, a.release);
+}
+
+// Runs of 5 .. 32 lookups, records loaded one run ahead.  Fixed shares would
+// leave the kernel to the group with the most lookups: each group claims
+// `grab` run segments at a time, its first ones by its index, the rest from a
+// counter; one at a time when they are few, so that every run starts at once.
+template <int V, bool SEG, int ROWS>
 __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_short(RowArgs ra, RunArgs a) {
     pdl_enter();
     if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_short, (unsigned long long)a.n + 1)) return;
-    const uint32_t U = min(a.cur->n_short, a.n);  // a list never holds more runs than lookups
-    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane / G;
+    const uint32_t nseg = SEG ? ra.nseg : 1u, N = min(a.cur->n_short, a.n) * nseg;  // a list never holds more runs than lookups
+    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane >> ra.gshift;
     const unsigned gmask = group_mask(G, gid);
-    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = (gridDim.x * blockDim.x) / G;
-    // Runs take 5 .. 32 lookups, so fixed shares would leave the kernel to the
-    // group with the most lookups: each group claims chunks of `grab` runs, its
-    // first chunk by its index, the rest from a counter (one atomic a chunk).
-    // With fewer runs than MLKV_SHORT_GRAB per group, one run at a time: every
-    // run then starts at once instead of queueing behind others.
-    const uint32_t grab = U >= ngroups * (uint32_t)MLKV_SHORT_GRAB ? (uint32_t)MLKV_SHORT_GRAB : 1u;
+    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) >> ra.gshift;
+    const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
+    const uint32_t grab = N >= ngroups * (uint32_t)MLKV_SHORT_GRAB ? (uint32_t)MLKV_SHORT_GRAB : 1u;
+    auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
     uint32_t base = group * grab;
-    while (base < U) {  // uniform within the group
-        const uint32_t end = min(U, base + grab);
-        uint4 next = run_meta(a, base, end);
-        for (uint32_t u = base; u < end; ++u) {
+    while (base < N) {  // uniform within the group
+        const uint32_t end = min(N, base + grab);
+        uint4 next = __ldg(a.runs + run_of(base));
+        for (uint32_t v = base; v < end; ++v) {
             const uint4 m = next;  // (start, end, row, first lookup)
-            next = run_meta(a, u + 1, end);
-            short_run<V, KV, ROWS>(ra, a, m.x, m.y - m.x, m.z, m.w, glane, gmask);
+            if (v + 1 < end) next = __ldg(a.runs + run_of(v + 1));
+            const int j = glane + G * (int)(v - run_of(v) * nseg);
+            short_run<V, ROWS>(ra, a, m.x, m.y, m.z, m.w, j, G, glane, gmask);
         }
         uint32_t c = 0;
         if (glane == 0) c = atomicAdd(&a.cur->short_next, grab);
@@ -636,325 +849,131 @@ __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_
     if (a.release) release_counters(a.cur, a.release);
 }
 
-// One lane group per run of one lookup (most runs of a Zipf batch): its row,
-// state and gradient row, SINGLES runs at a time, records loaded one round
-// ahead; the sum is the gradient row itself (0 + g), then the Adagrad step.
-// With no loop over positions it needs few registers, so more warps (and
-// rows) are in flight than in k_short.
-template <int V, int KV, int SG = MLKV_SINGLES>
+// Runs of 2 .. kSmallRun lookups, records loaded one run ahead.
+template <int V, bool SEG>
+__global__ void __launch_bounds__(256, MLKV_SMALL_MIN_BLOCKS) k_small(RowArgs ra, RunArgs a) {
+    pdl_enter();
+    if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_small, (unsigned long long)a.n + 1)) return;
+    const uint32_t nseg = SEG ? ra.nseg : 1u, N = min(a.cur->n_small, a.n) * nseg;
+    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1);
+    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) >> ra.gshift;
+    const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
+    auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
+    uint4 next = group < N ? __ldg(a.smalls + run_of(group)) : make_uint4(0u, 0u, 0u, 0u);
+    uint32_t next3 = group < N ? __ldg(a.small_p3 + run_of(group)) : NONE;
+    for (uint32_t v = group; v < N; v += ngroups) {  // uniform within the group
+        const uint4 m = next;
+        const uint32_t p3 = next3, x = v + ngroups;
+        if (x < N) {
+            next = __ldg(a.smalls + run_of(x));
+            next3 = __ldg(a.small_p3 + run_of(x));
+        }
+        small_run<V>(ra, a, m, p3, glane + G * (int)(v - run_of(v) * nseg));
+    }
+    if (a.release) release_counters(a.cur, a.release);
+}
+
+// Runs of one lookup (most runs of a Zipf batch): row, state and gradient row
+// loaded together, SG runs at a time, records loaded one round ahead.  With no
+// loop over positions it needs few registers, so many warps (and rows) are in
+// flight.
+template <int V, bool SEG, int SG>
 __global__ void __launch_bounds__(256, SG == 1 ? MLKV_SINGLE_MIN_BLOCKS : 4) k_single(RowArgs ra, RunArgs a) {
     pdl_enter();
     using VT = typename Vec<V>::T;
     if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_single, (unsigned long long)a.n + 1)) return;
-    const uint32_t U = min(a.cur->n_single, a.n);  // a list never holds more runs than lookups
+    const uint32_t nseg = SEG ? ra.nseg : 1u, N = min(a.cur->n_single, a.n) * nseg;
     const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1);
-    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = (gridDim.x * blockDim.x) / G;
+    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) >> ra.gshift;
+    const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
     const uint2 none = make_uint2(0xFFFFFFFFu, 0u);
+    auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
     uint2 next[SG];
 #pragma unroll
-    for (int j = 0; j < SG; ++j) next[j] = group * SG + j < U ? __ldg(a.singles + group * SG + j) : none;
-    for (uint32_t u = group * SG; u < U; u += ngroups * SG) {  // uniform within the group
+    for (int i = 0; i < SG; ++i) next[i] = group * SG + i < N ? __ldg(a.singles + run_of(group * SG + i)) : none;
+    for (uint32_t v = group * SG; v < N; v += ngroups * SG) {  // uniform within the group
         uint2 m[SG];
+        VT w[SG], Gs[SG], g[SG];
 #pragma unroll
-        for (int j = 0; j < SG; ++j) {
-            m[j] = next[j];
-            const uint32_t v = u + ngroups * SG + j;
-            next[j] = v < U ? __ldg(a.singles + v) : none;
+        for (int i = 0; i < SG; ++i) {
+            m[i] = next[i];
+            const uint32_t x = v + ngroups * SG + i;
+            next[i] = x < N ? __ldg(a.singles + run_of(x)) : none;
         }
-        VT w[SG][KV], Gs[SG][KV], g[SG][KV];
 #pragma unroll
-        for (int j = 0; j < SG; ++j) {
-            if (m[j].x == 0xFFFFFFFFu) continue;
-            if (MLKV_CHECK && !(in_bounds(a.err, kChkSingleRow, m[j].x, ra.nrows) &&
-                                in_bounds(a.err, kChkSinglePos, m[j].y, a.n))) {
-                m[j].x = 0xFFFFFFFFu;
+        for (int i = 0; i < SG; ++i) {
+            const int j = glane + G * (int)(v + i - run_of(v + i) * nseg);
+            if (m[i].x == none.x || j >= ra.NV) {
+                m[i].x = none.x;
                 continue;
             }
-            load_row_state<V, KV>(ra, m[j].x, w[j], Gs[j], glane);
-            const VT* src = reinterpret_cast<const VT*>(a.grads + (size_t)m[j].y * ra.d);
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                const int jj = glane + G * k;
-                if (jj < ra.NV) g[j][k] = __ldcs(src + jj);
+            if (MLKV_CHECK && !(in_bounds(a.err, kChkSingleRow, m[i].x, ra.nrows) &&
+                                in_bounds(a.err, kChkSinglePos, m[i].y, a.n))) {
+                m[i].x = none.x;
+                continue;
             }
+            const VT* p = row_vec<V>(ra, m[i].x, j);
+            w[i] = p[0];
+            Gs[i] = *beside(ra, p);
+            g[i] = __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)m[i].y * ra.d) + j);
         }
 #pragma unroll
-        for (int j = 0; j < SG; ++j) {
-            if (m[j].x == 0xFFFFFFFFu) continue;
-            VT acc[KV];
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                acc[k] = Vec<V>::zero();
-                if (glane + G * k < ra.NV) Vec<V>::add(acc[k], g[j][k]);  // 0 + g, as in a longer run
-            }
-            adagrad_store<V, KV>(ra, m[j].x, w[j], Gs[j], acc, glane, a.lr, a.eps);
+        for (int i = 0; i < SG; ++i) {
+            if (m[i].x == none.x) continue;
+            VT acc = Vec<V>::zero();
+            Vec<V>::add(acc, g[i]);  // 0 + g, as in a longer run
+            adagrad_store<V>(ra, m[i].x, glane + G * (int)(v + i - run_of(v + i) * nseg), w[i], Gs[i], acc, a.lr,
+                             a.eps);
         }
     }
     if (a.release) release_counters(a.cur, a.release);
 }
 
-// One lane group per run of 2 .. kSmallRun lookups (most runs of more than one
-// lookup in a Zipf batch).  k_heads put the run's positions in its record, so
-// the row, the state and every gradient row of the run load together, in one
-// round trip (records loaded one run ahead); then the sum 0 + g0 + g1 + ... in
-// occurrence order and the Adagrad step.  No loop over positions: few
-// registers and many warps, as in k_single.
-template <int V, int KV>
-__global__ void __launch_bounds__(256, KV >= 4 ? 2 : MLKV_SMALL_MIN_BLOCKS) k_small(RowArgs ra, RunArgs a) {
-    pdl_enter();
-    using VT = typename Vec<V>::T;
-    if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_small, (unsigned long long)a.n + 1)) return;
-    const uint32_t U = min(a.cur->n_small, a.n);  // a list never holds more runs than lookups
-    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1);
-    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = (gridDim.x * blockDim.x) / G;
-    uint4 next = group < U ? __ldg(a.smalls + group) : make_uint4(0u, 0u, 0u, 0u);
-    uint32_t next3 = group < U ? __ldg(a.small_p3 + group) : NONE;
-    for (uint32_t u = group; u < U; u += ngroups) {  // uniform within the group
-        const uint4 m = next;  // (row, p0, p1, p2)
-        const uint32_t p3 = next3;
-        const uint32_t v = u + ngroups;
-        next = v < U ? __ldg(a.smalls + v) : make_uint4(0u, 0u, 0u, 0u);
-        next3 = v < U ? __ldg(a.small_p3 + v) : NONE;
-        VT w[KV], Gs[KV], g[kSmallRun][KV];
-        if (MLKV_CHECK && !(in_bounds(a.err, kChkSmallRow, m.x, ra.nrows) && in_bounds(a.err, kChkSmallPos, m.y, a.n) &&
-                            in_bounds(a.err, kChkSmallPos, m.z, a.n) &&
-                            (m.w == NONE || in_bounds(a.err, kChkSmallPos, m.w, a.n)) &&
-                            (p3 == NONE || in_bounds(a.err, kChkSmallPos, p3, a.n))))
-            continue;
-        load_row_state<V, KV>(ra, m.x, w, Gs, glane);
-        const uint32_t ps[kSmallRun] = {m.y, m.z, m.w, p3};
-#pragma unroll
-        for (int i = 0; i < kSmallRun; ++i) {
-            if (ps[i] == NONE) continue;  // uniform within the group
-            const VT* src = reinterpret_cast<const VT*>(a.grads + (size_t)ps[i] * ra.d);
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                const int j = glane + G * k;
-                if (j < ra.NV) g[i][k] = __ldcs(src + j);
-            }
-        }
-        VT acc[KV];
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            acc[k] = Vec<V>::zero();
-            if (glane + G * k >= ra.NV) continue;
-#pragma unroll
-            for (int i = 0; i < kSmallRun; ++i)
-                if (ps[i] != NONE) Vec<V>::add(acc[k], g[i][k]);  // 0 + g0 + g1 + ...: occurrence order
-        }
-        adagrad_store<V, KV>(ra, m.x, w, Gs, acc, glane, a.lr, a.eps);
-    }
-    if (a.release) release_counters(a.cur, a.release);  // when it is its stream's last kernel
+using RunKernel = void (*)(RowArgs, RunArgs);
+
+// Narrow rows (on at most 16 lanes: dim <= 64): runs of one lookup two at a
+// time per lane group on at most 3 blocks per SM, runs of 5-32 lookups with 4
+// gradient rows in flight at 3 blocks per SM (more warps).
+struct RunKernels {
+    RunKernel longs, shorts, smalls, singles;
+};
+
+template <int V>
+RunKernels run_kernels(bool seg, bool narrow) {
+    if (seg) return {k_long<V, true>, k_short<V, true, MLKV_SHORT_ROWS>, k_small<V, true>, k_single<V, true, 1>};
+    if (narrow) return {k_long<V, false>, k_short<V, false, 4>, k_small<V, false>, k_single<V, false, 2>};
+    return {k_long<V, false>, k_short<V, false, MLKV_SHORT_ROWS>, k_small<V, false>, k_single<V, false, 1>};
 }
 
-template <int V, int KV>
-__global__ void __launch_bounds__(256, MLKV_LONG_MIN_BLOCKS) k_long_sum(RowArgs ra, RunArgs a) {
-    pdl_enter();
-    using VT = typename Vec<V>::T;
-    const uint32_t NI = min(a.cur->n_items, a.max_items);
-    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane / G;
-    const unsigned gmask = group_mask(G, gid);
-    const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = (gridDim.x * blockDim.x) / G;
-    for (uint32_t it = group; it < NI; it += ngroups) {
-        const uint32_t s = __ldg(a.item_s + it), e = __ldg(a.item_e + it);
-        if (MLKV_CHECK && !in_bounds(a.err, kChkLongItem, e, (unsigned long long)a.n + 1)) continue;
-        VT acc[KV], cmp[KV];
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            acc[k] = Vec<V>::zero();
-            cmp[k] = Vec<V>::zero();
-        }
-        sum_rows<V, KV, MLKV_LONG_ROWS_IN_FLIGHT, false, true>(acc, cmp, a.grads, a.spos, s, e > s ? e - s : 0u,
-                                                               ra.d, ra.NV, G, glane, gmask, a.err, kChkLongPos,
-                                                               a.n);
-        // the chunk's (sum, compensation) pair
-        VT* part = reinterpret_cast<VT*>(a.partial + (size_t)it * 2 * ra.dpad);
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            const int j = glane + G * k;
-            if (j < ra.NV) {
-                __stcg(part + j, acc[k]);
-                __stcg(part + ra.dpad / V + j, cmp[k]);
-            }
-        }
-    }
-}
-
-
-// (acc, cmp) += the chunk pairs base + k0 .. base + k1 - 1, in that order, with
-// eight vectors per lane in flight: each chunk's sum added with compensation,
-// then its own compensation added to cmp.
-template <int V, int KV>
-__device__ __forceinline__ void sum_partials(typename Vec<V>::T (&acc)[KV], typename Vec<V>::T (&cmp)[KV],
-                                             const RowArgs& ra, const float* partial, uint32_t base, uint32_t k0,
-                                             uint32_t k1, int glane) {
-    using VT = typename Vec<V>::T;
-    constexpr int UNR = KV >= 4 ? 1 : 4 / KV;
-    const int half = ra.dpad / V;
-    for (uint32_t x = k0; x < k1; x += UNR) {
-        VT g[UNR][KV], c[UNR][KV];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const VT* src = reinterpret_cast<const VT*>(partial + (size_t)(base + x + u) * 2 * ra.dpad);
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                const int j = glane + ra.G * k;
-                if (x + u < k1 && j < ra.NV) {
-                    g[u][k] = __ldcg(src + j);
-                    c[u][k] = __ldcg(src + half + j);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u)
-#pragma unroll
-            for (int k = 0; k < KV; ++k)
-                if (x + u < k1 && glane + ra.G * k < ra.NV) {
-                    Vec<V>::cadd(acc[k], cmp[k], g[u][k]);
-                    Vec<V>::add(cmp[k], c[u][k]);
-                }
-    }
-}
-
-// One launch for every long run.  A run of more than a.big chunk sums (the
-// hottest rows) takes a whole block: its lane groups split the sums in a fixed
-// way, then group 0 adds the groups' results in order.  Every other long run
-// takes one lane group, which adds its sums in order.  Then the Adagrad step.
-template <int V, int KV>
-__global__ void __launch_bounds__(1024) k_long_combine(RowArgs ra, RunArgs a, DevState* ds) {
-    pdl_enter();
-    using VT = typename Vec<V>::T;
-    extern __shared__ float sh[];  // [groups][2][dpad]: each group's (sum, compensation) pair
-    const uint32_t nl = min(a.cur->n_long, a.max_long), nb = a.cur->n_big;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        ds->last_unique = a.cur->n_single + a.cur->n_small + a.cur->n_short + a.cur->n_long;  // one run per row
-    const int G = ra.G, glane = threadIdx.x & (G - 1);
-    const int group = threadIdx.x / G;
-    const int ngroups = blockDim.x / G;
-    for (uint32_t i = blockIdx.x; i < nb; i += gridDim.x) {  // block-uniform
-        if (MLKV_CHECK && !in_bounds(a.err, kChkCombineRun, i, a.max_long)) break;
-        const uint32_t h = a.big_runs[i];
-        if (MLKV_CHECK && !in_bounds(a.err, kChkCombineRun, h, nl)) continue;
-        const uint32_t base = a.long_base[h];
-        const uint32_t m = (a.long_e[h] - a.long_s[h] + a.chunk - 1) / a.chunk;
-        if (MLKV_CHECK && !(in_bounds(a.err, kChkCombineRun, base + m, (unsigned long long)a.max_items + 1) &&
-                            in_bounds(a.err, kChkCombineRow, a.long_row[h], ra.nrows)))
-            continue;
-        const uint32_t per = (m + ngroups - 1) / ngroups;
-        const uint32_t k0 = min(m, group * per), k1 = min(m, k0 + per);
-        VT acc[KV], cmp[KV];
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            acc[k] = Vec<V>::zero();
-            cmp[k] = Vec<V>::zero();
-        }
-        sum_partials<V, KV>(acc, cmp, ra, a.partial, base, k0, k1, glane);
-        VT* mine = reinterpret_cast<VT*>(sh + (size_t)group * 2 * ra.dpad);
-        const int half = ra.dpad / V;
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            const int j = glane + G * k;
-            if (j < ra.NV) {
-                mine[j] = acc[k];
-                mine[half + j] = cmp[k];
-            }
-        }
-        __syncthreads();
-        if (group == 0) {
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                acc[k] = Vec<V>::zero();
-                cmp[k] = Vec<V>::zero();
-            }
-            for (int gi = 0; gi < ngroups; ++gi) {
-                const VT* src = reinterpret_cast<const VT*>(sh + (size_t)gi * 2 * ra.dpad);
-#pragma unroll
-                for (int k = 0; k < KV; ++k) {
-                    const int j = glane + G * k;
-                    if (j < ra.NV) {
-                        Vec<V>::cadd(acc[k], cmp[k], src[j]);
-                        Vec<V>::add(cmp[k], src[half + j]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < KV; ++k) Vec<V>::add(acc[k], cmp[k]);  // the sum, rounded once
-            VT w[KV], Gs[KV];
-            const uint32_t row = a.long_row[h];
-            load_row_state<V, KV>(ra, row, w, Gs, glane);
-            adagrad_store<V, KV>(ra, row, w, Gs, acc, glane, a.lr, a.eps);
-        }
-        __syncthreads();
-    }
-    // the other long runs: on the blocks that took no big run (all blocks when
-    // the big runs outnumber them)
-    const uint32_t b0 = nb < gridDim.x ? nb : 0u;
-    const uint32_t gg = (blockIdx.x - b0) * ngroups + group, ngg = (gridDim.x - b0) * ngroups;
-    for (uint32_t h = blockIdx.x < b0 ? nl : gg; h < nl; h += ngg) {  // uniform within the group
-        const uint32_t m = (a.long_e[h] - a.long_s[h] + a.chunk - 1) / a.chunk;
-        if (m > a.big) continue;
-        if (MLKV_CHECK && !(in_bounds(a.err, kChkCombineRun, a.long_base[h] + m, (unsigned long long)a.max_items + 1) &&
-                            in_bounds(a.err, kChkCombineRow, a.long_row[h], ra.nrows)))
-            continue;
-        VT acc[KV], cmp[KV], w[KV], Gs[KV];
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            acc[k] = Vec<V>::zero();
-            cmp[k] = Vec<V>::zero();
-        }
-        const uint32_t row = a.long_row[h];
-        load_row_state<V, KV>(ra, row, w, Gs, glane);
-        sum_partials<V, KV>(acc, cmp, ra, a.partial, a.long_base[h], 0u, m, glane);
-#pragma unroll
-        for (int k = 0; k < KV; ++k) Vec<V>::add(acc[k], cmp[k]);  // the sum, rounded once
-        adagrad_store<V, KV>(ra, row, w, Gs, acc, glane, a.lr, a.eps);
-    }
-    if (a.release) release_counters(a.cur, a.release);
-}
-
-template <int V, int KV>
-void launch_short(mlkv_table* t, bool narrow, int grid, cudaStream_t st, const RowArgs& ra, const RunArgs& a) {
-    if (narrow)
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SHORT, (k_short<V, KV, 4>), grid, 256, 0, st, ra, a);
-    else
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SHORT, (k_short<V, KV>), grid, 256, 0, st, ra, a);
-}
-
-template <int V, int KV>
+template <int V>
 cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* srow, const uint32_t* spos,
                        int64_t n, uint32_t sent, cudaStream_t st, CallCounters* cur) {
-    RowArgs ra{t->slots, t->geom.stride, t->geom.dpad, t->geom.NV, t->geom.G, t->geom.d,
+    const uint32_t nseg = (uint32_t)((t->geom.NV + t->geom.G - 1) / t->geom.G);
+    RowArgs ra{t->slots, t->geom.stride, t->geom.dpad, t->geom.NV, t->geom.G, __builtin_ctz((unsigned)t->geom.G),
+               t->geom.d, nseg,
                (uint32_t)(t->tiered ? t->cfg.hbm_cache_rows : t->cfg.capacity)};
     RunArgs a{grads, srow, spos, (uint32_t)n, sent, cur, t->s.short_runs, t->s.single_runs, t->s.small_runs,
-              t->s.small_p3, t->s.long_s, t->s.long_e,
-              t->s.long_row, t->s.long_base, t->s.item_s, t->s.item_e, t->s.big_runs, t->s.partial,
-              (uint32_t)t->s.max_long,
-              (uint32_t)t->s.max_items, n >= kSmallBatch ? kChunkLarge : kChunkSmall,
-              n >= kSmallBatch ? kBigRunLarge : kBigRunSmall,
+              t->s.small_p3, t->s.long_runs, t->s.nodes, t->s.items, t->s.partial, t->s.node_cnt,
+              (uint32_t)t->s.max_long, (uint32_t)t->s.max_nodes, (uint32_t)t->s.max_items,
+              n >= kSmallBatch ? kChunkLarge : kChunkSmall,
               ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}, t->cfg.lr, t->cfg.eps};
     // a warp per 32 positions, the windows dealt out grid-stride over at most
     // one wave of blocks
-#ifndef MLKV_HEADS_ONE_WAVE
-#define MLKV_HEADS_ONE_WAVE 1
-#endif
-    const int64_t cap = MLKV_HEADS_ONE_WAVE ? persistent_blocks(t, (const void*)k_heads, 256) : (int64_t)t->num_sms * 8;
+    const int64_t cap = persistent_blocks(t, (const void*)k_heads, 256);
     int64_t gh = (n + 255) / 256;
     if (gh > cap) gh = cap;
     if (gh < 1) gh = 1;
     MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_heads, (unsigned)gh, 256, 0, st, a);
     // The runs of one lookup, of 2 .. kSmallRun and of up to
-    // MLKV_SEQ_SEGMENT_MAX lookups, and the long runs (chunk sums, then their
-    // combine) touch disjoint rows and scratch: they run on three streams at
-    // once, each filling the others' tails, and join at the end of the call;
-    // the last kernel of each stream releases the counters they read.
+    // MLKV_SEQ_SEGMENT_MAX lookups, and the long runs touch disjoint rows and
+    // scratch: they run on three streams at once, each filling the others'
+    // tails, and join at the end of the call; the last kernel of each stream
+    // releases the counters they read.  While a kernel class is being timed
+    // (mlkv_time_kernel) they run one after another: on three streams a
+    // kernel's events would also span the time it waits for the SMs the others
+    // hold.
     cudaStream_t s1 = st, s2 = st;
-    // While a kernel class is being timed (mlkv_time_kernel) the reduce kernels
-    // run one after another: on three streams a kernel's events would also
-    // span the time it waits for the SMs the others hold.
-    const bool branches = MLKV_REDUCE_BRANCHES && t->timer.kernel_id == 0;
+    const bool branches = t->timer.kernel_id == 0;
     if (branches) {
         cudaError_t e;
         if ((e = cudaEventRecord(t->ev_fork, st)) != cudaSuccess ||
@@ -964,48 +983,31 @@ cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* srow, 
         s1 = t->branch[0];
         s2 = t->branch[1];
     }
-    const int gl = persistent_blocks(t, (const void*)k_long_sum<V, KV>, 256);
-    const int g2 = persistent_blocks(t, (const void*)k_small<V, KV>, 256);
-    const bool narrow = MLKV_NARROW_ROWS && t->geom.G <= 16;
-    const void* short_k = narrow ? (const void*)k_short<V, KV, 4> : (const void*)k_short<V, KV>;
-    const void* single_k = narrow ? (const void*)k_single<V, KV, 2> : (const void*)k_single<V, KV>;
-    const int gs = persistent_blocks(t, short_k, 256);
-    int g1 = persistent_blocks(t, single_k, 256);
-    if (MLKV_SINGLE_PER_SM > 0 && g1 > MLKV_SINGLE_PER_SM * t->num_sms) g1 = MLKV_SINGLE_PER_SM * t->num_sms;
+    const bool narrow = t->geom.G <= 16;
+    const RunKernels k = run_kernels<V>(nseg > 1, narrow);
+    const int gl = persistent_blocks(t, (const void*)k.longs, 256);
+    const int g2 = persistent_blocks(t, (const void*)k.smalls, 256);
+    const int gs = persistent_blocks(t, (const void*)k.shorts, 256);
+    int g1 = persistent_blocks(t, (const void*)k.singles, 256);
     if (narrow && g1 > 3 * t->num_sms) g1 = 3 * t->num_sms;
-    // the combine's block (MLKV_COMBINE_THREADS): the groups' (sum,
-    // compensation) pairs must fit the default 48 KB of shared memory
-    int big = MLKV_COMBINE_THREADS;
-    while (big > 64 && (size_t)(big / t->geom.G) * 2 * t->geom.dpad * sizeof(float) > 48 * 1024) big /= 2;
-    const size_t smem = (size_t)(big / t->geom.G) * 2 * t->geom.dpad * sizeof(float);
-    // 1024 threads per SM: 4,864 lane groups of 32 for the ordinary long runs
-    const int gc = t->num_sms * (1024 / big);
-    // The counters are released by the apply's last kernels: the last of each
-    // stream (the combine, the last of the runs of 2-4 and of 5-32, the runs
-    // of one), or the combine alone when all run in stream order.
+    // In a call of fewer than kSmallBatch lookups the runs of 5-32 (the longest
+    // per run of the three) go before those of 2-4: they would otherwise be last
+    // to start, after the runs of one had filled the SMs.
+    const bool short_first = n < (int64_t)kSmallBatch;
     RunArgs last = a;
-    const bool short_first = MLKV_SHORT_FIRST == 1 || (MLKV_SHORT_FIRST == 2 && n < (int64_t)kSmallBatch);
-    last.release = (uint32_t)(gc + (branches ? g1 + (short_first ? g2 : gs) : 0));
+    const int gc = t->num_sms * 4;  // 1024 threads per SM
+    last.release = branches ? (uint32_t)(gc + g1 + (short_first ? g2 : gs)) : (uint32_t)g1;
     const RunArgs& tail = branches ? last : a;
-    const cudaStream_t s_long = s2, s_single = st;
-    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_LONG, (k_long_sum<V, KV>), gl, 256, 0, s_long, ra, a);
-    if (branches)
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_LONG_COMBINE, (k_long_combine<V, KV>), gc, big, smem, s_long, ra, last,
-                               t->dstate);
+    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_LONG, k.longs, gl, 256, 0, s2, ra, a);
+    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_LONG_COMBINE, (k_combine<V>), gc, kCombineThreads, 0, s2, ra, tail, t->dstate);
     if (short_first) {
-        // the runs of 5-32 (the longest per run of the three) before those of
-        // 2-4: in a small batch the runs of 5-32 would otherwise be last to
-        // start, after the runs of one had filled the SMs
-        launch_short<V, KV>(t, narrow, gs, s1, ra, a);
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SMALL, (k_small<V, KV>), g2, 256, 0, s1, ra, tail);
+        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SHORT, k.shorts, gs, 256, 0, s1, ra, a);
+        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SMALL, k.smalls, g2, 256, 0, s1, ra, tail);
     } else {
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SMALL, (k_small<V, KV>), g2, 256, 0, s1, ra, a);
-        launch_short<V, KV>(t, narrow, gs, s1, ra, tail);
+        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SMALL, k.smalls, g2, 256, 0, s1, ra, a);
+        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SHORT, k.shorts, gs, 256, 0, s1, ra, tail);
     }
-    if (narrow)
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SINGLE, (k_single<V, KV, 2>), g1, 256, 0, s_single, ra, tail);
-    else
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SINGLE, (k_single<V, KV>), g1, 256, 0, s_single, ra, tail);
+    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SINGLE, k.singles, g1, 256, 0, st, ra, last);
     if (branches) {
         cudaError_t e;
         if ((e = cudaEventRecord(t->ev_join[0], s1)) != cudaSuccess ||
@@ -1013,41 +1015,33 @@ cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* srow, 
             (e = cudaStreamWaitEvent(st, t->ev_join[0], 0)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(st, t->ev_join[1], 0)) != cudaSuccess)
             return e;
-    } else {
-        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_LONG_COMBINE, (k_long_combine<V, KV>), gc, big, smem, st, ra, last,
-                               t->dstate);
     }
     return cudaGetLastError();
 }
 
 }  // namespace
 
-int64_t long_runs_bound(int64_t max_batch) { return max_batch / (MLKV_SEQ_SEGMENT_MAX + 1) + 1; }
-
-int64_t long_items_bound(int64_t max_batch) {
-    // chunks of kChunkLarge lookups in calls of at least kSmallBatch lookups, of kChunkSmall below
+void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& items) {
+    // chunks of kChunkLarge lookups in calls of at least kSmallBatch lookups, of
+    // kChunkSmall (or kChunkLarge) below, and one partial chunk per long run
     const int64_t small = std::min<int64_t>(max_batch, (int64_t)kSmallBatch - 1) / kChunkSmall;
-    return std::max<int64_t>(max_batch / kChunkLarge, small) + long_runs_bound(max_batch) + 1;
+    runs = max_batch / (MLKV_SEQ_SEGMENT_MAX + 1) + 1;
+    items = std::max<int64_t>(max_batch / kChunkLarge, small) + runs + 1;
+    // a run cut into nodes has more than kGroupChunks chunks, one partial node
+    nodes = items / kNode + items / (kGroupChunks + 1) + 2;
+}
+
+int64_t node_counters(int64_t max_items, int dim) {
+    // segments per row of the widest split: the scalar kernels' (dim <= 256) or the float4 kernels'
+    const int64_t nseg = std::max<int64_t>((std::min(dim, 256) + 31) / 32, (dim + 127) / 128);
+    return max_items * nseg;
 }
 
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
                                 const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
                                 CallCounters* cur) {
-    const RowGeom& g = t->geom;
-    if (g.V == 4) {
-        switch (g.KV) {
-            case 1: return run_reduce<4, 1>(t, grads, srow, spos, n, sent, st, cur);
-            case 2: return run_reduce<4, 2>(t, grads, srow, spos, n, sent, st, cur);
-            case 4: return run_reduce<4, 4>(t, grads, srow, spos, n, sent, st, cur);
-            default: return run_reduce<4, 8>(t, grads, srow, spos, n, sent, st, cur);
-        }
-    }
-    switch (g.KV) {
-        case 1: return run_reduce<1, 1>(t, grads, srow, spos, n, sent, st, cur);
-        case 2: return run_reduce<1, 2>(t, grads, srow, spos, n, sent, st, cur);
-        case 4: return run_reduce<1, 4>(t, grads, srow, spos, n, sent, st, cur);
-        default: return run_reduce<1, 8>(t, grads, srow, spos, n, sent, st, cur);
-    }
+    return t->geom.V == 4 ? run_reduce<4>(t, grads, srow, spos, n, sent, st, cur)
+                          : run_reduce<1>(t, grads, srow, spos, n, sent, st, cur);
 }
 
 }  // namespace mlkv

@@ -56,10 +56,11 @@ struct CallCounters {
     uint32_t n_valid;    // lookups with a row
     uint32_t n_long;     // runs longer than MLKV_SEQ_SEGMENT_MAX
     uint32_t n_items;    // chunks of the long runs
+    uint32_t n_group;    // long runs combined by a lane group
+    uint32_t n_nodes;    // nodes of the other long runs
     uint32_t n_short;    // runs of at most MLKV_SEQ_SEGMENT_MAX lookups
-    uint32_t n_big;      // long runs whose chunk sums are combined by the wide blocks
     uint32_t n_single;   // runs of one lookup
-    uint32_t short_next; // next chunk of short runs to claim (k_short's dynamic hand-out)
+    uint32_t short_next;  // run segments claimed (k_short's dynamic hand-out)
     uint32_t n_small;    // runs of 2 .. kSmallRun lookups (their positions in the record)
     uint32_t bar[4];     // arrivals at the miss kernel's grid barriers
     uint32_t done;       // blocks of the call's last kernel that have finished (release_counters)
@@ -113,16 +114,15 @@ struct Scratch {
     uint2* single_runs;     // [max_batch] its runs of one lookup: (row, lookup position)
     uint4* small_runs;      // [max_batch] runs of 2 .. kSmallRun lookups: (row, p0, p1, p2)
     uint32_t* small_p3;     // [max_batch] their fourth position (or none)
-    uint32_t* long_s;       // [max_long] long runs: first sorted position
-    uint32_t* long_e;       // [max_long] one past the last
-    uint32_t* long_row;     // [max_long]
-    uint32_t* long_base;    // [max_long] first chunk item
-    uint32_t* item_s;       // [max_items] first sorted position of each chunk
-    uint32_t* item_e;       // [max_items] one past its last
-    uint32_t* big_runs;     // [max_long] long runs with many chunks (combined by wide blocks)
+    uint4* long_runs;       // [max_long] long runs of few chunks (RunArgs)
+    uint4* nodes;           // [max_nodes] nodes of the other long runs
+    uint4* items;           // [max_items] chunks of the long runs
     float* partial;         // [max_items][2][dpad] chunk sums: compensated (sum, compensation) pairs
+    uint32_t* node_cnt;     // [node_counters()] counts of the long runs' combine, zero at rest
     int64_t max_long;
+    int64_t max_nodes;
     int64_t max_items;
+    int64_t node_cnt_bytes;
     int64_t tile_sums_len;
     int64_t sort_counts_bytes;
 };
@@ -193,9 +193,9 @@ struct mlkv_table {
     cudaEvent_t* ev_apply;       // [ring]: apply number j records ev_apply[j % ring]
     cudaEvent_t ev_other;        // after the last call other than an apply
     int other_recorded;
-    // The apply's independent reduce kernels run on the call's stream and
-    // these, forked after the run lists are made and joined before the long
-    // runs' combine.
+    // The apply's reduce kernels of a call of many lookups run on the call's
+    // stream and these, forked after the run lists are made and joined at the
+    // end of the call.
     cudaStream_t branch[2];
     cudaEvent_t ev_fork;
     cudaEvent_t ev_join[2];
@@ -515,8 +515,9 @@ cudaError_t launch_tier_init(mlkv_table* t, cudaStream_t st);
 cudaError_t launch_gather_lines(mlkv_table* t, const uint32_t* rows, int64_t n, float* out, cudaStream_t st);
 
 // mlkv_apply.cu
-int64_t long_runs_bound(int64_t max_batch);   // runs longer than MLKV_SEQ_SEGMENT_MAX, worst case
-int64_t long_items_bound(int64_t max_batch);  // chunks of those runs, worst case
+// Runs longer than MLKV_SEQ_SEGMENT_MAX, their combine's nodes, and their chunks, worst case.
+void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& items);
+int64_t node_counters(int64_t max_items, int dim);  // counters of the combine's nodes
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
                                 const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
                                 CallCounters* cur);

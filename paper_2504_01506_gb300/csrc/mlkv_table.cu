@@ -573,8 +573,8 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
     // Scratch arena, carved in 256-byte aligned pieces.
     const int64_t B = c.max_batch;
     Scratch& s = t->s;
-    s.max_long = long_runs_bound(B);
-    s.max_items = long_items_bound(B);
+    long_bounds(B, s.max_long, s.max_nodes, s.max_items);
+    s.node_cnt_bytes = node_counters(s.max_items, c.dim) * 4;
     s.tile_sums_len = std::max<int64_t>(tiles_of(B) + 1, t->num_sms);
     // the sort's tiles: 4096 lookups, 1024 in batches under kSortSmallBatch
     const int64_t sort_tiles = std::max<int64_t>(
@@ -595,11 +595,9 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.sort_counts2, 512 * sort_tiles * 4},
         {(void**)&s.sort_offsets, 512 * sort_tiles * 4},
         {(void**)&s.sort_dtot, kSortMaxPasses * 512 * 4},
-        {(void**)&s.seg_start, (B + 1) * 4},  {(void**)&s.long_s, s.max_long * 4},
-        {(void**)&s.long_e, s.max_long * 4},   {(void**)&s.long_row, s.max_long * 4},
-        {(void**)&s.long_base, s.max_long * 4}, {(void**)&s.item_s, s.max_items * 4},
-        {(void**)&s.item_e, s.max_items * 4},   {(void**)&s.run_row, B * 4},
-        {(void**)&s.big_runs, s.max_long * 4},
+        {(void**)&s.seg_start, (B + 1) * 4},  {(void**)&s.run_row, B * 4},
+        {(void**)&s.long_runs, s.max_long * 16}, {(void**)&s.nodes, s.max_nodes * 16},
+        {(void**)&s.items, s.max_items * 16}, {(void**)&s.node_cnt, s.node_cnt_bytes},
         {(void**)&s.short_runs, B * 16},
         {(void**)&s.single_runs, B * 8},
         {(void**)&s.small_runs, B * 16},
@@ -914,6 +912,7 @@ int mlkv_clear_status(mlkv_table* t) {
     CK(t, cudaMemset(t->s.sort_counts, 0, t->s.sort_counts_bytes));
     CK(t, cudaMemset(t->s.sort_counts2, 0, t->s.sort_counts_bytes));
     CK(t, cudaMemset(t->s.sort_dtot, 0, kSortMaxPasses * 512 * 4));
+    CK(t, cudaMemset(t->s.node_cnt, 0, (size_t)t->s.node_cnt_bytes));
     CK(t, cudaDeviceSynchronize());
     *(volatile uint32_t*)t->status_host = 0;
     t->last_error[0] = 0;
