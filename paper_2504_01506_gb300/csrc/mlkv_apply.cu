@@ -1040,8 +1040,9 @@ int64_t node_counters(int64_t max_items, int dim) {
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
                                 const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
                                 CallCounters* cur) {
-    return t->geom.V == 4 ? run_reduce<4>(t, grads, srow, spos, n, sent, st, cur)
-                          : run_reduce<1>(t, grads, srow, spos, n, sent, st, cur);
+    if (t->geom.V == 4) return run_reduce<4>(t, grads, srow, spos, n, sent, st, cur);
+    if (t->geom.V == 2) return run_reduce<2>(t, grads, srow, spos, n, sent, st, cur);
+    return run_reduce<1>(t, grads, srow, spos, n, sent, st, cur);
 }
 
 }  // namespace mlkv

@@ -185,46 +185,48 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
 }
 
 // Group-cooperative copy of one row (or NaN) into dst.
-template <int V, int KV>
+template <int V>
 __device__ __forceinline__ void copy_row(const float* __restrict__ src, float* __restrict__ dst,
                                          int NV, int G, int glane, bool absent) {
     using VT = typename Vec<V>::T;
     const VT* s = reinterpret_cast<const VT*>(src);
     VT* o = reinterpret_cast<VT*>(dst);
-#pragma unroll
-    for (int k = 0; k < KV; ++k) {
-        const int j = glane + G * k;
-        if (j < NV) __stcs(o + j, absent ? Vec<V>::nan() : __ldg(s + j));
-    }
+#pragma unroll 2
+    for (int j = glane; j < NV; j += G) __stcs(o + j, absent ? Vec<V>::nan() : __ldg(s + j));
 }
 
-// The fused Get: each warp probes 32 consecutive lookups (one per lane), then
-// its lane groups gather the 32 rows with vector loads, streaming the output.
-// Lookups of new keys are left to the miss path.
+// The fused Get: each warp probes `lpw` consecutive lookups (one per lane), then
+// its lane groups gather their rows with vector loads, streaming the output.
+// Lookups of new keys are left to the miss path.  A row wider than 32 vectors
+// (SEG) is copied two vectors a lane at a time, whatever its dim: with all of
+// them in flight (4 a lane at dim 512) the kernel spilled at the 32 registers
+// that let 64 warps reside on an SM (65,536 lookups of dim 512: 49 us, 39 so;
+// 48 warps of 40 registers for these rows: 64 spill again and cost 524k rows of
+// 1 KiB 5 us).
 // Tuning (set at build time): minimum resident blocks per SM for the Get
-// kernel's register allocation, and rows each lane group has in flight.
+// kernel's register allocation.
 #ifndef MLKV_GET_MIN_BLOCKS
 #define MLKV_GET_MIN_BLOCKS 8
 #endif
-#ifndef MLKV_GET_ROWS_IN_FLIGHT
-#define MLKV_GET_ROWS_IN_FLIGHT 1
+#ifndef MLKV_GET_SEG_MIN_BLOCKS
+#define MLKV_GET_SEG_MIN_BLOCKS 6
 #endif
 
-template <int V, int KV, bool INSERT>
-__global__ void __launch_bounds__(256, MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, RowArgs ra,
+template <int V, bool SEG, bool INSERT>
+__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, RowArgs ra,
                                              const int64_t* __restrict__ keys, uint32_t n,
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
-                                             CallCounters* nxt, Memo memo) {
+                                             CallCounters* nxt, Memo memo, int lpw) {
     pdl_enter();
     using VT = typename Vec<V>::T;
     zero_counters(nxt);
     const int lane = threadIdx.x & 31;
-    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u;
+    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     if (base >= n) return;  // warp-uniform
     const uint32_t p = base + lane;
     uint32_t row = ROW_PENDING;  // lanes past the end skip the gather
-    if (p < n) {
+    if (lane < lpw && p < n) {
         uint32_t slot = 0;
         const int64_t key = keys[p];
         row = probe_key<INSERT>(ia, (unsigned long long)key, p, slot);
@@ -233,36 +235,33 @@ __global__ void __launch_bounds__(256, MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, 
         memo.key[p] = key;
         memo.row[p] = row;
     }
-    const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
-    constexpr int UNR = KV >= MLKV_GET_ROWS_IN_FLIGHT ? 1 : MLKV_GET_ROWS_IN_FLIGHT / KV;
-    for (int it0 = 0; it0 < G; it0 += UNR) {
-        VT v[UNR][KV];
-        uint32_t rr[UNR];
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int q = (it0 + u) * R + gid;
-            const uint32_t r = __shfl_sync(0xffffffffu, row, q & 31);
-            rr[u] = (it0 + u < G) ? r : ROW_PENDING;
-            if (rr[u] < ROW_ABSENT) {
-                const VT* src = reinterpret_cast<const VT*>(ra.slots + (size_t)rr[u] * ra.stride);
-#pragma unroll
-                for (int k = 0; k < KV; ++k) {
-                    const int j = glane + G * k;
-                    if (j < ra.NV) v[u][k] = __ldg(src + j);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (rr[u] == ROW_PENDING) continue;
-            const int q = (it0 + u) * R + gid;
+    if (SEG) {
+        for (int q = 0; q < lpw; ++q) {
+            const uint32_t r = __shfl_sync(0xffffffffu, row, q);
+            if (r == ROW_PENDING) continue;
+            const VT* src = reinterpret_cast<const VT*>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride);
             VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q) * ra.d);
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                const int j = glane + G * k;
-                if (j < ra.NV) __stcs(dst + j, rr[u] == ROW_ABSENT ? Vec<V>::nan() : v[u][k]);
+            for (int j0 = 0; j0 < ra.NV; j0 += 64) {  // uniform
+                const int j = j0 + lane, k = j + 32;
+                VT v0, v1;
+                if (j < ra.NV) v0 = __ldg(src + j);
+                if (k < ra.NV) v1 = __ldg(src + k);
+                if (j < ra.NV) __stcs(dst + j, r == ROW_ABSENT ? Vec<V>::nan() : v0);
+                if (k < ra.NV) __stcs(dst + k, r == ROW_ABSENT ? Vec<V>::nan() : v1);
             }
         }
+        return;
+    }
+    const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
+    for (int q0 = 0; q0 < lpw; q0 += R) {
+        const int q = q0 + gid;
+        const uint32_t r = __shfl_sync(0xffffffffu, row, q);
+        VT v;
+        if (r < ROW_ABSENT && glane < ra.NV)
+            v = __ldg(reinterpret_cast<const VT*>(ra.slots + (size_t)r * ra.stride) + glane);
+        if (r == ROW_PENDING) continue;
+        VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q) * ra.d);
+        if (glane < ra.NV) __stcs(dst + glane, r == ROW_ABSENT ? Vec<V>::nan() : v);
     }
 }
 
@@ -452,7 +451,7 @@ __device__ __forceinline__ uint32_t miss_block_scan(uint32_t v, uint32_t& total)
     return before + x - v;
 }
 
-template <int V, int KV>
+template <int V>
 __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, RowArgs ra, const int64_t* __restrict__ keys,
                                                        uint32_t n, const uint32_t* __restrict__ miss_pos,
                                                        const uint32_t* __restrict__ miss_slot,
@@ -531,10 +530,7 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, RowArgs ra,
         float* w = ra.slots + (size_t)r * ra.stride;
         VT* wv = reinterpret_cast<VT*>(w);
         VT* gv = reinterpret_cast<VT*>(w + ra.dpad);
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            const int j = glane + G * k;
-            if (j >= ra.NV) continue;
+        for (int j = glane; j < ra.NV; j += G) {
             if (init_row) {
                 float e[V];
 #pragma unroll
@@ -566,7 +562,7 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, RowArgs ra,
             }
         }
         if (out)
-            copy_row<V, KV>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride,
+            copy_row<V>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride,
                             out + (size_t)p * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
     }
     if (release) release_counters(cur, gridDim.x);
@@ -582,7 +578,10 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, RowArgs ra,
 // the hot keys, the others find them marked.  kMarkPerSm = 2 blocks of 256
 // threads per SM: more make the first round's burst longer, fewer leave too few
 // reads in flight.
-constexpr int kMarkPerSm = 2;
+#ifndef MLKV_MARK_PER_SM
+#define MLKV_MARK_PER_SM 2
+#endif
+constexpr int kMarkPerSm = MLKV_MARK_PER_SM;
 __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, const uint32_t* __restrict__ row_of_pos,
                                                   const uint32_t* __restrict__ slot_of_pos, uint32_t n) {
     pdl_enter();
@@ -605,48 +604,65 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
     }
 }
 
-// Put 2/2: the winning occurrence writes the row and puts aux back to idle.
-template <int V, int KV>
+// Put 2/2: the winning occurrence writes the row and puts aux back to idle.  A
+// warp finds the winners among its lpw lookups, one per lane (row and slot, then
+// the slot's mark), and its lane groups copy their rows, kPutRows vectors a lane
+// in flight.  (With a lane group walking its lookups one by one, each copy
+// waited for its own mark: 75 us for 524k Puts of 1 KiB, Zipf(0.99); 70 so, 88
+// with 2 vectors in flight.)
+#ifndef MLKV_PUT_ROWS
+#define MLKV_PUT_ROWS 4
+#endif
+template <int V>
 __global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, RowArgs ra,
                                                      const uint32_t* __restrict__ row_of_pos,
                                                      const uint32_t* __restrict__ slot_of_pos,
                                                      const float* __restrict__ vals,
-                                                     const float* __restrict__ state, uint32_t n) {
+                                                     const float* __restrict__ state, uint32_t n, int lpw) {
     pdl_enter();
     using VT = typename Vec<V>::T;
-    const int lane = threadIdx.x & 31, G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
-    const uint32_t warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
-    for (uint32_t b = warp * R; b < n; b += nwarps * R) {  // warp-uniform
-        const uint32_t p = b + gid;
-        bool win = false;
-        uint32_t r = 0, s = 0;
-        if (p < n) {
-            r = row_of_pos[p];
-            s = slot_of_pos[p];
-            win = r < ROW_ABSENT && index[s].aux == 0xFFFFFFFEu - p;
-        }
-        __syncwarp();
-        if (win) {
-            const VT* src = reinterpret_cast<const VT*>(vals + (size_t)p * ra.d);
-            VT* dst = reinterpret_cast<VT*>(ra.slots + (size_t)r * ra.stride);
-#pragma unroll
-            for (int k = 0; k < KV; ++k) {
-                const int j = glane + G * k;
-                if (j < ra.NV) dst[j] = __ldg(src + j);
-            }
-            if (state) {  // import: the state too
-                const VT* ssrc = reinterpret_cast<const VT*>(state + (size_t)p * ra.d);
-                VT* sdst = reinterpret_cast<VT*>(ra.slots + (size_t)r * ra.stride + ra.dpad);
-#pragma unroll
-                for (int k = 0; k < KV; ++k) {
-                    const int j = glane + G * k;
-                    if (j < ra.NV) sdst[j] = __ldg(ssrc + j);
-                }
-            }
-            if (glane == 0) index[s].aux = AUX_IDLE;
+    constexpr int kPutRows = MLKV_PUT_ROWS;
+    __shared__ uint2 wins[8][32];  // (row, lookup) of the warp's winners
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
+    const uint32_t p = (blockIdx.x * (blockDim.x >> 5) + wib) * (uint32_t)lpw + lane;
+    bool win = false;
+    uint32_t r = 0;
+    if (lane < lpw && p < n) {
+        r = __ldg(row_of_pos + p);
+        const uint32_t s = __ldg(slot_of_pos + p);
+        if (r < ROW_ABSENT && index[s].aux == 0xFFFFFFFEu - p) {
+            win = true;
+            index[s].aux = AUX_IDLE;  // its other lookups hold other marks
         }
     }
+    const unsigned m = __ballot_sync(0xffffffffu, win);
+    if (win) wins[wib][__popc(m & lanemask_lt())] = make_uint2(r, p);
+    __syncwarp();
+    // vectors of the winners' rows, G at a time: segment x of the list
+    const int nseg = (ra.NV + G - 1) / G, items = __popc(m) * nseg;
+    auto copy = [&](const float* __restrict__ src, int off) {
+        for (int x0 = 0; x0 < items; x0 += R * kPutRows) {  // uniform
+            VT v[kPutRows];
+            VT* to[kPutRows];
+#pragma unroll
+            for (int i = 0; i < kPutRows; ++i) {
+                const int x = x0 + i * R + gid;
+                const int w = nseg == 1 ? x : x / nseg, j = glane + (x - w * nseg) * G;
+                to[i] = nullptr;
+                if (x < items && j < ra.NV) {
+                    const uint2 rp = wins[wib][w];
+                    v[i] = __ldcs(reinterpret_cast<const VT*>(src + (size_t)rp.y * ra.d) + j);
+                    to[i] = reinterpret_cast<VT*>(ra.slots + (size_t)rp.x * ra.stride + off) + j;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kPutRows; ++i)
+                if (to[i]) *to[i] = v[i];
+        }
+    };
+    copy(vals, 0);
+    if (state) copy(state, ra.dpad);  // import: the state too
 }
 
 __global__ void __launch_bounds__(256) k_find(IndexArgs ia, const int64_t* __restrict__ keys,
@@ -670,26 +686,27 @@ struct ExportTier {
     const float* host;
 };
 
-template <int V, int KV>
+template <int V>
 __global__ void __launch_bounds__(256) k_export(IndexArgs ia, RowArgs ra,
                                                 const int64_t* __restrict__ keys, uint32_t n,
                                                 float* __restrict__ rows_out,
                                                 float* __restrict__ state_out, CallCounters* nxt,
-                                                ExportTier et) {
+                                                ExportTier et, int lpw) {
     pdl_enter();
+    using VT = typename Vec<V>::T;
     zero_counters(nxt);
     const int lane = threadIdx.x & 31;
-    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u;
+    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     if (base >= n) return;
     const uint32_t p = base + lane;
     uint32_t row = ROW_PENDING;
-    if (p < n) {
+    if (lane < lpw && p < n) {
         uint32_t slot = 0;
         row = probe_key<false>(ia, (unsigned long long)keys[p], p, slot);
     }
     const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
-    for (int it = 0; it < G; ++it) {
-        const int q = it * R + gid;
+    for (int q0 = 0; q0 < lpw; q0 += R) {
+        const int q = q0 + gid;
         const uint32_t r = __shfl_sync(0xffffffffu, row, q);
         if (r == ROW_PENDING) continue;
         const float* src = ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride;
@@ -697,29 +714,25 @@ __global__ void __launch_bounds__(256) k_export(IndexArgs ia, RowArgs ra,
             const uint32_t l = et.row_loc[r];
             src = l < LOC_HOST ? et.cache + (size_t)l * ra.stride : et.host + (size_t)(l & ~LOC_HOST) * ra.stride;
         }
-        if (rows_out) copy_row<V, KV>(src, rows_out + (size_t)(base + q) * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
-        if (state_out)
-            copy_row<V, KV>(src + ra.dpad, state_out + (size_t)(base + q) * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
+        const VT* ws = reinterpret_cast<const VT*>(src);
+        const VT* gs = reinterpret_cast<const VT*>(src + ra.dpad);
+        for (int j = glane; j < ra.NV; j += G) {  // row and state in flight together
+            VT w, g;
+            if (rows_out) w = __ldg(ws + j);
+            if (state_out) g = __ldg(gs + j);
+            const size_t o = (size_t)(base + q) * ra.d;
+            if (rows_out) __stcs(reinterpret_cast<VT*>(rows_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : w);
+            if (state_out) __stcs(reinterpret_cast<VT*>(state_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : g);
+        }
     }
 }
 
-// Dispatch over (V, KV) for the row kernels.
-template <template <int, int> class F, typename... A>
+// Dispatch over V for the row kernels.
+template <template <int> class F, typename... A>
 cudaError_t dispatch_row(const RowGeom& g, A&&... a) {
-    if (g.V == 4) {
-        switch (g.KV) {
-            case 1: return F<4, 1>::run(a...);
-            case 2: return F<4, 2>::run(a...);
-            case 4: return F<4, 4>::run(a...);
-            default: return F<4, 8>::run(a...);
-        }
-    }
-    switch (g.KV) {
-        case 1: return F<1, 1>::run(a...);
-        case 2: return F<1, 2>::run(a...);
-        case 4: return F<1, 4>::run(a...);
-        default: return F<1, 8>::run(a...);
-    }
+    if (g.V == 4) return F<4>::run(a...);
+    if (g.V == 2) return F<2>::run(a...);
+    return F<1>::run(a...);
 }
 
 inline unsigned grid_for(int64_t items, int per_block) {
@@ -757,7 +770,7 @@ int bulk_grid(mlkv_table* t, size_t smem, int64_t n) {
     return (int)(g < cap ? g : cap);
 }
 
-template <int V, int KV>
+template <int V>
 struct GetRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* out,
                            cudaStream_t st, CallCounters* cur, CallCounters* nxt) {
@@ -774,27 +787,25 @@ struct GetRun {
                             t->s.miss_slot, cur, nxt, Memo{t->s.memo_key, t->s.memo_row});
             return cudaGetLastError();
         }
-        const unsigned grid = grid_for(n, 256);  // 8 warps x 32 lookups per block
-        if (t->cfg.insert_on_miss)
-            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, (k_get<V, KV, true>), grid, 256, 0, st, index_args(t),
-                        row_args(t), keys, (uint32_t)n, out, t->s.miss_pos, t->s.miss_slot, cur, nxt,
-                        Memo{t->s.memo_key, t->s.memo_row});
-        else
-            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, (k_get<V, KV, false>), grid, 256, 0, st, index_args(t),
-                        row_args(t), keys, (uint32_t)n, out, t->s.miss_pos, t->s.miss_slot, cur, nxt,
-                        Memo{t->s.memo_key, t->s.memo_row});
+        const bool seg = t->geom.NV > t->geom.G, ins = t->cfg.insert_on_miss != 0;
+        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
+        const auto kernel = seg ? (ins ? k_get<V, true, true> : k_get<V, true, false>)
+                                : (ins ? k_get<V, false, true> : k_get<V, false, false>);
+        MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t), row_args(t), keys,
+                    (uint32_t)n, out, t->s.miss_pos, t->s.miss_slot, cur, nxt, Memo{t->s.memo_key, t->s.memo_row},
+                    lpw);
         return cudaGetLastError();
     }
 };
 
-template <int V, int KV>
+template <int V>
 struct MissRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode, float* out,
                            cudaStream_t st, CallCounters* cur, bool release, const FirstCounts* fc) {
         const float span = t->cfg.init_hi - t->cfg.init_lo;
         RowArgs init_ra = row_args(t);  // new rows live in the host tier when tiered
         if (t->tiered) init_ra.slots = t->tier.host_dev;
-        MLKV_LAUNCH(t, 0, (k_miss<V, KV>), t->num_sms, kMissThreads, 0, st, index_args(t), init_ra, keys,
+        MLKV_LAUNCH(t, 0, (k_miss<V>), t->num_sms, kMissThreads, 0, st, index_args(t), init_ra, keys,
                     (uint32_t)n, t->s.miss_pos, t->s.miss_slot, t->s.first_flag, t->s.rank, t->s.tile_sums,
                     mode == MissMode::Get ? nullptr : t->s.row_of_pos, mode == MissMode::Get ? out : nullptr, cur,
                     t->dstate, (unsigned long long)t->cfg.capacity, mode == MissMode::Put ? 0 : 1,
@@ -804,14 +815,14 @@ struct MissRun {
     }
 };
 
-template <int V, int KV>
+template <int V>
 struct PutRun {
     static cudaError_t run(mlkv_table* t, const float* vals, const float* state, int64_t n, cudaStream_t st) {
         MLKV_LAUNCH(t, 0, k_put_mark, capped_grid(t, n, 256, kMarkPerSm), 256, 0, st, t->index, t->s.row_of_pos,
                     t->s.slot_of_pos, (uint32_t)n);
-        const unsigned g = capped_grid(t, n * (int64_t)t->geom.G, 256, 8);
-        MLKV_LAUNCH(t, MLKV_K_PUT_SCATTER, (k_put_scatter<V, KV>), g, 256, 0, st, t->index, row_args(t),
-                    t->s.row_of_pos, t->s.slot_of_pos, vals, state, (uint32_t)n);
+        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
+        MLKV_LAUNCH(t, MLKV_K_PUT_SCATTER, (k_put_scatter<V>), grid_for(n, 8 * lpw), 256, 0, st, t->index, row_args(t),
+                    t->s.row_of_pos, t->s.slot_of_pos, vals, state, (uint32_t)n, lpw);
         return cudaGetLastError();
     }
 };
@@ -829,14 +840,15 @@ __global__ void __launch_bounds__(256) k_dump_keys(const Slot* __restrict__ inde
     }
 }
 
-template <int V, int KV>
+template <int V>
 struct ExportRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* rows, float* state,
                            cudaStream_t st, CallCounters* nxt) {
         ExportTier et{nullptr, nullptr, nullptr};
         if (t->tiered) et = ExportTier{t->tier.row_loc, t->tier.cache, t->tier.host_dev};
-        MLKV_LAUNCH(t, 0, (k_export<V, KV>), grid_for(n, 256), 256, 0, st, index_args(t),
-                    row_args(t), keys, (uint32_t)n, rows, state, nxt, et);
+        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
+        MLKV_LAUNCH(t, 0, (k_export<V>), grid_for(n, 8 * lpw), 256, 0, st, index_args(t),
+                    row_args(t), keys, (uint32_t)n, rows, state, nxt, et, lpw);
         return cudaGetLastError();
     }
 };

@@ -76,13 +76,12 @@ struct DevState {
 };
 
 // Row-kernel geometry: a row of d floats is NV vectors of V floats; a group of
-// G lanes (a power of two <= 32) owns one row, each lane KV vectors of it.
+// G lanes (a power of two <= 32) takes one row, G vectors of it at a time.
 struct RowGeom {
     int d;        // dim
-    int V;        // 4 (float4) or 1
+    int V;        // 4 (float4), 2 or 1
     int NV;       // vectors per row
     int G;        // lanes per row
-    int KV;       // vectors per lane, 1/2/4/8
     int dpad;     // row and state stride inside a slot (floats, multiple of 8)
     int stride;   // floats per slot (row + state) = 2 * dpad
 };
@@ -389,10 +388,22 @@ template <> struct Vec<4> {
     }
     static __device__ __forceinline__ T splat(float v) { return make_float4(v, v, v, v); }
     static __device__ __forceinline__ T from(const float* e) { return make_float4(e[0], e[1], e[2], e[3]); }
-    static __device__ __forceinline__ T shfl_down(const T& v, int delta) {
-        return make_float4(__shfl_down_sync(0xffffffffu, v.x, delta), __shfl_down_sync(0xffffffffu, v.y, delta),
-                           __shfl_down_sync(0xffffffffu, v.z, delta), __shfl_down_sync(0xffffffffu, v.w, delta));
+};
+template <> struct Vec<2> {
+    using T = float2;
+    static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ T nan() {
+        float q = __int_as_float(0x7fc00000);
+        return make_float2(q, q);
     }
+    static __device__ __forceinline__ void add(T& a, const T& b) { a = add_x2(a, b); }
+    static __device__ __forceinline__ void cadd(T& s, T& c, const T& x) { comp_add_x2(s, c, x); }
+    static __device__ __forceinline__ void adagrad(T& w, T& G, const T& g, float lr, float eps) {
+        adagrad_element(w.x, G.x, g.x, lr, eps);
+        adagrad_element(w.y, G.y, g.y, lr, eps);
+    }
+    static __device__ __forceinline__ T splat(float v) { return make_float2(v, v); }
+    static __device__ __forceinline__ T from(const float* e) { return make_float2(e[0], e[1]); }
 };
 template <> struct Vec<1> {
     using T = float;
@@ -405,9 +416,6 @@ template <> struct Vec<1> {
     }
     static __device__ __forceinline__ T splat(float v) { return v; }
     static __device__ __forceinline__ T from(const float* e) { return e[0]; }
-    static __device__ __forceinline__ T shfl_down(const T& v, int delta) {
-        return __shfl_down_sync(0xffffffffu, v, delta);
-    }
 };
 
 // Programmatic dependent launch.  MLKV_LAUNCH lets a kernel start while the
@@ -521,6 +529,22 @@ int64_t node_counters(int64_t max_items, int dim);  // counters of the combine's
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
                                 const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
                                 CallCounters* cur);
+
+// Lookups per warp of the kernels that copy a warp's rows one after another: 32,
+// or as few as fill the GPU (kWarpsWanted warps per SM) in a small call, at
+// least `least` (the rows a warp copies at a time).  With 32 always, an export
+// of 100,003 rows of dim 50 ran on 20 warps per SM: 52 us, 20 with 8 lookups
+// (and 8-byte vectors); wanting 16 warps costs it 4 us, and a Get of 65,536
+// rows of dim 512 14.
+#ifndef MLKV_WARPS_WANTED
+#define MLKV_WARPS_WANTED 64
+#endif
+constexpr int kWarpsWanted = MLKV_WARPS_WANTED;
+inline int lookups_per_warp(const mlkv_table* t, int64_t n, int least) {
+    int lpw = 32;
+    while (lpw > least && lpw > 1 && n < (int64_t)lpw * t->num_sms * kWarpsWanted) lpw /= 2;
+    return lpw;
+}
 
 // mlkv_table.cu: launch bookkeeping and optional per-kernel timing; the host
 // side of mlkv_debug_fail's wait injection (true once, for the armed launch).

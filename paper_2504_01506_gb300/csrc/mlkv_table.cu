@@ -217,16 +217,13 @@ int next_pow2_int(int x) {
     return p;
 }
 
-// Row-kernel geometry for vector width V (4 needs dim % 4 == 0).
+// Row-kernel geometry for vector width V (needs dim % V == 0; below 4, dim <= 256).
 bool make_geom(int d, int V, RowGeom& g) {
-    if (V == 4 && d % 4) return false;
+    if (d % V || (V < 4 && d > 256)) return false;
     g.d = d;
     g.V = V;
-    g.NV = (d + V - 1) / V;
+    g.NV = d / V;
     g.G = next_pow2_int(g.NV) < 32 ? next_pow2_int(g.NV) : 32;
-    g.KV = (g.NV + g.G - 1) / g.G;
-    if (g.KV > 8) return false;
-    g.KV = g.KV <= 1 ? 1 : g.KV <= 2 ? 2 : g.KV <= 4 ? 4 : 8;
     g.dpad = (int)round_up(d, 8);
     g.stride = 2 * g.dpad;
     return true;
@@ -346,18 +343,13 @@ int check_call(mlkv_table* t, const void* keys, int64_t n, const void* buf, bool
     return n == 0 ? -1 : MLKV_OK;
 }
 
-// Chooses the float4 kernels when every row buffer of the call is 16-byte aligned.
+// Chooses the widest vectors that the dim and the alignment of every row buffer
+// of the call allow (the slots are 32-byte aligned): 16 bytes, 8 (an even dim:
+// at dim 50 a row is one load of 25 lanes instead of two of 32 and 18) or 4.
 int choose_geom(mlkv_table* t, const void* a, const void* b) {
-    const bool al = ((uintptr_t)a % 16 == 0) && ((uintptr_t)b % 16 == 0);
-    RowGeom g;
-    if (al && make_geom(t->cfg.dim, 4, g)) {
-        t->geom = g;
-        return MLKV_OK;
-    }
-    if (make_geom(t->cfg.dim, 1, g)) {
-        t->geom = g;
-        return MLKV_OK;
-    }
+    const uintptr_t al = (uintptr_t)a | (uintptr_t)b;
+    for (int V = 4; V >= 1; V /= 2)
+        if (al % (4 * V) == 0 && make_geom(t->cfg.dim, V, t->geom)) return MLKV_OK;
     return set_error(t, MLKV_ERR_INVALID, "dim %d needs 16-byte aligned row buffers", t->cfg.dim);
 }
 

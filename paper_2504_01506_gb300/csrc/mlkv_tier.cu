@@ -202,37 +202,35 @@ __global__ void __launch_bounds__(256) k_tier_remap(TierArgs ta, uint32_t* __res
     row_of_pos[p] = l < LOC_HOST ? l : ROW_ABSENT;
 }
 
-// Get from the cache: the warp's lane groups copy the rows of 32 lookups.
-template <int V, int KV>
+// Get from the cache: a warp's lane groups copy the rows of lpw lookups.
+template <int V>
 __global__ void __launch_bounds__(256) k_gather_lines(const float* __restrict__ slots, int stride, int d, int NV,
                                                       int G, const uint32_t* __restrict__ row_of_pos, uint32_t n,
-                                                      float* __restrict__ out) {
+                                                      float* __restrict__ out, int lpw) {
     pdl_enter();
     using VT = typename Vec<V>::T;
     const int lane = threadIdx.x & 31;
-    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u;
+    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     if (base >= n) return;
-    const uint32_t row = base + lane < n ? row_of_pos[base + lane] : ROW_PENDING;
+    const uint32_t row = lane < lpw && base + lane < n ? row_of_pos[base + lane] : ROW_PENDING;
     const int R = 32 / G, glane = lane & (G - 1), gid = lane / G;
-    for (int it = 0; it < G; ++it) {
-        const int q = it * R + gid;
+    for (int q0 = 0; q0 < lpw; q0 += R) {
+        const int q = q0 + gid;
         const uint32_t r = __shfl_sync(0xffffffffu, row, q);
         if (r == ROW_PENDING) continue;
         const VT* src = reinterpret_cast<const VT*>(slots + (size_t)(r < ROW_ABSENT ? r : 0) * stride);
         VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q) * d);
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {
-            const int j = glane + G * k;
-            if (j < NV) __stcs(dst + j, r >= ROW_ABSENT ? Vec<V>::nan() : __ldg(src + j));
-        }
+#pragma unroll 2
+        for (int j = glane; j < NV; j += G) __stcs(dst + j, r >= ROW_ABSENT ? Vec<V>::nan() : __ldg(src + j));
     }
 }
 
-template <int V, int KV>
+template <int V>
 cudaError_t run_gather(mlkv_table* t, const uint32_t* rows, int64_t n, float* out, cudaStream_t st) {
     const RowGeom& g = t->geom;
-    MLKV_LAUNCH(t, MLKV_K_GET_GATHER, (k_gather_lines<V, KV>), (unsigned)((n + 255) / 256), 256, 0, st, t->slots,
-                g.stride, g.d, g.NV, g.G, rows, (uint32_t)n, out);
+    const int lpw = lookups_per_warp(t, n, 32 / g.G);
+    MLKV_LAUNCH(t, MLKV_K_GET_GATHER, (k_gather_lines<V>), (unsigned)((n + 8 * lpw - 1) / (8 * lpw)), 256, 0, st,
+                t->slots, g.stride, g.d, g.NV, g.G, rows, (uint32_t)n, out, lpw);
     return cudaGetLastError();
 }
 
@@ -292,21 +290,9 @@ cudaError_t launch_tier_resolve(mlkv_table* t, const TierArgs& ta, uint32_t* row
 }
 
 cudaError_t launch_gather_lines(mlkv_table* t, const uint32_t* rows, int64_t n, float* out, cudaStream_t st) {
-    const RowGeom& g = t->geom;
-    if (g.V == 4) {
-        switch (g.KV) {
-            case 1: return run_gather<4, 1>(t, rows, n, out, st);
-            case 2: return run_gather<4, 2>(t, rows, n, out, st);
-            case 4: return run_gather<4, 4>(t, rows, n, out, st);
-            default: return run_gather<4, 8>(t, rows, n, out, st);
-        }
-    }
-    switch (g.KV) {
-        case 1: return run_gather<1, 1>(t, rows, n, out, st);
-        case 2: return run_gather<1, 2>(t, rows, n, out, st);
-        case 4: return run_gather<1, 4>(t, rows, n, out, st);
-        default: return run_gather<1, 8>(t, rows, n, out, st);
-    }
+    if (t->geom.V == 4) return run_gather<4>(t, rows, n, out, st);
+    if (t->geom.V == 2) return run_gather<2>(t, rows, n, out, st);
+    return run_gather<1>(t, rows, n, out, st);
 }
 
 }  // namespace mlkv
