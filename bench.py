@@ -283,6 +283,12 @@ def kernel_bytes(stats: dict, kid: int, sort_passes: int) -> float:
         return stats["B"] * 16.0  # per pass: (row id, position) read and written
     if kid == 2:
         return stats["B"] * 12.0 + stats["U"] * 32.0
+    if kid == 12:  # a small apply's runs of every length in one kernel
+        return (stats["reduce_short"] + stats["reduce_single"] + stats["reduce_small"] + stats["reduce_long"] +
+                stats["long_combine"])
+    if kid == 13:  # a small apply's probe, sort and run lists: keys read, index sectors, positions and records written
+        return (stats["B"] * 12.0 + stats["U"] * 32.0 + stats["U1"] * 8.0 + stats["Usm"] * 20.0 +
+                stats["Um"] * 16.0)
     if kid == 6:  # each sorted row id read twice and each position once; the run records written
         return stats["B"] * 12.0 + stats["U1"] * 8.0 + stats["Usm"] * 20.0 + stats["Um"] * 16.0
     return 0.0
@@ -292,16 +298,20 @@ KERNEL_NAMES = {1: "k_get (probe + row gather)", 2: "k_probe", 3: "k_sort_scatte
                 4: "k_short (run sum + Adagrad)", 5: "k_long (chunk sums of long runs)",
                 6: "k_heads (runs found in the sorted ids)", 7: "k_combine (chunk sums + Adagrad)",
                 8: "k_tier_fetch (host <-> HBM row swap)", 9: "k_put_scatter (Put: last occurrence writes)",
-                10: "k_single (runs of one lookup + Adagrad)", 11: "k_small (runs of 2-4 lookups + Adagrad)"}
+                10: "k_single (runs of one lookup + Adagrad)", 11: "k_small (runs of 2-4 lookups + Adagrad)",
+                12: "k_reduce (runs of every length + Adagrad, small applies)",
+                13: "k_plan (probe + sort + run lists, small applies)"}
 KERNEL_SOURCES = {1: "mlkv_index.cu", 2: "mlkv_index.cu", 3: "mlkv_sort.cu", 4: "mlkv_apply.cu",
                   5: "mlkv_apply.cu", 6: "mlkv_apply.cu", 7: "mlkv_apply.cu", 8: "mlkv_tier.cu",
-                  9: "mlkv_index.cu", 10: "mlkv_apply.cu", 11: "mlkv_apply.cu"}
+                  9: "mlkv_index.cu", 10: "mlkv_apply.cu", 11: "mlkv_apply.cu", 12: "mlkv_apply.cu",
+                  13: "mlkv_plan.cu"}
 
 
 # ncu kernel names (demangled, without the namespace) -> kernel class
 KERNEL_PATTERNS = [("k_get_bulk<", 1), ("k_get<", 1), ("k_probe<", 2), ("k_sort_scatter", 3), ("k_short<", 4),
                    ("k_long<", 5), ("k_heads", 6), ("k_combine<", 7), ("k_tier_fetch", 8),
-                   ("k_put_scatter", 9), ("k_single<", 10), ("k_small<", 11)]
+                   ("k_put_scatter", 9), ("k_single<", 10), ("k_small<", 11), ("k_reduce<", 12),
+                   ("k_plan<", 13)]
 TRAFFIC_PATH = os.path.join(ROOT, "profiles", "traffic.json")
 
 
@@ -612,7 +622,7 @@ def measure(args, cfg, dist, rank, local, world, dev, headline: bool, steps: int
     # The HBM store cycles a pool of batches.  The tiered store gets a fresh batch
     # every step (a cycled pool would end up resident in its cache): one per
     # kernel-class prepass step, warm-up step, timed step, and the last look-ahead.
-    kinds = (1, 2, 9) if kv else (1, 2, 3, 4, 5, 6, 7, 10, 11) + ((8,) if tiered else ())
+    kinds = (1, 2, 9) if kv else (1, 2, 3, 4, 5, 6, 7, 10, 11, 12, 13) + ((8,) if tiered else ())
     base = len(kinds) if tiered else 0
     pool = base + args.warmup + steps + 1 if tiered else max(1, min(args.pool, steps + args.warmup))
     ngrad = max(1, min(args.pool, pool))

@@ -307,7 +307,9 @@ int mlkv_tier_stats(mlkv_table* t, int64_t* rows_fetched, int64_t* rows_written_
  * the number of timed launches since the last reset.  While it is on, a
  * gradient apply launches its reduce kernels one after another on the call's
  * stream (otherwise they run on three streams at once), so that each timed
- * launch's events bracket that kernel alone. */
+ * launch's events bracket that kernel alone.  An apply of few lookups is two
+ * kernels: MLKV_K_PLAN (probe, sort and run lists) and MLKV_K_REDUCE (runs of
+ * every length). */
 #define MLKV_K_GET_GATHER 1
 #define MLKV_K_PROBE 2
 #define MLKV_K_SORT_SCATTER 3
@@ -319,6 +321,8 @@ int mlkv_tier_stats(mlkv_table* t, int64_t* rows_fetched, int64_t* rows_written_
 #define MLKV_K_PUT_SCATTER 9
 #define MLKV_K_REDUCE_SINGLE 10
 #define MLKV_K_REDUCE_SMALL 11
+#define MLKV_K_REDUCE 12
+#define MLKV_K_PLAN 13
 int mlkv_time_kernel(mlkv_table* t, int32_t kernel_id);
 int mlkv_kernel_time(mlkv_table* t, double* total_ms, int64_t* launches);
 

@@ -31,6 +31,8 @@
 //                 compensated, to scratch as a (sum, compensation) pair.
 //  k_combine      per long run: the chunk pairs added in a fixed order with
 //                 compensation, the sum rounded once, and the row updated.
+//  k_reduce       all of these in one launch, for small calls (whose run lists
+//                 the plan of mlkv_plan.cu makes in place of k_heads).
 //
 // The row kernels' unit of work is one segment of a run: a lane group (G
 // lanes, the power of two that holds a row of up to 32 vectors) reduces G
@@ -52,42 +54,11 @@
 // not depend on scheduling.
 #include <algorithm>
 
-#include "mlkv_internal.cuh"
+#include "mlkv_runs.cuh"
 
 namespace mlkv {
 
 namespace {
-
-// Long runs are summed in chunks: of kChunkLarge lookups in calls of at least
-// MLKV_SMALL_BATCH lookups, of kChunkSmall in smaller ones (few long runs:
-// more chunks to sum in parallel).  Set at build time.
-#ifndef MLKV_SMALL_BATCH
-#define MLKV_SMALL_BATCH (1u << 19)
-#endif
-#ifndef MLKV_CHUNK_SMALL
-#define MLKV_CHUNK_SMALL 16
-#endif
-constexpr uint32_t kChunkLarge = 64, kChunkSmall = MLKV_CHUNK_SMALL, kSmallBatch = MLKV_SMALL_BATCH;
-// In a small call a run of more small chunks than this is cut into large ones:
-// up to here a block combines them in one node.  (At 64, a knowledge-graph step
-// of 200k lookups lost 7 us in k_long: its runs of some thousand lookups were
-// cut into too few chunks to fill the GPU.)
-constexpr uint32_t kFewChunks = 256;
-
-// Lookups per chunk of a long run of len lookups (`chunk`: the call's).
-__device__ __forceinline__ uint32_t run_chunk(uint32_t len, uint32_t chunk) {
-    return len > chunk * kFewChunks ? kChunkLarge : chunk;
-}
-#ifndef MLKV_GROUP_CHUNKS
-#define MLKV_GROUP_CHUNKS 16
-#endif
-#ifndef MLKV_NODE
-#define MLKV_NODE 256
-#endif
-constexpr uint32_t NONE = 0xFFFFFFFFu;  // no position (a small run's record past its end)
-// k_combine: a lane group adds up the chunk sums of a run of at most
-// kGroupChunks chunks; of longer runs, a block takes kNode chunks at a time.
-constexpr uint32_t kGroupChunks = MLKV_GROUP_CHUNKS, kNode = MLKV_NODE;
 
 // Tuning (set at build time): gradient rows in flight per lane group in a long
 // chunk and in a run of 5-32 lookups, and the resident blocks per SM the
@@ -125,44 +96,6 @@ struct RowArgs {
     int d;
     uint32_t nseg;   // segments of G vectors per row: a lane group reduces one segment of a run at a time
     uint32_t nrows;  // rows of the slot array (bounds-checked build)
-};
-
-// Sites of the bounds-checked build (in_bounds).
-enum CheckSite : uint32_t {
-    kChkSingleRow = 1, kChkSinglePos, kChkSmallRow, kChkSmallPos, kChkShortRun, kChkShortRow, kChkShortPos,
-    kChkLongItem, kChkLongPos, kChkLongRow, kChkHeadsPos, kChkListEntry
-};
-
-constexpr uint32_t kItemLenBits = 7;  // a chunk holds at most 64 lookups; a run at most 2^24 chunks of 64
-static_assert(kChunkLarge < (1u << kItemLenBits) && kChunkSmall < (1u << kItemLenBits), "chunk lengths fit their bits");
-
-struct RunArgs {
-    const float* grads;
-    const uint32_t* srow;  // sorted row ids; lookups without a row hold `sent` and come last
-    const uint32_t* spos;  // their lookup positions
-    uint32_t n;
-    uint32_t sent;
-    CallCounters* cur;
-    uint4* runs;           // [max_batch] short runs of 2 or more lookups: (first sorted position, one
-                           //   past the last, row, first lookup position)
-    uint2* singles;        // [max_batch] runs of one lookup: (row, lookup position)
-    uint4* smalls;         // [max_batch] runs of 2 .. kSmallRun lookups: (row, p0, p1, p2), positions in
-                           //   occurrence order, NONE past the run's end
-    uint32_t* small_p3;    // [max_batch] their fourth position (or NONE)
-    uint4* long_runs;      // [max_long] long runs of at most kGroupChunks chunks: (first chunk, chunks, row, -)
-    uint4* nodes;          // [max_nodes] kNode chunks each of the longer runs: (the run's first chunk, its chunks,
-                           //   row, node of the run)
-    uint4* items;          // [max_items] chunks of the long runs: (first sorted position, lookups |
-                           //   chunks of the run << kItemLenBits, row, the run's first chunk)
-    float* partial;        // [max_items][2][dpad] sums of chunks, and of nodes in their first chunk's place
-    uint32_t* node_cnt;    // [max_items][nseg] nodes of a run done (at its first chunk's entry), zero at rest
-    uint32_t max_long;
-    uint32_t max_nodes;
-    uint32_t max_items;
-    uint32_t chunk;        // lookups per chunk of a long run (kChunkLarge or kChunkSmall)
-    ErrSink err;
-    float lr, eps;
-    uint32_t release;      // non-zero in the apply's last kernels: the blocks of all of them (release_counters)
 };
 
 __device__ __forceinline__ unsigned group_mask(int G, int gid) {
@@ -290,58 +223,6 @@ __device__ __forceinline__ uint32_t scan_end(const uint32_t* __restrict__ srow, 
     return run_end(srow, n, q0 + 1023u, row, lane);
 }
 
-// What the long runs qs[k] .. qe[k] (k < nq) add to the lists: chunks, runs
-// combined by a lane group, and nodes.
-struct LongCounts {
-    uint32_t items, runs, nodes;
-};
-
-__device__ __forceinline__ uint32_t warp_inclusive(uint32_t x, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
-
-// This lane's run's counts, their exclusive prefix over the lanes, and the sums
-// (the whole warp).
-__device__ __forceinline__ LongCounts long_counts(const uint32_t* qs, const uint32_t* qe, int nq, int lane,
-                                                  uint32_t chunk, LongCounts& mine, LongCounts& excl) {
-    const uint32_t len = lane < nq ? qe[lane] - qs[lane] : 0u;
-    const uint32_t c = run_chunk(len, chunk);
-    mine.items = (len + c - 1) / c;
-    mine.runs = lane < nq && mine.items <= kGroupChunks;
-    mine.nodes = mine.items > kGroupChunks ? (mine.items + kNode - 1) / kNode : 0u;
-    const LongCounts in = {warp_inclusive(mine.items, lane), warp_inclusive(mine.runs, lane),
-                           warp_inclusive(mine.nodes, lane)};
-    excl = {in.items - mine.items, in.runs - mine.runs, in.nodes - mine.nodes};
-    return {__shfl_sync(0xffffffffu, in.items, 31), __shfl_sync(0xffffffffu, in.runs, 31),
-            __shfl_sync(0xffffffffu, in.nodes, 31)};
-}
-
-// Writes the chunks of the long runs qs[k], qe[k], qr[k] (k < nq: start, end,
-// row) and their runs or nodes at list entries base.. (the whole warp).
-__device__ __forceinline__ void write_long_runs(const RunArgs& a, const uint32_t* qs, const uint32_t* qe,
-                                                const uint32_t* qr, int nq, const LongCounts& base, int lane) {
-    LongCounts mine, excl;
-    long_counts(qs, qe, nq, lane, a.chunk, mine, excl);
-    if (mine.runs) a.long_runs[base.runs + excl.runs] = make_uint4(base.items + excl.items, mine.items, qr[lane], 0u);
-    for (int k = 0; k < nq; ++k) {
-        const uint32_t s = qs[k], e = qe[k], row = qr[k], chunk = run_chunk(e - s, a.chunk);
-        const uint32_t m = __shfl_sync(0xffffffffu, mine.items, k);
-        const uint32_t ib = base.items + __shfl_sync(0xffffffffu, excl.items, k);
-        const uint32_t nodes = __shfl_sync(0xffffffffu, mine.nodes, k);
-        const uint32_t nb = base.nodes + __shfl_sync(0xffffffffu, excl.nodes, k);
-        for (uint32_t c = lane; c < m; c += 32) {
-            const uint32_t cs = s + c * chunk;
-            a.items[ib + c] = make_uint4(cs, min(chunk, e - cs) | m << kItemLenBits, row, ib);
-        }
-        for (uint32_t c = lane; c < nodes; c += 32) a.nodes[nb + c] = make_uint4(ib, m, row, c);
-    }
-}
-
 // A warp per window of 32 sorted positions (windows dealt out grid-stride).
 // A run starts where a row id differs from its left neighbour; it ends at the
 // next change of value in the window (the next run, or the absent lookups
@@ -407,10 +288,6 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
                 __syncwarp();
             }
         }
-    };
-    auto room = [&](const LongCounts& base, const LongCounts& tot) {
-        return base.items + tot.items <= a.max_items && base.runs + tot.runs <= a.max_long &&
-               base.nodes + tot.nodes <= a.max_nodes;
     };
     auto emit_long = [&](const LongCounts& base) {
         if (nq) write_long_runs(a, qs[wib], qe[wib], qr[wib], nq, base, lane);
@@ -489,7 +366,7 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
                 base.items = __shfl_sync(0xffffffffu, base.items, 0);
                 base.runs = __shfl_sync(0xffffffffu, base.runs, 0);
                 base.nodes = __shfl_sync(0xffffffffu, base.nodes, 0);
-                if (!room(base, tot)) {
+                if (!long_room(a, base, tot)) {
                     if (lane == 0) record_error(a.err, MLKV_ERR_FULL);
                     nq = 0;
                 } else {
@@ -555,7 +432,7 @@ __global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a)
         a.small_p3[ws2[wib] + k] = sp3[wib][k];
     }
     const LongCounts base = wlc[wib];
-    if (!room(base, tot)) {
+    if (!long_room(a, base, tot)) {
         if (lane == 0 && nq) record_error(a.err, MLKV_ERR_FULL);
         return;
     }
@@ -929,6 +806,212 @@ __global__ void __launch_bounds__(256, SG == 1 ? MLKV_SINGLE_MIN_BLOCKS : 4) k_s
     if (a.release) release_counters(a.cur, a.release);
 }
 
+// Calls of at most this many run segments reduce all their runs in k_reduce.
+#ifndef MLKV_FUSED_MAX
+#define MLKV_FUSED_MAX (1 << 15)
+#endif
+constexpr uint32_t kFusedMax = MLKV_FUSED_MAX;
+
+// --- calls of few lookups: one kernel ------------------------------------------
+
+// Levels of the combine tree: 32^5 chunks of 64 lookups exceed the largest batch.
+constexpr int kTreeLevels = 5;
+constexpr uint32_t kFanShift = 5, kFan = 1u << kFanShift;  // its fan-in
+#ifndef MLKV_SINGLES
+#define MLKV_SINGLES 1
+#endif
+
+// One segment of a chunk of a long run, by one lane group.  The chunk sums of a
+// run are combined in a tree of fan-in kFan, always in chunk order: the group
+// whose entry is the last of a node to arrive (an atomic count per node) adds
+// the node's entries up and goes on to the next level; at the root the sum is
+// rounded once and the row updated.  No group waits for another.
+template <int V>
+__device__ __forceinline__ void long_chunk(const RowArgs& ra, const RunArgs& a, uint32_t it, uint32_t seg, int G,
+                                           int glane, unsigned gmask) {
+    using VT = typename Vec<V>::T;
+    const uint4 rec = __ldg(a.items + it);
+    const uint32_t m = rec.y >> kItemLenBits, ib = rec.w;
+    const int j = glane + G * (int)seg;
+    const bool act = j < ra.NV;
+    VT acc, cmp;
+    if (!chunk_sum<V>(acc, cmp, ra, a, rec, j, G, glane, gmask)) return;
+    uint32_t idx = it - ib, count = m, stride = 1;
+    for (int level = 0; count > 1; ++level) {
+        if (act) store_pair<V>(ra, a, ib + idx * stride, j, acc, cmp);
+        const uint32_t node = idx >> kFanShift, first = node << kFanShift;
+        const uint32_t width = min(kFan, count - first);
+        __threadfence();
+        __syncwarp(gmask);
+        uint32_t arrived = 0;
+        if (glane == 0) {
+            uint32_t* ctr = a.node_cnt + ((size_t)level * a.max_items + ib + first * stride) * ra.nseg + seg;
+            arrived = atomicAdd(ctr, 1u);
+            if (arrived == width - 1) *ctr = 0u;  // zero again for the next call
+        }
+        arrived = __shfl_sync(gmask, arrived, 0, G);
+        if (arrived != width - 1) return;
+        __threadfence();
+        sum_pairs<V>(acc, cmp, ra, a.partial, ib + first * stride, stride, width, j, act);
+        idx = node;
+        count = (count + kFan - 1) >> kFanShift;
+        stride <<= kFanShift;
+    }
+    if (act) finish_long<V>(ra, a, rec.z, j, acc, cmp);
+}
+
+// k_reduce's units of runs: [0, us) of 5 .. 32 lookups, [us, um) of 2 ..
+// kSmallRun, [um, uc) and [uc, units) of one; ls, lm, lc, lf run segments each.
+struct Units {
+    uint32_t NS, NM, NC, N1;  // run segments of each kind (NC: those of one lookup in coarse units)
+    uint32_t ls, lm, lc, lf;
+    uint32_t us, um, uc, units;
+};
+
+__device__ __forceinline__ Units make_units(const RunArgs& a, uint32_t R, uint32_t nwarps, uint32_t nseg) {
+    Units q;
+    q.NS = min(a.cur->n_short, a.n) * nseg;
+    q.NM = min(a.cur->n_small, a.n) * nseg;
+    q.N1 = min(a.cur->n_single, a.n) * nseg;
+    q.NC = q.N1 - q.N1 / 4;
+    // segments per lane group so that each warp gets some `rounds` units, at most 32 a unit
+    auto unit = [&](uint32_t work, uint32_t rounds, uint32_t most) {
+        return R * max(1u, min(min(work / (R * nwarps * rounds), most), 32u / R));
+    };
+    q.ls = unit(q.NS, 2, 4);
+    q.lm = unit(q.NM, 2, 8);
+    q.lc = unit(q.N1, 4, 24);
+    q.lf = R * max(1u, q.lc / R / 4);
+    q.us = (q.NS + q.ls - 1) / q.ls;
+    q.um = q.us + (q.NM + q.lm - 1) / q.lm;
+    q.uc = q.um + (q.NC + q.lc - 1) / q.lc;
+    q.units = q.uc + (q.N1 - q.NC + q.lf - 1) / q.lf;
+    return q;
+}
+
+// Every run's sum and its row's Adagrad step, in one launch, for calls of at
+// most kFusedMax run segments: latency is all that counts there, and the
+// kernels per run length cost five launches, three event records and four
+// waits.  (Apply + Get of 4,096 lookups: 41 us with those, 36 with this; 13,312:
+// 48 and 42; 32,768 segments: equal.  In large calls those are faster: this
+// kernel's 128 registers leave 16 warps a SM, too few for the square roots and
+// divisions between a run's loads: 1.7M lookups 556 us, 637 with this.)
+//   1. The chunks of the long runs, in fixed shares (a lane group each).
+//   2. Everything else as units of up to 32 runs, claimed from one counter by
+//      the warps as they get free: runs of 5-32 lookups, of 2-4, of one in
+//      coarse units and the last quarter of those in fine ones, so that the
+//      warps end together.  A unit's run records are loaded by one coalesced
+//      load and handed round with shuffles; the next unit is claimed before
+//      this one is worked on.
+template <int V>
+__global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevState* ds) {
+    pdl_enter();
+    using VT = typename Vec<V>::T;
+    const uint32_t nseg = ra.nseg;
+    const uint32_t NI = min(a.cur->n_items, a.max_items);
+    // a list never holds more runs than lookups
+    if (MLKV_CHECK && !(in_bounds(a.err, kChkListEntry, a.cur->n_short, (unsigned long long)a.n + 1) &&
+                        in_bounds(a.err, kChkListEntry, a.cur->n_small, (unsigned long long)a.n + 1) &&
+                        in_bounds(a.err, kChkListEntry, a.cur->n_single, (unsigned long long)a.n + 1)))
+        return;
+    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane >> ra.gshift;
+    const uint32_t R = 32u >> ra.gshift;  // lane groups per warp
+    const unsigned gmask = group_mask(G, gid);
+    // neighbouring warps of the order are on different SMs: a batch with little work spreads
+    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    // the units' layout, in shared memory: read once a unit, it would only hold registers
+    __shared__ Units q;
+    if (threadIdx.x == 0) {
+        q = make_units(a, R, nwarps, nseg);
+        if (blockIdx.x == 0)
+            ds->last_unique = a.cur->n_single + a.cur->n_small + a.cur->n_short + a.cur->n_long;  // one run per row
+    }
+    for (uint32_t v = warp * R + gid; v < NI * nseg; v += nwarps * R) {
+        const uint32_t it = nseg == 1 ? v : v / nseg;
+        long_chunk<V>(ra, a, it, v - it * nseg, G, glane, gmask);
+    }
+    __syncthreads();
+    uint32_t u = warp;
+    while (u < q.units) {  // warp-uniform
+        uint32_t claim = 0;
+        if (lane == 0) claim = atomicAdd(&a.cur->short_next, 1u);
+        if (u < q.us) {  // runs of 5 .. 32 lookups
+            const uint32_t v0 = u * q.ls, cnt = min(q.ls, q.NS - v0);
+            const uint32_t mine = v0 + min((uint32_t)lane, cnt - 1);
+            const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
+            const uint4 mrec = __ldg(a.runs + mrun);  // (start, end, row, first lookup)
+            const uint32_t mseg = mine - mrun * nseg;
+            for (uint32_t k = 0; k < cnt; k += R) {
+                const int src = (int)min(k + gid, cnt - 1);
+                const uint32_t s = __shfl_sync(0xffffffffu, mrec.x, src), e = __shfl_sync(0xffffffffu, mrec.y, src);
+                const uint32_t row = __shfl_sync(0xffffffffu, mrec.z, src), p0 = __shfl_sync(0xffffffffu, mrec.w, src);
+                const int j = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
+                if (k + gid < cnt)
+                    short_run<V, MLKV_SHORT_ROWS>(ra, a, s, e, row, p0, j, G, glane, gmask);
+                __syncwarp();
+            }
+        } else if (u < q.um) {  // runs of 2 .. kSmallRun lookups, their positions in the record
+            const uint32_t v0 = (u - q.us) * q.lm, cnt = min(q.lm, q.NM - v0);
+            const uint32_t mine = v0 + min((uint32_t)lane, cnt - 1);
+            const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
+            const uint4 mrec = __ldg(a.smalls + mrun);  // (row, p0, p1, p2)
+            const uint32_t mp3 = __ldg(a.small_p3 + mrun), mseg = mine - mrun * nseg;
+            for (uint32_t k = 0; k < cnt; k += R) {
+                const int src = (int)min(k + gid, cnt - 1);
+                const uint4 m = make_uint4(__shfl_sync(0xffffffffu, mrec.x, src), __shfl_sync(0xffffffffu, mrec.y, src),
+                                           __shfl_sync(0xffffffffu, mrec.z, src), __shfl_sync(0xffffffffu, mrec.w, src));
+                const uint32_t p3 = __shfl_sync(0xffffffffu, mp3, src);
+                const int j = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
+                if (k + gid < cnt) small_run<V>(ra, a, m, p3, j);
+                __syncwarp();
+            }
+        } else {  // runs of one lookup
+            constexpr int SG = MLKV_SINGLES;
+            const bool coarse = u < q.uc;
+            const uint32_t v0 = coarse ? (u - q.um) * q.lc : q.NC + (u - q.uc) * q.lf;
+            const uint32_t cnt = coarse ? min(q.lc, q.NC - v0) : min(q.lf, q.N1 - v0);
+            const uint32_t mine = v0 + min((uint32_t)lane, cnt - 1);
+            const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
+            const uint2 mrec = __ldg(a.singles + mrun);  // (row, lookup)
+            const uint32_t mseg = mine - mrun * nseg;
+            for (uint32_t k = 0; k < cnt; k += R * SG) {
+                VT w[SG], Gs[SG], g[SG];
+                uint32_t row[SG];
+                int jj[SG];  // the lane's column, or NV where there is no run
+#pragma unroll
+                for (int i = 0; i < SG; ++i) {
+                    const uint32_t idx = k + i * R + gid;
+                    const int src = (int)min(idx, cnt - 1);
+                    row[i] = __shfl_sync(0xffffffffu, mrec.x, src);
+                    const uint32_t p = __shfl_sync(0xffffffffu, mrec.y, src);
+                    jj[i] = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
+                    if (idx >= cnt) jj[i] = ra.NV;
+                    if (MLKV_CHECK && jj[i] < ra.NV && !(in_bounds(a.err, kChkSingleRow, row[i], ra.nrows) &&
+                                                         in_bounds(a.err, kChkSinglePos, p, a.n)))
+                        jj[i] = ra.NV;
+                    if (jj[i] < ra.NV) {
+                        const VT* src_row = row_vec<V>(ra, row[i], jj[i]);
+                        w[i] = src_row[0];
+                        Gs[i] = *beside(ra, src_row);
+                        g[i] = __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)p * ra.d) + jj[i]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < SG; ++i) {
+                    if (jj[i] >= ra.NV) continue;
+                    VT acc = Vec<V>::zero();
+                    Vec<V>::add(acc, g[i]);  // 0 + g, as in a longer run
+                    adagrad_store<V>(ra, row[i], jj[i], w[i], Gs[i], acc, a.lr, a.eps);
+                }
+                __syncwarp();
+            }
+        }
+        u = nwarps + __shfl_sync(0xffffffffu, claim, 0);
+    }
+    release_counters(a.cur, gridDim.x);  // the apply's last kernel
+}
+
 using RunKernel = void (*)(RowArgs, RunArgs);
 
 // Narrow rows (on at most 16 lanes: dim <= 64): runs of one lookup two at a
@@ -946,24 +1029,22 @@ RunKernels run_kernels(bool seg, bool narrow) {
 }
 
 template <int V>
-cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* srow, const uint32_t* spos,
-                       int64_t n, uint32_t sent, cudaStream_t st, CallCounters* cur) {
+cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n, cudaStream_t st,
+                       CallCounters* cur) {
     const uint32_t nseg = (uint32_t)((t->geom.NV + t->geom.G - 1) / t->geom.G);
     RowArgs ra{t->slots, t->geom.stride, t->geom.dpad, t->geom.NV, t->geom.G, __builtin_ctz((unsigned)t->geom.G),
                t->geom.d, nseg,
                (uint32_t)(t->tiered ? t->cfg.hbm_cache_rows : t->cfg.capacity)};
-    RunArgs a{grads, srow, spos, (uint32_t)n, sent, cur, t->s.short_runs, t->s.single_runs, t->s.small_runs,
-              t->s.small_p3, t->s.long_runs, t->s.nodes, t->s.items, t->s.partial, t->s.node_cnt,
-              (uint32_t)t->s.max_long, (uint32_t)t->s.max_nodes, (uint32_t)t->s.max_items,
-              n >= kSmallBatch ? kChunkLarge : kChunkSmall,
-              ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}, t->cfg.lr, t->cfg.eps};
-    // a warp per 32 positions, the windows dealt out grid-stride over at most
-    // one wave of blocks
-    const int64_t cap = persistent_blocks(t, (const void*)k_heads, 256);
-    int64_t gh = (n + 255) / 256;
-    if (gh > cap) gh = cap;
-    if (gh < 1) gh = 1;
-    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_heads, (unsigned)gh, 256, 0, st, a);
+    const RunArgs a = run_args(t, grads, nullptr, spos, n, 0u, cur);
+    const int64_t segs = n * (int64_t)nseg;
+    if (segs <= (int64_t)kFusedMax) {
+        // one wave, or as many blocks as give every lane group a segment of a lookup
+        int64_t gr = (segs * t->geom.G + 255) / 256;
+        const int64_t wave = persistent_blocks(t, (const void*)k_reduce<V>, 256);
+        if (gr > wave) gr = wave;
+        MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE, (k_reduce<V>), (unsigned)gr, 256, 0, st, ra, a, t->dstate);
+        return cudaGetLastError();
+    }
     // The runs of one lookup, of 2 .. kSmallRun and of up to
     // MLKV_SEQ_SEGMENT_MAX lookups, and the long runs touch disjoint rows and
     // scratch: they run on three streams at once, each filling the others'
@@ -1034,15 +1115,27 @@ void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& item
 int64_t node_counters(int64_t max_items, int dim) {
     // segments per row of the widest split: the scalar kernels' (dim <= 256) or the float4 kernels'
     const int64_t nseg = std::max<int64_t>((std::min(dim, 256) + 31) / 32, (dim + 127) / 128);
-    return max_items * nseg;
+    return kTreeLevels * max_items * nseg;
 }
 
-cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
-                                const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
-                                CallCounters* cur) {
-    if (t->geom.V == 4) return run_reduce<4>(t, grads, srow, spos, n, sent, st, cur);
-    if (t->geom.V == 2) return run_reduce<2>(t, grads, srow, spos, n, sent, st, cur);
-    return run_reduce<1>(t, grads, srow, spos, n, sent, st, cur);
+cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,
+                         cudaStream_t st, CallCounters* cur) {
+    const RunArgs a = run_args(t, nullptr, srow, spos, n, sent, cur);
+    // a warp per 32 positions, the windows dealt out grid-stride over at most
+    // one wave of blocks
+    const int64_t cap = persistent_blocks(t, (const void*)k_heads, 256);
+    int64_t gh = (n + 255) / 256;
+    if (gh > cap) gh = cap;
+    if (gh < 1) gh = 1;
+    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_heads, (unsigned)gh, 256, 0, st, a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
+                                cudaStream_t st, CallCounters* cur) {
+    if (t->geom.V == 4) return run_reduce<4>(t, grads, spos, n, st, cur);
+    if (t->geom.V == 2) return run_reduce<2>(t, grads, spos, n, st, cur);
+    return run_reduce<1>(t, grads, spos, n, st, cur);
 }
 
 }  // namespace mlkv

@@ -12,106 +12,11 @@
 // atomicMin; the lookup whose position survives is the first occurrence; an
 // exclusive scan over first-occurrence flags gives each new key its rank, and
 // row = rows handed out so far + rank.
-#include "mlkv_internal.cuh"
+#include "mlkv_probe.cuh"
 
 namespace mlkv {
 
 namespace {
-
-// Device-scope relaxed loads: they see slots published by compare-and-swap in
-// the same kernel and still hit in L2 (the coherence point of GPU accesses);
-// a volatile load would be a system-scope access.
-__device__ __forceinline__ ulonglong2 ld_slot_relaxed(const Slot* s) {
-    ulonglong2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(s) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ uint32_t ld_u32_relaxed(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Probes `key`.  Returns its row, ROW_ABSENT, or (INSERT only) ROW_PENDING
-// with `slot_out` = the slot that now holds the key and the slot's aux
-// lowered to `pos`.
-template <bool INSERT>
-__device__ __forceinline__ uint32_t probe_key(const IndexArgs& ia, unsigned long long key,
-                                              uint32_t pos, uint32_t& slot_out) {
-    if (key == EMPTY_KEY) {
-        record_error(ia.err, MLKV_ERR_INVALID);
-        return ROW_ABSENT;
-    }
-    unsigned long long s = (ia.identity_hash ? key : hash_key(key)) & ia.mask;
-    for (int i = 0; i < PROBE_LIMIT; ++i) {
-        ulonglong2 v = INSERT ? ld_slot_relaxed(ia.index + s)
-                              : __ldg(reinterpret_cast<const ulonglong2*>(ia.index + s));
-        if (v.x == key) {
-            uint32_t row = (uint32_t)v.y;
-            slot_out = (uint32_t)s;
-            if (row != ROW_PENDING || !INSERT) return row == ROW_PENDING ? ROW_ABSENT : row;
-            atomicMin(&ia.index[s].aux, pos);
-            return ROW_PENDING;
-        }
-        if (v.x == EMPTY_KEY) {
-            if (!INSERT) return ROW_ABSENT;
-            unsigned long long old = atomicCAS(&ia.index[s].key, EMPTY_KEY, key);
-            if (old == EMPTY_KEY || old == key) {
-                slot_out = (uint32_t)s;
-                uint32_t row = ld_u32_relaxed(&ia.index[s].row);
-                if (row != ROW_PENDING) return row;
-                atomicMin(&ia.index[s].aux, pos);
-                return ROW_PENDING;
-            }
-            // another key took this slot first: keep probing
-        }
-        s = (s + 1) & ia.mask;
-    }
-    record_error(ia.err, MLKV_ERR_PROBE_LIMIT);
-    return ROW_ABSENT;
-}
-
-// Appends (pos, slot) to the miss list with one atomic per converged group of
-// lanes.  The list holds at most one entry per lookup (n): an entry past that
-// could only come from a counter left set, and is not written.
-__device__ __forceinline__ void append_miss(CallCounters* cur, uint32_t* miss_pos,
-                                            uint32_t* miss_slot, uint32_t pos, uint32_t slot, uint32_t n) {
-    const unsigned m = __activemask();
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(m) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&cur->n_miss, (uint32_t)__popc(m));
-    base = __shfl_sync(m, base, leader);
-    const uint32_t i = base + __popc(m & lanemask_lt());
-    if (i < n) {
-        miss_pos[i] = pos;
-        miss_slot[i] = slot;
-    }
-}
-
-__device__ __forceinline__ void zero_counters(CallCounters* nxt) {
-    if (nxt && blockIdx.x == 0 && threadIdx.x < sizeof(CallCounters) / 4)
-        reinterpret_cast<uint32_t*>(nxt)[threadIdx.x] = 0u;
-}
-
-struct RowArgs {
-    float* slots;
-    int stride;
-    int dpad;
-    int d;
-    int NV;
-    int G;
-};
-
-RowArgs row_args(mlkv_table* t) {
-    return RowArgs{t->slots, t->geom.stride, t->geom.dpad, t->geom.d, t->geom.NV, t->geom.G};
-}
-
-IndexArgs index_args(mlkv_table* t) {
-    return IndexArgs{t->index, t->index_mask, (t->cfg.flags & MLKV_IDENTITY_HASH) ? 1u : 0u,
-                     ErrSink{&t->dstate->status, t->status_dev_alias}};
-}
 
 // ---------------------------------------------------------------------------
 // row_of_pos[p] (and the slot) for every position.  Each thread takes
@@ -184,17 +89,6 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
     }
 }
 
-// Group-cooperative copy of one row (or NaN) into dst.
-template <int V>
-__device__ __forceinline__ void copy_row(const float* __restrict__ src, float* __restrict__ dst,
-                                         int NV, int G, int glane, bool absent) {
-    using VT = typename Vec<V>::T;
-    const VT* s = reinterpret_cast<const VT*>(src);
-    VT* o = reinterpret_cast<VT*>(dst);
-#pragma unroll 2
-    for (int j = glane; j < NV; j += G) __stcs(o + j, absent ? Vec<V>::nan() : __ldg(s + j));
-}
-
 // The fused Get: each warp probes `lpw` consecutive lookups (one per lane), then
 // its lane groups gather their rows with vector loads, streaming the output.
 // Lookups of new keys are left to the miss path.  A row wider than 32 vectors
@@ -213,7 +107,7 @@ __device__ __forceinline__ void copy_row(const float* __restrict__ src, float* _
 #endif
 
 template <int V, bool SEG, bool INSERT>
-__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, RowArgs ra,
+__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, IndexRows ra,
                                              const int64_t* __restrict__ keys, uint32_t n,
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
@@ -310,7 +204,7 @@ __device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_
 }
 
 template <bool INSERT>
-__global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, RowArgs ra, const int64_t* __restrict__ keys,
+__global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, IndexRows ra, const int64_t* __restrict__ keys,
                                                            uint32_t n, float* __restrict__ out, uint32_t* miss_pos,
                                                            uint32_t* miss_slot, CallCounters* cur, CallCounters* nxt,
                                                            Memo memo) {
@@ -360,22 +254,6 @@ __global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, RowArgs
     if (stored && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// ---------------------------------------------------------------------------
-// The miss path: new keys of a call get rows.  One kernel, one block per SM.
-// In steady-state training nothing misses and every block returns at once; a
-// call with misses runs four phases separated by grid barriers:
-//   1. flag the first occurrence of each new key (the lookup whose position
-//      survived in the slot's aux);
-//   2. rank the flags: an exclusive scan over the call's positions, block b
-//      owning positions [b * per, (b + 1) * per);
-//   3. each first occurrence takes row = rows handed out so far + rank and
-//      writes its init row (not for Put) and state_init;
-//   4. every missed lookup reads its key's row (a Get gathers it into its
-//      output), flags and the slot's aux go back to idle, the row counter
-//      advances.
-// Data written by other blocks within the kernel is read from L2 (ld.cg).
-constexpr int kMissThreads = 512;
-constexpr int kMissWarps = kMissThreads / 32;
 constexpr uint32_t kBarrierSpins = 1u << 21;  // with its L2 load and 100 ns sleep, 1-2 s a barrier
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
@@ -413,157 +291,40 @@ __device__ bool grid_barrier(uint32_t* ctr, uint32_t extra, const ErrSink& err) 
     return ok != 0;
 }
 
-// Sum over the block of one value per thread.
-__device__ __forceinline__ uint32_t miss_block_sum(uint32_t v) {
-    __shared__ uint32_t part[kMissWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) part[w] = v;
-    __syncthreads();
-    uint32_t t = 0;
-#pragma unroll
-    for (int k = 0; k < kMissWarps; ++k) t += part[k];
-    return t;
-}
-
-// Exclusive scan over the block of one value per thread; *total = the sum.
-__device__ __forceinline__ uint32_t miss_block_scan(uint32_t v, uint32_t& total) {
-    __shared__ uint32_t part[kMissWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    __syncthreads();
-    if (lane == 31) part[w] = x;
-    __syncthreads();
-    uint32_t before = 0;
-    total = 0;
-#pragma unroll
-    for (int k = 0; k < kMissWarps; ++k) {
-        if (k < w) before += part[k];
-        total += part[k];
-    }
-    return before + x - v;
-}
+// The miss path in a kernel of its own, one block per SM (see miss_path).  In
+// steady-state training nothing misses and every block returns at once.
+constexpr int kMissThreads = 512;
 
 template <int V>
-__global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, RowArgs ra, const int64_t* __restrict__ keys,
-                                                       uint32_t n, const uint32_t* __restrict__ miss_pos,
-                                                       const uint32_t* __restrict__ miss_slot,
-                                                       uint32_t* __restrict__ flag, uint32_t* __restrict__ rank,
-                                                       uint32_t* __restrict__ block_sums,
-                                                       uint32_t* __restrict__ row_of_pos, float* __restrict__ out,
-                                                       CallCounters* cur, DevState* ds,
-                                                       unsigned long long capacity, int init_row,
-                                                       unsigned long long seed, float lo, float span,
-                                                       float state_init, uint32_t bar_extra, int release,
-                                                       FirstCounts fc) {
+__global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows ra, MissArgs ma, uint32_t bar_extra,
+                                                       int release, FirstCounts fc) {
     // waits for the kernel before it, like every kernel; lets the next one
     // launch only once the grid barriers are behind it (see grid_barrier)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint32_t m = min(cur->n_miss, n);  // never more misses than lookups
+    CallCounters* cur = ma.cur;
+    const uint32_t m = min(cur->n_miss, ma.n);  // never more misses than lookups
     if (m == 0) {
         if (release) release_counters(cur, gridDim.x);
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         return;
     }
-    using VT = typename Vec<V>::T;
-    const uint32_t nthreads = gridDim.x * blockDim.x;
-    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int G = ra.G, glane = threadIdx.x & (G - 1);
-    const uint32_t group = tid / G, ngroups = nthreads / G;
-    // A block whose wait ran out returns at once; the first sort pass's counts
-    // (an apply's) still get its share of the missed lookups, which keep no row
-    // (the phase-4 share, so that every lookup is counted once).
-    auto give_up = [&]() {
-        if (fc.counts && glane == 0)
-            for (uint32_t i = group; i < m; i += ngroups) {
-                const uint32_t p = miss_pos[i];
-                const uint32_t dig = fc.sent & (uint32_t)(fc.radix - 1);
-                atomicAdd(&fc.counts[(size_t)dig * fc.ntiles + (p >> fc.tile_shift)], 1u);
-                atomicAdd(fc.dtot + dig, 1u);
-            }
+    // the first sort pass's count (an apply's) of a missed lookup's digit in its tile
+    auto count = [&](uint32_t p, uint32_t r) {
+        if (!fc.counts) return;
+        const uint32_t dig = (r >= ROW_ABSENT ? fc.sent : r) & (uint32_t)(fc.radix - 1);
+        atomicAdd(&fc.counts[(size_t)dig * fc.ntiles + (p >> fc.tile_shift)], 1u);
+        atomicAdd(fc.dtot + dig, 1u);
     };
-    // 1. first occurrences
-    for (uint32_t i = tid; i < m; i += nthreads) {
-        const uint32_t p = miss_pos[i];
-        if (ia.index[miss_slot[i]].aux == p) flag[p] = 1u;
-    }
-    if (!grid_barrier(&cur->bar[0], bar_extra, ia.err)) return give_up();
-    // 2. ranks: the first occurrences at earlier positions
-    const uint32_t per = (n + gridDim.x - 1) / gridDim.x;
-    const uint32_t p_lo = min(n, blockIdx.x * per), p_hi = min(n, p_lo + per);
-    uint32_t cnt = 0;
-    for (uint32_t p = p_lo + threadIdx.x; p < p_hi; p += blockDim.x) cnt += __ldcg(flag + p);
-    const uint32_t mine = miss_block_sum(cnt);
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = mine;
-    if (!grid_barrier(&cur->bar[1], bar_extra, ia.err)) return give_up();
-    uint32_t b_before = 0;
-    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += blockDim.x) b_before += __ldcg(block_sums + b);
-    uint32_t run = miss_block_sum(b_before);
-    for (uint32_t p0 = p_lo; p0 < p_hi; p0 += blockDim.x) {  // uniform
-        const uint32_t p = p0 + threadIdx.x;
-        const uint32_t f = p < p_hi ? __ldcg(flag + p) : 0u;
-        uint32_t tot;
-        const uint32_t ex = miss_block_scan(f, tot);
-        if (f) rank[p] = run + ex;
-        run += tot;
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) cur->n_new = run;  // every first occurrence
-    if (!grid_barrier(&cur->bar[2], bar_extra, ia.err)) return give_up();
-    // 3. rows of the first occurrences
-    const unsigned long long next = ds->next_row;
-    for (uint32_t i = group; i < m; i += ngroups) {
-        const uint32_t p = miss_pos[i], s = miss_slot[i];
-        if (ia.index[s].aux != p) continue;
-        const unsigned long long r = next + __ldcg(rank + p);
-        if (r >= capacity) {
-            if (glane == 0) record_error(ia.err, MLKV_ERR_FULL);
-            continue;
-        }
-        const unsigned long long key = (unsigned long long)keys[p];
-        float* w = ra.slots + (size_t)r * ra.stride;
-        VT* wv = reinterpret_cast<VT*>(w);
-        VT* gv = reinterpret_cast<VT*>(w + ra.dpad);
-        for (int j = glane; j < ra.NV; j += G) {
-            if (init_row) {
-                float e[V];
-#pragma unroll
-                for (int c = 0; c < V; ++c) e[c] = init_element(seed, key, (uint32_t)(j * V + c), lo, span);
-                wv[j] = Vec<V>::from(e);
-            }
-            gv[j] = Vec<V>::splat(state_init);
-        }
-        if (glane == 0) ia.index[s].row = (uint32_t)r;
-    }
-    if (!grid_barrier(&cur->bar[3], bar_extra, ia.err)) return give_up();
-    // 4. every missed lookup takes its key's row
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const unsigned long long nr = next + __ldcg(&cur->n_new);
-        ds->next_row = nr < capacity ? nr : capacity;
-    }
-    for (uint32_t i = group; i < m; i += ngroups) {
-        const uint32_t p = miss_pos[i], s = miss_slot[i];
-        const uint32_t r0 = ld_u32_relaxed(&ia.index[s].row);
-        const uint32_t r = r0 == ROW_PENDING ? ROW_ABSENT : r0;
-        if (glane == 0) {
-            if (row_of_pos) row_of_pos[p] = r;
-            flag[p] = 0u;
-            ia.index[s].aux = AUX_IDLE;
-            if (fc.counts) {  // the first sort pass's count of this lookup's digit in its tile
-                const uint32_t dig = (r >= ROW_ABSENT ? fc.sent : r) & (uint32_t)(fc.radix - 1);
-                atomicAdd(&fc.counts[(size_t)dig * fc.ntiles + (p >> fc.tile_shift)], 1u);
-                atomicAdd(fc.dtot + dig, 1u);
-            }
-        }
-        if (out)
-            copy_row<V>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride,
-                            out + (size_t)p * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
+    const bool done = miss_path<V, kMissThreads>(
+        ia, ra, ma, m, [&](int i) { return grid_barrier(&cur->bar[i], bar_extra, ia.err); }, count);
+    if (!done) {
+        // A block whose wait ran out returns at once; the first sort pass's counts
+        // still get its share of the missed lookups, which keep no row (the last
+        // phase's share, so that every lookup is counted once).
+        const uint32_t G = ra.G, tid = blockIdx.x * blockDim.x + threadIdx.x;
+        if ((tid & (G - 1)) == 0)
+            for (uint32_t i = tid / G; i < m; i += gridDim.x * blockDim.x / G) count(ma.miss_pos[i], ROW_ABSENT);
+        return;
     }
     if (release) release_counters(cur, gridDim.x);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -614,7 +375,7 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
 #define MLKV_PUT_ROWS 4
 #endif
 template <int V>
-__global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, RowArgs ra,
+__global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
                                                      const uint32_t* __restrict__ row_of_pos,
                                                      const uint32_t* __restrict__ slot_of_pos,
                                                      const float* __restrict__ vals,
@@ -687,7 +448,7 @@ struct ExportTier {
 };
 
 template <int V>
-__global__ void __launch_bounds__(256) k_export(IndexArgs ia, RowArgs ra,
+__global__ void __launch_bounds__(256) k_export(IndexArgs ia, IndexRows ra,
                                                 const int64_t* __restrict__ keys, uint32_t n,
                                                 float* __restrict__ rows_out,
                                                 float* __restrict__ state_out, CallCounters* nxt,
@@ -802,14 +563,11 @@ template <int V>
 struct MissRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode, float* out,
                            cudaStream_t st, CallCounters* cur, bool release, const FirstCounts* fc) {
-        const float span = t->cfg.init_hi - t->cfg.init_lo;
-        RowArgs init_ra = row_args(t);  // new rows live in the host tier when tiered
+        IndexRows init_ra = row_args(t);  // new rows live in the host tier when tiered
         if (t->tiered) init_ra.slots = t->tier.host_dev;
-        MLKV_LAUNCH(t, 0, (k_miss<V>), t->num_sms, kMissThreads, 0, st, index_args(t), init_ra, keys,
-                    (uint32_t)n, t->s.miss_pos, t->s.miss_slot, t->s.first_flag, t->s.rank, t->s.tile_sums,
-                    mode == MissMode::Get ? nullptr : t->s.row_of_pos, mode == MissMode::Get ? out : nullptr, cur,
-                    t->dstate, (unsigned long long)t->cfg.capacity, mode == MissMode::Put ? 0 : 1,
-                    (unsigned long long)t->cfg.seed, t->cfg.init_lo, span, t->cfg.state_init,
+        const MissArgs ma = miss_args(t, keys, n, mode, mode == MissMode::Get ? nullptr : t->s.row_of_pos,
+                                      mode == MissMode::Get ? out : nullptr, cur);
+        MLKV_LAUNCH(t, 0, (k_miss<V>), t->num_sms, kMissThreads, 0, st, index_args(t), init_ra, ma,
                     take_injected_wait() ? 1u : 0u, release ? 1 : 0, fc ? *fc : FirstCounts{});
         return cudaGetLastError();
     }

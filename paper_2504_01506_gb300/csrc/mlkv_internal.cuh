@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "../../include/mlkv_gpu.h"
@@ -60,7 +61,7 @@ struct CallCounters {
     uint32_t n_nodes;    // nodes of the other long runs
     uint32_t n_short;    // runs of at most MLKV_SEQ_SEGMENT_MAX lookups
     uint32_t n_single;   // runs of one lookup
-    uint32_t short_next;  // run segments claimed (k_short's dynamic hand-out)
+    uint32_t short_next;  // run segments or units claimed (dynamic hand-out of k_short, k_reduce)
     uint32_t n_small;    // runs of 2 .. kSmallRun lookups (their positions in the record)
     uint32_t bar[4];     // arrivals at the miss kernel's grid barriers
     uint32_t done;       // blocks of the call's last kernel that have finished (release_counters)
@@ -169,6 +170,7 @@ struct mlkv_table {
     int sort_bits;               // bits of the ids being sorted incl. the absent sentinel
     int bits_rows;               // ... for row ids
     int bits_lines;              // ... for cache line ids (tiered)
+    int plan_cluster;            // largest cluster of the plan kernels (plan_prepare)
     int tiered;
     mlkv::Tier tier;
     mlkv::DevState* dstate;      // device
@@ -515,6 +517,20 @@ cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t*
                              int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
                              CallCounters* cur);
 
+// mlkv_plan.cu
+// Applies of at most this many lookups are planned by one cluster (why here: mlkv_plan.cu).
+#ifndef MLKV_PLAN_MAX
+#define MLKV_PLAN_MAX (1 << 15)
+#endif
+constexpr uint32_t kPlanMax = MLKV_PLAN_MAX;
+int plan_prepare();  // the largest cluster the plan kernels can run as on the current device (0: none)
+bool plan_fits(const mlkv_table* t, int64_t n);
+// Probe (insert: absent keys get rows; rows: they are in row_of_pos already),
+// sort and run lists of an apply of n lookups (plan_fits); spos: the sorted
+// positions.  The call's first kernel.
+cudaError_t launch_plan(mlkv_table* t, const int64_t* keys, int64_t n, bool insert, bool memo, bool rows,
+                        cudaStream_t st, CallCounters* cur, CallCounters* nxt, const uint32_t** spos);
+
 // mlkv_tier.cu
 TierArgs tier_args(mlkv_table* t, uint32_t epoch, uint32_t keep_from, int strict);
 cudaError_t launch_tier_resolve(mlkv_table* t, const TierArgs& ta, uint32_t* row_of_pos, int64_t n,
@@ -526,9 +542,11 @@ cudaError_t launch_gather_lines(mlkv_table* t, const uint32_t* rows, int64_t n, 
 // Runs longer than MLKV_SEQ_SEGMENT_MAX, their combine's nodes, and their chunks, worst case.
 void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& items);
 int64_t node_counters(int64_t max_items, int dim);  // counters of the combine's nodes
-cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* srow,
-                                const uint32_t* spos, int64_t n, uint32_t sent, cudaStream_t st,
-                                CallCounters* cur);
+// The run lists of sorted rows; and the reduce of the listed runs.
+cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,
+                         cudaStream_t st, CallCounters* cur);
+cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
+                                cudaStream_t st, CallCounters* cur);
 
 // Lookups per warp of the kernels that copy a warp's rows one after another: 32,
 // or as few as fill the GPU (kWarpsWanted warps per SM) in a small call, at
@@ -549,6 +567,7 @@ inline int lookups_per_warp(const mlkv_table* t, int64_t n, int least) {
 // mlkv_table.cu: launch bookkeeping and optional per-kernel timing; the host
 // side of mlkv_debug_fail's wait injection (true once, for the armed launch).
 bool take_injected_wait();
+bool wait_injection_armed();
 void timer_before(mlkv_table* t, int kernel_id, cudaStream_t st);
 void timer_after(mlkv_table* t, int kernel_id, cudaStream_t st);
 int persistent_blocks(mlkv_table* t, const void* kernel, int threads);

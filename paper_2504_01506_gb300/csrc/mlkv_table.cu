@@ -359,6 +359,8 @@ namespace mlkv {
 
 bool take_injected_wait() { return injected(g_fail_wait); }
 
+bool wait_injection_armed() { return g_fail_wait.load() > 0; }
+
 void timer_before(mlkv_table* t, int kid, cudaStream_t st) {
     KernelTimer& tm = t->timer;
     if (!kid || kid != tm.kernel_id || tm.n_events >= KernelTimer::kMax) return;
@@ -493,6 +495,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         return fail(MLKV_ERR_CUDA);
     if (!make_geom(c.dim, c.dim % 4 == 0 ? 4 : 1, t->geom)) return fail(MLKV_ERR_INVALID);
 
+    t->plan_cluster = plan_prepare();
     const int64_t stride = t->geom.stride;
     t->tiered = c.hbm_cache_rows > 0;
     if (!t->tiered) {
@@ -732,23 +735,35 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
     // may be the next Get's; the apply inserts nothing and probes every key
     const bool ins = t->cfg.insert_on_miss != 0 && !beside && t->stale == 0;
     const MemoUse memo = t->stale ? MemoUse::None : MemoUse::Read;
-    // On an HBM-resident table the probe also counts the sort's first pass (the
-    // tiered apply sorts cache lines, known only after the probe).
-    const FirstCounts fc = first_counts(t, n);
-    CK(t, launch_probe(t, d_keys, n, ins, memo, false, !ins, st, cs.cur, cs.nxt, nullptr,
-                       t->tiered ? nullptr : &fc));
-    if (ins)
-        CK(t, launch_resolve_misses(t, d_keys, n, MissMode::Init, nullptr, st, cs.cur, false,
-                                    t->tiered ? nullptr : &fc));
-    if (t->tiered) {
-        const uint32_t e = beside ? t->tier.epoch : ++t->tier.epoch;
-        if ((rc = tier_map(t, e, beside ? 1 : 0, n, st))) return rc;
-        t->sort_bits = t->bits_lines;
-    }
     const uint32_t *srow, *spos;
-    const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);  // the sort's key of a lookup without a row
-    cudaError_t err = launch_sort_rows(t, n, st, &srow, &spos, !t->tiered);
-    if (err == cudaSuccess) err = launch_reduce_apply(t, d_grads, srow, spos, n, sent, st, cs.cur);
+    cudaError_t err = cudaSuccess;
+    // (an injected wait exists in the miss kernel alone: the plan's blocks meet at
+    // the cluster's barrier)
+    if (!t->tiered && plan_fits(t, n) && !wait_injection_armed()) {
+        err = launch_plan(t, d_keys, n, ins, memo == MemoUse::Read, false, st, cs.cur, cs.nxt, &spos);
+    } else {
+        // On an HBM-resident table the probe also counts the sort's first pass (the
+        // tiered apply sorts cache lines, known only after the probe).
+        const FirstCounts fc = first_counts(t, n);
+        CK(t, launch_probe(t, d_keys, n, ins, memo, false, !ins, st, cs.cur, cs.nxt, nullptr,
+                           t->tiered ? nullptr : &fc));
+        if (ins)
+            CK(t, launch_resolve_misses(t, d_keys, n, MissMode::Init, nullptr, st, cs.cur, false,
+                                        t->tiered ? nullptr : &fc));
+        if (t->tiered) {
+            const uint32_t e = beside ? t->tier.epoch : ++t->tier.epoch;
+            if ((rc = tier_map(t, e, beside ? 1 : 0, n, st))) return rc;
+            t->sort_bits = t->bits_lines;
+        }
+        if (t->tiered && plan_fits(t, n)) {
+            err = launch_plan(t, d_keys, n, false, false, true, st, cs.cur, nullptr, &spos);
+        } else {
+            const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);  // the sort's key of a lookup without a row
+            err = launch_sort_rows(t, n, st, &srow, &spos, !t->tiered);
+            if (err == cudaSuccess) err = launch_heads(t, srow, spos, n, sent, st, cs.cur);
+        }
+    }
+    if (err == cudaSuccess) err = launch_reduce_apply(t, d_grads, spos, n, st, cs.cur);
     t->sort_bits = t->bits_rows;
     if (err != cudaSuccess) return cuda_error(t, err, "apply_grad launches");
     return MLKV_OK;
