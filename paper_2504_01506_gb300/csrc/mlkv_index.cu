@@ -106,25 +106,24 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
 #define MLKV_GET_SEG_MIN_BLOCKS 6
 #endif
 
-template <int V, bool SEG, bool INSERT>
-__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, IndexRows ra,
-                                             const int64_t* __restrict__ keys, uint32_t n,
-                                             float* __restrict__ out, uint32_t* miss_pos,
-                                             uint32_t* miss_slot, CallCounters* cur,
-                                             CallCounters* nxt, Memo memo, int lpw) {
-    pdl_enter();
+// The rows of one warp's lookups base .. base + lpw - 1, UNR rows of a lane group
+// in flight (a row of one segment); true where this lane's key is new.
+template <int V, bool SEG, bool INSERT, int UNR>
+__device__ __forceinline__ bool get_rows(const IndexArgs& ia, const IndexRows& ra, const int64_t* __restrict__ keys,
+                                         uint32_t n, float* __restrict__ out, uint32_t* miss_pos,
+                                         uint32_t* miss_slot, CallCounters* cur, const Memo& memo, uint32_t base,
+                                         int lpw) {
     using VT = typename Vec<V>::T;
-    zero_counters(nxt);
     const int lane = threadIdx.x & 31;
-    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
-    if (base >= n) return;  // warp-uniform
     const uint32_t p = base + lane;
     uint32_t row = ROW_PENDING;  // lanes past the end skip the gather
+    bool fresh = false;
     if (lane < lpw && p < n) {
         uint32_t slot = 0;
         const int64_t key = keys[p];
         row = probe_key<INSERT>(ia, (unsigned long long)key, p, slot);
-        if (INSERT && row == ROW_PENDING) append_miss(cur, miss_pos, miss_slot, p, slot, n);
+        fresh = INSERT && row == ROW_PENDING;
+        if (fresh) append_miss(cur, miss_pos, miss_slot, p, slot, n);
         if (!INSERT && row == ROW_ABSENT) record_error(ia.err, MLKV_ERR_NOT_FOUND);
         memo.key[p] = key;
         memo.row[p] = row;
@@ -144,19 +143,56 @@ __global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_
                 if (k < ra.NV) __stcs(dst + k, r == ROW_ABSENT ? Vec<V>::nan() : v1);
             }
         }
-        return;
+        return fresh;
     }
     const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
-    for (int q0 = 0; q0 < lpw; q0 += R) {
-        const int q = q0 + gid;
-        const uint32_t r = __shfl_sync(0xffffffffu, row, q);
-        VT v;
-        if (r < ROW_ABSENT && glane < ra.NV)
-            v = __ldg(reinterpret_cast<const VT*>(ra.slots + (size_t)r * ra.stride) + glane);
-        if (r == ROW_PENDING) continue;
-        VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q) * ra.d);
-        if (glane < ra.NV) __stcs(dst + glane, r == ROW_ABSENT ? Vec<V>::nan() : v);
+    for (int q0 = 0; q0 < lpw; q0 += R * UNR) {
+        VT v[UNR];
+        uint32_t rr[UNR];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const int q = q0 + u * R + gid;
+            const uint32_t r = __shfl_sync(0xffffffffu, row, q & 31);
+            rr[u] = UNR == 1 || q < lpw ? r : ROW_PENDING;
+            if (rr[u] < ROW_ABSENT && glane < ra.NV)
+                v[u] = __ldg(reinterpret_cast<const VT*>(ra.slots + (size_t)rr[u] * ra.stride) + glane);
+        }
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            if (rr[u] == ROW_PENDING) continue;
+            VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q0 + u * R + gid) * ra.d);
+            if (glane < ra.NV) __stcs(dst + glane, rr[u] == ROW_ABSENT ? Vec<V>::nan() : v[u]);
+        }
     }
+    return fresh;
+}
+
+template <int V, bool SEG, bool INSERT>
+__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, IndexRows ra,
+                                             const int64_t* __restrict__ keys, uint32_t n,
+                                             float* __restrict__ out, uint32_t* miss_pos,
+                                             uint32_t* miss_slot, CallCounters* cur,
+                                             CallCounters* nxt, Memo memo, int lpw) {
+    pdl_enter();
+    zero_counters(nxt);
+    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
+    if (base >= n) return;  // warp-uniform
+    get_rows<V, SEG, INSERT, 1>(ia, ra, keys, n, out, miss_pos, miss_slot, cur, memo, base, lpw);
+}
+
+// The Get and its miss path in one launch (see finish_get): a warp per lpw
+// lookups, in a grid that can wait for itself.
+template <int V, bool SEG>
+__global__ void __launch_bounds__(256) k_get_small(IndexArgs ia, IndexRows ra, MissArgs ma, CallCounters* nxt,
+                                                   Memo memo, int lpw) {
+    pdl_enter();
+    zero_counters(nxt);
+    const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
+    bool fresh = false;
+    if (base < ma.n)
+        fresh = get_rows<V, SEG, true, 4>(ia, ra, ma.keys, ma.n, ma.out, const_cast<uint32_t*>(ma.miss_pos),
+                                       const_cast<uint32_t*>(ma.miss_slot), ma.cur, memo, base, lpw);
+    finish_get<V, 256>(ia, ra, ma, fresh);
 }
 
 // The Get with its rows moved by the SM's asynchronous copies, for calls of
@@ -254,43 +290,6 @@ __global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, IndexRo
     if (stored && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-constexpr uint32_t kBarrierSpins = 1u << 21;  // with its L2 load and 100 ns sleep, 1-2 s a barrier
-
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Every block of the grid arrives at `ctr` (zero at the call's start) and waits
-// until all have.  Only blocks of this one grid wait here, and the kernel lets
-// the next kernel launch only after its last barrier, so every block of the
-// grid (one per SM) can become resident.  The wait is bounded: a spin that runs
-// out records MLKV_ERR_TIMEOUT and the block returns (false).
-// (`extra` is 0; mlkv_debug_fail's wait injection makes it 1, a count that
-// no grid reaches, so that the wait runs out.)
-__device__ bool grid_barrier(uint32_t* ctr, uint32_t extra, const ErrSink& err) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ok = 1;
-        __threadfence();
-        atomicAdd(ctr, 1u);
-        uint32_t spins = 0;
-        while (ld_acquire_u32(ctr) < gridDim.x + extra) {
-            if (++spins > kBarrierSpins) {
-                record_error(err, MLKV_ERR_TIMEOUT);
-                ok = 0;
-                break;
-            }
-            __nanosleep(100);
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
 // The miss path in a kernel of its own, one block per SM (see miss_path).  In
 // steady-state training nothing misses and every block returns at once.
 constexpr int kMissThreads = 512;
@@ -316,7 +315,8 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
         atomicAdd(fc.dtot + dig, 1u);
     };
     const bool done = miss_path<V, kMissThreads>(
-        ia, ra, ma, m, [&](int i) { return grid_barrier(&cur->bar[i], bar_extra, ia.err); }, count);
+        ia, ra, ma, m, gridDim.x, blockIdx.x,
+        [&](int i) { return grid_barrier(&cur->bar[i], gridDim.x + bar_extra, ia.err); }, count);
     if (!done) {
         // A block whose wait ran out returns at once; the first sort pass's counts
         // still get its share of the missed lookups, which keep no row (the last
@@ -531,11 +531,22 @@ int bulk_grid(mlkv_table* t, size_t smem, int64_t n) {
     return (int)(g < cap ? g : cap);
 }
 
+int small_get_lpw(const mlkv_table* t, int64_t n);
+
 template <int V>
 struct GetRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* out,
                            cudaStream_t st, CallCounters* cur, CallCounters* nxt) {
         const uint32_t rowbytes = (uint32_t)t->geom.d * 4;
+        const bool seg = t->geom.NV > t->geom.G, ins = t->cfg.insert_on_miss != 0;
+        if (small_get(t, n)) {
+            const int lpw = small_get_lpw(t, n);
+            const MissArgs ma = miss_args(t, keys, n, MissMode::Get, nullptr, out, cur);
+            const auto kernel = seg ? k_get_small<V, true> : k_get_small<V, false>;
+            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t), row_args(t), ma,
+                        nxt, Memo{t->s.memo_key, t->s.memo_row}, lpw);
+            return cudaGetLastError();
+        }
         if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && (uint64_t)n < kBulkMaxBatch) {
             const size_t smem = (size_t)4 * kBulkRows * rowbytes + 4 * 32 * 4;
             if (t->cfg.insert_on_miss)
@@ -548,7 +559,6 @@ struct GetRun {
                             t->s.miss_slot, cur, nxt, Memo{t->s.memo_key, t->s.memo_row});
             return cudaGetLastError();
         }
-        const bool seg = t->geom.NV > t->geom.G, ins = t->cfg.insert_on_miss != 0;
         const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
         const auto kernel = seg ? (ins ? k_get<V, true, true> : k_get<V, true, false>)
                                 : (ins ? k_get<V, false, true> : k_get<V, false, false>);
@@ -654,6 +664,22 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
         MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<false, 0>), g, 256, 0, st, index_args(t), keys,
                     (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, ra, m, (int)memo, none);
     return cudaGetLastError();
+}
+
+namespace {
+// Lookups per warp of k_get_small: as few as a grid of two blocks of 8 warps per
+// SM allows (like the miss kernel's one block of 16: several tables' waiting
+// grids fit the GPU together), at least the rows a warp copies at a time.
+int small_get_lpw(const mlkv_table* t, int64_t n) {
+    int lpw = 32 / t->geom.G;
+    while (lpw < 32 && n > (int64_t)lpw * 8 * 2 * t->num_sms) lpw *= 2;
+    return lpw;
+}
+}  // namespace
+
+bool small_get(const mlkv_table* t, int64_t n) {
+    return t->cfg.insert_on_miss != 0 && n <= (int64_t)MLKV_SMALL_GET_MAX &&
+           n <= (int64_t)small_get_lpw(t, n) * 8 * 2 * t->num_sms && !wait_injection_armed();
 }
 
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,

@@ -63,7 +63,7 @@ struct CallCounters {
     uint32_t n_single;   // runs of one lookup
     uint32_t short_next;  // run segments or units claimed (dynamic hand-out of k_short, k_reduce)
     uint32_t n_small;    // runs of 2 .. kSmallRun lookups (their positions in the record)
-    uint32_t bar[4];     // arrivals at the miss kernel's grid barriers
+    uint32_t bar[5];     // arrivals at the miss path's barriers
     uint32_t done;       // blocks of the call's last kernel that have finished (release_counters)
 };
 
@@ -487,6 +487,13 @@ enum class MissMode : int { Init = 0, Put = 1, Get = 2 };
 cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool insert, MemoUse memo,
                          bool want_slot, bool report_absent, cudaStream_t st, CallCounters* cur,
                          CallCounters* nxt, uint32_t* rows_out = nullptr, const FirstCounts* fc = nullptr);
+// A Get that inserts, of at most this many lookups, runs its miss path in its
+// own launch.  Above, the one-warp-per-few-lookups grid that can wait for itself
+// is too small for the GPU (16,384 lookups already take 8 a warp).
+#ifndef MLKV_SMALL_GET_MAX
+#define MLKV_SMALL_GET_MAX (1 << 14)
+#endif
+bool small_get(const mlkv_table* t, int64_t n);  // launch_get then needs no launch_resolve_misses
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,
                        CallCounters* cur, CallCounters* nxt);
 // release: the miss kernel is the last of the call to read its counters, and

@@ -85,6 +85,46 @@ __device__ __forceinline__ void zero_counters(CallCounters* nxt) {
         reinterpret_cast<uint32_t*>(nxt)[threadIdx.x] = 0u;
 }
 
+constexpr uint32_t kBarrierSpins = 1u << 21;  // with its L2 load and 100 ns sleep, 1-2 s a barrier
+
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Waits (one thread) until the count ctr & mask reaches `want`.  The wait is
+// bounded: a spin that runs out records MLKV_ERR_TIMEOUT and returns false.
+__device__ __forceinline__ bool wait_count(const uint32_t* ctr, uint32_t mask, uint32_t want, const ErrSink& err) {
+    uint32_t spins = 0;
+    while ((ld_acquire_u32(ctr) & mask) < want) {
+        if (++spins > kBarrierSpins) {
+            record_error(err, MLKV_ERR_TIMEOUT);
+            return false;
+        }
+        __nanosleep(100);
+    }
+    return true;
+}
+
+// `want` blocks arrive at `ctr` (zero at the call's start) and wait until all
+// have, or until one's wait has run out (false).  Only blocks of this one grid
+// wait here, and a grid that does is small enough for all its blocks to be
+// resident.  (mlkv_debug_fail's wait injection asks for one arrival more than
+// there are, so that the wait runs out.)
+__device__ __forceinline__ bool grid_barrier(uint32_t* ctr, uint32_t want, const ErrSink& err) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(ctr, 1u);
+        ok = wait_count(ctr, 0xFFFFFFFFu, want, err);
+        __threadfence();
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 // The slot array as the index kernels use it.
 struct IndexRows {
     float* slots;
@@ -117,7 +157,7 @@ __device__ __forceinline__ void copy_row(const float* __restrict__ src, float* _
 
 // ---------------------------------------------------------------------------
 // The miss path: new keys of a call get rows, in four phases separated by
-// barriers of all the grid's blocks (`barrier`):
+// barriers of all its blocks (`barrier`; `nblocks` blocks, this one `block`):
 //   1. flag the first occurrence of each new key (the lookup whose position
 //      survived in the slot's aux);
 //   2. rank the flags: an exclusive scan over the call's positions, block b
@@ -197,10 +237,10 @@ __device__ __forceinline__ uint32_t miss_block_scan(uint32_t v, uint32_t& total)
 
 template <int V, int THREADS, class Barrier, class OnRow>
 __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& ra, const MissArgs& ma, uint32_t m,
-                                          Barrier barrier, OnRow on_row) {
+                                          uint32_t nblocks, uint32_t block, Barrier barrier, OnRow on_row) {
     using VT = typename Vec<V>::T;
-    const uint32_t nthreads = gridDim.x * blockDim.x;
-    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t nthreads = nblocks * blockDim.x;
+    const uint32_t tid = block * blockDim.x + threadIdx.x;
     const int G = ra.G, glane = threadIdx.x & (G - 1);
     const uint32_t group = tid / G, ngroups = nthreads / G;
     // 1. first occurrences
@@ -210,15 +250,15 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
     }
     if (!barrier(0)) return false;
     // 2. ranks: the first occurrences at earlier positions
-    const uint32_t per = (ma.n + gridDim.x - 1) / gridDim.x;
-    const uint32_t p_lo = min(ma.n, blockIdx.x * per), p_hi = min(ma.n, p_lo + per);
+    const uint32_t per = (ma.n + nblocks - 1) / nblocks;
+    const uint32_t p_lo = min(ma.n, block * per), p_hi = min(ma.n, p_lo + per);
     uint32_t cnt = 0;
     for (uint32_t p = p_lo + threadIdx.x; p < p_hi; p += blockDim.x) cnt += __ldcg(ma.flag + p);
     const uint32_t mine = miss_block_sum<THREADS>(cnt);
-    if (threadIdx.x == 0) ma.block_sums[blockIdx.x] = mine;
+    if (threadIdx.x == 0) ma.block_sums[block] = mine;
     if (!barrier(1)) return false;
     uint32_t b_before = 0;
-    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += blockDim.x) b_before += __ldcg(ma.block_sums + b);
+    for (uint32_t b = threadIdx.x; b < block; b += blockDim.x) b_before += __ldcg(ma.block_sums + b);
     uint32_t run = miss_block_sum<THREADS>(b_before);
     for (uint32_t p0 = p_lo; p0 < p_hi; p0 += blockDim.x) {  // uniform
         const uint32_t p = p0 + threadIdx.x;
@@ -228,7 +268,7 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
         if (f) ma.rank[p] = run + ex;
         run += tot;
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) ma.cur->n_new = run;  // every first occurrence
+    if (block == nblocks - 1 && threadIdx.x == 0) ma.cur->n_new = run;  // every first occurrence
     if (!barrier(2)) return false;
     // 3. rows of the first occurrences
     const unsigned long long next = ma.ds->next_row;
@@ -257,7 +297,7 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
     }
     if (!barrier(3)) return false;
     // 4. every missed lookup takes its key's row
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (block == 0 && threadIdx.x == 0) {
         const unsigned long long nr = next + __ldcg(&ma.cur->n_new);
         ma.ds->next_row = nr < ma.capacity ? nr : ma.capacity;
     }
@@ -276,6 +316,48 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
                         ma.out + (size_t)p * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
     }
     return true;
+}
+
+// The end of a Get whose grid is small enough to wait for itself: new keys get
+// their rows, and the call's counters are released, in the same launch.  Every
+// block arrives once it has copied its rows, with a mark where it met a new
+// key.  Where no block did, the last to arrive zeroes the counters and nothing
+// waits; else the marked blocks, alone, wait for the others and run the miss
+// path.  (A miss kernel of its own that finds nothing to do cost a Get of 416
+// lookups 4 of its 15 us, and the step of 4,096 lookups 2.5 of 36.)  The whole
+// block calls it.
+template <int V, int THREADS>
+__device__ __forceinline__ void finish_get(const IndexArgs& ia, const IndexRows& ra, const MissArgs& ma,
+                                           bool new_key) {
+    __shared__ uint32_t share[2];  // marked blocks, this block among them
+    CallCounters* cur = ma.cur;
+    const uint32_t grid = gridDim.x;
+    const int marked = __syncthreads_or(new_key);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const uint32_t old = atomicAdd(&cur->bar[0], marked ? 0x10001u : 1u);
+        share[1] = old >> 16;
+        if (!marked) {
+            if (old == grid - 1) {  // the last, and no block is marked
+                uint32_t* w = reinterpret_cast<uint32_t*>(cur);
+                for (unsigned i = 0; i < sizeof(CallCounters) / 4; ++i) w[i] = 0u;
+            }
+        } else {
+            share[0] = wait_count(&cur->bar[0], 0xFFFFu, grid, ia.err) ? ld_acquire_u32(&cur->bar[0]) >> 16 : 0u;
+            __threadfence();
+        }
+    }
+    if (!marked) return;
+    __syncthreads();
+    const uint32_t blocks = share[0];
+    if (!blocks) return;  // the wait ran out
+    const uint32_t m = min(ld_u32_relaxed(&cur->n_miss), ma.n);
+    if (!miss_path<V, THREADS>(
+            ia, ra, ma, m, blocks, share[1],
+            [&](int i) { return grid_barrier(&cur->bar[i + 1], blocks, ia.err); },
+            [](uint32_t, uint32_t) {}))
+        return;
+    release_counters(cur, blocks);
 }
 
 }  // namespace

@@ -178,3 +178,35 @@ def test_put_of_hot_keys_keeps_the_last_value(n):
         ref.put(keys, values)
         _check_table(store, ref, keys, f"Put of {n}")
     store.close()
+
+
+@pytest.mark.parametrize("dim", [4, 50, 128, 260])
+@pytest.mark.parametrize("n", [1, 9, 2432, 2433, 4865, 16_384, 16_385])
+def test_get_gives_new_keys_rows(n, dim):
+    """Gets with no new key, new keys in one warp, some everywhere, and all new, on
+    both sides of the sizes whose miss path runs inside the Get's kernel; each
+    Get starts from the counters the one before left."""
+    torch_cuda()
+    store, ref = make_pair(_cfg(dim), capacity=60_000, max_batch=n)
+    rng = np.random.default_rng(n + dim)
+    fresh = iter(rng.choice(1 << 40, 55_000, replace=False).astype(np.int64))
+    known = np.array([next(fresh) for _ in range(50)], np.int64)
+    store.insert(dev(known[: min(n, 50)]))
+    ref.insert(known[: min(n, 50)])
+    known = known[: min(n, 50)]
+    for share in (0.0, 0.0, 1.0 / n, 0.3, 0.0, 1.0):
+        keys = known[rng.integers(0, len(known), n)]
+        new = np.array([next(fresh) for _ in range(int(np.ceil(n * share * 0.8)))], np.int64)
+        at = rng.choice(n, int(round(n * share)), replace=False)
+        if len(at):
+            keys[at] = new[rng.integers(0, len(new), len(at))]  # some of them more than once
+        want, _, _ = ref.get(keys)
+        assert_bits(host(store.get(dev(keys))), want, f"Get, {share:.2f} of the lookups new")
+        assert store.size() == ref.size()
+        assert np.array_equal(host(store.find(dev(keys))), ref.find(keys))
+    grads = _grads(rng, n, dim)
+    store.apply_grad(dev(keys), dev(grads))
+    ref.apply_grad(keys, grads)
+    _check_table(store, ref, keys, "apply after the Gets")
+    assert store.sync() == 0
+    store.close()
