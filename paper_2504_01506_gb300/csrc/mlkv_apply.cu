@@ -236,8 +236,9 @@ __device__ __forceinline__ uint32_t scan_end(const uint32_t* __restrict__ srow, 
 #ifndef MLKV_HEADS_MIN_BLOCKS
 #define MLKV_HEADS_MIN_BLOCKS 4
 #endif
-__global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a) {
+__global__ void __launch_bounds__(256, MLKV_HEADS_MIN_BLOCKS) k_heads(RunArgs a, SortTail tail) {
     pdl_enter();
+    zero_tail(tail);
     constexpr int kList = 128, kListS = 64, kQueue = 16;
     __shared__ uint4 lst[8][kListS];  // (start, end, row, first lookup) of short runs
     __shared__ uint2 sgl[8][kList];   // (row, lookup) of runs of one lookup
@@ -1119,7 +1120,7 @@ int64_t node_counters(int64_t max_items, int dim) {
 }
 
 cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,
-                         cudaStream_t st, CallCounters* cur) {
+                         cudaStream_t st, CallCounters* cur, const SortTail& tail) {
     const RunArgs a = run_args(t, nullptr, srow, spos, n, sent, cur);
     // a warp per 32 positions, the windows dealt out grid-stride over at most
     // one wave of blocks
@@ -1127,7 +1128,7 @@ cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* sp
     int64_t gh = (n + 255) / 256;
     if (gh > cap) gh = cap;
     if (gh < 1) gh = 1;
-    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_heads, (unsigned)gh, 256, 0, st, a);
+    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_heads, (unsigned)gh, 256, 0, st, a, tail);
     return cudaGetLastError();
 }
 

@@ -24,7 +24,7 @@ namespace {
 // together (the probe is latency-bound: a key load, then a random slot load).
 // With CT > 0 (the gradient apply on an HBM-resident table) a block of CT
 // threads covers one tile of the sort (CT * kProbeKeys lookups: 1024 threads
-// for 4096-lookup tiles, 256 for 1024) and also counts the first sort pass's
+// for 4096-lookup tiles, 512 for 2048) and also counts the first sort pass's
 // digits of its rows (see FirstCounts).
 constexpr int kProbeKeys = 4;
 
@@ -81,11 +81,7 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
     }
     if (COUNT) {
         __syncthreads();
-        for (int d = threadIdx.x; d < fc.radix; d += blockDim.x) {
-            const uint32_t c = hist[d];
-            fc.counts[(size_t)d * fc.ntiles + blockIdx.x] = c;
-            if (c) atomicAdd(fc.dtot + d, c);
-        }
+        put_counts(hist, fc.counts, fc.packed != 0, fc.ntiles, fc.radix, blockIdx.x, fc.dtot);
     }
 }
 
@@ -311,7 +307,7 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
     auto count = [&](uint32_t p, uint32_t r) {
         if (!fc.counts) return;
         const uint32_t dig = (r >= ROW_ABSENT ? fc.sent : r) & (uint32_t)(fc.radix - 1);
-        atomicAdd(&fc.counts[(size_t)dig * fc.ntiles + (p >> fc.tile_shift)], 1u);
+        add_count(fc.counts, fc.packed != 0, fc.ntiles, fc.radix, p >> fc.tile_shift, dig, 1u);
         atomicAdd(fc.dtot + dig, 1u);
     };
     const bool done = miss_path<V, kMissThreads>(

@@ -31,19 +31,18 @@ constexpr int kSortMaxPasses = 4;      // row ids have at most 31 bits
 constexpr int kSortMaxDigitBits = 9;   // radix <= 512
 constexpr int kSortMaxRadix = 1 << kSortMaxDigitBits;
 constexpr int kSortTile = 4096;        // lookups per tile of a sort pass ...
-#ifndef MLKV_SORT_SMALL_TILE_SHIFT
-#define MLKV_SORT_SMALL_TILE_SHIFT 10
-#endif
-constexpr int kSortTileSmallShift = MLKV_SORT_SMALL_TILE_SHIFT;
+constexpr int kSortTileSmallShift = 11;
 constexpr int kSortTileSmall = 1 << kSortTileSmallShift;  // ... and in batches of fewer than kSortSmallBatch lookups
-static_assert(kSortTileSmallShift >= 9 && kSortTileSmallShift <= 11, "small tiles of 512 .. 2048 lookups");
 #ifndef MLKV_SORT_SMALL_BATCH
 #define MLKV_SORT_SMALL_BATCH (1u << 19)
 #endif
 constexpr uint32_t kSortSmallBatch = MLKV_SORT_SMALL_BATCH;
 // log2 of the sort's tile for a batch of n lookups: small batches take small
 // tiles, so that a pass still spreads over the SMs (200k lookups are 49 tiles
-// of 4096 but 196 of 1024)
+// of 4096 but 98 of 2048).  Their tiles are few enough for every block of a
+// pass to add up the counts of the tiles before its own, so they need no
+// offsets kernel (mlkv_sort.cu); their counts are packed, [tile][digit] with 16
+// bits a digit, the large tiles' are [digit][tile].
 inline int sort_tile_shift(int64_t n) { return n < (int64_t)kSortSmallBatch ? kSortTileSmallShift : 12; }
 constexpr int kSmallRun = 4;           // runs of 2 .. kSmallRun lookups carry their positions in their record
 constexpr int64_t kMaxStaleness = MLKV_MAX_STALENESS;  // largest bound kept below no bound
@@ -102,8 +101,7 @@ struct Scratch {
     uint32_t* rank;         // [max_batch]
     uint32_t* sk[2];        // sort keys (row ids), ping-pong [max_batch]
     uint32_t* sv[2];        // sort values (positions), ping-pong [max_batch]
-    uint32_t* sort_counts;  // [512][tiles] digit counts of the sort's even passes ...
-    uint32_t* sort_counts2; // ... and of its odd passes (zero between sorts)
+    uint32_t* sort_counts[3];  // digit counts of the sort's passes, in turn (all but the first zero between sorts)
     uint32_t* sort_offsets; // [tiles][512] output position of each tile's first element of each digit
     uint32_t* sort_dtot;    // [kSortMaxPasses][512] digit totals of each pass, zero between sorts
     uint32_t* tile_sums;    // [max(scan tiles, SMs)]: per-tile sums of the dedup's scan, per-block of the miss kernel
@@ -477,7 +475,41 @@ struct FirstCounts {
     int radix;       // digits of the first pass
     uint32_t sent;   // sort key of a lookup without a row
     int tile_shift;  // log2 of the sort's tile (sort_tile_shift)
+    int packed;      // the counts' layout (sort_tile_shift)
 };
+
+// Adds c to the count of digit dig of a tile; a packed tile holds fewer than
+// 2^16 lookups.
+__device__ __forceinline__ void add_count(uint32_t* counts, bool packed, uint32_t ntiles, int radix, uint32_t tile,
+                                          uint32_t dig, uint32_t c) {
+    if (packed) atomicAdd(counts + (size_t)tile * (radix / 2) + dig / 2, c << (16 * (dig & 1u)));
+    else atomicAdd(counts + (size_t)dig * ntiles + tile, c);
+}
+
+// Writes a tile's counts hist[radix] whole, and adds them to the totals (the block).
+__device__ __forceinline__ void put_counts(const uint32_t* hist, uint32_t* counts, bool packed, uint32_t ntiles,
+                                           int radix, uint32_t tile, uint32_t* dtot) {
+    for (int d = threadIdx.x; d < radix; d += blockDim.x) {
+        const uint32_t c = hist[d];
+        if (!packed) counts[(size_t)d * ntiles + tile] = c;
+        else if (!(d & 1)) counts[(size_t)tile * (radix / 2) + d / 2] = c | hist[d + 1] << 16;
+        if (c) atomicAdd(dtot + d, c);
+    }
+}
+
+// What the sort's last pass leaves for the kernel after it to zero.
+struct SortTail {
+    uint32_t* counts;
+    uint32_t words;
+    uint32_t* dtot;
+    uint32_t radix;
+};
+
+__device__ __forceinline__ void zero_tail(const SortTail& t) {
+    const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (uint32_t i = i0; i < t.words; i += step) t.counts[i] = 0u;
+    for (uint32_t i = i0; i < t.radix; i += step) t.dtot[i] = 0u;
+}
 
 // ---------------------------------------------------------------------------
 // Host-side launchers (each returns cudaGetLastError() of its launches).
@@ -516,10 +548,11 @@ cudaError_t launch_export(mlkv_table* t, const int64_t* keys, int64_t n, float* 
 FirstCounts first_counts(mlkv_table* t, int64_t n);
 // first_counted: the first pass's counts were made by the apply's probe and
 // miss kernel (FirstCounts).
+// tail: for the kernel launched next, which zeroes it.
 cudaError_t launch_sort_rows(mlkv_table* t, int64_t n, cudaStream_t st, const uint32_t** srow,
-                             const uint32_t** spos, bool first_counted = false);
+                             const uint32_t** spos, bool first_counted, SortTail& tail);
 cudaError_t launch_segments(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n,
-                            cudaStream_t st, CallCounters* cur);
+                            cudaStream_t st, CallCounters* cur, const SortTail& tail);
 cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t* spos, int64_t n,
                              int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
                              CallCounters* cur);
@@ -551,7 +584,7 @@ void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& item
 int64_t node_counters(int64_t max_items, int dim);  // counters of the combine's nodes
 // The run lists of sorted rows; and the reduce of the listed runs.
 cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,
-                         cudaStream_t st, CallCounters* cur);
+                         cudaStream_t st, CallCounters* cur, const SortTail& tail);
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
                                 cudaStream_t st, CallCounters* cur);
 

@@ -6,19 +6,27 @@
 // 40-bit keys), and the sorted order visits rows in memory order.  An absent
 // lookup is given the all-ones digit pattern and sorts last.
 //
-// Each pass is a reduce-then-scan pass over tiles of 4096 elements (1024 in
+// Each pass is a reduce-then-scan pass over tiles of 4096 elements (2048 in
 // batches of fewer than kSortSmallBatch lookups, which would otherwise cover a
 // fraction of the SMs): the digit counts of every tile and the pass's digit
-// totals come first; one kernel gives every (tile, digit) the output position
-// of its first element (the elements of lower digits plus those of the digit
-// in earlier tiles); a second ranks each tile's elements stably (over rounds
-// of 32, in order) and scatters them.  The counts of the first pass are made
-// by a histogram kernel, or in a gradient apply by the probe and the miss
-// kernel (FirstCounts); those of every later pass by the scatter before it,
-// which knows the tile each element lands in and adds the element's next digit
-// to that tile's count (one add per run of equal targets in a warp), so no
-// pass after the first reads its input twice.  No block waits on another, so
-// a pass costs the same when the sort shares the GPU with other kernels.  (A
+// totals come first; then every (tile, digit) needs the output position of its
+// first element (the elements of lower digits plus those of the digit in
+// earlier tiles); and the scatter ranks each tile's elements stably (over
+// rounds of 32, in order) and writes them out.  The positions are made by a
+// kernel of their own in large batches (416 tiles of a 1.7M-lookup batch), and
+// in small ones by each block of the scatter for itself: it reads the packed
+// counts of the tiles before its own (200k lookups: at most 97 rows of 512 or
+// 1,024 bytes) beside its elements, which costs less than the launch of a
+// kernel between two passes.  (Apply + Get of 200k lookups of dim 100: 153 ->
+// 140 us; apply + export of 100,003 of dim 50: 88.7 -> 78.  At 2^19 lookups the
+// blocks read 33 MB of counts a pass, as long as the offsets kernel takes.)  The
+// counts of the first pass are made by a histogram
+// kernel, or in a gradient apply by the probe and the miss kernel
+// (FirstCounts); those of every later pass by the scatter before it, which
+// knows the tile each element lands in and adds the element's next digit to
+// that tile's count (one add per run of equal targets in a warp), so no pass
+// after the first reads its input twice.  No block waits on another, so a pass
+// costs the same when the sort shares the GPU with other kernels.  (A
 // single-pass decoupled look-back sort was slower here: a batch is about one
 // wave of tiles, and the chain of tiles that know their prefix grows one
 // window per round trip.)
@@ -33,7 +41,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kItems = 16;
 constexpr int kTile = kThreads * kItems;  // 4096
-constexpr int kWarps = kThreads / 32;
 
 // Exclusive scan of one value per thread over a block of THREADS threads.
 template <int THREADS>
@@ -117,7 +124,7 @@ template <int TILE>
 __global__ void __launch_bounds__(TILE >= 1024 ? kThreads : TILE / 4) k_sort_hist(const uint32_t* __restrict__ kin, uint32_t n,
                                                         uint32_t* __restrict__ counts, uint32_t* __restrict__ dtot,
                                                         uint32_t ntiles, int shift, int radix, uint32_t sent,
-                                                        int first) {
+                                                        int first, int packed) {
     constexpr int kHThreads = TILE >= 1024 ? kThreads : TILE / 4;
     constexpr int kItems = TILE / kHThreads;
     static_assert(kItems % 4 == 0, "whole 16-byte loads");
@@ -155,11 +162,7 @@ __global__ void __launch_bounds__(TILE >= 1024 ? kThreads : TILE / 4) k_sort_his
     }
     if (cnt) atomicAdd(&hist[cur], cnt);
     __syncthreads();
-    for (int d = threadIdx.x; d < radix; d += kHThreads) {
-        const uint32_t c = hist[d];
-        counts[(size_t)d * ntiles + blockIdx.x] = c;
-        if (c) atomicAdd(dtot + d, c);
-    }
+    put_counts(hist, counts, packed != 0, ntiles, radix, blockIdx.x, dtot);
 }
 
 // Output position of the first element of every (tile, digit): the elements
@@ -239,47 +242,68 @@ __global__ void __launch_bounds__(kOThreads) k_sort_offsets(const uint32_t* __re
 // tile's elements of digit d.  With nshift >= 0 the element's digit of the
 // next pass (bits nshift ..) is added to the count of the tile of the next
 // pass that holds its output position, ncounts[digit][dst / TILE] (zero on
-// entry), and to the next pass's digit totals ndtot.  The counts this pass's
-// offsets came from (`counts`, read by the offsets kernel, which has
-// finished) are zeroed, for the pass after next to count into.
-// threads of the scatter's block for the small tiles (4 elements a thread)
-#ifndef MLKV_SCATTER_SMALL_THREADS
-#define MLKV_SCATTER_SMALL_THREADS (kSortTileSmall / 4)
-#endif
+// entry), and to the next pass's digit totals ndtot.  The counts and totals of
+// the pass before (zcounts, zdtot) are zeroed here: every block of this pass
+// reads its own pass's, so the next kernel zeroes those.
+// With SELF the block adds up offsets from `counts` (packed) itself.
 #ifndef MLKV_SCATTER_MIN_BLOCKS
 #define MLKV_SCATTER_MIN_BLOCKS 3
 #endif
-template <int TILE, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLOCKS : 4) k_sort_scatter(
-    const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, uint32_t n, const uint32_t* __restrict__ offsets, uint32_t ntiles, int shift,
-    int radix, uint32_t sent, int first, uint32_t* __restrict__ dtot, int nshift, uint32_t* __restrict__ ncounts,
-    uint32_t* __restrict__ ndtot, uint32_t* __restrict__ counts) {
+struct ScatterArgs {
+    const uint32_t* kin;
+    const uint32_t* vin;
+    uint32_t* kout;
+    uint32_t* vout;
+    uint32_t n;
+    const uint32_t* offsets;  // [tile][radix] (without SELF)
+    const uint32_t* counts;   // this pass's counts and digit totals (SELF)
+    const uint32_t* dtot;
+    uint32_t ntiles;
+    int shift, radix;
+    uint32_t sent;
+    int first;
+    int nshift;
+    uint32_t* ncounts;
+    uint32_t* ndtot;
+    uint32_t* zcounts;  // or null
+    uint32_t* zdtot;
+};
+
+template <int TILE, int THREADS, bool SELF>
+__global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k_sort_scatter(ScatterArgs s) {
     constexpr int kSWarps = THREADS / 32;
     constexpr int kSItems = TILE / THREADS;
-    constexpr int kTileShift = TILE == 4096 ? 12 : TILE == 2048 ? 11 : TILE == 1024 ? 10 : 9;
-    static_assert(TILE == (1 << kTileShift), "tiles of 512 .. 4096");
+    constexpr int kTileShift = TILE == 4096 ? 12 : 11;
+    static_assert(TILE == (1 << kTileShift), "tiles of 2048 or 4096");
     pdl_enter();
-    // the pass's digit totals were read by the offsets kernel, which has
-    // finished: zero them for the next sort (the totals are zero between sorts)
-    if (blockIdx.x == 0)
-        for (int d = threadIdx.x; d < radix; d += THREADS) dtot[d] = 0u;
-    // ... and this tile's column of the counts (radix x ntiles, a column a block)
-    for (int d = threadIdx.x; d < radix; d += THREADS) counts[(size_t)d * ntiles + blockIdx.x] = 0u;
+    const uint32_t* __restrict__ kin = s.kin;
+    const uint32_t* __restrict__ vin = s.vin;
+    const uint32_t n = s.n, sent = s.sent, ntiles = s.ntiles;
+    const int shift = s.shift, radix = s.radix, first = s.first, nshift = s.nshift;
+    if (s.zcounts) {
+        // this tile's share of the counts of the pass before
+        const uint32_t words = SELF ? radix / 2 : radix;
+        for (uint32_t d = threadIdx.x; d < words; d += THREADS) {
+            if (SELF) s.zcounts[(size_t)blockIdx.x * words + d] = 0u;
+            else s.zcounts[(size_t)d * ntiles + blockIdx.x] = 0u;
+        }
+        if (blockIdx.x == 0)
+            for (int d = threadIdx.x; d < radix; d += THREADS) s.zdtot[d] = 0u;
+    }
     // the per-warp digit counts, then (once every position is known) the sorted tile
-    __shared__ uint32_t pool[2 * TILE];
-    constexpr bool kShare = kSWarps * kMaxRadix <= 2 * TILE;  // the counts fit the tile buffer
-    __shared__ uint32_t wpool[kShare ? 1 : kSWarps * kMaxRadix];
-    uint32_t (*wcnt)[kMaxRadix] = reinterpret_cast<uint32_t (*)[kMaxRadix]>(kShare ? pool : wpool);
+    constexpr int kPool = 2 * TILE > kSWarps * kMaxRadix ? 2 * TILE : kSWarps * kMaxRadix;
+    __shared__ uint32_t pool[kPool];
+    uint32_t (*wcnt)[kMaxRadix] = reinterpret_cast<uint32_t (*)[kMaxRadix]>(pool);
     uint32_t* skey = pool;
     uint32_t* sval = pool + TILE;
+    __shared__ uint32_t part[SELF ? 2 * THREADS : 1];  // per group of threads: counts of the tiles before this one
     __shared__ uint32_t gbase[kMaxRadix];   // output position of the tile's first element of each digit
     __shared__ uint32_t lbase[kMaxRadix];   // position in the sorted tile of its first element of each digit
     __shared__ uint32_t ntot[kMaxRadix];    // the tile's elements of each digit of the next pass
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kSWarps * kMaxRadix; i += THREADS) (&wcnt[0][0])[i] = 0;
     for (int d = threadIdx.x; d < radix; d += THREADS) {
-        gbase[d] = offsets[(size_t)blockIdx.x * radix + d];
+        if (!SELF) gbase[d] = s.offsets[(size_t)blockIdx.x * radix + d];
         ntot[d] = 0u;
     }
     __syncthreads();
@@ -294,6 +318,27 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLO
         const uint32_t i = base + r * 32 + lane;
         key[r] = i < n ? sort_key(kin[i], sent, first) : 0u;
         val[r] = i < n ? (first ? i : vin[i]) : 0u;
+    }
+    if (SELF) {  // beside them, the counts of the tiles before: a group of radix / 2 threads per row
+        const uint32_t words = radix / 2, groups = THREADS / words;
+        const uint32_t grp = threadIdx.x / words, x = threadIdx.x & (words - 1);
+        uint32_t lo = 0, hi = 0;
+        constexpr int kRows = 16;  // in flight
+        for (uint32_t t0 = grp; t0 < blockIdx.x; t0 += groups * kRows) {
+            uint32_t c[kRows];
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+                const uint32_t t = t0 + k * groups;
+                c[k] = t < blockIdx.x ? __ldg(s.counts + (size_t)t * words + x) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+                lo += c[k] & 0xFFFFu;
+                hi += c[k] >> 16;
+            }
+        }
+        part[grp * radix + 2 * x] = lo;
+        part[grp * radix + 2 * x + 1] = hi;
     }
 #pragma unroll
     for (int r = 0; r < kSItems; ++r) {
@@ -328,6 +373,15 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLO
     }
     uint32_t all;
     uint32_t run = block_exclusive_scan_n<THREADS>(mine, all);
+    if (SELF) {  // the elements of lower digits, and the digit's in the tiles before
+        const int d = threadIdx.x;
+        uint32_t total;
+        uint32_t at = block_exclusive_scan_n<THREADS>(d < radix ? __ldg(s.dtot + d) : 0u, total);
+        if (d < radix) {
+            for (int g = 0; g < 2 * THREADS / radix; ++g) at += part[g * radix + d];
+            gbase[d] = at;
+        }
+    }
 #pragma unroll
     for (int j = 0; j < kDpt; ++j) {
         const int d = threadIdx.x * dpt + j;
@@ -356,8 +410,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLO
             const uint32_t k = skey[l];
             const uint32_t dig = (k >> shift) & (radix - 1);
             const uint32_t dst = gbase[dig] + (l - lbase[dig]);
-            kout[dst] = k;
-            vout[dst] = sval[l];
+            s.kout[dst] = k;
+            s.vout[dst] = sval[l];
         }
         return;
     }
@@ -370,10 +424,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLO
             const uint32_t k = skey[l];
             const uint32_t dig = (k >> shift) & (radix - 1);
             const uint32_t dst = gbase[dig] + (l - lbase[dig]);
-            kout[dst] = k;
-            vout[dst] = sval[l];
+            s.kout[dst] = k;
+            s.vout[dst] = sval[l];
             e = (k >> nshift) & (radix - 1);
-            target = e * ntiles + (dst >> kTileShift);
+            target = SELF ? (dst >> kTileShift) * (uint32_t)radix + e : e * ntiles + (dst >> kTileShift);
         }
         // consecutive lanes with one target (a hot row's lookups, a digit's
         // run within one tile) add their count once, from the run's first lane
@@ -384,14 +438,15 @@ __global__ void __launch_bounds__(THREADS, THREADS == 512 ? MLKV_SCATTER_MIN_BLO
         if (head) {
             const uint32_t later = heads & ~((2u << lane) - 1u);
             const uint32_t len = (later ? (uint32_t)(__ffs(later) - 1) : nvalid) - (uint32_t)lane;
-            atomicAdd(ncounts + target, len);
+            if (SELF) atomicAdd(s.ncounts + target / 2, len << (16 * (target & 1u)));  // packed
+            else atomicAdd(s.ncounts + target, len);
             atomicAdd(&ntot[e], len);
         }
     }
     __syncthreads();
     for (int d = threadIdx.x; d < radix; d += THREADS) {
         const uint32_t c = ntot[d];
-        if (c) atomicAdd(ndtot + d, c);
+        if (c) atomicAdd(s.ndtot + d, c);
     }
 }
 
@@ -403,8 +458,10 @@ __device__ __forceinline__ bool is_head(const uint32_t* srow, uint32_t p, uint32
 }
 
 __global__ void __launch_bounds__(kThreads) k_seg_reduce(const uint32_t* __restrict__ srow, uint32_t n,
-                                                         uint32_t sent, uint32_t* __restrict__ tile_sums) {
+                                                         uint32_t sent, uint32_t* __restrict__ tile_sums,
+                                                         SortTail tail) {
     pdl_enter();
+    zero_tail(tail);
     const uint32_t base = blockIdx.x * kTile;
     uint32_t s = 0;
 #pragma unroll 4
@@ -489,72 +546,84 @@ inline unsigned sort_tiles(int64_t n) {
 FirstCounts first_counts(mlkv_table* t, int64_t n) {
     int passes, D;
     sort_geometry(t->sort_bits, passes, D);
-    return FirstCounts{t->s.sort_counts, t->s.sort_dtot, sort_tiles(n), 1 << D,
-                       (uint32_t)((1ull << t->sort_bits) - 1), sort_tile_shift(n)};
+    const int shift = sort_tile_shift(n);
+    return FirstCounts{t->s.sort_counts[0], t->s.sort_dtot, sort_tiles(n), 1 << D,
+                       (uint32_t)((1ull << t->sort_bits) - 1), shift, shift == kSortTileSmallShift ? 1 : 0};
 }
 
 namespace {
-template <int TILE, int THREADS>
+template <int TILE, int THREADS, bool SELF>
 void sort_passes(mlkv_table* t, int64_t n, cudaStream_t st, const uint32_t** srow, const uint32_t** spos,
-                 bool first_counted, int passes, int D) {
+                 bool first_counted, int passes, int D, SortTail& tail) {
     const int radix = 1 << D;
     const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);
     const unsigned nt = sort_tiles(n);
-    // two count buffers in turn: pass p's counts are in counts[p & 1], and its
-    // scatter counts pass p + 1 into counts[(p + 1) & 1]
-    uint32_t* counts[2] = {t->s.sort_counts, t->s.sort_counts2};
-    uint32_t* offsets = t->s.sort_offsets;
-    // the digit totals of every pass, and the second count buffer, are zero
-    // between sorts (the arena starts zeroed; each pass's scatter zeroes its
-    // pass's totals and the counts its offsets came from; the first pass's
-    // counts are written whole by the probe or the histogram kernel)
-    const uint32_t* kin = t->s.row_of_pos;
-    const uint32_t* vin = nullptr;
+    // Three count buffers in turn: pass p reads counts[p % 3], counts pass p + 1
+    // into counts[(p + 1) % 3] and zeroes the one pass p - 1 read; the kernel
+    // after the sort zeroes the last pass's (tail).  So all are zero between
+    // sorts but the first pass's, which is written whole, by the probe or the
+    // histogram kernel.  The digit totals likewise, one array a pass.
+    ScatterArgs a{};
+    a.kin = t->s.row_of_pos;
+    a.n = (uint32_t)n;
+    a.offsets = t->s.sort_offsets;
+    a.ntiles = nt;
+    a.radix = radix;
+    a.sent = sent;
     int out = 0;
     for (int p = 0; p < passes; ++p) {
-        const int first = p == 0;
+        uint32_t* counts = t->s.sort_counts[p % 3];
         uint32_t* dtot = t->s.sort_dtot + p * kMaxRadix;
-        if (first && !first_counted)
-            MLKV_LAUNCH(t, 0, k_sort_hist<TILE>, nt, TILE >= 1024 ? kThreads : TILE / 4, 0, st, kin, (uint32_t)n,
-                        counts[0], dtot, nt, 0,
-                        radix, sent, first);
+        if (p == 0 && !first_counted)
+            MLKV_LAUNCH(t, 0, k_sort_hist<TILE>, nt, kThreads, 0, st, a.kin, (uint32_t)n, counts, dtot, nt, 0, radix,
+                        sent, 1, SELF ? 1 : 0);
         // launched after the kernel before it has finished, not beside its
         // drain: placed early, its few blocks landed on the SMs the scatter
         // left room on (a tenth of them) and took twice as long
-        MLKV_LAUNCH_PDL(MLKV_OFFSETS_PDL != 0, t, 0, k_sort_offsets,
-                        (unsigned)((radix + kOThreads / 32 - 1) / (kOThreads / 32)), kOThreads, 0, st,
-                        counts[p & 1], dtot, offsets, nt, radix);
+        if (!SELF)
+            MLKV_LAUNCH_PDL(MLKV_OFFSETS_PDL != 0, t, 0, k_sort_offsets,
+                            (unsigned)((radix + kOThreads / 32 - 1) / (kOThreads / 32)), kOThreads, 0, st, counts, dtot,
+                            t->s.sort_offsets, nt, radix);
         // every pass but the last counts the next one
-        const int nshift = p + 1 < passes ? (p + 1) * D : -1;
-        MLKV_LAUNCH(t, MLKV_K_SORT_SCATTER, (k_sort_scatter<TILE, THREADS>), nt, THREADS, 0, st, kin, vin,
-                    t->s.sk[out], t->s.sv[out], (uint32_t)n, offsets, nt, p * D, radix, sent, first, dtot, nshift,
-                    counts[(p + 1) & 1], nshift < 0 ? nullptr : t->s.sort_dtot + (p + 1) * kMaxRadix,
-                    counts[p & 1]);
-        kin = t->s.sk[out];
-        vin = t->s.sv[out];
+        a.kout = t->s.sk[out];
+        a.vout = t->s.sv[out];
+        a.counts = counts;
+        a.dtot = dtot;
+        a.shift = p * D;
+        a.first = p == 0;
+        a.nshift = p + 1 < passes ? (p + 1) * D : -1;
+        a.ncounts = t->s.sort_counts[(p + 1) % 3];
+        a.ndtot = dtot + kMaxRadix;
+        a.zcounts = p ? t->s.sort_counts[(p - 1) % 3] : nullptr;
+        a.zdtot = p ? dtot - kMaxRadix : nullptr;
+        MLKV_LAUNCH(t, MLKV_K_SORT_SCATTER, (k_sort_scatter<TILE, THREADS, SELF>), nt, THREADS, 0, st, a);
+        tail = SortTail{counts, (uint32_t)radix * nt / (SELF ? 2u : 1u), dtot, (uint32_t)radix};
+        a.kin = t->s.sk[out];
+        a.vin = t->s.sv[out];
         out ^= 1;
     }
-    *srow = kin;
-    *spos = vin;
+    *srow = a.kin;
+    *spos = a.vin;
 }
 }  // namespace
 
 cudaError_t launch_sort_rows(mlkv_table* t, int64_t n, cudaStream_t st, const uint32_t** srow,
-                             const uint32_t** spos, bool first_counted) {
+                             const uint32_t** spos, bool first_counted, SortTail& tail) {
     int passes, D;
     sort_geometry(t->sort_bits, passes, D);
     if (sort_tile_shift(n) == 12)
-        sort_passes<kSortTile, 512>(t, n, st, srow, spos, first_counted, passes, D);
+        sort_passes<kSortTile, 512, false>(t, n, st, srow, spos, first_counted, passes, D, tail);
     else
-        sort_passes<kSortTileSmall, MLKV_SCATTER_SMALL_THREADS>(t, n, st, srow, spos, first_counted, passes, D);
+        sort_passes<kSortTileSmall, 512, true>(t, n, st, srow, spos, first_counted, passes, D, tail);
     return cudaGetLastError();
 }
 
 cudaError_t launch_segments(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n,
-                            cudaStream_t st, CallCounters* cur) {
+                            cudaStream_t st, CallCounters* cur, const SortTail& tail) {
     const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);
     const unsigned nt = tiles(n);
-    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_reduce, nt, kThreads, 0, st, srow, (uint32_t)n, sent, t->s.tile_sums);
+    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_reduce, nt, kThreads, 0, st, srow, (uint32_t)n, sent, t->s.tile_sums,
+                tail);
     MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_down, nt, kThreads, 0, st, srow, spos, (uint32_t)n, sent,
                 t->s.tile_sums, t->s.seg_start, t->s.run_row, t->s.run_p0, cur, t->dstate);
     return cudaGetLastError();

@@ -571,7 +571,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
     long_bounds(B, s.max_long, s.max_nodes, s.max_items);
     s.node_cnt_bytes = node_counters(s.max_items, c.dim) * 4;
     s.tile_sums_len = std::max<int64_t>(tiles_of(B) + 1, t->num_sms);
-    // the sort's tiles: 4096 lookups, 1024 in batches under kSortSmallBatch
+    // the sort's tiles: 4096 lookups, kSortTileSmall in batches under kSortSmallBatch
     const int64_t sort_tiles = std::max<int64_t>(
         tiles_of(B), (std::min<int64_t>(B, (int64_t)kSortSmallBatch - 1) + kSortTileSmall - 1) / kSortTileSmall);
     struct Piece {
@@ -586,8 +586,9 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.sk[0], B * 4},          {(void**)&s.sk[1], B * 4},
         {(void**)&s.sv[0], B * 4},          {(void**)&s.sv[1], B * 4},
         {(void**)&s.tile_sums, s.tile_sums_len * 4},
-        {(void**)&s.sort_counts, s.sort_counts_bytes = 512 * sort_tiles * 4},
-        {(void**)&s.sort_counts2, 512 * sort_tiles * 4},
+        {(void**)&s.sort_counts[0], s.sort_counts_bytes = 512 * sort_tiles * 4},
+        {(void**)&s.sort_counts[1], s.sort_counts_bytes},
+        {(void**)&s.sort_counts[2], s.sort_counts_bytes},
         {(void**)&s.sort_offsets, 512 * sort_tiles * 4},
         {(void**)&s.sort_dtot, kSortMaxPasses * 512 * 4},
         {(void**)&s.seg_start, (B + 1) * 4},  {(void**)&s.run_row, B * 4},
@@ -760,8 +761,9 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
             err = launch_plan(t, d_keys, n, false, false, true, st, cs.cur, nullptr, &spos);
         } else {
             const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);  // the sort's key of a lookup without a row
-            err = launch_sort_rows(t, n, st, &srow, &spos, !t->tiered);
-            if (err == cudaSuccess) err = launch_heads(t, srow, spos, n, sent, st, cs.cur);
+            SortTail tail;
+            err = launch_sort_rows(t, n, st, &srow, &spos, !t->tiered, tail);
+            if (err == cudaSuccess) err = launch_heads(t, srow, spos, n, sent, st, cs.cur, tail);
         }
     }
     if (err == cudaSuccess) err = launch_reduce_apply(t, d_grads, spos, n, st, cs.cur);
@@ -835,8 +837,9 @@ int mlkv_dedup(mlkv_table* t, const int64_t* d_keys, int64_t n, int64_t* d_uniqu
     CallScope cs = begin_call(t, st);
     CK(t, launch_probe(t, d_keys, n, false, MemoUse::None, false, false, st, cs.cur, cs.nxt));
     const uint32_t *srow, *spos;
-    CK(t, launch_sort_rows(t, n, st, &srow, &spos));
-    CK(t, launch_segments(t, srow, spos, n, st, cs.cur));
+    SortTail tail;
+    CK(t, launch_sort_rows(t, n, st, &srow, &spos, false, tail));
+    CK(t, launch_segments(t, srow, spos, n, st, cs.cur, tail));
     CK(t, launch_dedup_out(t, d_keys, spos, n, d_unique_keys, d_counts, d_num_unique, st, cs.cur));
     return MLKV_OK;
 }
@@ -917,8 +920,7 @@ int mlkv_clear_status(mlkv_table* t) {
     CK(t, cudaMemset(t->dstate->cc, 0, sizeof(t->dstate->cc)));
     CK(t, cudaMemset(t->dstate->cca, 0, sizeof(t->dstate->cca)));
     // ... and the sort's counts and digit totals, zero between sorts
-    CK(t, cudaMemset(t->s.sort_counts, 0, t->s.sort_counts_bytes));
-    CK(t, cudaMemset(t->s.sort_counts2, 0, t->s.sort_counts_bytes));
+    for (uint32_t* counts : t->s.sort_counts) CK(t, cudaMemset(counts, 0, t->s.sort_counts_bytes));
     CK(t, cudaMemset(t->s.sort_dtot, 0, kSortMaxPasses * 512 * 4));
     CK(t, cudaMemset(t->s.node_cnt, 0, (size_t)t->s.node_cnt_bytes));
     CK(t, cudaDeviceSynchronize());
