@@ -52,8 +52,6 @@ constexpr int64_t kMaxStaleness = MLKV_MAX_STALENESS;  // largest bound kept bel
 struct CallCounters {
     uint32_t n_miss;     // lookups whose key had no row yet
     uint32_t n_new;      // distinct new keys (first occurrences)
-    uint32_t n_unique;   // distinct rows after the sort
-    uint32_t n_valid;    // lookups with a row
     uint32_t n_long;     // runs longer than MLKV_SEQ_SEGMENT_MAX
     uint32_t n_items;    // chunks of the long runs
     uint32_t n_group;    // long runs combined by a lane group
@@ -105,9 +103,6 @@ struct Scratch {
     uint32_t* sort_offsets; // [tiles][512] output position of each tile's first element of each digit
     uint32_t* sort_dtot;    // [kSortMaxPasses][512] digit totals of each pass, zero between sorts
     uint32_t* tile_sums;    // [max(scan tiles, SMs)]: per-tile sums of the dedup's scan, per-block of the miss kernel
-    uint32_t* seg_start;    // [max_batch + 1] run starts in sorted order (dedup)
-    uint32_t* run_row;      // [max_batch] row of each run (dedup)
-    uint32_t* run_p0;       // [max_batch] first lookup position of each run (dedup)
     uint4* short_runs;      // [max_batch] the apply's runs of 2 .. MLKV_SEQ_SEGMENT_MAX lookups
     uint2* single_runs;     // [max_batch] its runs of one lookup: (row, lookup position)
     uint4* small_runs;      // [max_batch] runs of 2 .. kSmallRun lookups: (row, p0, p1, p2)
@@ -551,11 +546,9 @@ FirstCounts first_counts(mlkv_table* t, int64_t n);
 // tail: for the kernel launched next, which zeroes it.
 cudaError_t launch_sort_rows(mlkv_table* t, int64_t n, cudaStream_t st, const uint32_t** srow,
                              const uint32_t** spos, bool first_counted, SortTail& tail);
-cudaError_t launch_segments(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n,
-                            cudaStream_t st, CallCounters* cur, const SortTail& tail);
-cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t* spos, int64_t n,
-                             int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
-                             CallCounters* cur);
+cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t* srow, const uint32_t* spos,
+                             int64_t n, int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
+                             const SortTail& tail);
 
 // mlkv_plan.cu
 // Applies of at most this many lookups are planned by one cluster (why here: mlkv_plan.cu).

@@ -1,5 +1,5 @@
 // Dedup of a gradient batch: a stable LSD radix sort of (row id, position)
-// pairs, then the segment starts of the sorted row ids.
+// pairs, then the runs of the sorted row ids.
 //
 // The sort key is the 32-bit row id, not the 64-bit key: rows are dense in
 // [0, capacity), so 3 passes of 9 bits cover 10^8 rows (against 5+ passes for
@@ -36,8 +36,8 @@ namespace mlkv {
 
 namespace {
 
-// the tiles of the segment scan (k_seg_*), and the block of the histogram and
-// offsets kernels
+// the tiles of the dedup's output (k_seg_count, k_dedup_out), and the block of
+// the histogram and offsets kernels
 constexpr int kThreads = 256;
 constexpr int kItems = 16;
 constexpr int kTile = kThreads * kItems;  // 4096
@@ -450,79 +450,103 @@ __global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k
     }
 }
 
-// --- segments -------------------------------------------------------------------
-__device__ __forceinline__ bool is_head(const uint32_t* srow, uint32_t p, uint32_t n, uint32_t sent) {
-    if (p >= n) return false;
-    const uint32_t r = srow[p];
-    return r != sent && (p == 0 || srow[p - 1] != r);
+// --- the dedup's output ----------------------------------------------------------
+// The runs of the sorted row ids, as (first lookup's key, length) in order: the
+// run heads of every tile of 4096 counted, then every tile finds its heads
+// again, knows from the counts how many are before them, and writes its runs.
+// A thread takes 16 consecutive elements (four 16-byte loads).  Bound by the
+// sorted arrays' 8 bytes a lookup in L2 and the random 8-byte key of each run.
+// (1.7M lookups, 0.31M runs: 44 us for three kernels that read a thread's 16
+// elements one by one and kept the runs' starts in memory between them, 19 for
+// these two.)
+
+// A bit per element of this thread's 16 from position `first`: a run starts there.
+__device__ __forceinline__ uint32_t head_bits(const uint32_t* __restrict__ srow, uint32_t first, uint32_t n,
+                                              uint32_t sent) {
+    uint32_t r[kItems];
+    if (first + kItems <= n) {
+        const uint4* v = reinterpret_cast<const uint4*>(srow + first);
+#pragma unroll
+        for (int q = 0; q < kItems / 4; ++q) {
+            const uint4 x = __ldg(v + q);
+            r[4 * q] = x.x;
+            r[4 * q + 1] = x.y;
+            r[4 * q + 2] = x.z;
+            r[4 * q + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) r[k] = first + k < n ? __ldg(srow + first + k) : sent;
+    }
+    uint32_t left = first && first < n ? __ldg(srow + first - 1) : ~r[0];
+    uint32_t bits = 0;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        if (r[k] != left && r[k] != sent) bits |= 1u << k;
+        left = r[k];
+    }
+    return bits;
 }
 
-__global__ void __launch_bounds__(kThreads) k_seg_reduce(const uint32_t* __restrict__ srow, uint32_t n,
-                                                         uint32_t sent, uint32_t* __restrict__ tile_sums,
-                                                         SortTail tail) {
+__global__ void __launch_bounds__(kThreads) k_seg_count(const uint32_t* __restrict__ srow, uint32_t n, uint32_t sent,
+                                                        uint32_t* __restrict__ tile_sums, SortTail tail) {
     pdl_enter();
     zero_tail(tail);
-    const uint32_t base = blockIdx.x * kTile;
-    uint32_t s = 0;
-#pragma unroll 4
-    for (int k = 0; k < kItems; ++k) s += is_head(srow, base + k * kThreads + threadIdx.x, n, sent);
+    const uint32_t first = blockIdx.x * kTile + threadIdx.x * kItems;
     uint32_t total;
-    block_exclusive_scan(s, total);
+    block_exclusive_scan((uint32_t)__popc(head_bits(srow, first, n, sent)), total);
     if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kThreads) k_seg_down(const uint32_t* __restrict__ srow,
-                                                       const uint32_t* __restrict__ spos, uint32_t n,
-                                                       uint32_t sent, const uint32_t* __restrict__ tile_sums,
-                                                       uint32_t* __restrict__ seg_start,
-                                                       uint32_t* __restrict__ run_row,
-                                                       uint32_t* __restrict__ run_p0, CallCounters* cur,
-                                                       DevState* ds) {
-    pdl_enter();
-    const uint32_t base = blockIdx.x * kTile;
-    const uint32_t prefix = tiles_before(tile_sums, blockIdx.x);
-    // thread t owns items base + t*16 .. +15 (consecutive, for an in-order compaction)
-    const uint32_t first = base + threadIdx.x * kItems;
-    uint32_t flags = 0, cnt = 0;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        const uint32_t p = first + k;
-        if (is_head(srow, p, n, sent)) {
-            flags |= 1u << k;
-            ++cnt;
-        }
-        if (p < n && srow[p] != sent && (p + 1 == n || srow[p + 1] == sent)) cur->n_valid = p + 1;
+// The end of the run of `row` that holds position q - 1: the first position
+// from q on with another row, or n (the whole warp; the rows ascend).
+__device__ __forceinline__ uint32_t end_from(const uint32_t* __restrict__ srow, uint32_t n, uint32_t q, uint32_t row,
+                                             int lane) {
+    uint32_t lo = q, hi = n;  // every position before lo holds row; hi is n or holds another
+    while (lo < hi) {
+        const uint32_t step = (hi - lo + 31) / 32;
+        const unsigned long long at = (unsigned long long)lo + (unsigned long long)step * lane;
+        const bool eq = at < hi && __ldg(srow + at) == row;
+        const uint32_t c = __popc(__ballot_sync(0xffffffffu, eq));
+        if (c == 0) return lo;
+        const unsigned long long nhi = (unsigned long long)lo + (unsigned long long)step * c;
+        lo += step * (c - 1) + 1;
+        if (nhi < hi) hi = (uint32_t)nhi;
     }
-    uint32_t block_total;
-    uint32_t run = block_exclusive_scan(cnt, block_total) + prefix;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k)
-        if (flags & (1u << k)) {
-            const uint32_t p = first + k;
-            seg_start[run] = p;
-            run_row[run] = srow[p];
-            run_p0[run] = spos[p];
-            ++run;
-        }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        cur->n_unique = prefix + block_total;
-        ds->last_unique = prefix + block_total;
-    }
+    return hi;
 }
 
-__global__ void k_dedup_out(const int64_t* __restrict__ keys, const uint32_t* __restrict__ spos,
-                            const uint32_t* __restrict__ seg_start, CallCounters* cur,
-                            int64_t* __restrict__ uniq, int32_t* __restrict__ counts, int64_t* num) {
+__global__ void __launch_bounds__(kThreads) k_dedup_out(const int64_t* __restrict__ keys,
+                                                        const uint32_t* __restrict__ srow,
+                                                        const uint32_t* __restrict__ spos, uint32_t n, uint32_t sent,
+                                                        const uint32_t* __restrict__ tile_sums,
+                                                        int64_t* __restrict__ uniq, int32_t* __restrict__ counts,
+                                                        int64_t* num, DevState* ds) {
     pdl_enter();
-    const uint32_t U = cur->n_unique, nv = cur->n_valid;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *num = (int64_t)U;
-    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < U; u += gridDim.x * blockDim.x) {
-        const uint32_t s = seg_start[u];
-        const uint32_t e = u + 1 < U ? seg_start[u + 1] : nv;
-        uniq[u] = keys[spos[s]];
-        counts[u] = (int32_t)(e - s);
+    __shared__ uint32_t at[kTile + 1];  // the tile's run heads, in order
+    const uint32_t tile0 = blockIdx.x * kTile, first = tile0 + threadIdx.x * kItems;
+    const uint32_t bits = head_bits(srow, first, n, sent);
+    const uint32_t prefix = tiles_before(tile_sums, blockIdx.x);
+    uint32_t heads;
+    uint32_t r = block_exclusive_scan((uint32_t)__popc(bits), heads);
+    for (uint32_t m = bits; m; m &= m - 1) at[r++] = first + (uint32_t)__ffs(m) - 1u;
+    __syncthreads();
+    if (heads && threadIdx.x < 32) {  // the last run may go on in later tiles
+        const uint32_t s = at[heads - 1], row = __ldg(srow + s);
+        const uint32_t e = end_from(srow, n, s + 1, row, (int)threadIdx.x);
+        if (threadIdx.x == 0) at[heads] = e;
     }
-    release_counters(cur, gridDim.x);  // the dedup's last kernel
+    __syncthreads();
+    for (uint32_t u = threadIdx.x; u < heads; u += kThreads) {
+        const uint32_t s = at[u];
+        // between two heads of a tile there is nothing but runs; lookups without a row sort last
+        uniq[prefix + u] = __ldg(keys + __ldg(spos + s));
+        counts[prefix + u] = (int32_t)(at[u + 1] - s);
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        *num = (int64_t)(prefix + heads);
+        ds->last_unique = prefix + heads;
+    }
 }
 
 inline unsigned tiles(int64_t n) { return (unsigned)((n + kTile - 1) / kTile); }
@@ -618,24 +642,14 @@ cudaError_t launch_sort_rows(mlkv_table* t, int64_t n, cudaStream_t st, const ui
     return cudaGetLastError();
 }
 
-cudaError_t launch_segments(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n,
-                            cudaStream_t st, CallCounters* cur, const SortTail& tail) {
+cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t* srow, const uint32_t* spos,
+                             int64_t n, int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
+                             const SortTail& tail) {
     const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);
     const unsigned nt = tiles(n);
-    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_reduce, nt, kThreads, 0, st, srow, (uint32_t)n, sent, t->s.tile_sums,
-                tail);
-    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_down, nt, kThreads, 0, st, srow, spos, (uint32_t)n, sent,
-                t->s.tile_sums, t->s.seg_start, t->s.run_row, t->s.run_p0, cur, t->dstate);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t* spos, int64_t n,
-                             int64_t* uniq, int32_t* counts, int64_t* num, cudaStream_t st,
-                             CallCounters* cur) {
-    int64_t g = (n + 255) / 256;
-    if (g > (int64_t)t->num_sms * 8) g = (int64_t)t->num_sms * 8;
-    if (g < 1) g = 1;
-    MLKV_LAUNCH(t, 0, k_dedup_out, (unsigned)g, 256, 0, st, keys, spos, t->s.seg_start, cur, uniq, counts, num);
+    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_seg_count, nt, kThreads, 0, st, srow, (uint32_t)n, sent, t->s.tile_sums, tail);
+    MLKV_LAUNCH(t, MLKV_K_SEGMENTS, k_dedup_out, nt, kThreads, 0, st, keys, srow, spos, (uint32_t)n, sent,
+                t->s.tile_sums, uniq, counts, num, t->dstate);
     return cudaGetLastError();
 }
 

@@ -278,7 +278,7 @@ bool capturing(cudaStream_t st) {
 // enqueued and a call's copy is zero when it starts even where the host no
 // longer knows which copy is next: a captured graph replays a fixed sequence
 // of calls, which may be odd in number, without passing through the host.
-// (find and export use no counters; every other call's last kernel releases
+// (find, export and dedup use no counters; every other call's last kernel releases
 // them.)
 //
 // Stale-synchronous mode (staleness_bound s >= 1, Gets and applies on two
@@ -591,14 +591,12 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.sort_counts[2], s.sort_counts_bytes},
         {(void**)&s.sort_offsets, 512 * sort_tiles * 4},
         {(void**)&s.sort_dtot, kSortMaxPasses * 512 * 4},
-        {(void**)&s.seg_start, (B + 1) * 4},  {(void**)&s.run_row, B * 4},
         {(void**)&s.long_runs, s.max_long * 16}, {(void**)&s.nodes, s.max_nodes * 16},
         {(void**)&s.items, s.max_items * 16}, {(void**)&s.node_cnt, s.node_cnt_bytes},
         {(void**)&s.short_runs, B * 16},
         {(void**)&s.single_runs, B * 8},
         {(void**)&s.small_runs, B * 16},
         {(void**)&s.small_p3, B * 4},
-        {(void**)&s.run_p0, B * 4},
         {(void**)&s.partial, s.max_items * 2 * t->geom.dpad * 4},
     };
     int64_t total = 0;
@@ -835,12 +833,12 @@ int mlkv_dedup(mlkv_table* t, const int64_t* d_keys, int64_t n, int64_t* d_uniqu
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = wait_lookahead(t, st))) return rc;
     CallScope cs = begin_call(t, st);
-    CK(t, launch_probe(t, d_keys, n, false, MemoUse::None, false, false, st, cs.cur, cs.nxt));
+    const FirstCounts fc = first_counts(t, n);  // the probe also counts the sort's first pass
+    CK(t, launch_probe(t, d_keys, n, false, MemoUse::None, false, false, st, cs.cur, cs.nxt, nullptr, &fc));
     const uint32_t *srow, *spos;
     SortTail tail;
-    CK(t, launch_sort_rows(t, n, st, &srow, &spos, false, tail));
-    CK(t, launch_segments(t, srow, spos, n, st, cs.cur, tail));
-    CK(t, launch_dedup_out(t, d_keys, spos, n, d_unique_keys, d_counts, d_num_unique, st, cs.cur));
+    CK(t, launch_sort_rows(t, n, st, &srow, &spos, true, tail));
+    CK(t, launch_dedup_out(t, d_keys, srow, spos, n, d_unique_keys, d_counts, d_num_unique, st, tail));
     return MLKV_OK;
 }
 
