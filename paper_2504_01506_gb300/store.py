@@ -29,7 +29,9 @@ class MLKVError(RuntimeError):
 
 
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    """The current torch stream's handle.  (Without building a Stream object: 0.2 us
+    instead of 2.1, of 13 for a Get of 416 lookups.)"""
+    return torch._C._cuda_getCurrentRawStream(device.index)
 
 
 class EmbeddingStore:
@@ -102,7 +104,8 @@ class EmbeddingStore:
         n = keys.numel()
         if out is None:
             out = torch.empty((n, self.dim), dtype=torch.float32, device=self.device)
-        out = self._check_out(out, n)
+        else:
+            out = self._check_out(out, n)
         self._check(self.lib.mlkv_get(self.h, keys.data_ptr(), n, out.data_ptr(), _stream(self.device)))
         return out
 
@@ -154,10 +157,12 @@ class EmbeddingStore:
         n = keys.numel()
         uniq = torch.empty(max(n, 1), dtype=torch.int64, device=self.device)
         counts = torch.empty(max(n, 1), dtype=torch.int32, device=self.device)
-        num = torch.zeros(1, dtype=torch.int64, device=self.device)
+        # the kernel writes the number straight to pinned host memory (one synchronisation, no copy)
+        num = torch.zeros(1, dtype=torch.int64, pin_memory=True)
         self._check(self.lib.mlkv_dedup(self.h, keys.data_ptr(), n, uniq.data_ptr(), counts.data_ptr(),
-                                        num.data_ptr(), _stream(self.device)))
-        u = int(num.item())
+                                        num.data_ptr() if n else None, _stream(self.device)))
+        torch.cuda.current_stream(self.device).synchronize()
+        u = int(num[0])
         return uniq[:u], counts[:u]
 
     # -- checkpoints (keys in row order, rows, state) -----------------------------
