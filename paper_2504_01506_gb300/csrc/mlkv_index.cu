@@ -293,14 +293,13 @@ constexpr int kMissThreads = 512;
 template <int V>
 __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows ra, MissArgs ma, uint32_t bar_extra,
                                                        int release, FirstCounts fc) {
-    // waits for the kernel before it, like every kernel; lets the next one
-    // launch only once the grid barriers are behind it (see grid_barrier)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (the next kernel's blocks are placed once every block of this grid has
+    // started, so they keep none of these from becoming resident)
+    pdl_enter();
     CallCounters* cur = ma.cur;
     const uint32_t m = min(cur->n_miss, ma.n);  // never more misses than lookups
     if (m == 0) {
         if (release) release_counters(cur, gridDim.x);
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         return;
     }
     // the first sort pass's count (an apply's) of a missed lookup's digit in its tile
@@ -323,7 +322,6 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
         return;
     }
     if (release) release_counters(cur, gridDim.x);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Put 1/2: the last occurrence of each key wins: aux = min over its
