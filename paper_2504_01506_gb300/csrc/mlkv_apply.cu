@@ -25,10 +25,10 @@
 //                 state, first gradient row and the run's other positions
 //                 loaded together, the rest summed in occurrence order, then
 //                 the Adagrad step.
-//  k_long         chunks of 64 lookups (16 in calls of fewer than 2^19 lookups,
-//                 but 64 there too for runs of more than 4,096) of a long run
-//                 (Zipf-hot keys reach 10^4-10^5 lookups): the chunk's sum,
-//                 compensated, to scratch as a (sum, compensation) pair.
+//  k_long         chunks of 64 lookups (16 in calls of fewer than 2^19 lookups)
+//                 of a long run (Zipf-hot keys reach 10^4-10^5 lookups): the
+//                 chunk's sum, compensated, to scratch as a (sum, compensation)
+//                 pair.
 //  k_combine      per long run: the chunk pairs added in a fixed order with
 //                 compensation, the sum rounded once, and the row updated.
 //  k_reduce       all of these in one launch, for small calls (whose run lists
@@ -593,10 +593,10 @@ __global__ void __launch_bounds__(256, MLKV_LONG_MIN_BLOCKS) k_long(RowArgs ra, 
 // scratch and the block that finishes the run's last node adds the nodes' pairs
 // up the same way (nodes counted by an atomic: no block waits for another).
 // Every run of at most kGroupChunks chunks takes one lane group.  (With one
-// block for all chunks of a run, 8 lane groups each added up to a hundred
-// chunks one after another: 100,003 lookups, Zipf(1.0), dim 50, took 119 us for
-// apply + export, 113 with nodes.)  kGroupChunks = 16: 4 and 32 cost the 1.7M-
-// and 200k-lookup steps 1-2 us.
+// block for all chunks of a run, 8 lane groups each added up to a hundred chunks
+// one after another: 100,003 lookups, Zipf(1.0), dim 50, took 119 us for apply +
+// export, 113 with nodes.)  kGroupChunks = 8: 4, 16 and 32 cost the 1.7M- and
+// 200k-lookup steps about 1 us.
 // 256 threads fit the slots that retiring blocks of the other reduce kernels
 // free, where a 1024-thread block waits for a whole SM to drain.
 constexpr int kCombineThreads = 256;

@@ -9,8 +9,10 @@ namespace mlkv {
 namespace {
 
 // Long runs are summed in chunks: of kChunkLarge lookups in calls of at least
-// MLKV_SMALL_BATCH lookups, of kChunkSmall in smaller ones (few long runs:
-// more chunks to sum in parallel).  Set at build time.
+// MLKV_SMALL_BATCH lookups, of kChunkSmall in smaller ones (few long runs: more
+// chunks to sum in parallel; also in the runs of thousands of lookups, whose
+// chunks the combine takes 256 a block: 64-lookup chunks there cost 100,003
+// lookups of dim 50 78 us instead of 74).  Set at build time.
 #ifndef MLKV_SMALL_BATCH
 #define MLKV_SMALL_BATCH (1u << 19)
 #endif
@@ -18,18 +20,8 @@ namespace {
 #define MLKV_CHUNK_SMALL 16
 #endif
 constexpr uint32_t kChunkLarge = 64, kChunkSmall = MLKV_CHUNK_SMALL, kSmallBatch = MLKV_SMALL_BATCH;
-// In a small call a run of more small chunks than this is cut into large ones:
-// up to here a block combines them in one node.  (At 64, a knowledge-graph step
-// of 200k lookups lost 7 us in k_long: its runs of some thousand lookups were
-// cut into too few chunks to fill the GPU.)
-constexpr uint32_t kFewChunks = 256;
-
-// Lookups per chunk of a long run of len lookups (`chunk`: the call's).
-__device__ __forceinline__ uint32_t run_chunk(uint32_t len, uint32_t chunk) {
-    return len > chunk * kFewChunks ? kChunkLarge : chunk;
-}
 #ifndef MLKV_GROUP_CHUNKS
-#define MLKV_GROUP_CHUNKS 16
+#define MLKV_GROUP_CHUNKS 8
 #endif
 #ifndef MLKV_NODE
 #define MLKV_NODE 256
@@ -107,8 +99,7 @@ __device__ __forceinline__ uint32_t warp_inclusive(uint32_t x, int lane) {
 __device__ __forceinline__ LongCounts long_counts(const uint32_t* qs, const uint32_t* qe, int nq, int lane,
                                                   uint32_t chunk, LongCounts& mine, LongCounts& excl) {
     const uint32_t len = lane < nq ? qe[lane] - qs[lane] : 0u;
-    const uint32_t c = run_chunk(len, chunk);
-    mine.items = (len + c - 1) / c;
+    mine.items = (len + chunk - 1) / chunk;
     mine.runs = lane < nq && mine.items <= kGroupChunks;
     mine.nodes = mine.items > kGroupChunks ? (mine.items + kNode - 1) / kNode : 0u;
     const LongCounts in = {warp_inclusive(mine.items, lane), warp_inclusive(mine.runs, lane),
@@ -126,7 +117,7 @@ __device__ __forceinline__ void write_long_runs(const RunArgs& a, const uint32_t
     long_counts(qs, qe, nq, lane, a.chunk, mine, excl);
     if (mine.runs) a.long_runs[base.runs + excl.runs] = make_uint4(base.items + excl.items, mine.items, qr[lane], 0u);
     for (int k = 0; k < nq; ++k) {
-        const uint32_t s = qs[k], e = qe[k], row = qr[k], chunk = run_chunk(e - s, a.chunk);
+        const uint32_t s = qs[k], e = qe[k], row = qr[k], chunk = a.chunk;
         const uint32_t m = __shfl_sync(0xffffffffu, mine.items, k);
         const uint32_t ib = base.items + __shfl_sync(0xffffffffu, excl.items, k);
         const uint32_t nodes = __shfl_sync(0xffffffffu, mine.nodes, k);
