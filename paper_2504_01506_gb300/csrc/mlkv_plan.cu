@@ -48,7 +48,8 @@ struct __align__(16) PlanShared {
     uint32_t gbase[kPlanRadix];                 // sorted position of the block's first element of each digit
     uint32_t bits[kPlanThreads * kPlanItems / 32];  // a bit per sorted element: another row than its left neighbour's
     uint32_t words[kPlanItems];             // a bit per word of `bits`: not zero
-    uint32_t first;                         // sorted position of the first set bit, or NONE
+    uint32_t firsts[kPlanCluster];          // sorted position of every block's first set bit, or NONE
+    uint32_t halo[kSmallRun];               // the next block's first sorted positions' lookups
     uint32_t nlong;
     uint32_t cnt[3], base[3];               // runs of one, of 2 .. kSmallRun, of more lookups: count, list entry
     uint32_t warp_sums[kPlanWarps];
@@ -294,9 +295,16 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan(IndexArgs ia, IndexRow
                 f = tile0 + (uint32_t)(k * 32 + l) * 32u + (uint32_t)__ffs(__shfl_sync(0xffffffffu, b, l)) - 1u;
             }
         }
-        if (lane == 0) sh.first = f;
+        // ... which the other blocks are told (a run may end in a later block)
+        if ((uint32_t)lane < nblocks) {
+            uint32_t* to = nblocks > 1 ? cluster.map_shared_rank(sh.firsts, lane) : sh.firsts;
+            to[me] = f;
+        }
     }
-    meet();
+    // the next block's first positions, for a run of 2 .. kSmallRun that goes on there
+    if (me + 1 < nblocks && threadIdx.x >= 32 && threadIdx.x < 32 + kSmallRun)
+        sh.halo[threadIdx.x - 32] = cluster.map_shared_rank(skv, me + 1)[threadIdx.x - 32].y;
+    meet();  // the last: nothing of another block is read after it
     // the end of a run that starts at element e: the next set bit, here or in a later block
     auto run_end = [&](uint32_t e) {
         uint32_t wd = e >> 5;
@@ -312,8 +320,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan(IndexArgs ia, IndexRow
             }
         }
         for (uint32_t c = me + 1; c < nblocks; ++c) {
-            const uint32_t f = *cluster.map_shared_rank(&sh.first, c);
-            if (f != NONE) return f;
+            if (sh.firsts[c] != NONE) return sh.firsts[c];
         }
         return n;
     };
@@ -387,9 +394,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan(IndexArgs ia, IndexRow
         } else if (len[r] <= kSmallRun) {
             auto pos = [&](uint32_t k) -> uint32_t {
                 if (k >= len[r]) return NONE;
-                const uint32_t x = g + k;
-                return (x >> kTileShift) == me ? skv[x & (T - 1)].y
-                                               : cluster.map_shared_rank(skv, x >> kTileShift)[x & (T - 1)].y;
+                return e + k < T ? skv[e + k].y : sh.halo[e + k - T];
             };
             const uint32_t i = sh.base[1] + place[r];
             a.smalls[i] = make_uint4(key[r], val[r], pos(1), pos(2));
@@ -398,7 +403,6 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan(IndexArgs ia, IndexRow
             a.runs[sh.base[2] + place[r]] = make_uint4(g, g + len[r], key[r], val[r]);
         }
     }
-    meet();  // no block leaves while another reads its shared memory
 }
 
 template <int V, int ITEMS>
