@@ -556,7 +556,7 @@ cudaError_t launch_dedup_out(mlkv_table* t, const int64_t* keys, const uint32_t*
 #define MLKV_PLAN_MAX (1 << 15)
 #endif
 constexpr uint32_t kPlanMax = MLKV_PLAN_MAX;
-int plan_prepare();  // the largest cluster the plan kernels can run as on the current device (0: none)
+int plan_prepare(int device);  // the largest cluster the plan kernels can run as on the current device (0: none)
 bool plan_fits(const mlkv_table* t, int64_t n);
 // Probe (insert: absent keys get rows; rows: they are in row_of_pos already),
 // sort and run lists of an apply of n lookups (plan_fits); spos: the sorted

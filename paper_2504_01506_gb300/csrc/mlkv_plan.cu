@@ -23,6 +23,9 @@
 // dim 512: 156 -> 161), so kPlanMax = 32,768.
 #include <cooperative_groups.h>
 
+#include <mutex>
+#include <unordered_map>
+
 #include "mlkv_probe.cuh"
 #include "mlkv_runs.cuh"
 
@@ -461,13 +464,19 @@ bool prepare_items(int& largest) {
 
 }  // namespace
 
-int plan_prepare() {
+// A device's answer is kept: the attributes and occupancy queries take 0.1 ms.
+int plan_prepare(int device) {
+    static std::mutex mu;
+    static std::unordered_map<int, int> known;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(device);
+    if (it != known.end()) return it->second;
     int largest = kPlanCluster;
     if (!prepare_items<1>(largest) || !prepare_items<kPlanItems>(largest)) {
         cudaGetLastError();
-        return 0;
+        largest = 0;
     }
-    return largest;
+    return known[device] = largest;
 }
 
 bool plan_fits(const mlkv_table* t, int64_t n) {

@@ -495,7 +495,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         return fail(MLKV_ERR_CUDA);
     if (!make_geom(c.dim, c.dim % 4 == 0 ? 4 : 1, t->geom)) return fail(MLKV_ERR_INVALID);
 
-    t->plan_cluster = plan_prepare();
+    t->plan_cluster = plan_prepare(t->device);
     const int64_t stride = t->geom.stride;
     t->tiered = c.hbm_cache_rows > 0;
     if (!t->tiered) {
