@@ -298,10 +298,7 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
     pdl_enter();
     CallCounters* cur = ma.cur;
     const uint32_t m = min(cur->n_miss, ma.n);  // never more misses than lookups
-    if (m == 0) {
-        if (release) release_counters(cur, gridDim.x);
-        return;
-    }
+    if (m == 0) return;  // the call has touched no counter
     // the first sort pass's count (an apply's) of a missed lookup's digit in its tile
     auto count = [&](uint32_t p, uint32_t r) {
         if (!fc.counts) return;
