@@ -88,8 +88,8 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
 // The fused Get: each warp probes `lpw` consecutive lookups (one per lane), then
 // its lane groups gather their rows with vector loads, streaming the output.
 // Lookups of new keys are left to the miss path.  A row wider than 32 vectors
-// (SEG) is copied two vectors a lane at a time, whatever its dim: with all of
-// them in flight (4 a lane at dim 512) the kernel spilled at the 32 registers
+// is copied 2 or 4 vectors a lane at a time (row_vectors), whatever its dim: with
+// all of them in flight (4 a lane at dim 512) the kernel spilled at the 32 registers
 // that let 64 warps reside on an SM (65,536 lookups of dim 512: 49 us, 39 so;
 // 48 warps of 40 registers for these rows: 64 spill again and cost 524k rows of
 // 1 KiB 5 us).
@@ -102,9 +102,19 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
 #define MLKV_GET_SEG_MIN_BLOCKS 6
 #endif
 
-// The rows of one warp's lookups base .. base + lpw - 1, UNR rows of a lane group
-// in flight (a row of one segment); true where this lane's key is new.
-template <int V, bool SEG, bool INSERT, int UNR>
+// Vectors of a row that a lane copies at a time: 1 where a row has at most 32
+// vectors, 2 up to 64 (and, again and again, for wider rows of 16-byte
+// vectors), else 4.
+template <int V>
+constexpr int kMostVectors = V == 4 ? 2 : 4;
+template <int V>
+int row_vectors(const RowGeom& g) {
+    return g.NV <= 32 ? 1 : g.NV <= 64 ? 2 : kMostVectors<V>;
+}
+
+// The rows of one warp's lookups base .. base + lpw - 1, KV vectors a lane of UNR
+// rows of a lane group in flight; true where this lane's key is new.
+template <int V, int KV, bool WIDE, bool INSERT, int UNR>
 __device__ __forceinline__ bool get_rows(const IndexArgs& ia, const IndexRows& ra, const int64_t* __restrict__ keys,
                                          uint32_t n, float* __restrict__ out, uint32_t* miss_pos,
                                          uint32_t* miss_slot, CallCounters* cur, const Memo& memo, uint32_t base,
@@ -124,47 +134,38 @@ __device__ __forceinline__ bool get_rows(const IndexArgs& ia, const IndexRows& r
         memo.key[p] = key;
         memo.row[p] = row;
     }
-    if (SEG) {
-        for (int q = 0; q < lpw; ++q) {
-            const uint32_t r = __shfl_sync(0xffffffffu, row, q);
-            if (r == ROW_PENDING) continue;
-            const VT* src = reinterpret_cast<const VT*>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride);
-            VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q) * ra.d);
-            for (int j0 = 0; j0 < ra.NV; j0 += 64) {  // uniform
-                const int j = j0 + lane, k = j + 32;
-                VT v0, v1;
-                if (j < ra.NV) v0 = __ldg(src + j);
-                if (k < ra.NV) v1 = __ldg(src + k);
-                if (j < ra.NV) __stcs(dst + j, r == ROW_ABSENT ? Vec<V>::nan() : v0);
-                if (k < ra.NV) __stcs(dst + k, r == ROW_ABSENT ? Vec<V>::nan() : v1);
-            }
-        }
-        return fresh;
-    }
     const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
     for (int q0 = 0; q0 < lpw; q0 += R * UNR) {
-        VT v[UNR];
-        uint32_t rr[UNR];
+        // more vectors than KV a lane: in rounds (uniform; one, but for the widest rows)
+        for (int j0 = glane; WIDE ? j0 - glane < ra.NV : j0 == glane; j0 += G * KV) {
+            VT v[UNR][KV];
+            uint32_t rr[UNR];
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int q = q0 + u * R + gid;
-            const uint32_t r = __shfl_sync(0xffffffffu, row, q & 31);
-            rr[u] = UNR == 1 || q < lpw ? r : ROW_PENDING;
-            if (rr[u] < ROW_ABSENT && glane < ra.NV)
-                v[u] = __ldg(reinterpret_cast<const VT*>(ra.slots + (size_t)rr[u] * ra.stride) + glane);
-        }
+            for (int u = 0; u < UNR; ++u) {
+                const int q = q0 + u * R + gid;
+                const uint32_t r = __shfl_sync(0xffffffffu, row, q & 31);
+                rr[u] = UNR == 1 || q < lpw ? r : ROW_PENDING;
+                const VT* src = reinterpret_cast<const VT*>(ra.slots + (size_t)rr[u] * ra.stride) + j0;
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            if (rr[u] == ROW_PENDING) continue;
-            VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q0 + u * R + gid) * ra.d);
-            if (glane < ra.NV) __stcs(dst + glane, rr[u] == ROW_ABSENT ? Vec<V>::nan() : v[u]);
+                for (int k = 0; k < KV; ++k)
+                    if (rr[u] < ROW_ABSENT && j0 + G * k < ra.NV) v[u][k] = __ldg(src + G * k);
+            }
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                if (rr[u] == ROW_PENDING) continue;
+                VT* dst = reinterpret_cast<VT*>(out + (size_t)(base + q0 + u * R + gid) * ra.d) + j0;
+#pragma unroll
+                for (int k = 0; k < KV; ++k)
+                    if (j0 + G * k < ra.NV) __stcs(dst + G * k, rr[u] == ROW_ABSENT ? Vec<V>::nan() : v[u][k]);
+            }
+            if (!WIDE) break;
         }
     }
     return fresh;
 }
 
-template <int V, bool SEG, bool INSERT>
-__global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, IndexRows ra,
+template <int V, int KV, bool WIDE, bool INSERT>
+__global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_MIN_BLOCKS) k_get(IndexArgs ia, IndexRows ra,
                                              const int64_t* __restrict__ keys, uint32_t n,
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
@@ -173,12 +174,12 @@ __global__ void __launch_bounds__(256, SEG ? MLKV_GET_SEG_MIN_BLOCKS : MLKV_GET_
     zero_counters(nxt);
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     if (base >= n) return;  // warp-uniform
-    get_rows<V, SEG, INSERT, 1>(ia, ra, keys, n, out, miss_pos, miss_slot, cur, memo, base, lpw);
+    get_rows<V, KV, WIDE, INSERT, 1>(ia, ra, keys, n, out, miss_pos, miss_slot, cur, memo, base, lpw);
 }
 
 // The Get and its miss path in one launch (see finish_get): a warp per lpw
 // lookups, in a grid that can wait for itself.
-template <int V, bool SEG>
+template <int V, int KV, bool WIDE>
 __global__ void __launch_bounds__(256) k_get_small(IndexArgs ia, IndexRows ra, MissArgs ma, CallCounters* nxt,
                                                    Memo memo, int lpw) {
     pdl_enter();
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(256) k_get_small(IndexArgs ia, IndexRows ra, M
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     bool fresh = false;
     if (base < ma.n)
-        fresh = get_rows<V, SEG, true, 4>(ia, ra, ma.keys, ma.n, ma.out, const_cast<uint32_t*>(ma.miss_pos),
+        fresh = get_rows<V, KV, WIDE, true, 4 / KV>(ia, ra, ma.keys, ma.n, ma.out, const_cast<uint32_t*>(ma.miss_pos),
                                        const_cast<uint32_t*>(ma.miss_slot), ma.cur, memo, base, lpw);
     finish_get<V, 256>(ia, ra, ma, fresh);
 }
@@ -200,15 +201,16 @@ __global__ void __launch_bounds__(256) k_get_small(IndexArgs ia, IndexRows ra, M
 // the output rows are contiguous.  The store runs on while the warp probes its
 // next lookups; the stage is reused once the store has read it.  Rows of new
 // keys are left to the miss path, which writes their output rows after this
-// kernel.  Measured against k_get: faster where a call is too small to fill
-// the GPU with k_get's warps (latency-bound: 200k lookups, 45 -> 37 us),
-// slower on millions of lookups (194 -> 205 us), where k_get's 64 warps a SM
-// beat the few warps the stages leave room for.
+// kernel.  Measured against k_get (Gets of dim 128, 8M rows): faster where a
+// call is too small to fill the GPU with k_get's warps (20,000 lookups 10.3 us
+// against 12.5, 60,000 15.4 against 16.7, 100,000 22.0 against 24.1), slower
+// above (140,000 28.2 against 27.3, 500,000 88 against 80), where k_get's 64
+// warps a SM beat the few warps the stages leave room for.
 #ifndef MLKV_GET_BULK
 #define MLKV_GET_BULK 1
 #endif
 #ifndef MLKV_GET_BULK_MAX_BATCH
-#define MLKV_GET_BULK_MAX_BATCH (1u << 19)
+#define MLKV_GET_BULK_MAX_BATCH (1u << 17)
 #endif
 constexpr uint32_t kBulkMaxBatch = MLKV_GET_BULK_MAX_BATCH;
 constexpr int kBulkThreads = 128;  // 4 warps
@@ -358,14 +360,12 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
 
 // Put 2/2: the winning occurrence writes the row and puts aux back to idle.  A
 // warp finds the winners among its lpw lookups, one per lane (row and slot, then
-// the slot's mark), and its lane groups copy their rows, kPutRows vectors a lane
+// the slot's mark), and its lane groups copy their rows, KV * ROWS vectors a lane
 // in flight.  (With a lane group walking its lookups one by one, each copy
 // waited for its own mark: 75 us for 524k Puts of 1 KiB, Zipf(0.99); 70 so, 88
 // with 2 vectors in flight.)
-#ifndef MLKV_PUT_ROWS
-#define MLKV_PUT_ROWS 4
-#endif
-template <int V>
+// KV vectors a lane (row_vectors) of ROWS rows are in flight.
+template <int V, int KV, int ROWS>
 __global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
                                                      const uint32_t* __restrict__ row_of_pos,
                                                      const uint32_t* __restrict__ slot_of_pos,
@@ -373,7 +373,6 @@ __global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, I
                                                      const float* __restrict__ state, uint32_t n, int lpw) {
     pdl_enter();
     using VT = typename Vec<V>::T;
-    constexpr int kPutRows = MLKV_PUT_ROWS;
     __shared__ uint2 wins[8][32];  // (row, lookup) of the warp's winners
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int G = ra.G, R = 32 / G, glane = lane & (G - 1), gid = lane / G;
@@ -391,27 +390,28 @@ __global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, I
     const unsigned m = __ballot_sync(0xffffffffu, win);
     if (win) wins[wib][__popc(m & lanemask_lt())] = make_uint2(r, p);
     __syncwarp();
-    // vectors of the winners' rows, G at a time: segment x of the list
-    const int nseg = (ra.NV + G - 1) / G, items = __popc(m) * nseg;
+    const int nwin = __popc(m);
     auto copy = [&](const float* __restrict__ src, int off) {
-        for (int x0 = 0; x0 < items; x0 += R * kPutRows) {  // uniform
-            VT v[kPutRows];
-            VT* to[kPutRows];
+        for (int w0 = 0; w0 < nwin; w0 += R * ROWS)  // uniform
+            for (int j0 = glane; j0 - glane < ra.NV; j0 += G * KV) {
+                VT v[ROWS][KV];
+                VT* to[ROWS];
 #pragma unroll
-            for (int i = 0; i < kPutRows; ++i) {
-                const int x = x0 + i * R + gid;
-                const int w = nseg == 1 ? x : x / nseg, j = glane + (x - w * nseg) * G;
-                to[i] = nullptr;
-                if (x < items && j < ra.NV) {
-                    const uint2 rp = wins[wib][w];
-                    v[i] = __ldcs(reinterpret_cast<const VT*>(src + (size_t)rp.y * ra.d) + j);
-                    to[i] = reinterpret_cast<VT*>(ra.slots + (size_t)rp.x * ra.stride + off) + j;
+                for (int i = 0; i < ROWS; ++i) {
+                    const int x = w0 + i * R + gid;
+                    const uint2 rp = wins[wib][x < nwin ? x : 0];
+                    const VT* from = reinterpret_cast<const VT*>(src + (size_t)rp.y * ra.d) + j0;
+                    to[i] = x < nwin ? reinterpret_cast<VT*>(ra.slots + (size_t)rp.x * ra.stride + off) + j0 : nullptr;
+#pragma unroll
+                    for (int k = 0; k < KV; ++k)
+                        if (x < nwin && j0 + G * k < ra.NV) v[i][k] = __ldcs(from + G * k);
                 }
-            }
 #pragma unroll
-            for (int i = 0; i < kPutRows; ++i)
-                if (to[i]) *to[i] = v[i];
-        }
+                for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+                    for (int k = 0; k < KV; ++k)
+                        if (to[i] && j0 + G * k < ra.NV) to[i][G * k] = v[i][k];
+            }
     };
     copy(vals, 0);
     if (state) copy(state, ra.dpad);  // import: the state too
@@ -438,7 +438,7 @@ struct ExportTier {
     const float* host;
 };
 
-template <int V>
+template <int V, int KV>
 __global__ void __launch_bounds__(256) k_export(IndexArgs ia, IndexRows ra,
                                                 const int64_t* __restrict__ keys, uint32_t n,
                                                 float* __restrict__ rows_out,
@@ -468,13 +468,24 @@ __global__ void __launch_bounds__(256) k_export(IndexArgs ia, IndexRows ra,
         }
         const VT* ws = reinterpret_cast<const VT*>(src);
         const VT* gs = reinterpret_cast<const VT*>(src + ra.dpad);
-        for (int j = glane; j < ra.NV; j += G) {  // row and state in flight together
-            VT w, g;
-            if (rows_out) w = __ldg(ws + j);
-            if (state_out) g = __ldg(gs + j);
-            const size_t o = (size_t)(base + q) * ra.d;
-            if (rows_out) __stcs(reinterpret_cast<VT*>(rows_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : w);
-            if (state_out) __stcs(reinterpret_cast<VT*>(state_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : g);
+        constexpr int kVecs = KV;  // of the row and of the state, in flight together a lane
+        const size_t o = (size_t)(base + q) * ra.d;
+        for (int j0 = glane; j0 < ra.NV; j0 += G * kVecs) {
+            VT w[kVecs], g[kVecs];
+#pragma unroll
+            for (int k = 0; k < kVecs; ++k) {
+                const int j = j0 + G * k;
+                if (j < ra.NV && rows_out) w[k] = __ldg(ws + j);
+                if (j < ra.NV && state_out) g[k] = __ldg(gs + j);
+            }
+#pragma unroll
+            for (int k = 0; k < kVecs; ++k) {
+                const int j = j0 + G * k;
+                if (j >= ra.NV) continue;
+                if (rows_out) __stcs(reinterpret_cast<VT*>(rows_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : w[k]);
+                if (state_out)
+                    __stcs(reinterpret_cast<VT*>(state_out + o) + j, r == ROW_ABSENT ? Vec<V>::nan() : g[k]);
+            }
         }
     }
 }
@@ -529,11 +540,17 @@ struct GetRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* out,
                            cudaStream_t st, CallCounters* cur, CallCounters* nxt) {
         const uint32_t rowbytes = (uint32_t)t->geom.d * 4;
-        const bool seg = t->geom.NV > t->geom.G, ins = t->cfg.insert_on_miss != 0;
+        const int kv = row_vectors<V>(t->geom);
+        constexpr int M = kMostVectors<V>;
+        const bool wide = t->geom.NV > 32 * kv;
+        const bool ins = t->cfg.insert_on_miss != 0;
         if (small_get(t, n)) {
             const int lpw = small_get_lpw(t, n);
             const MissArgs ma = miss_args(t, keys, n, MissMode::Get, nullptr, out, cur);
-            const auto kernel = seg ? k_get_small<V, true> : k_get_small<V, false>;
+            const auto kernel = kv == 1   ? k_get_small<V, 1, false>
+                                : wide    ? k_get_small<V, M, true>
+                                : kv == 2 ? k_get_small<V, 2, false>
+                                          : k_get_small<V, M, false>;
             MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t), row_args(t), ma,
                         nxt, Memo{t->s.memo_key, t->s.memo_row}, lpw);
             return cudaGetLastError();
@@ -551,8 +568,10 @@ struct GetRun {
             return cudaGetLastError();
         }
         const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
-        const auto kernel = seg ? (ins ? k_get<V, true, true> : k_get<V, true, false>)
-                                : (ins ? k_get<V, false, true> : k_get<V, false, false>);
+        const auto kernel = kv == 1   ? (ins ? k_get<V, 1, false, true> : k_get<V, 1, false, false>)
+                            : wide    ? (ins ? k_get<V, M, true, true> : k_get<V, M, true, false>)
+                            : kv == 2 ? (ins ? k_get<V, 2, false, true> : k_get<V, 2, false, false>)
+                                      : (ins ? k_get<V, M, false, true> : k_get<V, M, false, false>);
         MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t), row_args(t), keys,
                     (uint32_t)n, out, t->s.miss_pos, t->s.miss_slot, cur, nxt, Memo{t->s.memo_key, t->s.memo_row},
                     lpw);
@@ -579,8 +598,10 @@ struct PutRun {
     static cudaError_t run(mlkv_table* t, const float* vals, const float* state, int64_t n, cudaStream_t st) {
         MLKV_LAUNCH(t, 0, k_put_mark, capped_grid(t, n, 256, kMarkPerSm), 256, 0, st, t->index, t->s.row_of_pos,
                     t->s.slot_of_pos, (uint32_t)n);
-        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
-        MLKV_LAUNCH(t, MLKV_K_PUT_SCATTER, (k_put_scatter<V>), grid_for(n, 8 * lpw), 256, 0, st, t->index, row_args(t),
+        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G), kv = row_vectors<V>(t->geom);
+        const auto kernel = kv == 1 ? k_put_scatter<V, 1, 4> : kv == 2 ? k_put_scatter<V, 2, 2>
+                                                                       : k_put_scatter<V, kMostVectors<V>, 2>;
+        MLKV_LAUNCH(t, MLKV_K_PUT_SCATTER, kernel, grid_for(n, 8 * lpw), 256, 0, st, t->index, row_args(t),
                     t->s.row_of_pos, t->s.slot_of_pos, vals, state, (uint32_t)n, lpw);
         return cudaGetLastError();
     }
@@ -606,7 +627,9 @@ struct ExportRun {
         ExportTier et{nullptr, nullptr, nullptr};
         if (t->tiered) et = ExportTier{t->tier.row_loc, t->tier.cache, t->tier.host_dev};
         const int lpw = lookups_per_warp(t, n, 32 / t->geom.G);
-        MLKV_LAUNCH(t, 0, (k_export<V>), grid_for(n, 8 * lpw), 256, 0, st, index_args(t),
+        const int kv = row_vectors<V>(t->geom);
+        const auto kernel = kv == 1 ? k_export<V, 1> : kv == 2 ? k_export<V, 2> : k_export<V, kMostVectors<V>>;
+        MLKV_LAUNCH(t, 0, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t),
                     row_args(t), keys, (uint32_t)n, rows, state, nxt, et, lpw);
         return cudaGetLastError();
     }

@@ -581,19 +581,23 @@ cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* sp
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
                                 cudaStream_t st, CallCounters* cur);
 
-// Lookups per warp of the kernels that copy a warp's rows one after another: 32,
-// or as few as fill the GPU (kWarpsWanted warps per SM) in a small call, at
-// least `least` (the rows a warp copies at a time).  With 32 always, an export
-// of 100,003 rows of dim 50 ran on 20 warps per SM: 52 us, 20 with 8 lookups
-// (and 8-byte vectors); wanting 16 warps costs it 4 us, and a Get of 65,536
-// rows of dim 512 14.
+// Lookups per warp of the kernels that copy a warp's rows one after another: 16
+// of dims above 64 and 32 of narrower ones, or as few as fill the GPU
+// (kWarpsWanted warps per SM) in a small call, at least `least` (the rows a warp
+// copies at a time).  Shorter warps leave the probes of some to hide behind the
+// copies of others to the end.  Apply + Get of 1.7M rows of dim 128: 554 us with
+// 32, 546 with 16, 548 with 8; a batch with two Gets and a Put of 524k rows of
+// 1 KiB: 372, 351, 355; a Get of 700,000 rows of dim 67: 91 with 32, 89 with 16;
+// 2.1M rows of dim 64: 597 with 32, 600 with 16.  An export of 100,003 rows of
+// dim 50 took 52 us with 32 (20 warps per SM) and 4-byte vectors, 20 with 8.
+// kWarpsWanted = 128: 64 costs the 200k-lookup step 2.5 us, 256 3.
 #ifndef MLKV_WARPS_WANTED
-#define MLKV_WARPS_WANTED 64
+#define MLKV_WARPS_WANTED 128
 #endif
 constexpr int kWarpsWanted = MLKV_WARPS_WANTED;
 inline int lookups_per_warp(const mlkv_table* t, int64_t n, int least) {
-    int lpw = 32;
-    while (lpw > least && lpw > 1 && n < (int64_t)lpw * t->num_sms * kWarpsWanted) lpw /= 2;
+    int lpw = t->geom.d > 64 ? 16 : 32;
+    while (lpw > least && n < (int64_t)lpw * t->num_sms * kWarpsWanted) lpw /= 2;
     return lpw;
 }
 
