@@ -539,6 +539,7 @@ cudaError_t launch_export(mlkv_table* t, const int64_t* keys, int64_t n, float* 
                           float* state, cudaStream_t st, CallCounters* nxt);
 
 // mlkv_sort.cu
+cudaError_t sort_prepare();  // the scatter kernels' shared memory, on the current device
 // The first pass's counts for the probe to make (t->sort_bits rows, n lookups).
 FirstCounts first_counts(mlkv_table* t, int64_t n);
 // first_counted: the first pass's counts were made by the apply's probe and

@@ -496,6 +496,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
     if (!make_geom(c.dim, c.dim % 4 == 0 ? 4 : 1, t->geom)) return fail(MLKV_ERR_INVALID);
 
     t->plan_cluster = plan_prepare(t->device);
+    if (sort_prepare() != cudaSuccess) return fail(MLKV_ERR_CUDA);
     const int64_t stride = t->geom.stride;
     t->tiered = c.hbm_cache_rows > 0;
     if (!t->tiered) {
