@@ -284,6 +284,19 @@ __global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k
     const uint32_t* __restrict__ vin = s.vin;
     const uint32_t n = s.n, sent = s.sent, ntiles = s.ntiles;
     const int shift = s.shift, radix = s.radix, first = s.first, nshift = s.nshift;
+    const uint32_t tile0 = blockIdx.x * TILE;
+    const uint32_t base = tile0 + (threadIdx.x >> 5) * (kSItems * 32);
+    uint32_t key[kSItems], val[kSItems];
+    // all loads together; with SELF (and its registers) beside the zeroing too
+    auto load = [&]() {
+#pragma unroll
+        for (int r = 0; r < kSItems; ++r) {
+            const uint32_t i = base + r * 32 + (threadIdx.x & 31);
+            key[r] = i < n ? sort_key(kin[i], sent, first) : 0u;
+            val[r] = i < n ? (first ? i : vin[i]) : 0u;
+        }
+    };
+    if (SELF) load();
     if (s.zcounts) {
         // this tile's share of the counts of the pass before
         const uint32_t words = SELF ? radix / 2 : radix;
@@ -320,18 +333,10 @@ __global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k
         ntot[d] = 0u;
     }
     __syncthreads();
-    const uint32_t tile0 = blockIdx.x * TILE;
-    const uint32_t base = tile0 + w * (kSItems * 32);
     const int digit_bits = __ffs(radix) - 1;
     const uint32_t lt = lanemask_lt();
-    uint32_t key[kSItems], val[kSItems], rnk[kSItems];
-    // all loads first, so they are in flight together
-#pragma unroll
-    for (int r = 0; r < kSItems; ++r) {
-        const uint32_t i = base + r * 32 + lane;
-        key[r] = i < n ? sort_key(kin[i], sent, first) : 0u;
-        val[r] = i < n ? (first ? i : vin[i]) : 0u;
-    }
+    uint32_t rnk[kSItems];
+    if (!SELF) load();
     if (SELF) {  // beside them, the counts of the tiles before: a group of radix / 2 threads per row
         const uint32_t words = radix / 2, groups = THREADS / words;
         const uint32_t grp = threadIdx.x / words, x = threadIdx.x & (words - 1);
