@@ -15,7 +15,7 @@
 //                 MLKV_SEQ_SEGMENT_MAX lookups go to three lists (one atomic
 //                 per block and list; any order: every run is summed on its
 //                 own), longer ones are measured (a warp-wide search for their
-//                 end) and listed for k_long_*.
+//                 end) and listed for k_long.
 //  k_single       runs of one lookup: row, state and the gradient row loaded
 //                 together, then the Adagrad step.
 //  k_small        runs of 2 .. kSmallRun lookups, whose positions k_heads wrote

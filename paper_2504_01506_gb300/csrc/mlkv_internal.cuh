@@ -459,10 +459,10 @@ struct Memo {
 };
 enum class MemoUse { None, Read, Save };
 
-// The first sort pass's digit counts, made by the gradient apply: its probe
-// writes every tile's column of counts[digit][tile] for the lookups whose row
-// it found (and adds them to the pass's totals dtot); the miss kernel adds the
-// lookups it gave rows.  The sort's first pass then needs no histogram kernel.
+// The first sort pass's digit counts, made by a gradient apply's or a dedup's
+// probe: it writes every tile's counts (laid out as add_count has it) of the
+// lookups whose row it found, and adds them to the pass's totals dtot; the miss
+// kernel adds the lookups it gave rows.  The sort's first pass then needs no histogram kernel.
 struct FirstCounts {
     uint32_t* counts;
     uint32_t* dtot;
@@ -525,7 +525,7 @@ cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out
                        CallCounters* cur, CallCounters* nxt);
 // release: the miss kernel is the last of the call to read its counters, and
 // zeroes them when done (release_counters).  fc: the first sort pass's counts
-// the apply's probe made, to which the lookups given rows here are added.
+// the probe made, to which the lookups given rows here are added.
 cudaError_t launch_resolve_misses(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode,
                                   float* out, cudaStream_t st, CallCounters* cur, bool release,
                                   const FirstCounts* fc = nullptr);
@@ -542,7 +542,7 @@ cudaError_t launch_export(mlkv_table* t, const int64_t* keys, int64_t n, float* 
 cudaError_t sort_prepare();  // the scatter kernels' shared memory, on the current device
 // The first pass's counts for the probe to make (t->sort_bits rows, n lookups).
 FirstCounts first_counts(mlkv_table* t, int64_t n);
-// first_counted: the first pass's counts were made by the apply's probe and
+// first_counted: the first pass's counts were made by the probe and the
 // miss kernel (FirstCounts).
 // tail: for the kernel launched next, which zeroes it.
 cudaError_t launch_sort_rows(mlkv_table* t, int64_t n, cudaStream_t st, const uint32_t** srow,
