@@ -20,9 +20,9 @@
 // kernel between two passes.  (Apply + Get of 200k lookups of dim 100: 153 ->
 // 140 us; apply + export of 100,003 of dim 50: 88.7 -> 78.  At 2^19 lookups the
 // blocks read 33 MB of counts a pass, as long as the offsets kernel takes.)  The
-// counts of the first pass are made by a histogram
-// kernel, or in a gradient apply by the probe and the miss kernel
-// (FirstCounts); those of every later pass by the scatter before it, which
+// counts of the first pass are made by the probe and the miss kernel
+// (FirstCounts), or by a histogram kernel where the rows come from elsewhere (a
+// tiered apply); those of every later pass by the scatter before it, which
 // knows the tile each element lands in and adds the element's next digit to
 // that tile's count (one add per run of equal targets in a warp), so no pass
 // after the first reads its input twice.  No block waits on another, so a pass
@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(kOThreads) k_sort_offsets(const uint32_t* __re
 // An element of digit d goes to offsets[tile][d] plus its rank among the
 // tile's elements of digit d.  With nshift >= 0 the element's digit of the
 // next pass (bits nshift ..) is added to the count of the tile of the next
-// pass that holds its output position, ncounts[digit][dst / TILE] (zero on
-// entry), and to the next pass's digit totals ndtot.  The counts and totals of
+// pass that holds its output position (dst / TILE; ncounts, laid out as
+// add_count has it, zero on entry), and to the next pass's digit totals ndtot.  The counts and totals of
 // the pass before (zcounts, zdtot) are zeroed here: every block of this pass
 // reads its own pass's, so the next kernel zeroes those.
 // With SELF the block adds up offsets from `counts` (packed) itself.
