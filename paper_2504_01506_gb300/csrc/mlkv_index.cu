@@ -546,13 +546,15 @@ struct GetRun {
         const bool ins = t->cfg.insert_on_miss != 0;
         if (small_get(t, n)) {
             const int lpw = small_get_lpw(t, n);
+            const unsigned grid = grid_for(n, 8 * lpw);
+            if (!miss_grid_fits(t, grid)) return cudaErrorInvalidConfiguration;
             const MissArgs ma = miss_args(t, keys, n, MissMode::Get, nullptr, out, cur);
             const auto kernel = kv == 1   ? k_get_small<V, 1, false>
                                 : wide    ? k_get_small<V, M, true>
                                 : kv == 2 ? k_get_small<V, 2, false>
                                           : k_get_small<V, M, false>;
-            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid_for(n, 8 * lpw), 256, 0, st, index_args(t), row_args(t), ma,
-                        nxt, Memo{t->s.memo_key, t->s.memo_row}, lpw);
+            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid, 256, 0, st, index_args(t), row_args(t), ma, nxt,
+                        Memo{t->s.memo_key, t->s.memo_row}, lpw);
             return cudaGetLastError();
         }
         if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && (uint64_t)n < kBulkMaxBatch) {
@@ -585,6 +587,7 @@ struct MissRun {
                            cudaStream_t st, CallCounters* cur, bool release, const FirstCounts* fc) {
         IndexRows init_ra = row_args(t);  // new rows live in the host tier when tiered
         if (t->tiered) init_ra.slots = t->tier.host_dev;
+        if (!miss_grid_fits(t, t->num_sms)) return cudaErrorInvalidConfiguration;
         const MissArgs ma = miss_args(t, keys, n, mode, mode == MissMode::Get ? nullptr : t->s.row_of_pos,
                                       mode == MissMode::Get ? out : nullptr, cur);
         MLKV_LAUNCH(t, 0, (k_miss<V>), t->num_sms, kMissThreads, 0, st, index_args(t), init_ra, ma,
@@ -681,19 +684,19 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
 }
 
 namespace {
-// Lookups per warp of k_get_small: as few as a grid of two blocks of 8 warps per
+// Lookups per warp of k_get_small: as few as a grid of kGetBlocksPerSm blocks of 8 warps per
 // SM allows (like the miss kernel's one block of 16: several tables' waiting
 // grids fit the GPU together), at least the rows a warp copies at a time.
 int small_get_lpw(const mlkv_table* t, int64_t n) {
     int lpw = 32 / t->geom.G;
-    while (lpw < 32 && n > (int64_t)lpw * 8 * 2 * t->num_sms) lpw *= 2;
+    while (lpw < 32 && n > (int64_t)lpw * 8 * kGetBlocksPerSm * t->num_sms) lpw *= 2;
     return lpw;
 }
 }  // namespace
 
 bool small_get(const mlkv_table* t, int64_t n) {
     return t->cfg.insert_on_miss != 0 && n <= (int64_t)MLKV_SMALL_GET_MAX &&
-           n <= (int64_t)small_get_lpw(t, n) * 8 * 2 * t->num_sms && !wait_injection_armed();
+           n <= (int64_t)small_get_lpw(t, n) * 8 * kGetBlocksPerSm * t->num_sms && !wait_injection_armed();
 }
 
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,

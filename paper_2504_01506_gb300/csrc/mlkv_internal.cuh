@@ -44,6 +44,14 @@ constexpr uint32_t kSortSmallBatch = MLKV_SORT_SMALL_BATCH;
 // offsets kernel (mlkv_sort.cu); their counts are packed, [tile][digit] with 16
 // bits a digit, the large tiles' are [digit][tile].
 inline int sort_tile_shift(int64_t n) { return n < (int64_t)kSortSmallBatch ? kSortTileSmallShift : 12; }
+constexpr int kGetBlocksPerSm = 2;     // blocks per SM, at most, of a Get's grid that waits for itself (k_get_small)
+constexpr int kPlanCluster = 16;       // most blocks of the plan's cluster (8 is the portable limit)
+// The most blocks the miss path runs in: the miss kernel has one per SM, a small
+// Get's grid kGetBlocksPerSm, the plan's cluster kPlanCluster.
+constexpr int64_t most_miss_blocks(int num_sms) {
+    const int64_t get = (int64_t)kGetBlocksPerSm * num_sms;
+    return get > kPlanCluster ? get : kPlanCluster;
+}
 constexpr int kSmallRun = 4;           // runs of 2 .. kSmallRun lookups carry their positions in their record
 constexpr int64_t kMaxStaleness = MLKV_MAX_STALENESS;  // largest bound kept below no bound
 
@@ -102,7 +110,8 @@ struct Scratch {
     uint32_t* sort_counts[3];  // digit counts of the sort's passes, in turn (all but the first zero between sorts)
     uint32_t* sort_offsets; // [tiles][512] output position of each tile's first element of each digit
     uint32_t* sort_dtot;    // [kSortMaxPasses][512] digit totals of each pass, zero between sorts
-    uint32_t* tile_sums;    // [max(scan tiles, SMs)]: per-tile sums of the dedup's scan, per-block of the miss kernel
+    uint32_t* tile_sums;    // [scan tiles + 1] per-tile sums of the dedup's scan
+    uint32_t* miss_sums;    // [max_miss_blocks] new keys of every block of the miss path
     uint4* short_runs;      // [max_batch] the apply's runs of 2 .. MLKV_SEQ_SEGMENT_MAX lookups
     uint2* single_runs;     // [max_batch] its runs of one lookup: (row, lookup position)
     uint4* small_runs;      // [max_batch] runs of 2 .. kSmallRun lookups: (row, p0, p1, p2)
@@ -116,7 +125,7 @@ struct Scratch {
     int64_t max_nodes;
     int64_t max_items;
     int64_t node_cnt_bytes;
-    int64_t tile_sums_len;
+    int64_t max_miss_blocks;
     int64_t sort_counts_bytes;
 };
 
@@ -230,14 +239,20 @@ __device__ __forceinline__ void release_counters(CallCounters* c, uint32_t total
     }
 }
 
-// Bounds-checked build (-DMLKV_CHECK=1): the reduce kernels test the indices
-// they are about to use (rows, lookup positions, list entries); a failed test
+// Bounds-checked build (-DMLKV_CHECK=1): the reduce kernels and the miss path test
+// the indices they are about to use (rows, lookup positions, list entries, a
+// block's place among the miss path's); a failed test
 // records the first failing site with its index and bound and
 // MLKV_ERR_INVALID, and the access is skipped.  mlkv_sync reports the site.
 // In the normal build every test is compiled out.
 #ifndef MLKV_CHECK
 #define MLKV_CHECK 0
 #endif
+// Sites of the bounds-checked build (in_bounds).
+enum CheckSite : uint32_t {
+    kChkSingleRow = 1, kChkSinglePos, kChkSmallRow, kChkSmallPos, kChkShortRun, kChkShortRow, kChkShortPos,
+    kChkLongItem, kChkLongPos, kChkLongRow, kChkHeadsPos, kChkListEntry, kChkMissBlock
+};
 __device__ __forceinline__ bool in_bounds(const ErrSink& e, uint32_t site, unsigned long long idx,
                                           unsigned long long bound) {
     if (!MLKV_CHECK || idx < bound) return true;

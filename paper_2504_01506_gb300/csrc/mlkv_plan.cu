@@ -40,7 +40,6 @@ constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kPlanDigitBits = 10;  // one digit per thread
 constexpr int kPlanRadix = 1 << kPlanDigitBits;
 constexpr int kPlanItems = 2;       // most lookups per thread
-constexpr int kPlanCluster = 16;    // most blocks (8 is the portable limit)
 constexpr int kLongBatch = 8;       // long runs a warp writes at a time
 
 // A tile of T = 1024 * items lookups per block.
@@ -492,6 +491,7 @@ cudaError_t launch_plan(mlkv_table* t, const int64_t* keys, int64_t n, bool inse
     const int64_t tile = (int64_t)kPlanThreads * items;
     int blocks = 1;
     while (blocks * tile < n) blocks *= 2;
+    if (!miss_grid_fits(t, blocks)) return cudaErrorInvalidConfiguration;
     const int passes = (t->sort_bits + kPlanDigitBits - 1) / kPlanDigitBits;
     PlanArgs pa{};
     pa.keys = keys;

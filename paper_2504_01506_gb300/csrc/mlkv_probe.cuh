@@ -141,7 +141,7 @@ inline IndexRows row_args(mlkv_table* t) {
 
 inline IndexArgs index_args(mlkv_table* t) {
     return IndexArgs{t->index, t->index_mask, (t->cfg.flags & MLKV_IDENTITY_HASH) ? 1u : 0u,
-                     ErrSink{&t->dstate->status, t->status_dev_alias}};
+                     ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}};
 }
 
 // Group-cooperative copy of one row (or NaN) into dst.
@@ -167,6 +167,7 @@ __device__ __forceinline__ void copy_row(const float* __restrict__ src, float* _
 //   4. every missed lookup reads its key's row (a Get gathers it into its
 //      output), flags and the slot's aux go back to idle, the row counter
 //      advances.
+// The host keeps nblocks within MissArgs::max_blocks (miss_grid_fits).
 // `on_row` is told every missed lookup's row in phase 4.  Data written by other
 // blocks within the kernel is read from L2 (ld.cg).
 struct MissArgs {
@@ -176,7 +177,8 @@ struct MissArgs {
     const uint32_t* miss_slot;
     uint32_t* flag;
     uint32_t* rank;
-    uint32_t* block_sums;
+    uint32_t* block_sums;  // [max_blocks]
+    uint32_t max_blocks;
     uint32_t* row_of_pos;
     float* out;
     CallCounters* cur;
@@ -189,11 +191,14 @@ struct MissArgs {
 
 inline MissArgs miss_args(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode, uint32_t* row_of_pos,
                           float* out, CallCounters* cur) {
-    return MissArgs{keys, (uint32_t)n, t->s.miss_pos, t->s.miss_slot, t->s.first_flag, t->s.rank, t->s.tile_sums,
-                    row_of_pos, out, cur, t->dstate, (unsigned long long)t->cfg.capacity,
+    return MissArgs{keys, (uint32_t)n, t->s.miss_pos, t->s.miss_slot, t->s.first_flag, t->s.rank, t->s.miss_sums,
+                    (uint32_t)t->s.max_miss_blocks, row_of_pos, out, cur, t->dstate, (unsigned long long)t->cfg.capacity,
                     mode == MissMode::Put ? 0 : 1, (unsigned long long)t->cfg.seed, t->cfg.init_lo,
                     t->cfg.init_hi - t->cfg.init_lo, t->cfg.state_init};
 }
+
+// Whether the miss path may run in this many blocks.
+inline bool miss_grid_fits(const mlkv_table* t, int64_t blocks) { return blocks <= t->s.max_miss_blocks; }
 
 // Sum over the block of one value per thread.
 template <int THREADS>
@@ -255,7 +260,7 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
     uint32_t cnt = 0;
     for (uint32_t p = p_lo + threadIdx.x; p < p_hi; p += blockDim.x) cnt += __ldcg(ma.flag + p);
     const uint32_t mine = miss_block_sum<THREADS>(cnt);
-    if (threadIdx.x == 0) ma.block_sums[block] = mine;
+    if (threadIdx.x == 0 && in_bounds(ia.err, kChkMissBlock, block, ma.max_blocks)) ma.block_sums[block] = mine;
     if (!barrier(1)) return false;
     uint32_t b_before = 0;
     for (uint32_t b = threadIdx.x; b < block; b += blockDim.x) b_before += __ldcg(ma.block_sums + b);

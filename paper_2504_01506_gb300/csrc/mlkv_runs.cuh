@@ -31,12 +31,6 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;  // no position (a small run's record pas
 // kGroupChunks chunks; of longer runs, a block takes kNode chunks at a time.
 constexpr uint32_t kGroupChunks = MLKV_GROUP_CHUNKS, kNode = MLKV_NODE;
 
-// Sites of the bounds-checked build (in_bounds).
-enum CheckSite : uint32_t {
-    kChkSingleRow = 1, kChkSinglePos, kChkSmallRow, kChkSmallPos, kChkShortRun, kChkShortRow, kChkShortPos,
-    kChkLongItem, kChkLongPos, kChkLongRow, kChkHeadsPos, kChkListEntry
-};
-
 constexpr uint32_t kItemLenBits = 7;  // a chunk holds at most 64 lookups; a run at most 2^24 chunks of 64
 static_assert(kChunkLarge < (1u << kItemLenBits) && kChunkSmall < (1u << kItemLenBits), "chunk lengths fit their bits");
 

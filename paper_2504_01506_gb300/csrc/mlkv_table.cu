@@ -571,7 +571,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
     Scratch& s = t->s;
     long_bounds(B, s.max_long, s.max_nodes, s.max_items);
     s.node_cnt_bytes = node_counters(s.max_items, c.dim) * 4;
-    s.tile_sums_len = std::max<int64_t>(tiles_of(B) + 1, t->num_sms);
+    s.max_miss_blocks = most_miss_blocks(t->num_sms);
     // the sort's tiles: 4096 lookups, kSortTileSmall in batches under kSortSmallBatch
     const int64_t sort_tiles = std::max<int64_t>(
         tiles_of(B), (std::min<int64_t>(B, (int64_t)kSortSmallBatch - 1) + kSortTileSmall - 1) / kSortTileSmall);
@@ -586,7 +586,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.first_flag, B * 4},     {(void**)&s.rank, B * 4},
         {(void**)&s.sk[0], B * 4},          {(void**)&s.sk[1], B * 4},
         {(void**)&s.sv[0], B * 4},          {(void**)&s.sv[1], B * 4},
-        {(void**)&s.tile_sums, s.tile_sums_len * 4},
+        {(void**)&s.tile_sums, (tiles_of(B) + 1) * 4}, {(void**)&s.miss_sums, s.max_miss_blocks * 4},
         {(void**)&s.sort_counts[0], s.sort_counts_bytes = 512 * sort_tiles * 4},
         {(void**)&s.sort_counts[1], s.sort_counts_bytes},
         {(void**)&s.sort_counts[2], s.sort_counts_bytes},

@@ -150,3 +150,52 @@ def test_stale_synchronous_calls_refuse_capture():
             with torch.cuda.graph(graph, stream=s):
                 store.get(keys)
     assert e.value.code == 2  # MLKV_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("n_apply", [40_000, 500_000])
+def test_new_keys_beside_a_large_apply(n_apply):
+    """Gets of new keys alone, of as many lookups as fill the Get's largest grid
+    (2,432 of dim 128: 304 blocks, every one of which counts its new keys), beside
+    applies that are in their sort: neither may write into the other's scratch.
+    Row ids, the Gets' rows and the table after each pair against the oracle;
+    the gradients are small multiples of 2^-10, so every sum is exact."""
+    torch = torch_cuda()
+    dim, n_get, steps, n_keys = 128, 2_432, 6, 30_000
+    cfg = W.tiny()
+    rng = np.random.default_rng(n_apply)
+    pre = rng.choice(1 << 40, n_keys, replace=False).astype(np.int64)
+    store = _store(cfg, 1, dim=dim, capacity=n_keys + steps * n_get + 8, max_batch=n_apply, lr=0.125)
+    ref = oracle.Table(dim, lr=0.125, eps=cfg.eps, state_init=cfg.state_init, init_lo=cfg.init_lo, init_hi=cfg.init_hi,
+                       seed=cfg.seed, precision=32)
+    store.insert(dev(pre))
+    ref.insert(pre)
+    new = [((1 << 41) + t * 10_000 + rng.permutation(n_get)).astype(np.int64) for t in range(steps)]
+    # an apply has some of the keys that the Get before it inserts
+    ak = [np.concatenate([rng.choice(new[t], n_apply // 8), rng.choice(pre, n_apply - n_apply // 8)])
+          for t in range(steps)]
+    ak = [rng.permutation(k) for k in ak]
+    grads = dev((rng.integers(-8, 9, size=(n_apply, dim)) * 2.0**-10).astype(np.float32))
+    kd, akd = [dev(k) for k in new], [dev(k) for k in ak]
+    outs = [torch.empty((n_get, dim), device="cuda:0") for _ in range(steps)]
+    torch.cuda.synchronize()
+    s_get, s_apply = torch.cuda.Stream(), torch.cuda.Stream()
+    for t in range(steps):
+        with torch.cuda.stream(s_get):
+            store.get(kd[t], out=outs[t])
+        with torch.cuda.stream(s_apply):
+            store.apply_grad(akd[t], grads)
+    torch.cuda.synchronize()
+    assert store.sync() == 0
+    for t in range(steps):
+        want, _, _ = ref.get(new[t])
+        assert_bits(host(outs[t]), want, f"rows of the new keys, step {t}")
+        ref.apply_grad(ak[t], host(grads))
+    allk = ref.keys()
+    assert store.size() == len(allk)
+    assert np.array_equal(host(store.keys()), allk)  # the same row ids
+    assert store.last_unique() == len(np.unique(ak[-1]))
+    for s in range(0, len(allk), n_apply):
+        w, G = store.export(dev(allk[s:s + n_apply]))
+        rw, rG = ref.export(allk[s:s + n_apply])
+        assert_bits(host(w), rw, "rows after the last apply")
+        assert_bits(host(G), rG, "state after the last apply")
