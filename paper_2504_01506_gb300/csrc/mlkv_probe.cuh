@@ -144,15 +144,16 @@ inline IndexArgs index_args(mlkv_table* t) {
                      ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}};
 }
 
-// Group-cooperative copy of one row (or NaN) into dst.
+// Group-cooperative copy of one row (or NaN) into dst.  The row was written by
+// another block of this kernel: read from L2.
 template <int V>
-__device__ __forceinline__ void copy_row(const float* __restrict__ src, float* __restrict__ dst,
+__device__ __forceinline__ void copy_row(const float* src, float* __restrict__ dst,
                                          int NV, int G, int glane, bool absent) {
     using VT = typename Vec<V>::T;
     const VT* s = reinterpret_cast<const VT*>(src);
     VT* o = reinterpret_cast<VT*>(dst);
 #pragma unroll 2
-    for (int j = glane; j < NV; j += G) __stcs(o + j, absent ? Vec<V>::nan() : __ldg(s + j));
+    for (int j = glane; j < NV; j += G) __stcs(o + j, absent ? Vec<V>::nan() : __ldcg(s + j));
 }
 
 // ---------------------------------------------------------------------------
