@@ -178,9 +178,10 @@ __global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : M
 }
 
 // The Get and its miss path in one launch (see finish_get): a warp per lpw
-// lookups, in a grid that can wait for itself.
+// lookups, in a grid that can wait for itself (its launch bounds leave room for
+// the kGetBlocksPerSm blocks per SM of the largest, and the launch asks).
 template <int V, int KV, bool WIDE>
-__global__ void __launch_bounds__(256) k_get_small(IndexArgs ia, IndexRows ra, MissArgs ma, CallCounters* nxt,
+__global__ void __launch_bounds__(256, kGetBlocksPerSm) k_get_small(IndexArgs ia, IndexRows ra, MissArgs ma, CallCounters* nxt,
                                                    Memo memo, int lpw) {
     pdl_enter();
     zero_counters(nxt);
@@ -533,28 +534,37 @@ int bulk_grid(mlkv_table* t, size_t smem, int64_t n) {
     return (int)(g < cap ? g : cap);
 }
 
-int small_get_lpw(const mlkv_table* t, int64_t n);
+// Lookups per warp of k_get_small: as few as a grid of kGetBlocksPerSm blocks of 8 warps per
+// SM allows (like the miss kernel's one block of 16: several tables' waiting
+// grids fit the GPU together), at least the rows a warp copies at a time.
+int small_get_lpw(const mlkv_table* t, int64_t n) {
+    int lpw = 32 / t->geom.G;
+    while (lpw < 32 && n > (int64_t)lpw * 8 * kGetBlocksPerSm * t->num_sms) lpw *= 2;
+    return lpw;
+}
 
 template <int V>
 struct GetRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* out,
-                           cudaStream_t st, CallCounters* cur, CallCounters* nxt) {
+                           cudaStream_t st, CallCounters* cur, CallCounters* nxt, bool& resolved) {
         const uint32_t rowbytes = (uint32_t)t->geom.d * 4;
         const int kv = row_vectors<V>(t->geom);
         constexpr int M = kMostVectors<V>;
         const bool wide = t->geom.NV > 32 * kv;
         const bool ins = t->cfg.insert_on_miss != 0;
-        if (small_get(t, n)) {
-            const int lpw = small_get_lpw(t, n);
-            const unsigned grid = grid_for(n, 8 * lpw);
-            if (!miss_grid_fits(t, grid)) return cudaErrorInvalidConfiguration;
+        const auto small = kv == 1   ? k_get_small<V, 1, false>
+                           : wide    ? k_get_small<V, M, true>
+                           : kv == 2 ? k_get_small<V, 2, false>
+                                     : k_get_small<V, M, false>;
+        const int small_lpw = small_get_lpw(t, n);
+        const unsigned grid = grid_for(n, 8 * small_lpw);
+        // every block resident at once, with a word each for its new keys
+        resolved = ins && n <= (int64_t)MLKV_SMALL_GET_MAX && !wait_injection_armed() && miss_grid_fits(t, grid) &&
+                   (int64_t)grid <= persistent_blocks(t, (const void*)small, 256);
+        if (resolved) {
             const MissArgs ma = miss_args(t, keys, n, MissMode::Get, nullptr, out, cur);
-            const auto kernel = kv == 1   ? k_get_small<V, 1, false>
-                                : wide    ? k_get_small<V, M, true>
-                                : kv == 2 ? k_get_small<V, 2, false>
-                                          : k_get_small<V, M, false>;
-            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, kernel, grid, 256, 0, st, index_args(t), row_args(t), ma, nxt,
-                        Memo{t->s.memo_key, t->s.memo_row}, lpw);
+            MLKV_LAUNCH(t, MLKV_K_GET_GATHER, small, grid, 256, 0, st, index_args(t), row_args(t), ma, nxt,
+                        Memo{t->s.memo_key, t->s.memo_row}, small_lpw);
             return cudaGetLastError();
         }
         if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && (uint64_t)n < kBulkMaxBatch) {
@@ -683,25 +693,9 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
     return cudaGetLastError();
 }
 
-namespace {
-// Lookups per warp of k_get_small: as few as a grid of kGetBlocksPerSm blocks of 8 warps per
-// SM allows (like the miss kernel's one block of 16: several tables' waiting
-// grids fit the GPU together), at least the rows a warp copies at a time.
-int small_get_lpw(const mlkv_table* t, int64_t n) {
-    int lpw = 32 / t->geom.G;
-    while (lpw < 32 && n > (int64_t)lpw * 8 * kGetBlocksPerSm * t->num_sms) lpw *= 2;
-    return lpw;
-}
-}  // namespace
-
-bool small_get(const mlkv_table* t, int64_t n) {
-    return t->cfg.insert_on_miss != 0 && n <= (int64_t)MLKV_SMALL_GET_MAX &&
-           n <= (int64_t)small_get_lpw(t, n) * 8 * kGetBlocksPerSm * t->num_sms && !wait_injection_armed();
-}
-
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,
-                       CallCounters* cur, CallCounters* nxt) {
-    return dispatch_row<GetRun>(t->geom, t, keys, n, out, st, cur, nxt);
+                       CallCounters* cur, CallCounters* nxt, bool& resolved) {
+    return dispatch_row<GetRun>(t->geom, t, keys, n, out, st, cur, nxt, resolved);
 }
 
 cudaError_t launch_resolve_misses(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode,

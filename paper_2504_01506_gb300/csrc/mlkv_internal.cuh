@@ -535,9 +535,9 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
 #ifndef MLKV_SMALL_GET_MAX
 #define MLKV_SMALL_GET_MAX (1 << 14)
 #endif
-bool small_get(const mlkv_table* t, int64_t n);  // launch_get then needs no launch_resolve_misses
+// resolved: whether this one does; else launch_resolve_misses has to follow.
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,
-                       CallCounters* cur, CallCounters* nxt);
+                       CallCounters* cur, CallCounters* nxt, bool& resolved);
 // release: the miss kernel is the last of the call to read its counters, and
 // zeroes them when done (release_counters).  fc: the first sort pass's counts
 // the probe made, to which the lookups given rows here are added.

@@ -663,9 +663,10 @@ int mlkv_get(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_out, void
         return MLKV_OK;
     }
     CallScope cs = begin_call(t, st, true);
-    const bool small = small_get(t, n);
-    CK(t, launch_get(t, d_keys, n, d_out, st, cs.cur, cs.nxt));
-    if (t->cfg.insert_on_miss && !small) CK(t, launch_resolve_misses(t, d_keys, n, MissMode::Get, d_out, st, cs.cur, true));
+    bool resolved = false;
+    CK(t, launch_get(t, d_keys, n, d_out, st, cs.cur, cs.nxt, resolved));
+    if (t->cfg.insert_on_miss && !resolved)
+        CK(t, launch_resolve_misses(t, d_keys, n, MissMode::Get, d_out, st, cs.cur, true));
     return MLKV_OK;
 }
 
