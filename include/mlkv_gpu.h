@@ -338,12 +338,15 @@ int64_t mlkv_last_unique(mlkv_table* t);
  * returns MLKV_ERR_NOMEM; for MLKV_FAULT_COPY a host <-> device copy of a
  * *_host call, which then returns MLKV_ERR_CUDA with nothing after it
  * enqueued; for MLKV_FAULT_WAIT a launch of the kernel that gives new keys
- * their rows (launched by every call that may insert), whose grid barriers then wait for one
- * block more than the grid has: if the call has new keys, every wait runs out
- * (in a second or two), MLKV_ERR_TIMEOUT is recorded and the keys get no rows
+ * their rows (a Get's own kernel in small Gets; launched by every call that may
+ * insert), in which blocks then wait for one block more than there is: if the
+ * call has new keys, the waits run out (in a second or two each),
+ * MLKV_ERR_TIMEOUT is recorded and the keys get no rows
  * (a gradient apply still updates the keys that had rows, as if the new keys'
  * lookups were not in the batch; mlkv_clear_status then makes the table whole
- * again).  nth = 0 disarms.  One countdown per kind, shared by the whole
+ * again).  While a wait is armed a gradient apply whose plan one thread-block
+ * cluster would make (it has no wait that can run out) takes the general
+ * kernels.  nth = 0 disarms.  One countdown per kind, shared by the whole
  * process.  No GPU work is affected: nothing faults on the device.  A failed
  * mlkv_open frees everything it allocated and leaves *out null; a failed
  * *_host call leaves the table usable.  Returns MLKV_ERR_INVALID for an

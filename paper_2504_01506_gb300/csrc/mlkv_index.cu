@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : M
 // the kGetBlocksPerSm blocks per SM of the largest, and the launch asks).
 template <int V, int KV, bool WIDE>
 __global__ void __launch_bounds__(256, kGetBlocksPerSm) k_get_small(IndexArgs ia, IndexRows ra, MissArgs ma, CallCounters* nxt,
-                                                   Memo memo, int lpw) {
+                                                                    Memo memo, int lpw, uint32_t bar_extra) {
     pdl_enter();
     zero_counters(nxt);
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256, kGetBlocksPerSm) k_get_small(IndexArgs ia
     if (base < ma.n)
         fresh = get_rows<V, KV, WIDE, true, 4 / KV>(ia, ra, ma.keys, ma.n, ma.out, const_cast<uint32_t*>(ma.miss_pos),
                                        const_cast<uint32_t*>(ma.miss_slot), ma.cur, memo, base, lpw);
-    finish_get<V, 256>(ia, ra, ma, fresh);
+    finish_get<V, 256>(ia, ra, ma, fresh, bar_extra);
 }
 
 // The Get with its rows moved by the SM's asynchronous copies, for calls of
@@ -559,12 +559,12 @@ struct GetRun {
         const int small_lpw = small_get_lpw(t, n);
         const unsigned grid = grid_for(n, 8 * small_lpw);
         // every block resident at once, with a word each for its new keys
-        resolved = ins && n <= (int64_t)MLKV_SMALL_GET_MAX && !wait_injection_armed() && miss_grid_fits(t, grid) &&
+        resolved = ins && n <= (int64_t)MLKV_SMALL_GET_MAX && miss_grid_fits(t, grid) &&
                    (int64_t)grid <= persistent_blocks(t, (const void*)small, 256);
         if (resolved) {
             const MissArgs ma = miss_args(t, keys, n, MissMode::Get, nullptr, out, cur);
             MLKV_LAUNCH(t, MLKV_K_GET_GATHER, small, grid, 256, 0, st, index_args(t), row_args(t), ma, nxt,
-                        Memo{t->s.memo_key, t->s.memo_row}, small_lpw);
+                        Memo{t->s.memo_key, t->s.memo_row}, small_lpw, take_injected_wait() ? 1u : 0u);
             return cudaGetLastError();
         }
         if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && (uint64_t)n < kBulkMaxBatch) {

@@ -331,10 +331,12 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
 // waits; else the marked blocks, alone, wait for the others and run the miss
 // path.  (A miss kernel of its own that finds nothing to do cost a Get of 416
 // lookups 4 of its 15 us, and the step of 4,096 lookups 2.5 of 36.)  The whole
-// block calls it.
+// block calls it.  (mlkv_debug_fail's wait injection, bar_extra, makes the first
+// marked block wait for one arrival too many; the other marked blocks then wait
+// for that one in the miss path, in vain too.)
 template <int V, int THREADS>
 __device__ __forceinline__ void finish_get(const IndexArgs& ia, const IndexRows& ra, const MissArgs& ma,
-                                           bool new_key) {
+                                           bool new_key, uint32_t bar_extra) {
     __shared__ uint32_t share[2];  // marked blocks, this block among them
     CallCounters* cur = ma.cur;
     const uint32_t grid = gridDim.x;
@@ -349,7 +351,8 @@ __device__ __forceinline__ void finish_get(const IndexArgs& ia, const IndexRows&
                 for (unsigned i = 0; i < sizeof(CallCounters) / 4; ++i) w[i] = 0u;
             }
         } else {
-            share[0] = wait_count(&cur->bar[0], 0xFFFFu, grid, ia.err) ? ld_acquire_u32(&cur->bar[0]) >> 16 : 0u;
+            const uint32_t want = grid + (share[1] ? 0u : bar_extra);
+            share[0] = wait_count(&cur->bar[0], 0xFFFFu, want, ia.err) ? ld_acquire_u32(&cur->bar[0]) >> 16 : 0u;
             __threadfence();
         }
     }

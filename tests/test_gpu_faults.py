@@ -19,7 +19,7 @@ import pytest
 
 import oracle
 import workloads as W
-from gpu_helpers import assert_bits, dev, host, torch_cuda
+from gpu_helpers import assert_bits, dev, host, make_pair, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -219,4 +219,88 @@ def test_apply_whose_miss_wait_runs_out_updates_only_known_keys():
     short = c <= 32
     assert_bits(host(w)[short], rw[short], "rows after the second apply")
     assert_bits(host(G)[short], rG[short], "state after the second apply")
+    store.close()
+
+
+@pytest.mark.parametrize("n,dim", [(40, 16), (2_432, 128), (16_384, 16)])  # one block, the largest grid, 8 lookups a warp
+def test_small_get_whose_wait_runs_out_hands_out_no_row(n, dim):
+    """A Get whose new keys get their rows in its own kernel, made to wait in
+    vain: the first block that met a new key gives up at its first wait, the
+    others in the miss path, where they wait for it.  No row is handed out, and
+    after mlkv_clear_status the same Get gives what the oracle gives."""
+    torch = torch_cuda()
+    L, lib = _lib()
+    cfg = W.tiny()
+    cfg.dim = dim
+    store, ref = make_pair(cfg, capacity=40_000, max_batch=n)
+    rng = np.random.default_rng(n)
+    known = rng.choice(1 << 40, 30, replace=False).astype(np.int64)
+    store.insert(dev(known))
+    ref.insert(known)
+    keys = known[rng.integers(0, 30, n)]
+    new = (1 << 45) + np.arange(max(n // 3, 1), dtype=np.int64) * 7919
+    at = rng.permutation(n)[: n // 2]
+    keys[at] = new[rng.integers(0, len(new), len(at))]  # in every block, some of them more than once
+    keys[0] = new[0]
+    lib.mlkv_debug_fail(L.FAULT_WAIT, 1)
+    t0 = time.time()
+    store.get(dev(keys))
+    rc = store.sync()
+    took = time.time() - t0
+    lib.mlkv_debug_fail(L.FAULT_WAIT, 0)
+    assert rc == L.ERR_TIMEOUT, rc
+    assert took < 60, took
+    assert store.size() == len(known)
+    store.clear_status()
+    for _ in range(2):  # the first inserts; the second starts from the counters it left
+        want, _, _ = ref.get(keys)
+        assert_bits(host(store.get(dev(keys))), want, "the same Get after the status was cleared")
+    assert store.sync() == 0
+    assert store.size() == ref.size() and np.array_equal(host(store.find(dev(keys))), ref.find(keys))
+    grads = (rng.integers(-8, 9, size=(n, dim)) * 2.0**-10).astype(np.float32)  # exact sums
+    store.apply_grad(dev(keys), dev(grads))
+    ref.apply_grad(keys, grads)
+    u = np.unique(keys)
+    w, G = store.export(dev(u))
+    rw, rG = ref.export(u)
+    assert_bits(host(w), rw, "rows after an apply")
+    assert_bits(host(G), rG, "state after an apply")
+    store.close()
+
+
+def test_large_apply_whose_miss_wait_runs_out_updates_only_known_keys():
+    """The same as above for an apply too large for the one-cluster plan, whose
+    miss kernel every such apply launches."""
+    torch = torch_cuda()
+    L, lib = _lib()
+    cfg = W.tiny()
+    cfg.dim = 4
+    n = 40_000
+    store, ref = make_pair(cfg, capacity=30_000, max_batch=n)
+    rng = np.random.default_rng(6)
+    known = rng.choice(1 << 40, 20_000, replace=False).astype(np.int64)
+    store.insert(dev(known))
+    ref.insert(known)
+    new = (1 << 45) + np.arange(5_000, dtype=np.int64) * 7919
+    keys = rng.choice(np.concatenate([known, new]), n)
+    grads = (rng.integers(-8, 9, size=(n, 4)) * 2.0**-10).astype(np.float32)  # exact sums
+    lib.mlkv_debug_fail(L.FAULT_WAIT, 1)
+    store.apply_grad(dev(keys), dev(grads))
+    rc = store.sync()
+    lib.mlkv_debug_fail(L.FAULT_WAIT, 0)
+    assert rc == L.ERR_TIMEOUT, rc
+    store.clear_status()
+    assert store.size() == len(known)
+    there = np.isin(keys, known)
+    ref.apply_grad(keys[there], grads[there])
+    for step in ("timed-out", "second"):
+        if step == "second":
+            store.apply_grad(dev(keys), dev(grads))
+            ref.apply_grad(keys, grads)
+        u = np.unique(keys[there] if step == "timed-out" else keys)
+        w, G = store.export(dev(u))
+        rw, rG = ref.export(u)
+        assert_bits(host(w), rw, f"rows after the {step} apply")
+        assert_bits(host(G), rG, f"state after the {step} apply")
+    assert store.sync() == 0 and store.size() == ref.size()
     store.close()
