@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan(IndexArgs ia, IndexRow
                 if (m) {  // the same for every block
                     auto none = [](uint32_t, uint32_t) {};
                     miss_path<V, kPlanThreads>(
-                        ia, ra, ma, m, nblocks, me,
+                        ia, ra, ma, m, even_share(ma.n, nblocks, me),
                         [&](int) {
                             __threadfence();
                             meet();

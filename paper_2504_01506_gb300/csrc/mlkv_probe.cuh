@@ -144,33 +144,25 @@ inline IndexArgs index_args(mlkv_table* t) {
                      ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}};
 }
 
-// Group-cooperative copy of one row (or NaN) into dst.  The row was written by
-// another block of this kernel: read from L2.
-template <int V>
-__device__ __forceinline__ void copy_row(const float* src, float* __restrict__ dst,
-                                         int NV, int G, int glane, bool absent) {
-    using VT = typename Vec<V>::T;
-    const VT* s = reinterpret_cast<const VT*>(src);
-    VT* o = reinterpret_cast<VT*>(dst);
-#pragma unroll 2
-    for (int j = glane; j < NV; j += G) __stcs(o + j, absent ? Vec<V>::nan() : __ldcg(s + j));
-}
-
 // ---------------------------------------------------------------------------
 // The miss path: new keys of a call get rows, in four phases separated by
-// barriers of all its blocks (`barrier`; `nblocks` blocks, this one `block`):
+// barriers of all its blocks (`barrier`; MissShare says which blocks they are):
 //   1. flag the first occurrence of each new key (the lookup whose position
 //      survived in the slot's aux);
-//   2. rank the flags: an exclusive scan over the call's positions, block b
-//      owning positions [b * per, (b + 1) * per);
+//   2. rank the flags: an exclusive scan over the call's positions, every block
+//      over a range of them of its own;
 //   3. each first occurrence takes row = rows handed out so far + rank and
 //      writes its init row (not for Put) and state_init;
 //   4. every missed lookup reads its key's row (a Get gathers it into its
 //      output), flags and the slot's aux go back to idle, the row counter
 //      advances.
-// The host keeps nblocks within MissArgs::max_blocks (miss_grid_fits).
 // `on_row` is told every missed lookup's row in phase 4.  Data written by other
 // blocks within the kernel is read from L2 (ld.cg).
+// Phases 3 and 4 take the miss list's entries as for_misses deals them out: a
+// warp loads up to 32 entries, one a lane, and its lane groups then write or copy
+// their rows one after another.  (With a lane group loading the entry of each
+// row it wrote, every row waited for three dependent loads: a Get of 16,384
+// lookups of dim 128 whose last 64 keys are new took 64 us, 25 so.)
 struct MissArgs {
     const int64_t* keys;
     uint32_t n;
@@ -241,86 +233,135 @@ __device__ __forceinline__ uint32_t miss_block_scan(uint32_t v, uint32_t& total)
     return before + x - v;
 }
 
+// The blocks of a miss path, and the positions this one ranks.  A block's
+// place in the order of positions is `order` of the `nsums` that blocks (not all
+// of them blocks of the miss path) have in MissArgs::block_sums.
+struct MissShare {
+    uint32_t nblocks, block;  // blocks of the miss path (the host keeps them within MissArgs::max_blocks), this one
+    uint32_t nsums, order;
+    uint32_t p_lo, p_hi;
+};
+
+// Every block of the grid, the positions in equal shares.
+__device__ __forceinline__ MissShare even_share(uint32_t n, uint32_t nblocks, uint32_t block) {
+    const uint32_t per = (n + nblocks - 1) / nblocks, lo = min(n, block * per);
+    return MissShare{nblocks, block, nblocks, block, lo, min(n, lo + per)};
+}
+
+// f(i, at_once) for this lane's entry i (or a value >= m) of every round of the
+// warp over the m entries of the miss list (the whole warp; at_once entries a
+// round, at least R = 32 / G: as few as leave every warp of the miss path some).
+template <int THREADS, class F>
+__device__ __forceinline__ void for_misses(uint32_t m, uint32_t nblocks, uint32_t block, uint32_t R, F f) {
+    const uint32_t warps = nblocks * (THREADS / 32), lane = threadIdx.x & 31;
+    uint32_t at_once = 32;
+    while (at_once > R && (unsigned long long)warps * (at_once / 2) >= m) at_once /= 2;
+    for (uint32_t i0 = (block * (THREADS / 32) + (threadIdx.x >> 5)) * at_once; i0 < m; i0 += warps * at_once)
+        f(lane < at_once ? i0 + lane : 0xFFFFFFFFu, at_once);
+}
+
 template <int V, int THREADS, class Barrier, class OnRow>
 __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& ra, const MissArgs& ma, uint32_t m,
-                                          uint32_t nblocks, uint32_t block, Barrier barrier, OnRow on_row) {
+                                          const MissShare& sh, Barrier barrier, OnRow on_row) {
     using VT = typename Vec<V>::T;
-    const uint32_t nthreads = nblocks * blockDim.x;
-    const uint32_t tid = block * blockDim.x + threadIdx.x;
-    const int G = ra.G, glane = threadIdx.x & (G - 1);
-    const uint32_t group = tid / G, ngroups = nthreads / G;
+    const uint32_t nthreads = sh.nblocks * THREADS;
+    const int lane = threadIdx.x & 31, G = ra.G, glane = lane & (G - 1), gid = lane / G;
+    const uint32_t R = 32u / G;
     // 1. first occurrences
-    for (uint32_t i = tid; i < m; i += nthreads) {
+    for (uint32_t i = sh.block * THREADS + threadIdx.x; i < m; i += nthreads) {
         const uint32_t p = __ldcg(ma.miss_pos + i);
         if (ld_u32_relaxed(&ia.index[__ldcg(ma.miss_slot + i)].aux) == p) ma.flag[p] = 1u;
     }
     if (!barrier(0)) return false;
     // 2. ranks: the first occurrences at earlier positions
-    const uint32_t per = (ma.n + nblocks - 1) / nblocks;
-    const uint32_t p_lo = min(ma.n, block * per), p_hi = min(ma.n, p_lo + per);
     uint32_t cnt = 0;
-    for (uint32_t p = p_lo + threadIdx.x; p < p_hi; p += blockDim.x) cnt += __ldcg(ma.flag + p);
+    for (uint32_t p = sh.p_lo + threadIdx.x; p < sh.p_hi; p += THREADS) cnt += __ldcg(ma.flag + p);
     const uint32_t mine = miss_block_sum<THREADS>(cnt);
-    if (threadIdx.x == 0 && in_bounds(ia.err, kChkMissBlock, block, ma.max_blocks)) ma.block_sums[block] = mine;
+    if (threadIdx.x == 0 && in_bounds(ia.err, kChkMissBlock, sh.order, ma.max_blocks)) ma.block_sums[sh.order] = mine;
     if (!barrier(1)) return false;
-    uint32_t b_before = 0;
-    for (uint32_t b = threadIdx.x; b < block; b += blockDim.x) b_before += __ldcg(ma.block_sums + b);
+    uint32_t b_before = 0, b_all = 0;
+    for (uint32_t b = threadIdx.x; b < sh.nsums; b += THREADS) {
+        const uint32_t c = __ldcg(ma.block_sums + b);
+        b_all += c;
+        if (b < sh.order) b_before += c;
+    }
     uint32_t run = miss_block_sum<THREADS>(b_before);
-    for (uint32_t p0 = p_lo; p0 < p_hi; p0 += blockDim.x) {  // uniform
+    if (sh.block == 0) {  // every first occurrence
+        const uint32_t all = miss_block_sum<THREADS>(b_all);
+        if (threadIdx.x == 0) ma.cur->n_new = all;
+    }
+    for (uint32_t p0 = sh.p_lo; p0 < sh.p_hi; p0 += THREADS) {  // uniform
         const uint32_t p = p0 + threadIdx.x;
-        const uint32_t f = p < p_hi ? __ldcg(ma.flag + p) : 0u;
+        const uint32_t f = p < sh.p_hi ? __ldcg(ma.flag + p) : 0u;
         uint32_t tot;
         const uint32_t ex = miss_block_scan<THREADS>(f, tot);
         if (f) ma.rank[p] = run + ex;
         run += tot;
     }
-    if (block == nblocks - 1 && threadIdx.x == 0) ma.cur->n_new = run;  // every first occurrence
     if (!barrier(2)) return false;
     // 3. rows of the first occurrences
     const unsigned long long next = ma.ds->next_row;
-    for (uint32_t i = group; i < m; i += ngroups) {
-        const uint32_t p = __ldcg(ma.miss_pos + i), s = __ldcg(ma.miss_slot + i);
-        if (ld_u32_relaxed(&ia.index[s].aux) != p) continue;
-        const unsigned long long r = next + __ldcg(ma.rank + p);
-        if (r >= ma.capacity) {
-            if (glane == 0) record_error(ia.err, MLKV_ERR_FULL);
-            continue;
-        }
-        const unsigned long long key = (unsigned long long)ma.keys[p];
-        float* w = ra.slots + (size_t)r * ra.stride;
-        VT* wv = reinterpret_cast<VT*>(w);
-        VT* gv = reinterpret_cast<VT*>(w + ra.dpad);
-        for (int j = glane; j < ra.NV; j += G) {
-            if (ma.init_row) {
-                float e[V];
-#pragma unroll
-                for (int c = 0; c < V; ++c) e[c] = init_element(ma.seed, key, (uint32_t)(j * V + c), ma.lo, ma.span);
-                wv[j] = Vec<V>::from(e);
+    for_misses<THREADS>(m, sh.nblocks, sh.block, R, [&](uint32_t i, uint32_t at_once) {
+        uint32_t row = ROW_ABSENT;
+        unsigned long long key = 0ull;
+        if (i < m) {
+            const uint32_t p = __ldcg(ma.miss_pos + i), s = __ldcg(ma.miss_slot + i);
+            if (ld_u32_relaxed(&ia.index[s].aux) == p) {
+                const unsigned long long r = next + __ldcg(ma.rank + p);
+                key = (unsigned long long)ma.keys[p];
+                if (r < ma.capacity) ia.index[s].row = row = (uint32_t)r;
+                else record_error(ia.err, MLKV_ERR_FULL);
             }
-            gv[j] = Vec<V>::splat(ma.state_init);
         }
-        if (glane == 0) ia.index[s].row = (uint32_t)r;
-    }
+        for (uint32_t q = 0; q < at_once; q += R) {
+            const uint32_t r = __shfl_sync(0xffffffffu, row, (int)q + gid);
+            const unsigned long long key_q = __shfl_sync(0xffffffffu, key, (int)q + gid);
+            if (r == ROW_ABSENT) continue;
+            float* w = ra.slots + (size_t)r * ra.stride;
+            VT* wv = reinterpret_cast<VT*>(w);
+            VT* gv = reinterpret_cast<VT*>(w + ra.dpad);
+            for (int j = glane; j < ra.NV; j += G) {
+                if (ma.init_row) {
+                    float e[V];
+#pragma unroll
+                    for (int c = 0; c < V; ++c) e[c] = init_element(ma.seed, key_q, (uint32_t)(j * V + c), ma.lo,
+                                                                          ma.span);
+                    wv[j] = Vec<V>::from(e);
+                }
+                gv[j] = Vec<V>::splat(ma.state_init);
+            }
+        }
+    });
     if (!barrier(3)) return false;
     // 4. every missed lookup takes its key's row
-    if (block == 0 && threadIdx.x == 0) {
+    if (sh.block == 0 && threadIdx.x == 0) {
         const unsigned long long nr = next + __ldcg(&ma.cur->n_new);
         ma.ds->next_row = nr < ma.capacity ? nr : ma.capacity;
     }
-    for (uint32_t i = group; i < m; i += ngroups) {
-        const uint32_t p = __ldcg(ma.miss_pos + i), s = __ldcg(ma.miss_slot + i);
-        const uint32_t r0 = ld_u32_relaxed(&ia.index[s].row);
-        const uint32_t r = r0 == ROW_PENDING ? ROW_ABSENT : r0;
-        if (glane == 0) {
-            if (ma.row_of_pos) ma.row_of_pos[p] = r;
+    for_misses<THREADS>(m, sh.nblocks, sh.block, R, [&](uint32_t i, uint32_t at_once) {
+        uint32_t p = 0, row = ROW_PENDING;  // lanes without an entry copy nothing
+        if (i < m) {
+            const uint32_t s = __ldcg(ma.miss_slot + i);
+            p = __ldcg(ma.miss_pos + i);
+            row = ld_u32_relaxed(&ia.index[s].row);
+            if (row == ROW_PENDING) row = ROW_ABSENT;
+            if (ma.row_of_pos) ma.row_of_pos[p] = row;
             ma.flag[p] = 0u;
             ia.index[s].aux = AUX_IDLE;
-            on_row(p, r);
+            on_row(p, row);
         }
-        if (ma.out)
-            copy_row<V>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride,
-                        ma.out + (size_t)p * ra.d, ra.NV, G, glane, r == ROW_ABSENT);
-    }
+        if (!ma.out) return;
+        for (uint32_t q = 0; q < at_once; q += R) {
+            const uint32_t r = __shfl_sync(0xffffffffu, row, (int)q + gid);
+            const uint32_t x = __shfl_sync(0xffffffffu, p, (int)q + gid);
+            if (r == ROW_PENDING) continue;
+            // (written by other blocks of this kernel)
+            const VT* src = reinterpret_cast<const VT*>(ra.slots + (size_t)(r == ROW_ABSENT ? 0 : r) * ra.stride);
+            VT* dst = reinterpret_cast<VT*>(ma.out + (size_t)x * ra.d);
+#pragma unroll 2
+            for (int j = glane; j < ra.NV; j += G) __stcs(dst + j, r == ROW_ABSENT ? Vec<V>::nan() : __ldcg(src + j));
+        }
+    });
     return true;
 }
 
@@ -331,17 +372,22 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
 // waits; else the marked blocks, alone, wait for the others and run the miss
 // path.  (A miss kernel of its own that finds nothing to do cost a Get of 416
 // lookups 4 of its 15 us, and the step of 4,096 lookups 2.5 of 36.)  The whole
-// block calls it.  (mlkv_debug_fail's wait injection, bar_extra, makes the first
+// block, whose lookups start at position p_lo and end before p_hi, calls it: it
+// ranks those positions, since a new key's are all in marked blocks.  (With the
+// marked blocks sharing all of the call's positions, a Get of 16,384 lookups
+// that met one new key had a single block scan them all: 52 us of dim 128 where
+// one without new keys takes 13; 21 so.)  (mlkv_debug_fail's wait injection, bar_extra, makes the first
 // marked block wait for one arrival too many; the other marked blocks then wait
 // for that one in the miss path, in vain too.)
 template <int V, int THREADS>
 __device__ __forceinline__ void finish_get(const IndexArgs& ia, const IndexRows& ra, const MissArgs& ma,
-                                           bool new_key, uint32_t bar_extra) {
+                                           bool new_key, uint32_t p_lo, uint32_t p_hi, uint32_t bar_extra) {
     __shared__ uint32_t share[2];  // marked blocks, this block among them
     CallCounters* cur = ma.cur;
     const uint32_t grid = gridDim.x;
     const int marked = __syncthreads_or(new_key);
     if (threadIdx.x == 0) {
+        if (!marked && in_bounds(ia.err, kChkMissBlock, blockIdx.x, ma.max_blocks)) ma.block_sums[blockIdx.x] = 0u;
         __threadfence();
         const uint32_t old = atomicAdd(&cur->bar[0], marked ? 0x10001u : 1u);
         share[1] = old >> 16;
@@ -362,7 +408,7 @@ __device__ __forceinline__ void finish_get(const IndexArgs& ia, const IndexRows&
     if (!blocks) return;  // the wait ran out
     const uint32_t m = min(ld_u32_relaxed(&cur->n_miss), ma.n);
     if (!miss_path<V, THREADS>(
-            ia, ra, ma, m, blocks, share[1],
+            ia, ra, ma, m, MissShare{blocks, share[1], grid, blockIdx.x, p_lo, p_hi},
             [&](int i) { return grid_barrier(&cur->bar[i + 1], blocks, ia.err); },
             [](uint32_t, uint32_t) {}))
         return;

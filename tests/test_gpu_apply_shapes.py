@@ -210,3 +210,34 @@ def test_get_gives_new_keys_rows(n, dim):
     _check_table(store, ref, keys, "apply after the Gets")
     assert store.sync() == 0
     store.close()
+
+
+@pytest.mark.parametrize("dim", [3, 64, 128, 512])
+@pytest.mark.parametrize("n", [65, 2432, 9728, 16_384])
+def test_get_whose_new_keys_are_in_few_blocks(n, dim):
+    """The blocks that met a new key rank the new keys of their own lookups and
+    share the rows: new keys in the first lookups, in the last ones (more of them
+    than a warp takes at a time), in two far ends, one alone, and again and again
+    the same one."""
+    torch_cuda()
+    store, ref = make_pair(_cfg(dim), capacity=4000, max_batch=n, state_init=0.25)
+    rng = np.random.default_rng(n + dim)
+    known = rng.choice(1 << 40, 500, replace=False).astype(np.int64)
+    for s in range(0, 500, n):
+        store.insert(dev(known[s:s + n]))
+        ref.insert(known[s:s + n])
+    fresh = iter((1 << 41) + rng.permutation(4000).astype(np.int64))
+    few, end = min(40, n), min(300, n)
+    for at in (np.arange(few), np.arange(n - end, n), np.r_[np.arange(few // 2), np.arange(n - few // 2, n)],
+               np.array([n // 2]), None, np.array([], np.int64)):
+        keys = known[rng.integers(0, 500, n)]
+        if at is None:
+            keys[rng.permutation(n)[: n // 2]] = next(fresh)
+        else:
+            keys[at] = [next(fresh) for _ in range(len(at))]
+        want, _, _ = ref.get(keys)
+        assert_bits(host(store.get(dev(keys))), want, "Get")
+        assert store.size() == ref.size()
+        _check_table(store, ref, keys, "after the Get")
+    assert store.sync() == 0
+    store.close()
