@@ -38,7 +38,8 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
     constexpr bool COUNT = CT > 0;
     static_assert(!COUNT || kProbeKeys * CT == kSortTile || kProbeKeys * CT == kSortTileSmall,
                   "a counting block covers one sort tile");
-    pdl_enter();
+    if (INSERT) pdl_enter_last();  // the miss kernel is next
+    else pdl_enter();
     zero_counters(nxt);
     __shared__ uint32_t hist[COUNT ? kSortMaxRadix : 1];
     if (COUNT) {
@@ -170,7 +171,8 @@ __global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : M
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
                                              CallCounters* nxt, Memo memo, int lpw) {
-    pdl_enter();
+    if (INSERT) pdl_enter_last();  // the miss kernel is next
+    else pdl_enter();
     zero_counters(nxt);
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
     if (base >= n) return;  // warp-uniform
@@ -244,7 +246,8 @@ __global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, IndexRo
                                                            uint32_t n, float* __restrict__ out, uint32_t* miss_pos,
                                                            uint32_t* miss_slot, CallCounters* cur, CallCounters* nxt,
                                                            Memo memo) {
-    pdl_enter();
+    if (INSERT) pdl_enter_last();  // the miss kernel is next
+    else pdl_enter();
     zero_counters(nxt);
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kWarps = kBulkThreads / 32;

@@ -440,6 +440,14 @@ template <> struct Vec<1> {
 //     scheduled (once every block of this grid has issued it or exited);
 //     they in turn wait for this grid.  Issued after the wait, it keeps at
 //     most one grid waiting ahead of the running one.
+// pdl_enter_last leaves the second out (the next kernel's blocks are then placed
+// when this grid's are done): for the kernels before the miss kernel, whose one
+// block per SM, placed early, piles up on the few SMs that have room first, up
+// to four on one, and finds new keys' rows there on a fraction of the GPU.
+// (Inserts of new keys alone, early -> late: 100,000 of dim 64 73 -> 72 us,
+// 500,000 of dim 128 262 -> 263, a million 1,348 -> 500; of dim 512 4,271 -> 1,259;
+// a Get of a million new keys of dim 128 1,203 -> 833.  Calls without new keys
+// take as long as before within 0.3 us.)
 #ifndef MLKV_PDL_TRIGGER_FIRST
 #define MLKV_PDL_TRIGGER_FIRST 0
 #endif
@@ -448,6 +456,7 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!MLKV_PDL_TRIGGER_FIRST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+__device__ __forceinline__ void pdl_enter_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
