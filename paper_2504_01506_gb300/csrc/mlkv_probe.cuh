@@ -250,12 +250,12 @@ __device__ __forceinline__ MissShare even_share(uint32_t n, uint32_t nblocks, ui
 
 // f(i, at_once) for this lane's entry i (or a value >= m) of every round of the
 // warp over the m entries of the miss list (the whole warp; at_once entries a
-// round, at least R = 32 / G: as few as leave every warp of the miss path some).
+// round, whole groups of R = 32 / G and at most 32: every warp gets about as many).
 template <int THREADS, class F>
 __device__ __forceinline__ void for_misses(uint32_t m, uint32_t nblocks, uint32_t block, uint32_t R, F f) {
     const uint32_t warps = nblocks * (THREADS / 32), lane = threadIdx.x & 31;
-    uint32_t at_once = 32;
-    while (at_once > R && (unsigned long long)warps * (at_once / 2) >= m) at_once /= 2;
+    const uint32_t rounds = (m + warps * 32 - 1) / (warps * 32);
+    const uint32_t at_once = ((m + warps * rounds - 1) / (warps * rounds) + R - 1) / R * R;
     for (uint32_t i0 = (block * (THREADS / 32) + (threadIdx.x >> 5)) * at_once; i0 < m; i0 += warps * at_once)
         f(lane < at_once ? i0 + lane : 0xFFFFFFFFu, at_once);
 }
