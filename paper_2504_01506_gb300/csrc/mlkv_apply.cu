@@ -166,6 +166,22 @@ __device__ __forceinline__ void adagrad_store(const RowArgs& ra, uint32_t row, i
     *beside(ra, p) = G;
 }
 
+// The rows that an apply's plan gave new keys, from row first_new on, hold nothing
+// yet: the lanes that reduce a row's run write its init values and its state
+// before they load them.  (The plan's 16 SMs at most took longer for the rows than
+// all the rest of an apply: 4,096 new keys of dim 128 111 us, 46 so, of dim 512 224
+// and 58; an apply without new keys pays one load and a comparison a unit.)
+__device__ __forceinline__ uint32_t first_new(const RunArgs& a) { return a.cur->new_base - 1u; }  // or NONE
+
+template <int V>
+__device__ __forceinline__ void make_new(const RowArgs& ra, const RunArgs& a, uint32_t row, uint32_t from, int j) {
+    if (row < from || j >= ra.NV) return;
+    typename Vec<V>::T* p = row_vec<V>(ra, row, j);
+    *p = init_vec<V>(a.new_rows.seed, (unsigned long long)__ldg(a.new_rows.keys + (row - from)), j, a.new_rows.lo,
+                     a.new_rows.span);
+    *beside(ra, p) = Vec<V>::splat(a.new_rows.state_init);
+}
+
 // Where the run of `row` that starts at sorted position s ends: the first
 // later position holding another row, or n.  The whole warp searches: 32
 // probes at doubling distances, then rounds of 32 evenly spaced probes, each
@@ -626,13 +642,14 @@ __device__ __forceinline__ void block_pairs(typename Vec<V>::T& acc, typename Ve
     __syncthreads();
 }
 
-template <int V>
+template <int V, bool NEW>
 __global__ void __launch_bounds__(kCombineThreads, 3) k_combine(RowArgs ra, RunArgs a, DevState* ds) {
     pdl_enter();
     using VT = typename Vec<V>::T;
     __shared__ VT sh[2 * kCombineThreads];
     __shared__ int last_node;
     const uint32_t nseg = ra.nseg;
+    const uint32_t from = NEW ? first_new(a) : NONE;
     const uint32_t NR = min(a.cur->n_group, a.max_long) * nseg, NN = min(a.cur->n_nodes, a.max_nodes) * nseg;
     if (blockIdx.x == 0 && threadIdx.x == 0)
         ds->last_unique = a.cur->n_single + a.cur->n_small + a.cur->n_short + a.cur->n_long;  // one run per row
@@ -671,7 +688,10 @@ __global__ void __launch_bounds__(kCombineThreads, 3) k_combine(RowArgs ra, RunA
             cnt = nodes;
         }
         if (!done) continue;
-        if (group == 0 && j < ra.NV) finish_long<V>(ra, a, nd.z, j, acc, cmp);
+        if (group == 0 && j < ra.NV) {
+            if (NEW) make_new<V>(ra, a, nd.z, from, j);
+            finish_long<V>(ra, a, nd.z, j, acc, cmp);
+        }
     }
     // the other long runs: on the blocks that took no node (all blocks when the
     // nodes outnumber them)
@@ -685,6 +705,7 @@ __global__ void __launch_bounds__(kCombineThreads, 3) k_combine(RowArgs ra, RunA
                             in_bounds(a.err, kChkLongRow, r.z, ra.nrows)))
             continue;
         if (j >= ra.NV) continue;
+        if (NEW) make_new<V>(ra, a, r.z, from, j);
         const VT* p = row_vec<V>(ra, r.z, j);
         const VT w = p[0], Gs = *beside(ra, p);  // beside the chunk sums
         VT acc, cmp;
@@ -699,7 +720,7 @@ __global__ void __launch_bounds__(kCombineThreads, 3) k_combine(RowArgs ra, RunA
 // leave the kernel to the group with the most lookups: each group claims
 // `grab` run segments at a time, its first ones by its index, the rest from a
 // counter; one at a time when they are few, so that every run starts at once.
-template <int V, bool SEG, int ROWS>
+template <int V, bool SEG, int ROWS, bool NEW>
 __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_short(RowArgs ra, RunArgs a) {
     pdl_enter();
     if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_short, (unsigned long long)a.n + 1)) return;
@@ -710,6 +731,7 @@ __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_
     const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
     const uint32_t grab = N >= ngroups * (uint32_t)MLKV_SHORT_GRAB ? (uint32_t)MLKV_SHORT_GRAB : 1u;
     auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
+    const uint32_t from = NEW ? first_new(a) : NONE;
     uint32_t base = group * grab;
     while (base < N) {  // uniform within the group
         const uint32_t end = min(N, base + grab);
@@ -718,6 +740,7 @@ __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_
             const uint4 m = next;  // (start, end, row, first lookup)
             if (v + 1 < end) next = __ldg(a.runs + run_of(v + 1));
             const int j = glane + G * (int)(v - run_of(v) * nseg);
+            if (NEW) make_new<V>(ra, a, m.z, from, j);
             short_run<V, ROWS>(ra, a, m.x, m.y, m.z, m.w, j, G, glane, gmask);
         }
         uint32_t c = 0;
@@ -728,7 +751,7 @@ __global__ void __launch_bounds__(256, ROWS >= 8 ? MLKV_SHORT_MIN_BLOCKS : 3) k_
 }
 
 // Runs of 2 .. kSmallRun lookups, records loaded one run ahead.
-template <int V, bool SEG>
+template <int V, bool SEG, bool NEW>
 __global__ void __launch_bounds__(256, MLKV_SMALL_MIN_BLOCKS) k_small(RowArgs ra, RunArgs a) {
     pdl_enter();
     if (MLKV_CHECK && !in_bounds(a.err, kChkListEntry, a.cur->n_small, (unsigned long long)a.n + 1)) return;
@@ -737,6 +760,10 @@ __global__ void __launch_bounds__(256, MLKV_SMALL_MIN_BLOCKS) k_small(RowArgs ra
     const uint32_t group = (blockIdx.x * blockDim.x + threadIdx.x) >> ra.gshift;
     const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
     auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
+    const uint32_t from = NEW ? first_new(a) : NONE;
+    if (NEW && from != NONE)
+        for (uint32_t v = group; v < N; v += ngroups)
+            make_new<V>(ra, a, __ldg(a.smalls + run_of(v)).x, from, glane + G * (int)(v - run_of(v) * nseg));
     uint4 next = group < N ? __ldg(a.smalls + run_of(group)) : make_uint4(0u, 0u, 0u, 0u);
     uint32_t next3 = group < N ? __ldg(a.small_p3 + run_of(group)) : NONE;
     for (uint32_t v = group; v < N; v += ngroups) {  // uniform within the group
@@ -755,7 +782,7 @@ __global__ void __launch_bounds__(256, MLKV_SMALL_MIN_BLOCKS) k_small(RowArgs ra
 // loaded together, SG runs at a time, records loaded one round ahead.  With no
 // loop over positions it needs few registers, so many warps (and rows) are in
 // flight.
-template <int V, bool SEG, int SG>
+template <int V, bool SEG, int SG, bool NEW>
 __global__ void __launch_bounds__(256, SG == 1 ? MLKV_SINGLE_MIN_BLOCKS : 4) k_single(RowArgs ra, RunArgs a) {
     pdl_enter();
     using VT = typename Vec<V>::T;
@@ -766,6 +793,11 @@ __global__ void __launch_bounds__(256, SG == 1 ? MLKV_SINGLE_MIN_BLOCKS : 4) k_s
     const uint32_t ngroups = (gridDim.x * blockDim.x) >> ra.gshift;
     const uint2 none = make_uint2(0xFFFFFFFFu, 0u);
     auto run_of = [&](uint32_t v) { return SEG ? v / nseg : v; };
+    const uint32_t from = NEW ? first_new(a) : NONE;
+    if (NEW && from != NONE)
+        for (uint32_t x = group * SG; x < N; x += ngroups * SG)
+            for (uint32_t v = x; v < min(x + SG, N); ++v)
+                make_new<V>(ra, a, __ldg(a.singles + run_of(v)).x, from, glane + G * (int)(v - run_of(v) * nseg));
     uint2 next[SG];
 #pragma unroll
     for (int i = 0; i < SG; ++i) next[i] = group * SG + i < N ? __ldg(a.singles + run_of(group * SG + i)) : none;
@@ -812,6 +844,7 @@ __global__ void __launch_bounds__(256, SG == 1 ? MLKV_SINGLE_MIN_BLOCKS : 4) k_s
 #define MLKV_FUSED_MAX (1 << 15)
 #endif
 constexpr uint32_t kFusedMax = MLKV_FUSED_MAX;
+static_assert(kPlanMax <= kFusedMax, "a plan's narrow rows go to k_reduce, which makes new ones (run_kernels)");
 
 // --- calls of few lookups: one kernel ------------------------------------------
 
@@ -827,8 +860,8 @@ constexpr int kTreeLevels = 30 / kFanShift + 1;  // more chunks than any batch h
 // the node's entries up and goes on to the next level; at the root the sum is
 // rounded once and the row updated.  No group waits for another.
 template <int V>
-__device__ __forceinline__ void long_chunk(const RowArgs& ra, const RunArgs& a, uint32_t it, uint32_t seg, int G,
-                                           int glane, unsigned gmask) {
+__device__ __forceinline__ void long_chunk(const RowArgs& ra, const RunArgs& a, uint32_t it, uint32_t seg, uint32_t from,
+                                           int G, int glane, unsigned gmask) {
     using VT = typename Vec<V>::T;
     const uint4 rec = __ldg(a.items + it);
     const uint32_t m = rec.y >> kItemLenBits, ib = rec.w;
@@ -857,7 +890,9 @@ __device__ __forceinline__ void long_chunk(const RowArgs& ra, const RunArgs& a, 
         count = (count + kFan - 1) >> kFanShift;
         stride <<= kFanShift;
     }
-    if (act) finish_long<V>(ra, a, rec.z, j, acc, cmp);
+    if (!act) return;
+    make_new<V>(ra, a, rec.z, from, j);
+    finish_long<V>(ra, a, rec.z, j, acc, cmp);
 }
 
 // k_reduce's units of runs: [0, us) of 5 .. 32 lookups, [us, um) of 2 ..
@@ -866,6 +901,7 @@ struct Units {
     uint32_t NS, NM, NC, N1;  // run segments of each kind (NC: those of one lookup in coarse units)
     uint32_t ls, lm, lc, lf;
     uint32_t us, um, uc, units;
+    uint32_t new_from;  // first row that holds nothing yet, or NONE
 };
 
 __device__ __forceinline__ Units make_units(const RunArgs& a, uint32_t R, uint32_t nwarps, uint32_t nseg) {
@@ -908,7 +944,7 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
     pdl_enter();
     using VT = typename Vec<V>::T;
     const uint32_t nseg = ra.nseg;
-    const uint32_t NI = min(a.cur->n_items, a.max_items);
+    const uint32_t NI = min(a.cur->n_items, a.max_items), from = first_new(a);
     // a list never holds more runs than lookups
     if (MLKV_CHECK && !(in_bounds(a.err, kChkListEntry, a.cur->n_short, (unsigned long long)a.n + 1) &&
                         in_bounds(a.err, kChkListEntry, a.cur->n_small, (unsigned long long)a.n + 1) &&
@@ -924,14 +960,25 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
     __shared__ Units q;
     if (threadIdx.x == 0) {
         q = make_units(a, R, nwarps, nseg);
+        q.new_from = from;
         if (blockIdx.x == 0)
             ds->last_unique = a.cur->n_single + a.cur->n_small + a.cur->n_short + a.cur->n_long;  // one run per row
     }
     for (uint32_t v = warp * R + gid; v < NI * nseg; v += nwarps * R) {
         const uint32_t it = nseg == 1 ? v : v / nseg;
-        long_chunk<V>(ra, a, it, v - it * nseg, G, glane, gmask);
+        long_chunk<V>(ra, a, it, v - it * nseg, from, G, glane, gmask);
     }
     __syncthreads();
+    // the new rows among a unit's cnt (row, segment) pairs, one a lane; a lane writes the vectors it loads next
+    auto new_rows = [&](uint32_t mrow, uint32_t mseg, uint32_t cnt) {
+        if (!__any_sync(0xffffffffu, mrow >= q.new_from)) return;
+        for (uint32_t k = 0; k < cnt; k += R) {
+            const int src = (int)min(k + gid, cnt - 1);
+            const uint32_t row = __shfl_sync(0xffffffffu, mrow, src);
+            const int j = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
+            if (k + gid < cnt) make_new<V>(ra, a, row, q.new_from, j);
+        }
+    };
     // first units from the other end: the warps that had a chunk get one last (4
     // of the 14 us of 4,096 lookups went by with both on the same warps)
     uint32_t u = nwarps - 1 - warp;
@@ -944,6 +991,7 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
             const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
             const uint4 mrec = __ldg(a.runs + mrun);  // (start, end, row, first lookup)
             const uint32_t mseg = mine - mrun * nseg;
+            new_rows(mrec.z, mseg, cnt);
             for (uint32_t k = 0; k < cnt; k += R) {
                 const int src = (int)min(k + gid, cnt - 1);
                 const uint32_t s = __shfl_sync(0xffffffffu, mrec.x, src), e = __shfl_sync(0xffffffffu, mrec.y, src);
@@ -959,6 +1007,7 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
             const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
             const uint4 mrec = __ldg(a.smalls + mrun);  // (row, p0, p1, p2)
             const uint32_t mp3 = __ldg(a.small_p3 + mrun), mseg = mine - mrun * nseg;
+            new_rows(mrec.x, mseg, cnt);
             for (uint32_t k = 0; k < cnt; k += R) {
                 const int src = (int)min(k + gid, cnt - 1);
                 const uint4 m = make_uint4(__shfl_sync(0xffffffffu, mrec.x, src), __shfl_sync(0xffffffffu, mrec.y, src),
@@ -977,6 +1026,7 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
             const uint32_t mrun = nseg == 1 ? mine : mine / nseg;
             const uint2 mrec = __ldg(a.singles + mrun);  // (row, lookup)
             const uint32_t mseg = mine - mrun * nseg;
+            new_rows(mrec.x, mseg, cnt);
             for (uint32_t k = 0; k < cnt; k += R * SG) {
                 VT w[SG], Gs[SG], g[SG];
                 uint32_t row[SG];
@@ -1021,18 +1071,32 @@ using RunKernel = void (*)(RowArgs, RunArgs);
 // gradient rows in flight at 3 blocks per SM (more warps).
 struct RunKernels {
     RunKernel longs, shorts, smalls, singles;
+    void (*combine)(RowArgs, RunArgs, DevState*);
 };
 
+// new_rows (make_new): after a plan, whose narrow rows' runs (seg not set) all go
+// to k_reduce.  Kernels of their own, since k_short's 8-byte vectors would pay for
+// the comparison with 7 registers and a block per SM (1.3M lookups of dim 50,
+// Zipf(1.1): 282 -> 292 us).
 template <int V>
-RunKernels run_kernels(bool seg, bool narrow) {
-    if (seg) return {k_long<V, true>, k_short<V, true, MLKV_SHORT_ROWS>, k_small<V, true>, k_single<V, true, 1>};
-    if (narrow) return {k_long<V, false>, k_short<V, false, 4>, k_small<V, false>, k_single<V, false, 2>};
-    return {k_long<V, false>, k_short<V, false, MLKV_SHORT_ROWS>, k_small<V, false>, k_single<V, false, 1>};
+RunKernels run_kernels(bool seg, bool narrow, bool new_rows) {
+    constexpr int R = MLKV_SHORT_ROWS;
+    if (seg && new_rows)
+        return {k_long<V, true>, k_short<V, true, R, true>, k_small<V, true, true>, k_single<V, true, 1, true>,
+                k_combine<V, true>};
+    if (seg)
+        return {k_long<V, true>, k_short<V, true, R, false>, k_small<V, true, false>, k_single<V, true, 1, false>,
+                k_combine<V, false>};
+    if (narrow)
+        return {k_long<V, false>, k_short<V, false, 4, false>, k_small<V, false, false>, k_single<V, false, 2, false>,
+                k_combine<V, false>};
+    return {k_long<V, false>, k_short<V, false, R, false>, k_small<V, false, false>, k_single<V, false, 1, false>,
+            k_combine<V, false>};
 }
 
 template <int V>
 cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n, cudaStream_t st,
-                       CallCounters* cur) {
+                       CallCounters* cur, bool new_rows) {
     const uint32_t nseg = (uint32_t)((t->geom.NV + t->geom.G - 1) / t->geom.G);
     RowArgs ra{t->slots, t->geom.stride, t->geom.dpad, t->geom.NV, t->geom.G, __builtin_ctz((unsigned)t->geom.G),
                t->geom.d, nseg,
@@ -1067,7 +1131,7 @@ cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* spos, 
         s2 = t->branch[1];
     }
     const bool narrow = t->geom.G <= 16;
-    const RunKernels k = run_kernels<V>(nseg > 1, narrow);
+    const RunKernels k = run_kernels<V>(nseg > 1, narrow, new_rows);
     const int gl = persistent_blocks(t, (const void*)k.longs, 256);
     const int g2 = persistent_blocks(t, (const void*)k.smalls, 256);
     const int gs = persistent_blocks(t, (const void*)k.shorts, 256);
@@ -1082,7 +1146,7 @@ cudaError_t run_reduce(mlkv_table* t, const float* grads, const uint32_t* spos, 
     last.release = branches ? (uint32_t)(gc + g1 + (short_first ? g2 : gs)) : (uint32_t)g1;
     const RunArgs& tail = branches ? last : a;
     MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_LONG, k.longs, gl, 256, 0, s2, ra, a);
-    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_LONG_COMBINE, (k_combine<V>), gc, kCombineThreads, 0, s2, ra, tail, t->dstate);
+    MLKV_LAUNCH_PERSISTENT(t, MLKV_K_LONG_COMBINE, k.combine, gc, kCombineThreads, 0, s2, ra, tail, t->dstate);
     if (short_first) {
         MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SHORT, k.shorts, gs, 256, 0, s1, ra, a);
         MLKV_LAUNCH_PERSISTENT(t, MLKV_K_REDUCE_SMALL, k.smalls, g2, 256, 0, s1, ra, tail);
@@ -1134,10 +1198,10 @@ cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* sp
 }
 
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
-                                cudaStream_t st, CallCounters* cur) {
-    if (t->geom.V == 4) return run_reduce<4>(t, grads, spos, n, st, cur);
-    if (t->geom.V == 2) return run_reduce<2>(t, grads, spos, n, st, cur);
-    return run_reduce<1>(t, grads, spos, n, st, cur);
+                                cudaStream_t st, CallCounters* cur, bool new_rows) {
+    if (t->geom.V == 4) return run_reduce<4>(t, grads, spos, n, st, cur, new_rows);
+    if (t->geom.V == 2) return run_reduce<2>(t, grads, spos, n, st, cur, new_rows);
+    return run_reduce<1>(t, grads, spos, n, st, cur, new_rows);
 }
 
 }  // namespace mlkv

@@ -60,6 +60,7 @@ constexpr int64_t kMaxStaleness = MLKV_MAX_STALENESS;  // largest bound kept bel
 struct CallCounters {
     uint32_t n_miss;     // lookups whose key had no row yet
     uint32_t n_new;      // distinct new keys (first occurrences)
+    uint32_t new_base;   // 1 + row of the first of them, where the miss path left their rows to the reduce; else 0
     uint32_t n_long;     // runs longer than MLKV_SEQ_SEGMENT_MAX
     uint32_t n_items;    // chunks of the long runs
     uint32_t n_group;    // long runs combined by a lane group
@@ -111,6 +112,7 @@ struct Scratch {
     uint32_t* sort_offsets; // [tiles][512] output position of each tile's first element of each digit
     uint32_t* sort_dtot;    // [kSortMaxPasses][512] digit totals of each pass, zero between sorts
     uint32_t* tile_sums;    // [scan tiles + 1] per-tile sums of the dedup's scan
+    int64_t* new_keys;      // [min(max_batch, kPlanMax)] keys of the rows a plan handed out, in row order
     uint32_t* miss_sums;    // [max_miss_blocks] new keys of every block of the miss path
     uint4* short_runs;      // [max_batch] the apply's runs of 2 .. MLKV_SEQ_SEGMENT_MAX lookups
     uint2* single_runs;     // [max_batch] its runs of one lookup: (row, lookup position)
@@ -428,6 +430,16 @@ template <> struct Vec<1> {
     static __device__ __forceinline__ T from(const float* e) { return e[0]; }
 };
 
+// Vector j of a key's init row.
+template <int V>
+__device__ __forceinline__ typename Vec<V>::T init_vec(unsigned long long seed, unsigned long long key, int j, float lo,
+                                                       float span) {
+    float e[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) e[c] = init_element(seed, key, (uint32_t)(j * V + c), lo, span);
+    return Vec<V>::from(e);
+}
+
 // Programmatic dependent launch.  MLKV_LAUNCH lets a kernel start while the
 // kernel before it on the stream drains, which hides the launch and ramp-up
 // of the ~25 kernels of a step.  Every kernel begins with pdl_enter():
@@ -585,7 +597,8 @@ int plan_prepare(int device);  // the largest cluster the plan kernels can run a
 bool plan_fits(const mlkv_table* t, int64_t n);
 // Probe (insert: absent keys get rows; rows: they are in row_of_pos already),
 // sort and run lists of an apply of n lookups (plan_fits); spos: the sorted
-// positions.  The call's first kernel.
+// positions.  The call's first kernel.  The rows of new keys hold nothing yet:
+// the reduce kernels write their init values first (RunArgs::new_rows).
 cudaError_t launch_plan(mlkv_table* t, const int64_t* keys, int64_t n, bool insert, bool memo, bool rows,
                         cudaStream_t st, CallCounters* cur, CallCounters* nxt, const uint32_t** spos);
 
@@ -603,8 +616,9 @@ int64_t node_counters(int64_t max_items, int dim);  // counters of the combine's
 // The run lists of sorted rows; and the reduce of the listed runs.
 cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,
                          cudaStream_t st, CallCounters* cur, const SortTail& tail);
+// new_rows: the runs' rows may be ones that a plan gave new keys.
 cudaError_t launch_reduce_apply(mlkv_table* t, const float* grads, const uint32_t* spos, int64_t n,
-                                cudaStream_t st, CallCounters* cur);
+                                cudaStream_t st, CallCounters* cur, bool new_rows);
 
 // Lookups per warp of the kernels that copy a warp's rows one after another: 16
 // of dims above 64 and 32 of narrower ones, or as few as fill the GPU

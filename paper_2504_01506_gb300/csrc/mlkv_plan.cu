@@ -508,7 +508,8 @@ cudaError_t launch_plan(mlkv_table* t, const int64_t* keys, int64_t n, bool inse
     *spos = pa.spos = t->s.sv[0];
     const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);
     const RunArgs a = run_args(t, nullptr, nullptr, *spos, n, sent, cur);
-    const MissArgs ma = miss_args(t, keys, n, MissMode::Init, t->s.row_of_pos, nullptr, cur);
+    MissArgs ma = miss_args(t, keys, n, MissMode::Init, t->s.row_of_pos, nullptr, cur);
+    ma.new_keys = t->s.new_keys;
     auto go = [&](auto v) {
         constexpr int V = decltype(v)::value;
         if (items == 1) return run_plan<V, 1>(t, blocks, ma, pa, a, st);

@@ -152,7 +152,8 @@ inline IndexArgs index_args(mlkv_table* t) {
 //   2. rank the flags: an exclusive scan over the call's positions, every block
 //      over a range of them of its own;
 //   3. each first occurrence takes row = rows handed out so far + rank and
-//      writes its init row (not for Put) and state_init;
+//      writes its init row (not for Put) and state_init (or, with new_keys, its
+//      key alone: the apply's plan, whose few SMs would be long about the rows);
 //   4. every missed lookup reads its key's row (a Get gathers it into its
 //      output), flags and the slot's aux go back to idle, the row counter
 //      advances.
@@ -178,6 +179,7 @@ struct MissArgs {
     DevState* ds;
     unsigned long long capacity;
     int init_row;
+    int64_t* new_keys;  // or null
     unsigned long long seed;
     float lo, span, state_init;
 };
@@ -186,7 +188,7 @@ inline MissArgs miss_args(mlkv_table* t, const int64_t* keys, int64_t n, MissMod
                           float* out, CallCounters* cur) {
     return MissArgs{keys, (uint32_t)n, t->s.miss_pos, t->s.miss_slot, t->s.first_flag, t->s.rank, t->s.miss_sums,
                     (uint32_t)t->s.max_miss_blocks, row_of_pos, out, cur, t->dstate, (unsigned long long)t->cfg.capacity,
-                    mode == MissMode::Put ? 0 : 1, (unsigned long long)t->cfg.seed, t->cfg.init_lo,
+                    mode == MissMode::Put ? 0 : 1, nullptr, (unsigned long long)t->cfg.seed, t->cfg.init_lo,
                     t->cfg.init_hi - t->cfg.init_lo, t->cfg.state_init};
 }
 
@@ -309,10 +311,14 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
             if (ld_u32_relaxed(&ia.index[s].aux) == p) {
                 const unsigned long long r = next + __ldcg(ma.rank + p);
                 key = (unsigned long long)ma.keys[p];
-                if (r < ma.capacity) ia.index[s].row = row = (uint32_t)r;
-                else record_error(ia.err, MLKV_ERR_FULL);
+                if (r >= ma.capacity) record_error(ia.err, MLKV_ERR_FULL);
+                else {
+                    ia.index[s].row = row = (uint32_t)r;
+                    if (ma.new_keys) ma.new_keys[r - next] = (int64_t)key;
+                }
             }
         }
+        if (ma.new_keys) return;
         for (uint32_t q = 0; q < at_once; q += R) {
             const uint32_t r = __shfl_sync(0xffffffffu, row, (int)q + gid);
             const unsigned long long key_q = __shfl_sync(0xffffffffu, key, (int)q + gid);
@@ -321,13 +327,7 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
             VT* wv = reinterpret_cast<VT*>(w);
             VT* gv = reinterpret_cast<VT*>(w + ra.dpad);
             for (int j = glane; j < ra.NV; j += G) {
-                if (ma.init_row) {
-                    float e[V];
-#pragma unroll
-                    for (int c = 0; c < V; ++c) e[c] = init_element(ma.seed, key_q, (uint32_t)(j * V + c), ma.lo,
-                                                                          ma.span);
-                    wv[j] = Vec<V>::from(e);
-                }
+                if (ma.init_row) wv[j] = init_vec<V>(ma.seed, key_q, j, ma.lo, ma.span);
                 gv[j] = Vec<V>::splat(ma.state_init);
             }
         }
@@ -337,6 +337,7 @@ __device__ __forceinline__ bool miss_path(const IndexArgs& ia, const IndexRows& 
     if (sh.block == 0 && threadIdx.x == 0) {
         const unsigned long long nr = next + __ldcg(&ma.cur->n_new);
         ma.ds->next_row = nr < ma.capacity ? nr : ma.capacity;
+        if (ma.new_keys) ma.cur->new_base = (uint32_t)next + 1u;
     }
     for_misses<THREADS>(m, sh.nblocks, sh.block, R, [&](uint32_t i, uint32_t at_once) {
         uint32_t p = 0, row = ROW_PENDING;  // lanes without an entry copy nothing

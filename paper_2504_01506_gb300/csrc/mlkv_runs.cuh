@@ -61,6 +61,11 @@ struct RunArgs {
     uint32_t chunk;        // lookups per chunk of a long run (kChunkLarge or kChunkSmall)
     ErrSink err;
     float lr, eps;
+    struct {               // what the new rows of a plan's apply start with (make_new)
+        const int64_t* keys;  // [new rows] their keys
+        unsigned long long seed;
+        float lo, span, state_init;
+    } new_rows;
     uint32_t release;      // non-zero in the apply's last kernels: the blocks of all of them (release_counters)
 };
 
@@ -70,7 +75,9 @@ inline RunArgs run_args(mlkv_table* t, const float* grads, const uint32_t* srow,
                    t->s.small_p3, t->s.long_runs, t->s.nodes, t->s.items, t->s.partial, t->s.node_cnt,
                    (uint32_t)t->s.max_long, (uint32_t)t->s.max_nodes, (uint32_t)t->s.max_items,
                    n >= kSmallBatch ? kChunkLarge : kChunkSmall,
-                   ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}, t->cfg.lr, t->cfg.eps, 0u};
+                   ErrSink{&t->dstate->status, t->status_dev_alias, t->dstate->chk}, t->cfg.lr, t->cfg.eps,
+                   {t->s.new_keys, (unsigned long long)t->cfg.seed, t->cfg.init_lo, t->cfg.init_hi - t->cfg.init_lo,
+                    t->cfg.state_init}, 0u};
 }
 
 // What the long runs qs[k] .. qe[k] (k < nq) add to the lists: chunks, runs

@@ -586,7 +586,7 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.first_flag, B * 4},     {(void**)&s.rank, B * 4},
         {(void**)&s.sk[0], B * 4},          {(void**)&s.sk[1], B * 4},
         {(void**)&s.sv[0], B * 4},          {(void**)&s.sv[1], B * 4},
-        {(void**)&s.tile_sums, (tiles_of(B) + 1) * 4}, {(void**)&s.miss_sums, s.max_miss_blocks * 4},
+        {(void**)&s.tile_sums, (tiles_of(B) + 1) * 4},
         {(void**)&s.sort_counts[0], s.sort_counts_bytes = 512 * sort_tiles * 4},
         {(void**)&s.sort_counts[1], s.sort_counts_bytes},
         {(void**)&s.sort_counts[2], s.sort_counts_bytes},
@@ -599,6 +599,9 @@ int mlkv_open(const mlkv_config* cfg, mlkv_table** out) {
         {(void**)&s.small_runs, B * 16},
         {(void**)&s.small_p3, B * 4},
         {(void**)&s.partial, s.max_items * 2 * t->geom.dpad * 4},
+        // (last: where the sort's arrays lie moves a large apply's time by up to 4%)
+        {(void**)&s.miss_sums, s.max_miss_blocks * 4},
+        {(void**)&s.new_keys, std::min<int64_t>(B, kPlanMax) * 8},
     };
     int64_t total = 0;
     for (auto& p : pieces) total += round_up(p.bytes, 256);
@@ -739,10 +742,12 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
     const MemoUse memo = t->stale ? MemoUse::None : MemoUse::Read;
     const uint32_t *srow, *spos;
     cudaError_t err = cudaSuccess;
+    bool new_rows = false;
     // (an injected wait exists in the miss kernel alone: the plan's blocks meet at
     // the cluster's barrier)
     if (!t->tiered && plan_fits(t, n) && !wait_injection_armed()) {
         err = launch_plan(t, d_keys, n, ins, memo == MemoUse::Read, false, st, cs.cur, cs.nxt, &spos);
+        new_rows = ins;
     } else {
         // On an HBM-resident table the probe also counts the sort's first pass (the
         // tiered apply sorts cache lines, known only after the probe).
@@ -766,7 +771,7 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
             if (err == cudaSuccess) err = launch_heads(t, srow, spos, n, sent, st, cs.cur, tail);
         }
     }
-    if (err == cudaSuccess) err = launch_reduce_apply(t, d_grads, spos, n, st, cs.cur);
+    if (err == cudaSuccess) err = launch_reduce_apply(t, d_grads, spos, n, st, cs.cur, new_rows);
     t->sort_bits = t->bits_rows;
     if (err != cudaSuccess) return cuda_error(t, err, "apply_grad launches");
     return MLKV_OK;

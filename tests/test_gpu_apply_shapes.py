@@ -241,3 +241,49 @@ def test_get_whose_new_keys_are_in_few_blocks(n, dim):
         _check_table(store, ref, keys, "after the Get")
     assert store.sync() == 0
     store.close()
+
+
+@pytest.mark.parametrize("dim", [1, 6, 50, 64, 128, 132, 512])
+@pytest.mark.parametrize("n", [700, 8192, 32_768])
+def test_apply_gives_new_keys_rows_before_it_reduces_them(n, dim):
+    """Applies whose keys are new (all of them, or some) in runs of every length,
+    through the one-cluster plan: each row starts from its init values and state,
+    whichever kernel (by n and dim) and run length reduces it; the next apply
+    finds none new; and a full table gives the first keys rows and skips the rest."""
+    torch_cuda()
+    lens = [n // 3, 9 * 16 + 1, 33, 32, 20, 5, 4, 4, 3, 2, 2]  # 16 lookups a chunk of a long run
+    opts = dict(max_batch=n, lr=0.125, eps=1e-8, state_init=0.25)
+    store, ref = make_pair(_cfg(dim), capacity=3 * n, **opts)
+    rng = np.random.default_rng(n + dim)
+    fresh = (1 << 41) + rng.permutation(6 * n).astype(np.int64)
+    used = 0
+    known = np.zeros(0, np.int64)
+    for share in (1.0, 0.0, 0.2):
+        runs = fresh[used:used + len(lens)]
+        ones = fresh[used + len(lens):used + n]
+        used += n
+        keys = np.concatenate([np.repeat(runs, lens), ones])[:n]
+        if share < 1:
+            at = rng.permutation(n)[: int(n * (1 - share))]
+            keys = rng.permutation(keys)
+            keys[at] = known[rng.integers(0, len(known), len(at))]
+        keys = rng.permutation(keys)
+        grads = _grads(rng, n, dim)
+        store.apply_grad(dev(keys), dev(grads))
+        ref.apply_grad(keys, grads)
+        assert store.size() == ref.size() and store.last_unique() == len(np.unique(keys))
+        _check_table(store, ref, keys, f"{share:.1f} of the lookups new")
+        known = np.unique(np.concatenate([known, keys]))
+    assert store.sync() == 0
+    store.close()
+    room = n // 2 + 3
+    store, ref = make_pair(_cfg(dim), capacity=room, **opts)
+    keys = fresh[used:used + n]
+    grads = _grads(rng, n, dim)
+    store.apply_grad(dev(keys), dev(grads))
+    assert store.sync() == 5  # MLKV_ERR_FULL
+    store.clear_status()
+    ref.apply_grad(keys[:room], grads[:room])
+    assert store.size() == ref.size() == room
+    _check_table(store, ref, keys[:room], "a table filled by an apply")
+    store.close()
