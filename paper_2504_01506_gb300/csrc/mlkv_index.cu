@@ -12,6 +12,8 @@
 // atomicMin; the lookup whose position survives is the first occurrence; an
 // exclusive scan over first-occurrence flags gives each new key its rank, and
 // row = rows handed out so far + rank.
+#include <algorithm>
+
 #include "mlkv_probe.cuh"
 
 namespace mlkv {
@@ -336,7 +338,8 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
 // slot that already holds a later position is only read: the first round marks
 // the hot keys, the others find them marked.  kMarkPerSm = 2 blocks of 256
 // threads per SM: more make the first round's burst longer, fewer leave too few
-// reads in flight.
+// reads in flight.  The lanes are matched by 32-bit rows (64-bit values: 1.3M Puts
+// of uniform keys of dim 4 118 us instead of 109; one atomic per lookup: 107).
 #ifndef MLKV_MARK_PER_SM
 #define MLKV_MARK_PER_SM 2
 #endif
@@ -356,9 +359,8 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
         row = j < n ? __ldg(row_of_pos + (n - 1 - j)) : ROW_ABSENT;
         slot = j < n ? __ldg(slot_of_pos + (n - 1 - j)) : 0u;
         const bool has = r < ROW_ABSENT;
-        const unsigned long long who = has ? (unsigned long long)s : ~0ull;
-        const unsigned peers = __match_any_sync(0xffffffffu, who);
-        // the lowest lane of a slot holds its last position
+        // lanes of one slot are those of one row; the lowest holds its last position
+        const unsigned peers = __match_any_sync(0xffffffffu, r);
         if (has && lane == __ffs(peers) - 1 && mark < ld_u32_relaxed(&index[s].aux)) atomicMin(&index[s].aux, mark);
     }
 }
@@ -369,9 +371,13 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
 // in flight.  (With a lane group walking its lookups one by one, each copy
 // waited for its own mark: 75 us for 524k Puts of 1 KiB, Zipf(0.99); 70 so, 88
 // with 2 vectors in flight.)
-// KV vectors a lane (row_vectors) of ROWS rows are in flight.
+// KV vectors a lane (row_vectors) of ROWS rows are in flight, and a warp takes at
+// least that many rows: with 1 or 2 a warp, 50,000 Puts of dim 64 took 27 us, 21
+// so (a lane group per lookup in a loop: 20).  6 blocks per SM: 40 registers; the
+// 48 to 53 taken without leave fewer warps (300,000 of dim 64: 52 us, 49 so), 32
+// spill (59).
 template <int V, int KV, int ROWS>
-__global__ void __launch_bounds__(256) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
+__global__ void __launch_bounds__(256, 6) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
                                                      const uint32_t* __restrict__ row_of_pos,
                                                      const uint32_t* __restrict__ slot_of_pos,
                                                      const float* __restrict__ vals,
@@ -616,7 +622,8 @@ struct PutRun {
     static cudaError_t run(mlkv_table* t, const float* vals, const float* state, int64_t n, cudaStream_t st) {
         MLKV_LAUNCH(t, 0, k_put_mark, capped_grid(t, n, 256, kMarkPerSm), 256, 0, st, t->index, t->s.row_of_pos,
                     t->s.slot_of_pos, (uint32_t)n);
-        const int lpw = lookups_per_warp(t, n, 32 / t->geom.G), kv = row_vectors<V>(t->geom);
+        const int kv = row_vectors<V>(t->geom), rows = kv == 1 ? 4 : 2;  // in flight a lane group
+        const int lpw = lookups_per_warp(t, n, std::min(32, rows * (32 / t->geom.G)));
         const auto kernel = kv == 1 ? k_put_scatter<V, 1, 4> : kv == 2 ? k_put_scatter<V, 2, 2>
                                                                        : k_put_scatter<V, kMostVectors<V>, 2>;
         MLKV_LAUNCH(t, MLKV_K_PUT_SCATTER, kernel, grid_for(n, 8 * lpw), 256, 0, st, t->index, row_args(t),
