@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256, 2 * kGetBlocksPerSm) k_get_small(IndexArg
 }
 
 // The Get with its rows moved by the SM's asynchronous copies, for calls of
-// fewer than kBulkMaxBatch lookups (rows of at most kBulkRowBytes, 16-byte
+// fewer than bulk_lookups lookups (rows of at most kBulkRowBytes, 16-byte
 // aligned buffers).  Each warp probes kBulkRows consecutive lookups as k_get
 // does, then copies their rows into its shared-memory stage with cp.async (16
 // bytes a lane, L2 only; no registers hold rows in flight, so all of them are
@@ -207,18 +207,23 @@ __global__ void __launch_bounds__(256, 2 * kGetBlocksPerSm) k_get_small(IndexArg
 // the output rows are contiguous.  The store runs on while the warp probes its
 // next lookups; the stage is reused once the store has read it.  Rows of new
 // keys are left to the miss path, which writes their output rows after this
-// kernel.  Measured against k_get (Gets of dim 128, 8M rows): faster where a
-// call is too small to fill the GPU with k_get's warps (20,000 lookups 10.3 us
-// against 12.5, 60,000 15.4 against 16.7, 100,000 22.0 against 24.1), slower
-// above (140,000 28.2 against 27.3, 500,000 88 against 80), where k_get's 64
-// warps a SM beat the few warps the stages leave room for.
+// kernel.  Faster where a call is too small to fill the GPU with k_get's warps,
+// slower above, where k_get's 64 warps a SM beat the few warps the stages leave
+// room for; rows of few bytes leave little to copy at once.  (us of a Get of keys
+// drawn uniformly from 4M rows, k_get / with this kernel; bulk_lookups lies where
+// the two cross:
+//   dim      60,000   131,000   250,000   420,000 lookups
+//     4    11.7/11.3  13.4/15.2  17.0/21.0  24.1/28.6
+//    16    10.7/10.9  14.9/15.4  21.4/21.9  28.5/31.3
+//    64    16.0/12.6  21.7/18.7  35.5/32.1  48.4/51.9
+//    96    18.0/14.9  29.5/25.0  48.5/44.1  69.1/70.6
+//   128    19.0/17.2  32.4/30.5  53.9/54.3  80.1/87.5)
 #ifndef MLKV_GET_BULK
 #define MLKV_GET_BULK 1
 #endif
-#ifndef MLKV_GET_BULK_MAX_BATCH
-#define MLKV_GET_BULK_MAX_BATCH (1u << 17)
-#endif
-constexpr uint32_t kBulkMaxBatch = MLKV_GET_BULK_MAX_BATCH;
+inline int64_t bulk_lookups(uint32_t rowbytes) {
+    return rowbytes <= 64 ? 1 << 16 : rowbytes < 128 || rowbytes > 384 ? 200'000 : 400'000;
+}
 constexpr int kBulkThreads = 128;  // 4 warps
 constexpr uint32_t kBulkRowBytes = 512;
 #ifndef MLKV_GET_BULK_ROWS
@@ -578,7 +583,7 @@ struct GetRun {
                         Memo{t->s.memo_key, t->s.memo_row}, small_lpw, take_injected_wait() ? 1u : 0u);
             return cudaGetLastError();
         }
-        if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && (uint64_t)n < kBulkMaxBatch) {
+        if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && n < bulk_lookups(rowbytes)) {
             const size_t smem = (size_t)4 * kBulkRows * rowbytes + 4 * 32 * 4;
             if (t->cfg.insert_on_miss)
                 MLKV_LAUNCH(t, MLKV_K_GET_GATHER, k_get_bulk<true>, bulk_grid<true>(t, smem, n), kBulkThreads, smem,

@@ -287,3 +287,28 @@ def test_apply_gives_new_keys_rows_before_it_reduces_them(n, dim):
     assert store.size() == ref.size() == room
     _check_table(store, ref, keys[:room], "a table filled by an apply")
     store.close()
+
+
+@pytest.mark.parametrize("dim,edge", [(16, 1 << 16), (20, 200_000), (32, 400_000), (96, 400_000), (100, 200_000)])
+@pytest.mark.parametrize("insert", [True, False])
+def test_get_at_the_edge_of_the_asynchronous_copies(dim, edge, insert):
+    """One lookup fewer and as many as where a Get leaves the kernel that moves
+    rows by asynchronous copies, known keys beside new (or absent) ones."""
+    torch_cuda()
+    store, ref = make_pair(_cfg(dim), capacity=30_000, max_batch=edge, insert_on_miss=insert)
+    rng = np.random.default_rng(dim)
+    universe = rng.choice(1 << 40, 29_000, replace=False).astype(np.int64)
+    store.insert(dev(universe[:20_000]))
+    ref.insert(universe[:20_000])
+    for n, known in ((edge - 1, 25_000), (edge, 29_000)):
+        keys = universe[rng.integers(0, known, n)]
+        want, _, _ = ref.get(keys)
+        got = host(store.get(dev(keys)))
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        assert_bits(np.nan_to_num(got), np.nan_to_num(want), f"Get of {n}")
+        if not insert:
+            assert store.sync() == 7  # MLKV_ERR_NOT_FOUND
+            store.clear_status()
+        assert store.size() == ref.size()
+    assert store.sync() == 0
+    store.close()
