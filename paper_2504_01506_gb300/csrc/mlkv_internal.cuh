@@ -458,8 +458,8 @@ __device__ __forceinline__ typename Vec<V>::T init_vec(unsigned long long seed, 
 // to four on one, and finds new keys' rows there on a fraction of the GPU.
 // (Inserts of new keys alone, early -> late: 100,000 of dim 64 73 -> 72 us,
 // 500,000 of dim 128 262 -> 263, a million 1,348 -> 500; of dim 512 4,271 -> 1,259;
-// a Get of a million new keys of dim 128 1,203 -> 833.  Calls without new keys
-// take as long as before within 0.3 us.)
+// a Get of a million new keys of dim 128 1,203 -> 833.  A call without new keys
+// pays 0.1 to 0.8 us for it.)
 #ifndef MLKV_PDL_TRIGGER_FIRST
 #define MLKV_PDL_TRIGGER_FIRST 0
 #endif

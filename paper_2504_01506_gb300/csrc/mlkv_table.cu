@@ -644,6 +644,17 @@ int tier_map(mlkv_table* t, uint32_t epoch, int strict, int64_t n, cudaStream_t 
     return MLKV_OK;
 }
 
+// Whether an apply issued beside a look-ahead takes the one-cluster plan: its
+// blocks need whole SMs, up to 16 of one GPU processing cluster at once, and wait
+// for them where the fetch's blocks sit; the general kernels fit beside those.
+// The line is where the fetch of about n rows gets longer than the plan saves.
+// (us of Get + look-ahead + apply, an eighth of the keys cold, with the plan /
+// the general kernels: dim 16 8,192 lookups 50/56, 16,384 59/59, 32,768 81/65;
+// dim 128 2,048 lookups 44/48, 4,096 74/66, 32,768 177/151.)
+bool plan_beside_fetch(const mlkv_table* t, int64_t n) {
+    return n <= 1 << 14 && n * t->geom.stride * (int64_t)sizeof(float) <= 2 << 20;
+}
+
 }  // namespace
 
 extern "C" {
@@ -762,7 +773,7 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
             if ((rc = tier_map(t, e, beside ? 1 : 0, n, st))) return rc;
             t->sort_bits = t->bits_lines;
         }
-        if (t->tiered && plan_fits(t, n)) {
+        if (t->tiered && plan_fits(t, n) && (!beside || plan_beside_fetch(t, n))) {
             err = launch_plan(t, d_keys, n, false, false, true, st, cs.cur, nullptr, &spos);
         } else {
             const uint32_t sent = (uint32_t)((1ull << t->sort_bits) - 1);  // the sort's key of a lookup without a row

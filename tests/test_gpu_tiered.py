@@ -142,3 +142,34 @@ def test_open_rejects_small_cache():
     with pytest.raises(MLKVError) as e:
         EmbeddingStore(dim=8, capacity=10_000, max_batch=1_000, hbm_cache_rows=1_500)
     assert e.value.code == 1
+
+
+@pytest.mark.parametrize("dim,n", [(16, 16_384), (16, 16_385), (128, 2_048), (128, 2_049), (4, 300)])
+def test_apply_beside_a_lookahead_on_either_plan(dim, n):
+    """On both sides of where an apply issued beside a look-ahead leaves the
+    one-cluster plan for the general kernels."""
+    torch = torch_cuda()
+    cfg = W.tiny()
+    cfg.dim, cfg.n_keys, cfg.batch = dim, 120_000, n
+    tiered, resident = _stores(cfg, 4 * n + 64)
+    rng = np.random.default_rng(n)
+    universe = rng.choice(1 << 40, cfg.n_keys, replace=False).astype(np.int64)
+    _insert(tiered, universe)
+    _insert(resident, universe)
+    batches = [np.where(rng.random(n) < 0.5, universe[rng.integers(0, 50, n)], universe[rng.integers(0, 120_000, n)])
+               for _ in range(7)]
+    grads = (rng.integers(-8, 9, size=(n, dim)) * 2.0**-10).astype(np.float32)  # exact sums
+    for step in range(6):
+        kd, g = dev(batches[step]), dev(grads)
+        assert_bits(host(tiered.get(kd)), host(resident.get(kd)), f"Get step {step}")
+        tiered.lookahead(dev(batches[step + 1]))
+        tiered.apply_grad(kd, g)
+        resident.apply_grad(kd, g)
+        assert tiered.last_unique() == resident.last_unique()
+    torch.cuda.synchronize()
+    assert tiered.sync() == 0 and resident.sync() == 0
+    touched = np.unique(np.concatenate(batches[:6]))
+    for got, want in zip(_export(tiered, touched), _export(resident, touched)):
+        assert_bits(got, want, "rows and state")
+    tiered.close()
+    resident.close()
