@@ -36,11 +36,12 @@ __global__ void __launch_bounds__(CT ? CT : 256) k_probe(IndexArgs ia, const int
                                                uint32_t* __restrict__ slot_of_pos,
                                                uint32_t* miss_pos, uint32_t* miss_slot,
                                                CallCounters* cur, CallCounters* nxt,
-                                               int report_absent, Memo memo, int memo_use, FirstCounts fc) {
+                                               int report_absent, Memo memo, int memo_use, FirstCounts fc,
+                                               int late_miss) {
     constexpr bool COUNT = CT > 0;
     static_assert(!COUNT || kProbeKeys * CT == kSortTile || kProbeKeys * CT == kSortTileSmall,
                   "a counting block covers one sort tile");
-    if (INSERT) pdl_enter_last();  // the miss kernel is next
+    if (INSERT && late_miss) pdl_enter_last();
     else pdl_enter();
     zero_counters(nxt);
     __shared__ uint32_t hist[COUNT ? kSortMaxRadix : 1];
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : M
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
                                              CallCounters* nxt, Memo memo, int lpw) {
-    if (INSERT) pdl_enter_last();  // the miss kernel is next
+    if (INSERT && wide_rows(ra.NV)) pdl_enter_last();
     else pdl_enter();
     zero_counters(nxt);
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
@@ -253,8 +254,7 @@ __global__ void __launch_bounds__(kBulkThreads) k_get_bulk(IndexArgs ia, IndexRo
                                                            uint32_t n, float* __restrict__ out, uint32_t* miss_pos,
                                                            uint32_t* miss_slot, CallCounters* cur, CallCounters* nxt,
                                                            Memo memo) {
-    if (INSERT) pdl_enter_last();  // the miss kernel is next
-    else pdl_enter();
+    pdl_enter();
     zero_counters(nxt);
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kWarps = kBulkThreads / 32;
@@ -674,28 +674,28 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
     uint32_t* rows = rows_out ? rows_out : t->s.row_of_pos;
     if (want_slot && memo == MemoUse::Read) memo = MemoUse::None;  // the memo holds no slots
     const Memo m{t->s.memo_key, t->s.memo_row};
-    const int ra = report_absent ? 1 : 0;
+    const int ra = report_absent ? 1 : 0, late = wide_rows(t->geom.NV) ? 1 : 0;
     if (fc) {  // one block per sort tile, counting the first pass
         const unsigned g = grid_for(n, 1 << fc->tile_shift);
         if (fc->tile_shift == 12) {
             if (insert)
                 MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<true, 1024>), g, 1024, 0, st, index_args(t), keys,
                             (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, 0, m,
-                            (int)memo, *fc);
+                            (int)memo, *fc, late);
             else
                 MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<false, 1024>), g, 1024, 0, st, index_args(t), keys,
                             (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, ra, m,
-                            (int)memo, *fc);
+                            (int)memo, *fc, late);
         } else {  // the small tiles: kSortTileSmall / kProbeKeys threads
             constexpr int CT = kSortTileSmall / kProbeKeys;
             if (insert)
                 MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<true, CT>), g, CT, 0, st, index_args(t), keys,
                             (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, 0, m,
-                            (int)memo, *fc);
+                            (int)memo, *fc, late);
             else
                 MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<false, CT>), g, CT, 0, st, index_args(t), keys,
                             (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, ra, m,
-                            (int)memo, *fc);
+                            (int)memo, *fc, late);
         }
         return cudaGetLastError();
     }
@@ -703,10 +703,10 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
     const unsigned g = grid_for(n, 256 * kProbeKeys);
     if (insert)
         MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<true, 0>), g, 256, 0, st, index_args(t), keys,
-                    (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, 0, m, (int)memo, none);
+                    (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, 0, m, (int)memo, none, late);
     else
         MLKV_LAUNCH(t, MLKV_K_PROBE, (k_probe<false, 0>), g, 256, 0, st, index_args(t), keys,
-                    (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, ra, m, (int)memo, none);
+                    (uint32_t)n, rows, slot_of_pos, t->s.miss_pos, t->s.miss_slot, cur, nxt, ra, m, (int)memo, none, late);
     return cudaGetLastError();
 }
 

@@ -453,13 +453,14 @@ __device__ __forceinline__ typename Vec<V>::T init_vec(unsigned long long seed, 
 //     they in turn wait for this grid.  Issued after the wait, it keeps at
 //     most one grid waiting ahead of the running one.
 // pdl_enter_last leaves the second out (the next kernel's blocks are then placed
-// when this grid's are done): for the kernels before the miss kernel, whose one
-// block per SM, placed early, piles up on the few SMs that have room first, up
-// to four on one, and finds new keys' rows there on a fraction of the GPU.
-// (Inserts of new keys alone, early -> late: 100,000 of dim 64 73 -> 72 us,
-// 500,000 of dim 128 262 -> 263, a million 1,348 -> 500; of dim 512 4,271 -> 1,259;
-// a Get of a million new keys of dim 128 1,203 -> 833.  A call without new keys
-// pays 0.1 to 0.8 us for it.)
+// when this grid's are done): for the kernels before the miss kernel where rows
+// are wide (wide_rows).  Its one block per SM, placed early, piles up on the few
+// SMs that have room first, up to four on one, and writes and copies new keys'
+// rows there on a fraction of the GPU, which wide rows feel at any size.  (New keys
+// alone, early -> late: a Get of 100,000 of dim 256 279 -> 177 us, of dim 512 483
+// -> 282, an insert of a million of dim 512 3,268 -> 1,229.  Without new keys a
+// call pays 0.3 to 0.8 us; for narrow rows that is not worth it: 100,000 of dim 64
+// insert in 65 us either way.)
 #ifndef MLKV_PDL_TRIGGER_FIRST
 #define MLKV_PDL_TRIGGER_FIRST 0
 #endif
@@ -468,6 +469,7 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!MLKV_PDL_TRIGGER_FIRST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+__host__ __device__ __forceinline__ bool wide_rows(int NV) { return NV > 32; }  // more vectors than lanes
 __device__ __forceinline__ void pdl_enter_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
