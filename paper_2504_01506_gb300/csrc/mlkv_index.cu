@@ -339,12 +339,13 @@ __global__ void __launch_bounds__(kMissThreads) k_miss(IndexArgs ia, IndexRows r
 // occurrences of (0xFFFFFFFE - p).  Atomics on one slot queue (about 2.7 ns
 // each): with one per lookup, a Zipf(0.99) batch of 524k Puts, 6% of them of
 // one key, took 89 us.  So the positions are walked from the last to the first
-// by a grid of few warps, a warp's lanes of one slot send one atomic, and a
-// slot that already holds a later position is only read: the first round marks
-// the hot keys, the others find them marked.  kMarkPerSm = 2 blocks of 256
+// by a grid of few warps, and a slot that already holds a later position is only
+// read: the first round, in which a warp's lanes of one slot send one atomic,
+// marks the hot keys, the others find them marked.  kMarkPerSm = 2 blocks of 256
 // threads per SM: more make the first round's burst longer, fewer leave too few
-// reads in flight.  The lanes are matched by 32-bit rows (64-bit values: 1.3M Puts
-// of uniform keys of dim 4 118 us instead of 109; one atomic per lookup: 107).
+// reads in flight.  Matching the lanes in every round cost 1.3M Puts of uniform
+// keys of dim 4 118 us instead of 109 (one atomic per lookup, as without hot keys:
+// 108), and Zipf(0.99) ones 67 instead of 61.
 #ifndef MLKV_MARK_PER_SM
 #define MLKV_MARK_PER_SM 2
 #endif
@@ -363,10 +364,12 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
         const uint32_t j = i + nthreads;
         row = j < n ? __ldg(row_of_pos + (n - 1 - j)) : ROW_ABSENT;
         slot = j < n ? __ldg(slot_of_pos + (n - 1 - j)) : 0u;
-        const bool has = r < ROW_ABSENT;
-        // lanes of one slot are those of one row; the lowest holds its last position
-        const unsigned peers = __match_any_sync(0xffffffffu, r);
-        if (has && lane == __ffs(peers) - 1 && mark < ld_u32_relaxed(&index[s].aux)) atomicMin(&index[s].aux, mark);
+        bool lead = r < ROW_ABSENT;
+        if (i - lane < nthreads) {  // the first round: the lowest lane of a slot holds its last position
+            const unsigned peers = __match_any_sync(0xffffffffu, lead ? (unsigned long long)s : ~0ull);
+            lead = lead && lane == __ffs(peers) - 1;
+        }
+        if (lead && mark < ld_u32_relaxed(&index[s].aux)) atomicMin(&index[s].aux, mark);
     }
 }
 
@@ -378,11 +381,11 @@ __global__ void __launch_bounds__(256) k_put_mark(Slot* __restrict__ index, cons
 // with 2 vectors in flight.)
 // KV vectors a lane (row_vectors) of ROWS rows are in flight, and a warp takes at
 // least that many rows: with 1 or 2 a warp, 50,000 Puts of dim 64 took 27 us, 21
-// so (a lane group per lookup in a loop: 20).  6 blocks per SM: 40 registers; the
-// 48 to 53 taken without leave fewer warps (300,000 of dim 64: 52 us, 49 so), 32
-// spill (59).
+// so (a lane group per lookup in a loop: 20).  6 blocks per SM with one vector a
+// lane: 40 registers; the 53 taken without leave fewer warps (300,000 of dim 64:
+// 52 us, 49 so), 32 spill (59); 5 with more, where 40 spill.
 template <int V, int KV, int ROWS>
-__global__ void __launch_bounds__(256, 6) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
+__global__ void __launch_bounds__(256, KV == 1 ? 6 : 5) k_put_scatter(Slot* __restrict__ index, IndexRows ra,
                                                      const uint32_t* __restrict__ row_of_pos,
                                                      const uint32_t* __restrict__ slot_of_pos,
                                                      const float* __restrict__ vals,
