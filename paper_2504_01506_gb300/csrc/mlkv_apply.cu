@@ -849,7 +849,16 @@ static_assert(kPlanMax <= kFusedMax, "a plan's narrow rows go to k_reduce, which
 // --- calls of few lookups: one kernel ------------------------------------------
 
 constexpr uint32_t kFanShift = 5, kFan = 1u << kFanShift;  // fan-in of the combine tree
-constexpr int kTreeLevels = 30 / kFanShift + 1;  // more chunks than any batch holds
+// ... its levels, and the counters of one level above the lowest: run segments'
+// chunks (of kChunkSmall lookups, one more a run) in a call of kFusedMax segments.
+constexpr int tree_levels() {
+    int levels = 1;
+    for (uint32_t m = kFusedMax / kChunkSmall + 1; m > kFan; m = (m + kFan - 1) / kFan) ++levels;
+    return levels;
+}
+constexpr int kMostSegs = 8;  // dim 256 in 4-byte vectors, dim 1,024 in 16-byte ones
+constexpr uint32_t kTreeEntries = kFusedMax / kChunkSmall + kFusedMax / (MLKV_SEQ_SEGMENT_MAX + 1) + 2 * kMostSegs;
+static_assert(MLKV_MAX_DIM <= kMostSegs * 128, "segments of the widest row");
 #ifndef MLKV_SINGLES
 #define MLKV_SINGLES 1
 #endif
@@ -878,7 +887,9 @@ __device__ __forceinline__ void long_chunk(const RowArgs& ra, const RunArgs& a, 
         __syncwarp(gmask);
         uint32_t arrived = 0;
         if (glane == 0) {
-            uint32_t* ctr = a.node_cnt + ((size_t)level * a.max_items + ib + first * stride) * ra.nseg + seg;
+            const uint32_t at = (ib + first * stride) * ra.nseg + seg;
+            uint32_t* ctr = a.node_cnt + at;
+            if (level) ctr += (size_t)a.max_items * ra.nseg + (size_t)(level - 1) * kTreeEntries;
             arrived = atomicAdd(ctr, 1u);
             if (arrived == width - 1) *ctr = 0u;  // zero again for the next call
         }
@@ -1181,7 +1192,7 @@ void long_bounds(int64_t max_batch, int64_t& runs, int64_t& nodes, int64_t& item
 int64_t node_counters(int64_t max_items, int dim) {
     // segments per row of the widest split: the scalar kernels' (dim <= 256) or the float4 kernels'
     const int64_t nseg = std::max<int64_t>((std::min(dim, 256) + 31) / 32, (dim + 127) / 128);
-    return kTreeLevels * max_items * nseg;
+    return max_items * nseg + (tree_levels() - 1) * (int64_t)kTreeEntries;
 }
 
 cudaError_t launch_heads(mlkv_table* t, const uint32_t* srow, const uint32_t* spos, int64_t n, uint32_t sent,

@@ -53,8 +53,9 @@ struct RunArgs {
     uint4* items;          // [max_items] chunks of the long runs: (first sorted position, lookups |
                            //   chunks of the run << kItemLenBits, row, the run's first chunk)
     float* partial;        // [max_items][2][dpad] sums of chunks, and of nodes in their first chunk's place
-    uint32_t* node_cnt;    // [levels][max_items][nseg] nodes of a run done (k_combine: level 0, at the run's first
-                           //   chunk's entry; k_reduce: arrivals at its trees' nodes), zero at rest
+    uint32_t* node_cnt;    // [max_items][nseg] nodes of a run done (k_combine, at the run's first chunk's entry), or
+                           //   arrivals at the lowest nodes of k_reduce's trees; behind them the higher levels',
+                           //   [levels - 1][kTreeEntries]; zero at rest
     uint32_t max_long;
     uint32_t max_nodes;
     uint32_t max_items;

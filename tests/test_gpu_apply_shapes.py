@@ -312,3 +312,23 @@ def test_get_at_the_edge_of_the_asynchronous_copies(dim, edge, insert):
         assert store.size() == ref.size()
     assert store.sync() == 0
     store.close()
+
+
+@pytest.mark.parametrize("n,dim,shift", [(4096, 256, 1), (4096, 1024, 0), (16_384, 256, 0), (32_768, 128, 0)])
+def test_trees_of_the_most_segments(n, dim, shift):
+    """One run of all of the batch's lookups, then runs just past 32, in as many
+    row segments as the one-kernel reduce takes: the combine trees' counters, of
+    every level, and again from what the first apply left."""
+    torch_cuda()
+    store, ref = make_pair(_cfg(dim), capacity=2000, max_batch=n, lr=0.125, eps=1e-8)
+    rng = np.random.default_rng(n + dim)
+    universe = rng.choice(1 << 40, 1990, replace=False).astype(np.int64)
+    store.insert(dev(universe))
+    ref.insert(universe)
+    for keys in (np.full(n, universe[3]), np.resize(np.repeat(universe, 33), n), np.full(n, universe[5])):
+        grads = _grads(rng, n, dim)
+        store.apply_grad(dev(keys), _shifted(grads, shift))
+        ref.apply_grad(keys, grads)
+        _check_table(store, ref, keys, "one apply")
+    assert store.sync() == 0
+    store.close()
