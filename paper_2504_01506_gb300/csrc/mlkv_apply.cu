@@ -859,9 +859,6 @@ constexpr int tree_levels() {
 constexpr int kMostSegs = 8;  // dim 256 in 4-byte vectors, dim 1,024 in 16-byte ones
 constexpr uint32_t kTreeEntries = kFusedMax / kChunkSmall + kFusedMax / (MLKV_SEQ_SEGMENT_MAX + 1) + 2 * kMostSegs;
 static_assert(MLKV_MAX_DIM <= kMostSegs * 128, "segments of the widest row");
-#ifndef MLKV_SINGLES
-#define MLKV_SINGLES 1
-#endif
 
 // One segment of a chunk of a long run, by one lane group.  The chunk sums of a
 // run are combined in a tree of fan-in kFan, always in chunk order: the group
@@ -1029,7 +1026,6 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
                 __syncwarp();
             }
         } else {  // runs of one lookup
-            constexpr int SG = MLKV_SINGLES;
             const bool coarse = u < q.uc;
             const uint32_t v0 = coarse ? (u - q.um) * q.lc : q.NC + (u - q.uc) * q.lf;
             const uint32_t cnt = coarse ? min(q.lc, q.NC - v0) : min(q.lf, q.N1 - v0);
@@ -1038,34 +1034,18 @@ __global__ void __launch_bounds__(256, 2) k_reduce(RowArgs ra, RunArgs a, DevSta
             const uint2 mrec = __ldg(a.singles + mrun);  // (row, lookup)
             const uint32_t mseg = mine - mrun * nseg;
             new_rows(mrec.x, mseg, cnt);
-            for (uint32_t k = 0; k < cnt; k += R * SG) {
-                VT w[SG], Gs[SG], g[SG];
-                uint32_t row[SG];
-                int jj[SG];  // the lane's column, or NV where there is no run
-#pragma unroll
-                for (int i = 0; i < SG; ++i) {
-                    const uint32_t idx = k + i * R + gid;
-                    const int src = (int)min(idx, cnt - 1);
-                    row[i] = __shfl_sync(0xffffffffu, mrec.x, src);
-                    const uint32_t p = __shfl_sync(0xffffffffu, mrec.y, src);
-                    jj[i] = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
-                    if (idx >= cnt) jj[i] = ra.NV;
-                    if (MLKV_CHECK && jj[i] < ra.NV && !(in_bounds(a.err, kChkSingleRow, row[i], ra.nrows) &&
-                                                         in_bounds(a.err, kChkSinglePos, p, a.n)))
-                        jj[i] = ra.NV;
-                    if (jj[i] < ra.NV) {
-                        const VT* src_row = row_vec<V>(ra, row[i], jj[i]);
-                        w[i] = src_row[0];
-                        Gs[i] = *beside(ra, src_row);
-                        g[i] = __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)p * ra.d) + jj[i]);
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < SG; ++i) {
-                    if (jj[i] >= ra.NV) continue;
+            for (uint32_t k = 0; k < cnt; k += R) {
+                const int src = (int)min(k + gid, cnt - 1);
+                const uint32_t row = __shfl_sync(0xffffffffu, mrec.x, src), p = __shfl_sync(0xffffffffu, mrec.y, src);
+                const int j = glane + G * (int)__shfl_sync(0xffffffffu, mseg, src);
+                if (k + gid < cnt && j < ra.NV && in_bounds(a.err, kChkSingleRow, row, ra.nrows) &&
+                    in_bounds(a.err, kChkSinglePos, p, a.n)) {
+                    const VT* src_row = row_vec<V>(ra, row, j);
+                    const VT w = src_row[0], Gs = *beside(ra, src_row);
+                    const VT g = __ldcs(reinterpret_cast<const VT*>(a.grads + (size_t)p * ra.d) + j);
                     VT acc = Vec<V>::zero();
-                    Vec<V>::add(acc, g[i]);  // 0 + g, as in a longer run
-                    adagrad_store<V>(ra, row[i], jj[i], w[i], Gs[i], acc, a.lr, a.eps);
+                    Vec<V>::add(acc, g);  // 0 + g, as in a longer run
+                    adagrad_store<V>(ra, row, j, w, Gs, acc, a.lr, a.eps);
                 }
                 __syncwarp();
             }

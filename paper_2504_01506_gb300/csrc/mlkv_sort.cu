@@ -123,16 +123,15 @@ __device__ __forceinline__ uint32_t digit_peers_by_mask(uint32_t* mask, uint32_t
 // counts the probe did not make.  A thread counts consecutive elements and
 // adds a run of equal digits with one atomic.
 template <int TILE>
-__global__ void __launch_bounds__(TILE >= 1024 ? kThreads : TILE / 4) k_sort_hist(const uint32_t* __restrict__ kin, uint32_t n,
+__global__ void __launch_bounds__(kThreads) k_sort_hist(const uint32_t* __restrict__ kin, uint32_t n,
                                                         uint32_t* __restrict__ counts, uint32_t* __restrict__ dtot,
                                                         uint32_t ntiles, int shift, int radix, uint32_t sent,
                                                         int first, int packed) {
-    constexpr int kHThreads = TILE >= 1024 ? kThreads : TILE / 4;
-    constexpr int kItems = TILE / kHThreads;
+    constexpr int kItems = TILE / kThreads;
     static_assert(kItems % 4 == 0, "whole 16-byte loads");
     pdl_enter();
     __shared__ uint32_t hist[kMaxRadix];
-    for (int d = threadIdx.x; d < radix; d += kHThreads) hist[d] = 0;
+    for (int d = threadIdx.x; d < radix; d += kThreads) hist[d] = 0;
     __syncthreads();
     const uint32_t i0 = blockIdx.x * TILE + threadIdx.x * kItems;
     uint32_t key[kItems];
@@ -375,28 +374,22 @@ __global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k
         rnk[r] = valid ? before + __popc(peers & lt) : 0xFFFFFFFFu;
     }
     __syncthreads();
-    // per digit: exclusive prefix over the warps; per tile: exclusive prefix
-    // over the digits (thread t owns digits t*dpt .. t*dpt+dpt-1, in order)
-    constexpr int kDpt = kMaxRadix > THREADS ? kMaxRadix / THREADS : 1;
-    const int dpt = radix > THREADS ? radix / THREADS : 1;
-    uint32_t tot[kDpt], mine = 0;
-#pragma unroll
-    for (int j = 0; j < kDpt; ++j) {
-        const int d = threadIdx.x * dpt + j;
-        tot[j] = 0;
-        if (j >= dpt || d >= radix) continue;
+    // per digit, a thread each: exclusive prefix over the warps; per tile: exclusive
+    // prefix over the digits
+    static_assert(THREADS >= kMaxRadix, "a thread per digit");
+    const int d = threadIdx.x;
+    uint32_t mine = 0;
+    if (d < radix) {
 #pragma unroll
         for (int ww = 0; ww < kSWarps; ++ww) {
             const uint32_t c = wcnts[ww * kMaxRadix + d];
-            wcnts[ww * kMaxRadix + d] = (Count)tot[j];
-            tot[j] += c;
+            wcnts[ww * kMaxRadix + d] = (Count)mine;
+            mine += c;
         }
-        mine += tot[j];
     }
     uint32_t all;
-    uint32_t run = block_exclusive_scan_n<THREADS>(mine, all);
+    const uint32_t run = block_exclusive_scan_n<THREADS>(mine, all);
     if (SELF) {  // the elements of lower digits, and the digit's in the tiles before
-        const int d = threadIdx.x;
         uint32_t total;
         uint32_t at = block_exclusive_scan_n<THREADS>(d < radix ? __ldg(s.dtot + d) : 0u, total);
         if (d < radix) {
@@ -404,13 +397,7 @@ __global__ void __launch_bounds__(THREADS, SELF ? 2 : MLKV_SCATTER_MIN_BLOCKS) k
             gbase[d] = at;
         }
     }
-#pragma unroll
-    for (int j = 0; j < kDpt; ++j) {
-        const int d = threadIdx.x * dpt + j;
-        if (j >= dpt || d >= radix) continue;
-        lbase[d] = run;
-        run += tot[j];
-    }
+    if (d < radix) lbase[d] = run;
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kSItems; ++r) {
