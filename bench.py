@@ -308,8 +308,8 @@ KERNEL_SOURCES = {1: "mlkv_index.cu", 2: "mlkv_index.cu", 3: "mlkv_sort.cu", 4: 
 
 
 # ncu kernel names (demangled, without the namespace) -> kernel class
-KERNEL_PATTERNS = [("k_get_bulk<", 1), ("k_get<", 1), ("k_probe<", 2), ("k_sort_scatter", 3), ("k_short<", 4),
-                   ("k_long<", 5), ("k_heads", 6), ("k_combine<", 7), ("k_tier_fetch", 8),
+KERNEL_PATTERNS = [("k_get_bulk<", 1), ("k_get_small<", 1), ("k_get<", 1), ("k_probe<", 2), ("k_sort_scatter", 3),
+                   ("k_short<", 4), ("k_long<", 5), ("k_heads", 6), ("k_combine<", 7), ("k_tier_fetch", 8),
                    ("k_put_scatter", 9), ("k_single<", 10), ("k_small<", 11), ("k_reduce<", 12),
                    ("k_plan<", 13)]
 TRAFFIC_PATH = os.path.join(ROOT, "profiles", "traffic.json")

@@ -149,3 +149,11 @@ def test_traffic_record_of_get_put_batches_uses_their_gets(tmp_path):
     want = bench.kernel_bytes(bench.ycsb_stats(read, write, cfg.dim), 1, 1)
     assert out["1"]["algorithmic_bytes_per_launch"] == want
     assert want < bench.kernel_bytes(bench.batch_stats(cfg.batch_keys(1), cfg.dim), 1, 1)
+
+
+def test_every_kernel_of_a_class_is_found_by_its_name():
+    """The names ncu prints, and the class each kernel is timed as: a Get's three kernels among them."""
+    for name, kid in (("k_get<4, 1, 0, 1>", 1), ("k_get_bulk<1>", 1), ("k_get_small<4, 1, 0>", 1), ("k_probe<1, 512>", 2),
+                      ("k_plan<4, 1>", 13), ("k_reduce<4>", 12), ("k_single<4, 0, 1, 0>", 10), ("k_combine<4, 0>", 7),
+                      ("k_miss<4>", None)):
+        assert bench.kernel_id_of(f"void mlkv::(anonymous namespace)::{name}(mlkv::IndexArgs)") == kid, name
