@@ -242,8 +242,9 @@ int mlkv_export(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_rows, 
 /* The dedup step of the gradient apply, exposed for checking: the distinct
  * present keys of d_keys ordered by row id, with their occurrence counts.
  * Absent keys are left out and never inserted.  d_unique_keys: int64 [n];
- * d_counts: int32 [n]; *d_num_unique (device int64) = number of distinct
- * present keys. */
+ * d_counts: int32 [n]; *d_num_unique (int64, in device memory, or for n > 0 in
+ * pinned host memory, which then holds it once the stream has synchronised) =
+ * number of distinct present keys. */
 int mlkv_dedup(mlkv_table* t, const int64_t* d_keys, int64_t n, int64_t* d_unique_keys,
                int32_t* d_counts, int64_t* d_num_unique, void* stream);
 

@@ -28,10 +28,15 @@ class MLKVError(RuntimeError):
         self.code = code
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(device) -> int:
-    """The current torch stream's handle.  (Without building a Stream object: 0.2 us
-    instead of 2.1, of 13 for a Get of 416 lookups.)"""
-    return torch._C._cuda_getCurrentRawStream(device.index)
+    """The current torch stream's handle.  (Without building a Stream object, where
+    this torch has the call: 0.2 us instead of 2.1, of 13 for a Get of 416 lookups.)"""
+    if _raw_stream is None:
+        return torch.cuda.current_stream(device).cuda_stream
+    return _raw_stream(device.index)
 
 
 class EmbeddingStore:

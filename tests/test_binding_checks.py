@@ -56,3 +56,18 @@ def test_host_buffer_calls_check_their_host_tensors():
         s.get_host(torch.arange(3, dtype=torch.int64), torch.zeros(4, 3).t())  # strided output
     with pytest.raises(TypeError):
         s.apply_grad_host(torch.arange(3, dtype=torch.int64), torch.zeros(2, 4))  # one gradient row short
+
+
+def test_stream_handle_without_the_raw_call(monkeypatch):
+    """A torch without the call that gives a stream's handle alone: the Stream object's."""
+    import types
+
+    from paper_2504_01506_gb300 import store
+
+    seen = []
+    monkeypatch.setattr(store, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda d: seen.append(d) or types.SimpleNamespace(cuda_stream=7))
+    device = torch.device("cuda", 1)
+    assert store._stream(device) == 7 and seen == [device]
+    monkeypatch.setattr(store, "_raw_stream", lambda index: 100 + index)
+    assert store._stream(device) == 101
