@@ -464,7 +464,7 @@ bool prepare_items(int& largest) {
 }  // namespace
 
 // A device's answer is kept: the attributes and occupancy queries take 0.1 ms.
-int plan_prepare(int device) {
+int plan_prepare(int device) try {
     static std::mutex mu;
     static std::unordered_map<int, int> known;
     std::lock_guard<std::mutex> lock(mu);
@@ -476,6 +476,8 @@ int plan_prepare(int device) {
         largest = 0;
     }
     return known[device] = largest;
+} catch (...) {  // no memory for the entry, under a C entry: the general kernels
+    return 0;
 }
 
 bool plan_fits(const mlkv_table* t, int64_t n) {

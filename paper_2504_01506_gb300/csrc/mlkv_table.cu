@@ -378,22 +378,19 @@ void timer_after(mlkv_table* t, int kid, cudaStream_t st) {
     tm.n_events++;
 }
 
-int persistent_blocks(mlkv_table* t, const void* kernel, int threads) {
+int persistent_blocks(mlkv_table* t, const void* kernel, int threads) try {
     static std::mutex mu;
     static std::unordered_map<const void*, int> cache;
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(kernel);
-    int per_sm;
-    if (it != cache.end()) {
-        per_sm = it->second;
-    } else {
-        per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        cache[kernel] = per_sm;
-    }
+    if (it != cache.end()) return it->second * t->num_sms;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    cache[kernel] = per_sm;
     return per_sm * t->num_sms;
+} catch (...) {  // no memory for the entry, under a C entry: one block per SM always fits
+    return t->num_sms;
 }
 
 }  // namespace mlkv
