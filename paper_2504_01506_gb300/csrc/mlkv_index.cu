@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256, V * KV >= 8 ? MLKV_GET_SEG_MIN_BLOCKS : M
                                              float* __restrict__ out, uint32_t* miss_pos,
                                              uint32_t* miss_slot, CallCounters* cur,
                                              CallCounters* nxt, Memo memo, int lpw) {
-    if (INSERT && wide_rows(ra.NV)) pdl_enter_last();
+    if (INSERT && late_miss_get(ra.NV, n)) pdl_enter_last();
     else pdl_enter();
     zero_counters(nxt);
     const uint32_t base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)lpw;
@@ -677,7 +677,7 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
     uint32_t* rows = rows_out ? rows_out : t->s.row_of_pos;
     if (want_slot && memo == MemoUse::Read) memo = MemoUse::None;  // the memo holds no slots
     const Memo m{t->s.memo_key, t->s.memo_row};
-    const int ra = report_absent ? 1 : 0, late = wide_rows(t->geom.NV) ? 1 : 0;
+    const int ra = report_absent ? 1 : 0, late = late_miss_probe(t->geom.NV, n) ? 1 : 0;
     if (fc) {  // one block per sort tile, counting the first pass
         const unsigned g = grid_for(n, 1 << fc->tile_shift);
         if (fc->tile_shift == 12) {

@@ -454,13 +454,7 @@ __device__ __forceinline__ typename Vec<V>::T init_vec(unsigned long long seed, 
 //     most one grid waiting ahead of the running one.
 // pdl_enter_last leaves the second out (the next kernel's blocks are then placed
 // when this grid's are done): for the kernels before the miss kernel where rows
-// are wide (wide_rows).  Its one block per SM, placed early, piles up on the few
-// SMs that have room first, up to four on one, and writes and copies new keys'
-// rows there on a fraction of the GPU, which wide rows feel at any size.  (New keys
-// alone, early -> late: a Get of 100,000 of dim 256 279 -> 177 us, of dim 512 483
-// -> 282, an insert of a million of dim 512 3,268 -> 1,229.  Without new keys a
-// call pays 0.3 to 0.8 us; for narrow rows that is not worth it: 100,000 of dim 64
-// insert in 65 us either way.)
+// are wide (late_miss_get, late_miss_probe).
 #ifndef MLKV_PDL_TRIGGER_FIRST
 #define MLKV_PDL_TRIGGER_FIRST 0
 #endif
@@ -469,8 +463,21 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!MLKV_PDL_TRIGGER_FIRST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-__host__ __device__ __forceinline__ bool wide_rows(int NV) { return NV > 32; }  // more vectors than lanes
 __device__ __forceinline__ void pdl_enter_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Whether the miss kernel is placed late behind a Get, or behind a probe, of n
+// lookups of rows of NV vectors.  Its one block per SM, placed early, piles up on
+// the few SMs that have room first, up to four on one, and writes and copies new
+// keys' rows on a fraction of the GPU; placed late it costs a call without new keys
+// 0.3 to 1 us.  The lines lie where the early one falls behind a kernel that needs
+// a whole SM a block.  (us, all keys new, such a kernel / early / late: a Get of
+// 100,000 of dim 256 206/279/177, of 500,000 1,698/1,166/679; of 100,000 of dim 512
+// 306/483/282, of 500,000 1,454/2,182/1,195; an insert of 500,000 of dim 512
+// 1,040/623/623, of a million 2,089/3,268/1,229.)
+__host__ __device__ __forceinline__ bool late_miss_get(int NV, uint32_t n) {
+    return NV > 64 || (NV > 32 && n < 1u << 18);
+}
+inline bool late_miss_probe(int NV, int64_t n) { return NV > 32 && n >= 1 << 19; }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
