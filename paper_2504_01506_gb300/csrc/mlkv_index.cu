@@ -222,6 +222,11 @@ __global__ void __launch_bounds__(256, 2 * kGetBlocksPerSm) k_get_small(IndexArg
 #ifndef MLKV_GET_BULK
 #define MLKV_GET_BULK 1
 #endif
+// Rows that are copied to the host next leave them at this many bytes: the copy
+// takes longer behind the bulk stores.  (us of a Get into host memory, k_get / with
+// this kernel: 100,000 of dim 100 235/248, 180,000 414/440, 180,000 of dim 64
+// 275/282; smaller ones 40,000 of dim 128 132/126, 80,000 of dim 32 82/78.)
+constexpr int64_t kBulkMaxToHost = 24 << 20;
 inline int64_t bulk_lookups(uint32_t rowbytes) {
     return rowbytes <= 64 ? 1 << 16 : rowbytes < 128 || rowbytes > 384 ? 200'000 : 400'000;
 }
@@ -565,7 +570,8 @@ int small_get_lpw(const mlkv_table* t, int64_t n) {
 template <int V>
 struct GetRun {
     static cudaError_t run(mlkv_table* t, const int64_t* keys, int64_t n, float* out,
-                           cudaStream_t st, CallCounters* cur, CallCounters* nxt, bool& resolved) {
+                           cudaStream_t st, CallCounters* cur, CallCounters* nxt, bool to_host,
+                           bool& resolved) {
         const uint32_t rowbytes = (uint32_t)t->geom.d * 4;
         const int kv = row_vectors<V>(t->geom);
         constexpr int M = kMostVectors<V>;
@@ -586,7 +592,8 @@ struct GetRun {
                         Memo{t->s.memo_key, t->s.memo_row}, small_lpw, take_injected_wait() ? 1u : 0u);
             return cudaGetLastError();
         }
-        if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && n < bulk_lookups(rowbytes)) {
+        if (MLKV_GET_BULK && V == 4 && rowbytes <= kBulkRowBytes && n < bulk_lookups(rowbytes) &&
+            !(to_host && n * (int64_t)rowbytes >= kBulkMaxToHost)) {
             const size_t smem = (size_t)4 * kBulkRows * rowbytes + 4 * 32 * 4;
             if (t->cfg.insert_on_miss)
                 MLKV_LAUNCH(t, MLKV_K_GET_GATHER, k_get_bulk<true>, bulk_grid<true>(t, smem, n), kBulkThreads, smem,
@@ -714,8 +721,8 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
 }
 
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,
-                       CallCounters* cur, CallCounters* nxt, bool& resolved) {
-    return dispatch_row<GetRun>(t->geom, t, keys, n, out, st, cur, nxt, resolved);
+                       CallCounters* cur, CallCounters* nxt, bool to_host, bool& resolved) {
+    return dispatch_row<GetRun>(t->geom, t, keys, n, out, st, cur, nxt, to_host, resolved);
 }
 
 cudaError_t launch_resolve_misses(mlkv_table* t, const int64_t* keys, int64_t n, MissMode mode,

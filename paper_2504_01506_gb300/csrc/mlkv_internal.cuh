@@ -565,9 +565,10 @@ cudaError_t launch_probe(mlkv_table* t, const int64_t* keys, int64_t n, bool ins
 #ifndef MLKV_SMALL_GET_MAX
 #define MLKV_SMALL_GET_MAX (1 << 14)
 #endif
-// resolved: whether this one does; else launch_resolve_misses has to follow.
+// to_host: the rows are copied to the host next.  resolved: whether this one
+// does; else launch_resolve_misses has to follow.
 cudaError_t launch_get(mlkv_table* t, const int64_t* keys, int64_t n, float* out, cudaStream_t st,
-                       CallCounters* cur, CallCounters* nxt, bool& resolved);
+                       CallCounters* cur, CallCounters* nxt, bool to_host, bool& resolved);
 // release: the miss kernel is the last of the call to read its counters, and
 // zeroes them when done (release_counters).  fc: the first sort pass's counts
 // the probe made, to which the lookups given rows here are added.

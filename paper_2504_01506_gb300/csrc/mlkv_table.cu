@@ -657,7 +657,7 @@ bool plan_beside_fetch(const mlkv_table* t, int64_t n) {
 
 extern "C" {
 
-int mlkv_get(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_out, void* stream) {
+static int get_rows(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_out, void* stream, bool to_host) {
     MLKV_RANGE("mlkv_get");
     int rc = check_call(t, d_keys, n, d_out, true, stream);
     if (rc) return rc < 0 ? MLKV_OK : rc;
@@ -676,10 +676,14 @@ int mlkv_get(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_out, void
     }
     CallScope cs = begin_call(t, st, true);
     bool resolved = false;
-    CK(t, launch_get(t, d_keys, n, d_out, st, cs.cur, cs.nxt, resolved));
+    CK(t, launch_get(t, d_keys, n, d_out, st, cs.cur, cs.nxt, to_host, resolved));
     if (t->cfg.insert_on_miss && !resolved)
         CK(t, launch_resolve_misses(t, d_keys, n, MissMode::Get, d_out, st, cs.cur, true));
     return MLKV_OK;
+}
+
+int mlkv_get(mlkv_table* t, const int64_t* d_keys, int64_t n, float* d_out, void* stream) {
+    return get_rows(t, d_keys, n, d_out, stream, false);
 }
 
 int mlkv_insert(mlkv_table* t, const int64_t* d_keys, int64_t n, void* stream) {
@@ -882,7 +886,7 @@ int mlkv_get_host(mlkv_table* t, const int64_t* h_keys, int64_t n, float* h_out,
     if ((rc = ensure_staging(t, false, set))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     CK(t, copy_async(t->stage_keys[set], h_keys, (size_t)n * 8, cudaMemcpyHostToDevice, st));
-    if ((rc = mlkv_get(t, t->stage_keys[set], n, t->stage_vals[set], stream))) return rc;
+    if ((rc = get_rows(t, t->stage_keys[set], n, t->stage_vals[set], stream, true))) return rc;
     CK(t, copy_async(h_out, t->stage_vals[set], (size_t)n * t->cfg.dim * 4, cudaMemcpyDeviceToHost, st));
     return MLKV_OK;
 }

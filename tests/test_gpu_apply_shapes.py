@@ -332,3 +332,22 @@ def test_trees_of_the_most_segments(n, dim, shift):
         _check_table(store, ref, keys, "one apply")
     assert store.sync() == 0
     store.close()
+
+
+@pytest.mark.parametrize("n", [62_914, 62_915])
+def test_get_into_host_memory_at_the_edge_of_the_asynchronous_copies(n):
+    """One row fewer and as many bytes as where a Get whose rows go to host memory leaves them."""
+    torch = torch_cuda()
+    store, ref = make_pair(_cfg(100), capacity=30_000, max_batch=n)
+    rng = np.random.default_rng(n)
+    universe = rng.choice(1 << 40, 29_000, replace=False).astype(np.int64)
+    store.insert(dev(universe[:20_000]))
+    ref.insert(universe[:20_000])
+    keys = universe[rng.integers(0, 29_000, n)]
+    out = torch.empty((n, 100), dtype=torch.float32).pin_memory()
+    store.get_host(torch.from_numpy(keys).pin_memory(), out)
+    assert store.sync() == 0
+    torch.cuda.synchronize()
+    want, _, _ = ref.get(keys)
+    assert_bits(out.numpy(), want, "Get into host memory")
+    store.close()
