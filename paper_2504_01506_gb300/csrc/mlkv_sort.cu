@@ -95,7 +95,8 @@ __device__ __forceinline__ uint32_t sort_key(uint32_t r, uint32_t sent, bool fir
 constexpr int kMaxRadix = kSortMaxRadix;
 
 // Lanes of the warp whose (valid, digit) equals this lane's: one ballot per
-// digit bit.
+// digit bit (the warp-level multisplit of Ashkiani, Davidson, Meyer and Owens,
+// "GPU Multisplit", 2016).
 __device__ __forceinline__ uint32_t digit_peers(uint32_t dig, bool valid, int bits) {
     const uint32_t vm = __ballot_sync(0xffffffffu, valid);
     uint32_t peers = valid ? vm : ~vm;

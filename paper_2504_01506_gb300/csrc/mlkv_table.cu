@@ -756,8 +756,8 @@ int mlkv_apply_grad(mlkv_table* t, const int64_t* d_keys, int64_t n, const float
     const uint32_t *srow, *spos;
     cudaError_t err = cudaSuccess;
     bool new_rows = false;
-    // (an injected wait exists in the miss kernel alone: the plan's blocks meet at
-    // the cluster's barrier)
+    // (the plan has no wait that can run out, its blocks meet at the cluster's
+    // barrier: an armed injection goes to the general kernels' miss kernel)
     if (!t->tiered && plan_fits(t, n) && !wait_injection_armed()) {
         err = launch_plan(t, d_keys, n, ins, memo == MemoUse::Read, false, st, cs.cur, cs.nxt, &spos);
         new_rows = ins;
