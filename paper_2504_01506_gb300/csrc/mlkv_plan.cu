@@ -21,6 +21,12 @@
 // 16,384 61 -> 48, 32,768 70 -> 62.  At 65,536 (4 lookups a thread) the 16 SMs
 // take as long as the general kernels take on all of them (dim 16: 77 -> 75,
 // dim 512: 156 -> 161), so kPlanMax = 32,768.
+//
+// A block takes an SM's whole register file (1,024 threads of 64 registers), and
+// all blocks start at once: beside a grid that keeps its blocks on many SMs for
+// long (another stream's) the plan waits until enough SMs of one processing
+// cluster are free, where the general kernels would run in what room there is.  An
+// apply beside the table's own look-ahead avoids that (plan_beside_fetch).
 #include <cooperative_groups.h>
 
 #include <mutex>
