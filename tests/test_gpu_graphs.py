@@ -146,3 +146,38 @@ def test_direct_calls_after_replays(last):
     assert_bits(G, pG, "state vs direct calls only")
     assert_bits(w, rw, "rows vs oracle")
     assert_bits(G, rG, "state vs oracle")
+
+
+@pytest.mark.parametrize("dim,n", [(16, 3_000), (512, 12_000)])  # all runs in one kernel, a kernel per run length
+def test_replayed_apply_gives_new_keys_rows(dim, n):
+    """A captured apply whose keys are new at its first replay and known at the
+    others; the keys are changed in place before the last, to new ones again."""
+    torch = torch_cuda()
+    cfg = W.tiny()
+    cfg.dim = dim
+    store, ref = make_pair(cfg, capacity=2 * n, max_batch=n, lr=0.125, eps=1e-8, state_init=0.25)
+    rng = np.random.default_rng(n)
+    first, second = ((1 << 41) * (i + 1) + rng.integers(0, n // 2, n) ** 2 // n for i in range(2))
+    grads = (rng.integers(-8, 9, size=(n, dim)) * 2.0**-10).astype(np.float32)  # exact sums
+    kd, gd = dev(first), dev(grads)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(graph, stream=s):
+            store.apply_grad(kd, gd)
+    torch.cuda.synchronize()
+    for keys in (first, first, second, second):
+        kd.copy_(torch.from_numpy(keys))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        ref.apply_grad(keys, grads)
+        u = np.unique(keys)
+        w, G = store.export(dev(u))
+        rw, rG = ref.export(u)
+        assert_bits(host(w), rw, "rows")
+        assert_bits(host(G), rG, "state")
+        assert store.size() == ref.size()
+    assert store.sync() == 0
+    store.close()
